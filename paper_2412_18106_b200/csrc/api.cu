@@ -541,9 +541,12 @@ int xy_attn_append_kv(xy_attn_ctx* ctx, const void* qkv, int64_t qkv_token_strid
       page_stride % 8 != 0 || page_stride < 1 || num_pages < 1 || block_table_stride < 1)
     return set_err(ctx, XY_ERR_INVALID_ARG, "bad K/V pool strides, num_pages or block_table_stride");
   XY_CUDA(ctx, cudaSetDevice(cfg.device));
+  // Only the caller's requests: the virtual requests of shared-prefix groups behind them own no new
+  // tokens and no block-table row, and their start positions are out of order.
+  const int num_reqs = static_cast<int>(p.q_start.size()) - 1;
   XY_CUDA(ctx, launch_append_kv(static_cast<const uint16_t*>(qkv), qkv_token_stride, static_cast<uint16_t*>(k_pool),
                                 static_cast<uint16_t*>(v_pool), page_stride, head_stride, token_stride, block_table,
-                                block_table_stride, ctx->d_reqs, static_cast<int>(p.reqs.size()),
+                                block_table_stride, ctx->d_reqs, num_reqs,
                                 static_cast<int>(p.total_q), cfg.num_q_heads, cfg.num_kv_heads, cfg.page_size,
                                 ctx->page_shift, static_cast<cudaStream_t>(stream)));
   return XY_OK;
@@ -644,7 +647,7 @@ int xy_attn_debug_gather(xy_attn_ctx* ctx, int32_t req, int32_t kv_head, const v
   if (ctx->host_only) return set_err(ctx, XY_ERR_UNSUPPORTED, "host-only context cannot run");
   if (ctx->cfg.kv_dtype != XY_KV_BF16) return set_err(ctx, XY_ERR_UNSUPPORTED, "gather serves bf16 caches only");
   if (!ctx->planned) return set_err(ctx, XY_ERR_NOT_PLANNED, "gather before plan");
-  if (req < 0 || req >= static_cast<int32_t>(ctx->plan.reqs.size()) || kv_head < 0 ||
+  if (req < 0 || req >= static_cast<int32_t>(ctx->plan.q_start.size()) - 1 || kv_head < 0 ||
       kv_head >= ctx->cfg.num_kv_heads || !k_pool || !v_pool || !block_table || !out_k || !out_v)
     return set_err(ctx, XY_ERR_INVALID_ARG, "bad gather argument");
   const ReqInfo& r = ctx->plan.reqs[req];

@@ -40,3 +40,18 @@ def test_append_kv_bit_exact_then_attention(page):
     with pytest.raises(xb.XYAttnError) as e:
         ctx2.append_kv(qkv_dev, d.k_pool, d.v_pool, d.block_table)
     assert e.value.code == xb.XY_ERR_NOT_PLANNED
+
+
+def test_append_kv_under_a_shared_prefix_plan():
+    """The virtual requests of the groups stand behind the caller's in the Token-Table; the append
+    must not take one of them for the owner of a token."""
+    b, groups = W.shared_prefix_decode(seed=5, num_groups=2, members=9, prefix=256, suffix_hi=70, hq=8, hkv=2)
+    t = W.make_tensors(b, fused_qkv=True)
+    d = H.DeviceBatch(b, t)
+    ctx = H.make_ctx(b)
+    ctx.plan_batch(b, groups=groups)
+    ctx.append_kv(t.qkv.cuda(), d.k_pool, d.v_pool, d.block_table)
+    torch.cuda.synchronize()
+    oracle.append_kv(b, t.qkv, t.k_pool, t.v_pool)
+    assert torch.equal(d.k_pool.cpu().view(torch.int16), t.k_pool.view(torch.int16))
+    assert torch.equal(d.v_pool.cpu().view(torch.int16), t.v_pool.view(torch.int16))
