@@ -6,7 +6,7 @@
 //   warp  8     producer (one lane): takes the next task, looks page ids up in the block table and
 //               stages 128-key K and V tiles (one TMA box per page and 64-element half) into a
 //               ring of four shared-memory stages; it runs ahead across task boundaries
-//   warps 9-10  tcgen05 issuers (one lane each), one per 128-row sub-tile of a dense task
+//   warp  9     tcgen05 issuer for both 128-row sub-tiles of a dense task
 // Shared-memory tiles use the 128-byte TMA swizzle: element (row, d) of a tile lives at
 //   (d / 64) * 16 KiB + row * 128 B + (((d % 64) / 8) ^ (row % 8)) * 16 B + (d % 8) * 2 B,
 // which both ldmatrix and the tcgen05 shared-memory descriptors read without bank conflicts.
@@ -53,7 +53,7 @@ constexpr float kLn2 = 0.6931471805599453f;
 struct __align__(8) SmemBarriers {
   uint64_t full[kStages];
   uint64_t empty[kStages];      // released by the eight consumer warps (warp-level MMA paths)
-  uint64_t empty_umma[kStages];  // released by two tcgen05.commit arrivals (tensor-memory path)
+  uint64_t empty_umma[kStages];  // released by a tcgen05.commit of the issuer (tensor-memory path)
 };
 
 constexpr int kSmemQ = 2 * kTileBytes;
@@ -699,9 +699,8 @@ struct __align__(8) UmmaBarriers {
   uint64_t s_full[2];  // MMA -> consumers: S = Q K^T of the next KV tile is in TMEM
   uint64_t p_full[2][2];  // consumers -> MMA: [sub-tile][half] 64 keys of P are in TMEM (O rescaled if need be)
   uint64_t o_done[2];  // MMA -> consumers: the task's last P V has completed
-  uint64_t drained[2];  // every MMA an issuer has issued has completed (waited for once, before exit)
+  uint64_t drained;  // every MMA the issuer has issued has completed (waited for once, before exit)
   uint32_t tmem_base;
-  volatile uint32_t turn;  // index of the next MMA group allowed onto the tensor pipe
 };
 
 static_assert(kStatusWaitLimit == kStatusWaitLimitWord, "one word, two names");
@@ -726,7 +725,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   float* qmult = reinterpret_cast<float*>(gen_base + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers) + 128 + 256);
   float* scale_ring = qmult + 128;  // [kScaleSlots][16]: K scales [0..7], V scales [8..15] of a tile's pages
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     unsigned long long now;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
@@ -734,12 +733,11 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&bars->full[s]), 1);
       mbar_init(smem_u32(&bars->empty[s]), kConsumerWarps);
-      mbar_init(smem_u32(&bars->empty_umma[s]), 2);
+      mbar_init(smem_u32(&bars->empty_umma[s]), 1);
     }
-    ub->turn = 0;
     for (int i = 0; i < kTaskRing; ++i) {
       mbar_init(smem_u32(&tq->full[i]), 1);
-      mbar_init(smem_u32(&tq->empty[i]), kConsumerWarps + (kUmma ? 2 : 0));
+      mbar_init(smem_u32(&tq->empty[i]), kConsumerWarps + (kUmma ? 1 : 0));
     }
     for (int X = 0; X < 2; ++X) {
       mbar_init(smem_u32(&ub->q_full[X]), 4);
@@ -747,8 +745,8 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       mbar_init(smem_u32(&ub->p_full[X][0]), 4);
       mbar_init(smem_u32(&ub->p_full[X][1]), 4);
       mbar_init(smem_u32(&ub->o_done[X]), 1);
-      mbar_init(smem_u32(&ub->drained[X]), 1);
     }
+    mbar_init(smem_u32(&ub->drained), 1);
     fence_mbar_init();
   }
   if (kUmma && warp == kConsumerWarps + 1) {
@@ -758,7 +756,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = kUmma ? ub->tmem_base : 0u;
+  const uint32_t tmem = kUmma ? __shfl_sync(0xffffffffu, ub->tmem_base, 0) : 0u;
 
   const int t_begin = a.worker_off[blockIdx.x], t_end = a.worker_off[blockIdx.x + 1];
   const bool dynamic = a.dynamic != 0;
@@ -988,17 +986,23 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // readers have long consumed it; a bounded wait after a failure).
       for (int s = 0; s < kStages; ++s)
         if (used & (1u << s)) mbar_wait_block(smem_u32(&bars->full[s]), (fill_par >> s) & 1u, a.status);
-    } else if (kUmma && (warp == kConsumerWarps + 1 || warp == kConsumerWarps + 2) && lane == 0) {
-      // ================================ tcgen05 MMA issuers =============================
-      // One issuing thread per sub-tile (on different schedulers), each walking its own chain
-      //   S_X(0);  for j: [P_X(j) ready] O_X += P_X(j) V(j);  S_X(j+1) = Q_X K(j+1)^T.
-      // The MMAs of one thread execute in order, which is what lets P overwrite S in place.
-      const int X = warp - (kConsumerWarps + 1);
+    } else if (kUmma && warp == kConsumerWarps + 1) {
+      // ================================ tcgen05 MMA issuer ==============================
+      // One warp issues for both 128-row sub-tiles.  Each sub-tile is a chain
+      //   S_X(0);  for j: [P_X(j) ready] O_X += P_X(j) V(j);  S_X(j+1) = Q_X K(j+1)^T
+      // and the two chains alternate (A, B, A, B, ... skipping a sub-tile that has nothing left),
+      // so that one sub-tile's softmax overlaps the other's MMAs.  MMAs execute in order, which is
+      // what lets P overwrite S in place.  The whole warp walks the loop and waits, so that every
+      // operand is warp-uniform; one elected lane issues.  (Two issuing lanes, one per sub-tile, that
+      // took turns through a polled shared-memory word: 3.65 k cycles per pair of 128 x 128 tiles,
+      // this form 3.27 k; 4 prompts of 4096 tokens 1172 -> 1136 us, tree verification 916 -> 879 us
+      // at the power cap.)
+      const bool elected = elect_one();
       uint32_t pos = 0;  // ring position: stage = pos % kStages, parity = (pos / kStages) & 1
       bool dead = false;
-      uint32_t ph_q = 0, ph_p = 0;
+      uint32_t ph_q = 0, ph_p = 0;  // bit X: parity of sub-tile X's next wait
       Tracer tr;
-      tr.init(a, 2, X == 0);
+      tr.init(a, 2, elected);
       auto wait_or_die = [&](uint32_t bar, uint32_t parity) {
         if (!dead && !mbar_wait_block(bar, parity, a.status)) {
           report_timeout(a);
@@ -1015,68 +1019,38 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // distance to the second 64-element half, for the MN-major V tile).
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
       constexpr uint64_t kDescHi64 = static_cast<uint64_t>(kDescHi) << 32;
-      const uint32_t ring_lo = (ring >> 4) & 0x3FFFu;
-      const uint32_t t_s = tmem + kTmemS + X * 128, t_o = tmem + kTmemO + X * 128;
-      // The issuing thread gets few issue slots next to the softmax warps, so everything an MMA
-      // needs is computed ahead of the turn: Q descriptors once, K / V descriptors per tile.
-      uint64_t qd[8];
-#pragma unroll
-      for (int ks = 0; ks < 8; ++ks) {
-        const uint32_t off = (ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2;
-        qd[ks] = kDescHi64 | (((((q_smem + X * kTileBytes) >> 4) & 0x3FFFu) + off) | (1u << 16));
-      }
-      // K tile (K-major): 8 k-steps of 16 elements, 32 B apart, the second half 16 KiB away
-      auto k_descs = [&](uint32_t p, uint64_t (&kd)[8]) {
-        const uint32_t b0 = (ring_lo + (p % kStages) * (kTileBytes >> 4)) | (1u << 16);
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks)
-          kd[ks] = kDescHi64 | (b0 + (ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2);
+      const uint32_t ring_lo = (ring >> 4) & 0x3FFFu, q_lo = (q_smem >> 4) & 0x3FFFu;
+      auto commit = [&](uint64_t* bar) {
+        if (elected) umma_commit(smem_u32(bar));
       };
-      // V tile (MN-major): 8 k-steps of 16 keys, 2 KiB apart; LBO = 16 KiB to the second half
-      auto v_descs = [&](uint32_t p, uint64_t (&vd)[8]) {
-        const uint32_t b0 = (ring_lo + (p % kStages) * (kTileBytes >> 4)) | ((kHalfBytes >> 4) << 16);
+      // S_X = Q_X K^T: 8 k-steps of 16 elements, 32 B apart, the second half 16 KiB away
+      auto issue_qk = [&](int X, uint32_t p) {
+        const uint32_t k0 = (ring_lo + (p % kStages) * (kTileBytes >> 4)) | (1u << 16);
+        const uint32_t q0 = (q_lo + X * (kTileBytes >> 4)) | (1u << 16);
+        if (elected && !dead) {
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) vd[ks] = kDescHi64 | (b0 + ks * 128);
-      };
-      auto issue_qk = [&](const uint64_t (&kd)[8]) {  // S_X = Q_X K^T
-        umma_ss64(t_s, qd[0], kd[0], kIdescQK, 0u);
-#pragma unroll
-        for (int ks = 1; ks < 8; ++ks) umma_ss64(t_s, qd[ks], kd[ks], kIdescQK, 1u);
-        umma_commit(smem_u32(&ub->s_full[X]));
+          for (int ks = 0; ks < 8; ++ks) {
+            const uint32_t off = (ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2;
+            umma_ss64(tmem + kTmemS + X * 128, kDescHi64 | (q0 + off), kDescHi64 | (k0 + off), kIdescQK, ks > 0 ? 1u : 0u);
+          }
+        }
+        commit(&ub->s_full[X]);
       };
       // O_X (+)= P_X V with P in TMEM, in two halves of 64 keys: the first half is issued while
-      // the softmax warps are still exponentiating the second.
-      auto issue_pv_lo = [&](const uint64_t (&vd)[8], bool accumulate) {
-        umma_ts64(t_o, t_s, vd[0], kIdescPV, accumulate ? 1u : 0u);
+      // the softmax warps are still exponentiating the second.  V (MN-major): 8 k-steps of 16
+      // keys, 2 KiB apart.
+      auto issue_pv = [&](int X, uint32_t p, int half, bool accumulate) {
+        const uint32_t v0 = (ring_lo + (p % kStages) * (kTileBytes >> 4)) | ((kHalfBytes >> 4) << 16);
+        if (elected && !dead) {
 #pragma unroll
-        for (int ks = 1; ks < 4; ++ks) umma_ts64(t_o, t_s + ks * 8, vd[ks], kIdescPV, 1u);
-      };
-      auto issue_pv_hi = [&](const uint64_t (&vd)[8]) {
-#pragma unroll
-        for (int ks = 4; ks < 8; ++ks) umma_ts64(t_o, t_s + ks * 8, vd[ks], kIdescPV, 1u);
-      };
-      // A stage's empty barrier counts two arrivals: one per sub-tile that reads it, or both
-      // from the only reader.
-      auto release = [&](uint32_t p, bool alone) {
-        umma_commit(smem_u32(&bars->empty_umma[p % kStages]));
-        if (alone) umma_commit(smem_u32(&bars->empty_umma[p % kStages]));
-      };
-      // The two issuers take strict turns on the tensor pipe (A, B, A, B, ... skipping a sub-tile
-      // that has nothing left), so that one sub-tile's softmax always overlaps the other's MMAs
-      // instead of both falling into lockstep.  `turn` counts the groups issued so far.
-      uint32_t g_base = 0;
-      auto take_turn = [&](uint32_t g) {
-        if (dead) return;
-        for (uint32_t spin = 0; ub->turn != g; ++spin) {
-          if (spin > (1u << 22) || ((spin & 4095u) == 4095u && wait_should_give_up(a.status, spin))) {
-            report_timeout(a);
-            dead = true;
-            return;
+          for (int k = 0; k < 4; ++k) {
+            const int ks = half * 4 + k;
+            umma_ts64(tmem + kTmemO + X * 128, tmem + kTmemS + X * 128 + ks * 8, kDescHi64 | (v0 + ks * 128), kIdescPV,
+                      (accumulate || ks > 0) ? 1u : 0u);
           }
         }
       };
-      auto pass_turn = [&](uint32_t g) { ub->turn = g + 1; };
-      for (int ti = next_task(false); ti >= 0; ti = next_task(false)) {
+      for (int ti = next_task(true); ti >= 0; ti = next_task(true)) {
         const xy_attn_task t = a.tasks[ti];
         const uint32_t n_all = t.kt_hi - t.kt_lo;
         const uint32_t pos0 = pos;
@@ -1084,61 +1058,50 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         if (t.kind == 1) continue;  // streaming tasks never touch the tensor-memory path
         const ReqInfo rq = a.reqs[t.req];
         const DenseShape ds = dense_shape(t, rq, G);
-        const int nX = ds.n[X], nY = ds.n[1 - X];
-        const int nA = ds.n[0], nB = ds.n[1];
-        const uint32_t g0 = g_base;                                  // first group of this task
-        const uint32_t g1 = g0 + (nA > 0 ? 1u : 0u) + (nB > 0 ? 1u : 0u);  // first group of the j loop
-        g_base = g1 + nA + nB;
-        if (nX == 0) continue;
-        wait_or_die(smem_u32(&ub->q_full[X]), ph_q);
-        ph_q ^= 1u;
-        uint64_t kd[8], vd[8];
-        k_descs(pos0, kd);
+        const int n_max = max(ds.n[0], ds.n[1]);
+        if (n_max == 0) continue;
         wait_full(pos0);
-        {
-          const uint32_t g = g0 + ((X == 1 && nA > 0) ? 1u : 0u);
-          take_turn(g);
-          if (!dead) {
-            issue_qk(kd);
-            release(pos0, nY == 0);
-          }
-          pass_turn(g);
+#pragma unroll
+        for (int X = 0; X < 2; ++X) {
+          if (ds.n[X] == 0) continue;
+          wait_or_die(smem_u32(&ub->q_full[X]), (ph_q >> X) & 1u);
+          ph_q ^= 1u << X;
+          tc_fence_after();
+          issue_qk(X, pos0);
         }
-        for (int j = 0; j < nX; ++j) {
+        commit(&bars->empty_umma[pos0 % kStages]);
+        for (int j = 0; j < n_max; ++j) {
           const uint32_t pv = pos0 + 2 * j + 1, pk = pv + 1;
-          const bool more = j + 1 < nX;
-          const uint32_t g = g1 + min(j, nA) + min(j, nB) + ((X == 1 && j < nA) ? 1u : 0u);
-          v_descs(pv, vd);
-          k_descs(pk, kd);
           wait_full(pv);
-          if (more) wait_full(pk);
-          wait_or_die(smem_u32(&ub->p_full[X][0]), ph_p);
-          tc_fence_after();
-          tr(12);
-          take_turn(g);
-          tr(19);
-          if (!dead) issue_pv_lo(vd, j > 0);
-          wait_or_die(smem_u32(&ub->p_full[X][1]), ph_p);  // second half of P
-          ph_p ^= 1u;
-          tc_fence_after();
-          if (!dead) {
-            issue_pv_hi(vd);
-            if (j == nX - 1) umma_commit(smem_u32(&ub->o_done[X]));
-            release(pv, j >= nY);
+#pragma unroll
+          for (int X = 0; X < 2; ++X) {
+            if (j >= ds.n[X]) continue;
+            const bool more = j + 1 < ds.n[X];
+            wait_or_die(smem_u32(&ub->p_full[X][0]), (ph_p >> X) & 1u);
+            tc_fence_after();
+            tr(12);
+            issue_pv(X, pv, 0, j > 0);
+            if (more) wait_full(pk);
+            wait_or_die(smem_u32(&ub->p_full[X][1]), (ph_p >> X) & 1u);  // second half of P
+            ph_p ^= 1u << X;
+            tc_fence_after();
+            issue_pv(X, pv, 1, true);
+            if (!more) commit(&ub->o_done[X]);
+            // the stage goes back to the producer behind its last reader
+            if (X == 1 || j >= ds.n[1]) commit(&bars->empty_umma[pv % kStages]);
             if (more) {
-              issue_qk(kd);
-              release(pk, j + 1 >= nY);
+              issue_qk(X, pk);
+              if (X == 1 || j + 1 >= ds.n[1]) commit(&bars->empty_umma[pk % kStages]);
             }
+            tr(16);
           }
-          pass_turn(g);
-          tr(16);
         }
       }
       // Tensor memory is freed after the final barrier: no MMA of this thread may still be in
       // flight then.  On the normal path they completed long ago (immediate); after a failure
       // this is a bounded wait.
-      umma_commit(smem_u32(&ub->drained[X]));
-      mbar_wait_block(smem_u32(&ub->drained[X]), 0u, a.status);
+      commit(&ub->drained);
+      mbar_wait_block(smem_u32(&ub->drained), 0u, a.status);
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsConsumer));
