@@ -1060,13 +1060,15 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         const DenseShape ds = dense_shape(t, rq, G);
         const int n_max = max(ds.n[0], ds.n[1]);
         if (n_max == 0) continue;
-        wait_full(pos0);
 #pragma unroll
         for (int X = 0; X < 2; ++X) {
           if (ds.n[X] == 0) continue;
+          // q_full first: streaming tasks are skipped without a look at the ring, so this warp may be
+          // several fills of a stage ahead, where the parity of `full` says nothing.  Q is there once
+          // the consumers are through with every earlier task, that is, with every earlier fill.
           wait_or_die(smem_u32(&ub->q_full[X]), (ph_q >> X) & 1u);
           ph_q ^= 1u << X;
-          tc_fence_after();
+          wait_full(pos0);
           issue_qk(X, pos0);
         }
         commit(&bars->empty_umma[pos0 % kStages]);
