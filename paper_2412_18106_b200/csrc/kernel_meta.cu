@@ -17,7 +17,7 @@
 //             warpgroup does the online softmax of one sub-tile (thread = row).  In the variant
 //             without tensor memory (kUmma = false) a dense task is one 128-row tile on
 //             mma.sync, each consumer warp owning 16 rows.
-//   streaming (rows <= 16: decode, tiny verify): each consumer warp owns 16 keys of every tile
+//   streaming (rows <= 16: decode, tiny verify; stream.cuh): each consumer warp owns 16 keys of every tile
 //             against all rows on mma.sync; the warps' partial (m, l, O) are merged in shared
 //             memory at the end of the task.  HBM-bound.
 // Online softmax runs in the log2 domain in fp32; P is rounded to bf16 before P V; masked scores
@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "ptx.cuh"
+#include "stream.cuh"
 #include "xy_kernels.h"
 
 namespace xy {
@@ -47,8 +48,6 @@ constexpr int kStages = 4;
 constexpr int kTileBytes = 32768;  // 2 halves x 128 rows x 128 B
 constexpr int kHalfBytes = 16384;
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kRescaleThresholdWarp = 8.0f;  // log2 units, warp-level MMA paths
-constexpr float kLn2 = 0.6931471805599453f;
 
 struct __align__(8) SmemBarriers {
   uint64_t full[kStages];
@@ -60,7 +59,6 @@ constexpr int kSmemQ = 2 * kTileBytes;
 constexpr int kSmemRing = kStages * kTileBytes;
 constexpr int kSmemMl = kConsumerWarps * 16 * 2 * 4;
 constexpr int kSmemFp8 = 1024;  // fp8 KV path: per-row Q factors [128] and a ring of per-tile page scales [8][16]
-constexpr int kScaleSlots = 8;
 constexpr int kSmemTotal = 1024 /*align slack*/ + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers) + 128 + 256 + kSmemFp8;
 
 __device__ __forceinline__ uint32_t swz(uint32_t row, uint32_t chunk16 /*0..15*/) {
@@ -82,18 +80,8 @@ struct MetaParams {
   RunArgs a;
 };
 
-// Visibility of key column `col` for new token i (Sections 4.1.2, 4.2.2, 5.2).
-__device__ __forceinline__ bool visible(const RunArgs& a, const ReqInfo& rq, int i, int col) {
-  if (col > rq.kv_len + i) return false;  // causal frontier; also excludes everything >= L
-  if (col < rq.kv_len || rq.mask_kind == XY_MASK_CAUSAL) return true;
-  const int jp = col - rq.kv_len;
-  const uint64_t w = __ldg(a.tree_mask + rq.tree_off + static_cast<int64_t>(i) * rq.tree_words + (jp >> 6));
-  return (w >> (jp & 63)) & 1ull;
-}
-
-// One consumer warp: 16 packed rows (x0 .. x0+15) against NT*8 keys (key offset koff inside
-// every 128-key tile).  Keeps m (log2 domain), l (thread-partial) and O in registers.
-// KEEPQ: Q fragments stay in registers for the whole task (streaming); otherwise they are
+// One consumer warp of a dense task without tensor memory: 16 packed rows (x0 .. x0+15) against
+// NT*8 keys.  Keeps m (log2 domain), l (thread-partial) and O in registers; the Q fragments are
 // re-read from shared memory at every k-step to leave registers for the 128-key score tile.
 // F16: operands are f16 (the fp8 KV-cache path: K / V widened exactly from e4m3, Q converted with a
 // power-of-two factor per row) and the scores carry per-row and per-page factors (FpScale).
@@ -108,12 +96,11 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
   if constexpr (F16) mma_f16_16816(c, a, b0, b1); else mma_bf16_16816(c, a, b0, b1);
 }
 
-template <int NT, bool KEEPQ, bool F16 = false>
+template <int NT, bool F16 = false>
 struct WarpTile {
   float o[16][4];
   float m_lo, m_hi, l_lo, l_hi;
-  uint32_t qf[KEEPQ ? 8 : 1][4];
-  uint32_t q_addr;  // this lane's ldmatrix row address for k-step 0 (!KEEPQ)
+  uint32_t q_addr, q_row7, q_hi;  // this lane's ldmatrix row address for k-step 0, row % 8, chunk parity
 
   __device__ __forceinline__ void init() {
 #pragma unroll
@@ -127,59 +114,13 @@ struct WarpTile {
   __device__ __forceinline__ void load_q(uint32_t q_smem, int x0, int lane) {
     const int mi = lane >> 3;
     const uint32_t row = x0 + (lane & 7) + (mi & 1) * 8;
-    if (KEEPQ) {
-#pragma unroll
-      for (int ks = 0; ks < 8; ++ks)
-        ldmatrix_x4(q_smem + swz(row, ks * 2 + (mi >> 1)), qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3]);
-    } else {
-      q_addr = q_smem + row * 128u;
-      q_row7 = row & 7u;
-      q_hi = mi >> 1;
-    }
+    q_addr = q_smem + row * 128u;
+    q_row7 = row & 7u;
+    q_hi = mi >> 1;
   }
-  uint32_t q_row7, q_hi;
 
   // S = Q K^T for this warp's keys; returns scores (raw dot products) in s.
   __device__ __forceinline__ void qk(uint32_t k_smem, int koff, int lane, float (&s)[NT][4]) {
-    if constexpr (NT == 2) {
-      // Streaming tile: all eight K fragments are fetched first (one shared-memory latency
-      // instead of eight), and even / odd k-steps accumulate separately so that the MMAs form
-      // four chains of four instead of two chains of eight.
-      const int mi = lane >> 3;
-      const uint32_t key = koff + (lane & 7) + (mi >> 1) * 8;
-      uint32_t kb[8][4];
-#pragma unroll
-      for (int ks = 0; ks < 8; ++ks)
-        ldmatrix_x4(k_smem + swz(key, ks * 2 + (mi & 1)), kb[ks][0], kb[ks][1], kb[ks][2], kb[ks][3]);
-      uint32_t qq[8][4];
-      if constexpr (!KEEPQ) {
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-          const uint32_t ch = ks * 2 + q_hi;
-          ldmatrix_x4(q_addr + (ch >> 3) * kHalfBytes + (((ch & 7u) ^ q_row7) << 4), qq[ks][0], qq[ks][1],
-                      qq[ks][2], qq[ks][3]);
-        }
-      }
-      float t[2][4];
-#pragma unroll
-      for (int n = 0; n < 2; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] = t[n][e] = 0.f;
-#pragma unroll
-      for (int ks = 0; ks < 8; ks += 2) {
-        const uint32_t(&qa)[4] = KEEPQ ? qf[KEEPQ ? ks : 0] : qq[ks];
-        const uint32_t(&qb)[4] = KEEPQ ? qf[KEEPQ ? ks + 1 : 0] : qq[ks + 1];
-        mma16816<F16>(s[0], qa, kb[ks][0], kb[ks][1]);
-        mma16816<F16>(s[1], qa, kb[ks][2], kb[ks][3]);
-        mma16816<F16>(t[0], qb, kb[ks + 1][0], kb[ks + 1][1]);
-        mma16816<F16>(t[1], qb, kb[ks + 1][2], kb[ks + 1][3]);
-      }
-#pragma unroll
-      for (int n = 0; n < 2; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] += t[n][e];
-      return;
-    }
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
@@ -187,12 +128,9 @@ struct WarpTile {
     const int mi = lane >> 3;
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      if (!KEEPQ) {
-        const uint32_t ch = ks * 2 + q_hi;
-        ldmatrix_x4(q_addr + (ch >> 3) * kHalfBytes + (((ch & 7u) ^ q_row7) << 4), qf[0][0], qf[0][1],
-                    qf[0][2], qf[0][3]);
-      }
-      const uint32_t(&qa)[4] = qf[KEEPQ ? ks : 0];
+      uint32_t qa[4];
+      const uint32_t ch = ks * 2 + q_hi;
+      ldmatrix_x4(q_addr + (ch >> 3) * kHalfBytes + (((ch & 7u) ^ q_row7) << 4), qa[0], qa[1], qa[2], qa[3]);
 #pragma unroll
       for (int np = 0; np < NT / 2; ++np) {
         const uint32_t key = koff + np * 16 + (lane & 7) + (mi >> 1) * 8;
@@ -281,19 +219,6 @@ struct WarpTile {
   // O += P V for this warp's keys.
   __device__ __forceinline__ void pv(uint32_t v_smem, int koff, int lane, const uint32_t (&p)[NT / 2][4]) {
     const int mi = lane >> 3;
-    if constexpr (NT == 2) {  // streaming tile: fetch the eight V fragments, then 16 MMAs
-      const uint32_t key = koff + (lane & 7) + (mi & 1) * 8;
-      uint32_t vb[8][4];
-#pragma unroll
-      for (int dp = 0; dp < 8; ++dp)
-        ldmatrix_x4_trans(v_smem + swz(key, dp * 2 + (mi >> 1)), vb[dp][0], vb[dp][1], vb[dp][2], vb[dp][3]);
-#pragma unroll
-      for (int dp = 0; dp < 8; ++dp) {
-        mma16816<F16>(o[2 * dp], p[0], vb[dp][0], vb[dp][1]);
-        mma16816<F16>(o[2 * dp + 1], p[0], vb[dp][2], vb[dp][3]);
-      }
-      return;
-    }
 #pragma unroll
     for (int kk = 0; kk < NT / 2; ++kk) {
       const uint32_t key = koff + kk * 16 + (lane & 7) + (mi & 1) * 8;
@@ -382,12 +307,6 @@ __device__ __forceinline__ void q_rows_to_f16(uint32_t q_smem, int row0, float* 
   if (lane % kLanesPerRow == 0) qmult[row] = up;
 }
 
-struct TaskView {
-  xy_attn_task t;
-  ReqInfo rq;
-  int G, rows;
-};
-
 // Destination of packed row x: final O / LSE or the fp32 partial.
 __device__ __forceinline__ void write_row_pair(const RunArgs& a, const TaskView& tv, int x, int col,
                                                float v0, float v1) {
@@ -428,229 +347,6 @@ struct Tracer {
   __device__ __forceinline__ void operator()(unsigned) {}
 #endif
 };
-
-// Word 0 of the status block is this run's (cleared at every launch, polled by every wait); the
-// sticky word is what xy_attn_device_status reads and clears.
-__device__ __forceinline__ void report_timeout(const RunArgs& a) {
-  atomicExch(a.status, XY_ERR_DEVICE_TIMEOUT);
-  atomicExch(a.status + kStatusSticky, XY_ERR_DEVICE_TIMEOUT);
-}
-
-// Merge of a split streaming unit inside the attention kernel (the cross-task Update stage of
-// Section 4.2.1, run by the task of the unit that finished last).  rows <= 16; one warp per row;
-// LSE_c in lanes, the partial rows read eight at a time straight from L2.
-__device__ __forceinline__ float ldcg_f(const float* p) { return __ldcg(p); }
-__device__ __forceinline__ void merge_unit_in_kernel(const RunArgs& a, const xy_attn_merge_unit& u, int G, int warp,
-                                                     int lane) {
-  const int rows = u.ntok * G, ns = u.nsplit;
-  const ReqInfo rq = a.reqs[u.req];
-  for (int x = warp; x < rows; x += kConsumerWarps) {
-    const int64_t row0 = static_cast<int64_t>(u.part0) + x;  // partial row of split c: row0 + c * rows
-    float mx = -INFINITY;
-    for (int c = lane; c < ns; c += 32) mx = fmaxf(mx, ldcg_f(a.lse_part + row0 + static_cast<int64_t>(c) * rows));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float z = 0.f;
-    for (int c = lane; c < ns; c += 32) {
-      const float lc = ldcg_f(a.lse_part + row0 + static_cast<int64_t>(c) * rows);
-      if (lc != -INFINITY) z += __expf(lc - mx);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    const float lse = mx + logf(z);
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int c0 = 0; c0 < ns; c0 += 8) {
-      float w[8];
-      float4 v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int c = c0 + e;
-        const float lc = c < ns ? ldcg_f(a.lse_part + row0 + static_cast<int64_t>(c) * rows) : -INFINITY;
-        w[e] = lc != -INFINITY ? __expf(lc - lse) : 0.f;
-        // an empty split (weight 0) is not read
-        v[e] = w[e] != 0.f ? __ldcg(reinterpret_cast<const float4*>(a.o_part + (row0 + static_cast<int64_t>(c) * rows) * kHeadDim) + lane)
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        acc.x += w[e] * v[e].x;
-        acc.y += w[e] * v[e].y;
-        acc.z += w[e] * v[e].z;
-        acc.w += w[e] * v[e].w;
-      }
-    }
-    const int i = u.tok0 + x / G, head = u.kv_head * G + x % G;
-    uint2 packed;
-    packed.x = pack_bf16(acc.x, acc.y);
-    packed.y = pack_bf16(acc.z, acc.w);
-    *reinterpret_cast<uint2*>(a.o + static_cast<int64_t>(rq.q_start + i) * a.o_token_stride + head * kHeadDim + lane * 4) = packed;
-    if (lane == 0) a.lse[static_cast<int64_t>(rq.q_start + i) * a.num_q_heads + head] = lse;
-  }
-}
-
-// ------------------------------------------------------------------------------------------
-// One streaming task (at most 16 packed rows: decode steps, short verify windows and the thin
-// tails of prefill chunks), run by the eight consumer warps.  Every warp owns 16 keys of each
-// 128-key tile, keeps its own online-softmax state over those keys, and the eight partial
-// results are merged through shared memory when the task ends (the in-CTA Update stage of
-// Section 4.2.1).  pipe_state: ring stage | phase << 8 | dead << 16, returned updated.
-// kFp8: the stages hold e4m3 bytes; every warp widens its 16 keys before use, the Q rows in shared
-// memory are f16 (converted by the caller), qmult / scale_ring carry the row and page factors and
-// tile_seq counts the key tiles this worker has consumed (it selects the scale slot).
-template <bool kFp8>
-__device__ __forceinline__ uint32_t stream_task(const RunArgs& a, const TaskView& tv, uint32_t q_smem, uint32_t ring,
-                                             SmemBarriers* bars, float* xch, float* ml, uint32_t pipe_state,
-                                             float scale_log2, const float* qmult, const float* scale_ring,
-                                             uint32_t& tile_seq, int unit) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  Pipe pipe{static_cast<int>(pipe_state & 0xFFu), (pipe_state >> 8) & 1u};
-  bool dead = (pipe_state >> 16) & 1u;
-  const int h = tv.rq.kv_len;
-  const bool tree = tv.rq.mask_kind == XY_MASK_TREE;
-  const int koff = warp * 16;
-  WarpTile<2, false, kFp8> w;
-  w.init();
-  w.load_q(q_smem, 0, lane);
-  FpScale fs{1.f, 1.f, scale_ring, a.page_shift};
-  if constexpr (kFp8) {
-    fs.q_lo = qmult[lane >> 2];
-    fs.q_hi = qmult[(lane >> 2) + 8];
-  }
-  const int r_lo = min(lane >> 2, tv.rows - 1), r_hi = min((lane >> 2) + 8, tv.rows - 1);
-  const int i_lo = tv.t.tok0 + r_lo / tv.G, i_hi = tv.t.tok0 + r_hi / tv.G;
-  const int i_max = tv.t.tok0 + tv.t.ntok - 1;
-  // Tiles that every row of the task sees in full need neither the mask nor the mask-aware
-  // skip test; the loop over them is compiled without either.  The last tiles (the causal
-  // frontier or the speculative corner) take the general step.
-#ifdef XY_ENABLE_TRACE
-  long long ph[6] = {0, 0, 0, 0, 0, 0};
-#define XY_PH(i) { const long long c_now = clock64(); ph[i] += c_now - c_prev; c_prev = c_now; }
-#else
-#define XY_PH(i)
-#endif
-  auto step = [&](int kt, auto tail_tag) {
-    constexpr bool kTail = decltype(tail_tag)::value;
-    const int col0 = kt * kKeyTile + koff;
-    const bool work = kTail ? (col0 <= h + i_max) : true;
-    float s[2][4];
-    uint32_t p[1][4];
-#ifdef XY_ENABLE_TRACE
-    long long c_prev = clock64();
-    ph[5] += 1;
-#endif
-    if (!dead && !mbar_wait_block(smem_u32(&bars->full[pipe.stage]), pipe.phase, a.status)) {
-      report_timeout(a);
-      dead = true;
-    }
-    XY_PH(0)
-    if constexpr (kFp8) {
-      fs.tile = scale_ring + (tile_seq % kScaleSlots) * 16;
-      ++tile_seq;
-      if (work) widen_rows16(ring + pipe.stage * kTileBytes, koff, lane);
-    }
-    if (work) w.qk(ring + pipe.stage * kTileBytes, koff, lane, s);
-    if constexpr (kFp8) fence_proxy_async_smem();  // the widened rows are overwritten by the next bulk copy
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
-    pipe.advance();
-    XY_PH(1)
-    if (work) {
-      const bool need_mask = kTail ? (tree ? (col0 + 16 > h) : (col0 + 16 > h + tv.t.tok0 + 1)) : false;
-      w.softmax(a, tv.rq, s, p, col0, i_lo, i_hi, need_mask, scale_log2, lane, &fs, koff);
-    }
-    XY_PH(2)
-    if (!dead && !mbar_wait_block(smem_u32(&bars->full[pipe.stage]), pipe.phase, a.status)) {
-      report_timeout(a);
-      dead = true;
-    }
-    XY_PH(3)
-    if constexpr (kFp8) {
-      if (work) widen_rows16(ring + pipe.stage * kTileBytes, koff, lane);
-    }
-    if (work) w.pv(ring + pipe.stage * kTileBytes, koff, lane, p);
-    if constexpr (kFp8) fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
-    pipe.advance();
-    XY_PH(4)
-  };
-  const int full_cols = tree ? h : h + tv.t.tok0 + 1;  // columns below this are visible to every row
-  const int kt_mid = max(tv.t.kt_lo, min(tv.t.kt_hi, full_cols / kKeyTile));
-  int kt = tv.t.kt_lo;
-  for (; kt < kt_mid; ++kt) step(kt, std::false_type{});
-  for (; kt < tv.t.kt_hi; ++kt) step(kt, std::true_type{});
-#ifdef XY_ENABLE_TRACE
-  if (a.trace != nullptr && blockIdx.x == 0 && threadIdx.x == 0)
-    for (int i = 0; i < 6; ++i) a.trace[4 * kTraceLen - 8 + i] += ph[i];
-#endif
-#undef XY_PH
-  // ---- merge the eight warps' partials (in-CTA Update stage)
-  w.reduce_l();
-  named_bar_sync(1, kConsumerThreads);  // every warp holds its Q fragments: Q smem is free
-  {
-    const int xl = lane >> 2, xh = xl + 8;
-    float* mine = xch + warp * (16 * kHeadDim);
-    // only the task's rows are merged below: padding rows (most of the 16 in a decode step) are
-    // not written
-    const bool has_lo = xl < tv.rows, has_hi = xh < tv.rows;
-#pragma unroll
-    for (int n = 0; n < 16; ++n) {
-      const int col = n * 8 + 2 * (lane & 3);
-      if (has_lo) *reinterpret_cast<float2*>(mine + xl * kHeadDim + col) = make_float2(w.o[n][0], w.o[n][1]);
-      if (has_hi) *reinterpret_cast<float2*>(mine + xh * kHeadDim + col) = make_float2(w.o[n][2], w.o[n][3]);
-    }
-    if ((lane & 3) == 0) {
-      ml[(warp * 16 + xl) * 2 + 0] = w.m_lo;
-      ml[(warp * 16 + xl) * 2 + 1] = w.l_lo;
-      ml[(warp * 16 + xh) * 2 + 0] = w.m_hi;
-      ml[(warp * 16 + xh) * 2 + 1] = w.l_hi;
-    }
-  }
-  named_bar_sync(1, kConsumerThreads);
-  {
-    const int x = threadIdx.x >> 4, seg = threadIdx.x & 15;  // row, 8-column segment
-    if (x < tv.rows) {
-      float M = -INFINITY;
-#pragma unroll
-      for (int ww = 0; ww < kConsumerWarps; ++ww) M = fmaxf(M, ml[(ww * 16 + x) * 2]);
-      float L = 0.f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int ww = 0; ww < kConsumerWarps; ++ww) {
-        const float mw = ml[(ww * 16 + x) * 2], lw = ml[(ww * 16 + x) * 2 + 1];
-        if (mw == -INFINITY) continue;
-        const float f = ex2(mw - M);
-        L += f * lw;
-        const float4* src = reinterpret_cast<const float4*>(xch + ww * (16 * kHeadDim) + x * kHeadDim + seg * 8);
-        const float4 v0 = src[0], v1 = src[1];
-        acc[0] += f * v0.x; acc[1] += f * v0.y; acc[2] += f * v0.z; acc[3] += f * v0.w;
-        acc[4] += f * v1.x; acc[5] += f * v1.y; acc[6] += f * v1.z; acc[7] += f * v1.w;
-      }
-      const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; e += 2)
-        write_row_pair(a, tv, x, seg * 8 + e, acc[e] * inv, acc[e + 1] * inv);
-      if (seg == 0) write_lse(a, tv, x, L > 0.f ? (M + log2f(L)) * kLn2 : -INFINITY);
-    }
-  }
-  if (unit >= 0) {
-    // This task is one KV split of a unit that is merged here: publish the partial, count the
-    // finished splits, and let the task that completes the unit merge it.  (Writers: stores, fence,
-    // barrier, one atomic; the last one: atomic, fence, loads that bypass L1.)
-    __shared__ int s_last;
-    __threadfence();
-    named_bar_sync(1, kConsumerThreads);
-    if (threadIdx.x == 0) {
-      const int ns = a.units[unit].nsplit;
-      s_last = atomicAdd(a.unit_count + unit, 1) == ns - 1 ? 1 : 0;
-    }
-    named_bar_sync(1, kConsumerThreads);
-    if (s_last) {
-      __threadfence();
-      merge_unit_in_kernel(a, a.units[unit], tv.G, warp, lane);
-    }
-  }
-  return static_cast<uint32_t>(pipe.stage) | (pipe.phase << 8) | (dead ? 1u << 16 : 0u);
-}
 
 // ------------------------------------------------------------------------------------------
 // tcgen05 dense path.  TMEM columns: S_A [0,128) S_B [128,256) O_A [256,384) O_B [384,512);
@@ -720,7 +416,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   SmemBarriers* bars = reinterpret_cast<SmemBarriers*>(gen_base + kSmemQ + kSmemRing + kSmemMl);
   UmmaBarriers* ub = reinterpret_cast<UmmaBarriers*>(gen_base + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers));
   TaskRing* tq = reinterpret_cast<TaskRing*>(gen_base + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers) + 128);
-  float* xch = reinterpret_cast<float*>(gen_base);  // streaming merge area, aliases the Q tiles
+  float* xch = reinterpret_cast<float*>(gen_base + kTileBytes);  // streaming merge area, aliases sub-tile B's Q
   static_assert(!(kUmma && kFp8), "the fp8 KV path runs on the warp-level MMA paths");
   float* qmult = reinterpret_cast<float*>(gen_base + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers) + 128 + 256);
   float* scale_ring = qmult + 128;  // [kScaleSlots][16]: K scales [0..7], V scales [8..15] of a tile's pages
@@ -1436,11 +1132,11 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         cp_async_commit_wait_all();
         named_bar_sync(1, kConsumerThreads);
         if constexpr (kFp8) {
-          // Q rows become f16 with a power-of-two factor per row (dense: each warp its own 16 rows;
-          // streaming: the 16 rows shared by all warps, two per warp)
-          if (stream) q_rows_to_f16<16>(q_smem, warp * 2, qmult, lane);
-          else q_rows_to_f16<2>(q_smem, warp * 16, qmult, lane);
-          named_bar_sync(1, kConsumerThreads);
+          // dense: the Q rows become f16 with a power-of-two factor per row, each warp its own 16 rows
+          if (!stream) {
+            q_rows_to_f16<2>(q_smem, warp * 16, qmult, lane);
+            named_bar_sync(1, kConsumerThreads);
+          }
         }
       }
 
@@ -1448,7 +1144,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         // ---------------- dense: this warp owns rows x0 .. x0+15 -------------------------
         const int x0 = warp * 16;
         const bool active = x0 < tv.rows;
-        WarpTile<16, false, kFp8> w;
+        WarpTile<16, kFp8> w;
         w.init();
         if (active) w.load_q(q_smem, x0, lane);
         FpScale fs{1.f, 1.f, scale_ring, a.page_shift};
@@ -1519,13 +1215,27 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         }
         named_bar_sync(1, kConsumerThreads);  // Q tile may be overwritten by the next task
       } else {
-        // ---------------- streaming (see stream_task) ----
-        const uint32_t st = stream_task<kFp8>(a, tv, q_smem, ring, bars, xch, ml, pipe.stage | (pipe.phase << 8) |
-                                              (dead ? 1u << 16 : 0u), scale_log2, qmult, scale_ring, tile_seq,
-                                              (a.task_unit != nullptr && tv.t.part >= 0) ? a.task_unit[ti] : -1);
-        pipe.stage = st & 0xFFu;
-        pipe.phase = (st >> 8) & 1u;
-        dead = (st >> 16) & 1u;
+        // ---------------- streaming (see stream.cuh) ----
+        __shared__ int s_last;
+        const int unit = (a.task_unit != nullptr && tv.t.part >= 0) ? a.task_unit[ti] : -1;
+        const StreamRing sr{ring + (kFp8 ? kHalfBytes : 0), kTileBytes, smem_u32(&bars->full[0]), smem_u32(&bars->empty[0])};
+        auto q_addr = [&](uint32_t row, uint32_t ch) { return q_smem + swz(row, ch); };
+        RingPos pos{pipe.stage, pipe.phase};
+        if (tv.rows <= 8) {
+          StreamWarp<kConsumerWarps, 1, kFp8> w;
+          w.init();
+          w.load_q(q_addr, lane);
+          stream_task<kConsumerWarps, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq,
+                                                        unit, warp, 1, &s_last);
+        } else {
+          StreamWarp<kConsumerWarps, 2, kFp8> w;
+          w.init();
+          w.load_q(q_addr, lane);
+          stream_task<kConsumerWarps, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq,
+                                                        unit, warp, 1, &s_last);
+        }
+        pipe.stage = pos.stage;
+        pipe.phase = pos.phase;
         named_bar_sync(1, kConsumerThreads);
       }
     }
