@@ -388,6 +388,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.queue = ctx->d_queue;
   a.queue_head = ctx->d_status + kStatusQueueHead;  // second cache line of the status block
   a.num_tasks = static_cast<int32_t>(p.tasks.size());
+  a.num_workers = ctx->num_workers;
   // Balanced plans are dealt dynamically by the meta-kernel; paper-mode plans keep the static
   // Task-Table (each worker walks its own list), as does the reference kernel.
   a.dynamic = (cfg.plan_mode == XY_PLAN_BALANCED && cfg.kernel != XY_KERNEL_REFERENCE) ? 1 : 0;
@@ -427,12 +428,17 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
     st.num_tasks = a.num_tasks - p.queue_dense;
     st.queue_head = a.queue_head + 1;  // its own head word, cleared by the same memset
     if (st.num_tasks > 0) {
-      XY_CUDA(ctx, launch_meta(st, ctx->num_workers, num_pages, false, &ctx->launch_cache, s));
+      XY_CUDA(ctx, launch_meta(st, num_pages, false, &ctx->launch_cache, s));
       ctx->last_launches += 1;
     }
     ctx->last_launches -= 1;  // counted once more below
+  } else if (cfg.kernel == XY_KERNEL_AUTO && a.dynamic && p.info.num_dense_tasks == 0) {
+    // Only streaming tasks: the kernel with two small CTAs per SM (faster from one request to a
+    // saturated decode batch, figures in kernel_stream.cu).  With dense tasks in the batch the
+    // meta-kernel runs both kinds side by side.
+    XY_CUDA(ctx, launch_stream(a, num_pages, &ctx->launch_cache, s));
   } else {
-    XY_CUDA(ctx, launch_meta(a, ctx->num_workers, num_pages,
+    XY_CUDA(ctx, launch_meta(a, num_pages,
                              (cfg.kernel == XY_KERNEL_AUTO || cfg.kernel == XY_KERNEL_PAIR) && p.info.num_dense_tasks > 0,
                              &ctx->launch_cache, s));
   }

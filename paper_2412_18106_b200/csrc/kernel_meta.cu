@@ -1299,19 +1299,10 @@ bool encode_pool_map(CUtensorMap* m, const void* pool, int64_t num_pages, int nu
 
 }  // namespace
 
-cudaError_t launch_meta(const RunArgs& a, int num_workers, int64_t num_pages, bool umma, MetaLaunchCache* cache,
-                        cudaStream_t s) {
+// The tensor maps of the pools, encoded when the pools differ from those of the last call.
+cudaError_t pool_maps(const RunArgs& a, int64_t num_pages, MetaLaunchCache* cache) {
   static_assert(sizeof(CUtensorMap) == 128, "MetaLaunchCache holds a tensor map in 128 bytes");
   const bool fp8 = a.kv_fp8 != 0;
-  if (fp8) umma = false;
-  auto kernel = fp8 ? meta_attention_kernel<false, true>
-                    : (umma ? meta_attention_kernel<true, false> : meta_attention_kernel<false, false>);
-  const int which = fp8 ? 2 : (umma ? 1 : 0);
-  if (!cache->attr_set[which]) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal);
-    if (e != cudaSuccess) return e;
-    cache->attr_set[which] = true;
-  }
   CUtensorMap* k_map = reinterpret_cast<CUtensorMap*>(cache->maps[0]);
   CUtensorMap* v_map = reinterpret_cast<CUtensorMap*>(cache->maps[1]);
   const bool same = cache->valid && cache->k_pool == a.k_pool && cache->v_pool == a.v_pool &&
@@ -1336,8 +1327,25 @@ cudaError_t launch_meta(const RunArgs& a, int num_workers, int64_t num_pages, bo
     cache->fp8 = fp8;
     cache->valid = true;
   }
+  return cudaSuccess;
+}
+
+cudaError_t launch_meta(const RunArgs& a, int64_t num_pages, bool umma, MetaLaunchCache* cache, cudaStream_t s) {
+  const bool fp8 = a.kv_fp8 != 0;
+  if (fp8) umma = false;
+  auto kernel = fp8 ? meta_attention_kernel<false, true>
+                    : (umma ? meta_attention_kernel<true, false> : meta_attention_kernel<false, false>);
+  const int which = fp8 ? 2 : (umma ? 1 : 0);
+  if (!cache->attr_set[which]) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal);
+    if (e != cudaSuccess) return e;
+    cache->attr_set[which] = true;
+  }
+  const cudaError_t e = pool_maps(a, num_pages, cache);
+  if (e != cudaSuccess) return e;
   MetaParams P{a};
-  kernel<<<num_workers, kThreads, kSmemTotal, s>>>(P, *k_map, *v_map);
+  kernel<<<a.num_workers, kThreads, kSmemTotal, s>>>(P, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
+                                                     *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
   return cudaGetLastError();
 }
 

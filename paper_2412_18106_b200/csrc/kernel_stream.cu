@@ -1,0 +1,320 @@
+// Attention kernel for batches without dense tiles (decode, tiny verify windows): HBM-bound.
+//
+// Two CTAs of 160 threads per SM: while one is between tasks (first tiles on their way, merge of
+// the warps, output), the other one keeps the SM's loads in flight.  Roles of a CTA:
+//   warps 0..3  consumers: 32 keys of every 128-key tile each (stream.cuh)
+//   warp  4     producer: takes the next task (the first by block index, the following ones from the
+//               head of the queue), copies its Q rows and its description into shared memory while
+//               the previous task is still being worked on, and keeps a ring of K and V tiles filled
+//               by TMA, its lanes issuing the boxes of a tile's pages side by side
+// What bounds it: the bytes of K and V.  96 KiB of tiles per CTA, 192 KiB per SM, are in flight
+// (fp8: 80 and 160).  Every wait is bounded and reports a timeout in the status word.
+// Measured (device time of one call) against the meta-kernel, whose single CTA per SM drains between
+// tasks: 13 requests of 300 - 2500 keys, 32/8 heads 34.9 -> 23.8 us; 24 requests up to 3000 keys, 64/8
+// heads 47.5 -> 38.6 us; 64 requests up to 8192 keys, 28/4 heads 101.3 -> 100.0 us (0.9 of the copy
+// bandwidth), over an fp8 cache 88.5 -> 56.6 us.
+#include <cuda.h>
+#include <cuda_runtime.h>
+
+#include "ptx.cuh"
+#include "stream.cuh"
+#include "xy_kernels.h"
+
+namespace xy {
+namespace {
+
+using namespace ptx;
+
+constexpr int kWarpsS = 4;
+constexpr int kThreadsS = (kWarpsS + 1) * 32;
+// Descriptions of tasks: the one being worked on and up to three that the look-ahead has reached.
+constexpr int kTaskSlots = 4;
+
+template <bool kFp8>
+struct StreamCfg {
+  static constexpr int kStageBytes = kFp8 ? 16384 : 32768;
+  static constexpr int kStages = kFp8 ? 5 : 3;
+  static constexpr int kRing = kStages * kStageBytes;
+  static constexpr int kXch = kStreamXchFloats<kWarpsS> * 4;
+  static constexpr int kQ = 16 * 256;
+  static constexpr int kMl = kWarpsS * 16 * 8;
+  static constexpr int kScales = kFp8 ? kScaleSlots * 64 : 0;
+  static constexpr int kSmem = kRing + kXch + kQ + kMl + kScales + kTaskSlots * 64 + 16 * kStages + 32;
+};
+
+struct TaskDesc {
+  xy_attn_task t;
+  ReqInfo rq;  // pad1: index of the unit the last finisher merges, or -1
+};
+static_assert(sizeof(TaskDesc) == 64, "the shared-memory layout reserves 64 bytes per description");
+
+template <bool kFp8>
+__global__ void __launch_bounds__(kThreadsS, 2)
+stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant__ CUtensorMap k_map,
+                        const __grid_constant__ CUtensorMap v_map) {
+  using Cfg = StreamCfg<kFp8>;
+  constexpr int kStages = Cfg::kStages;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  float* xch = reinterpret_cast<float*>(smem + Cfg::kRing);
+  uint8_t* q_gen = smem + Cfg::kRing + Cfg::kXch;
+  float* ml = reinterpret_cast<float*>(q_gen + Cfg::kQ);
+  float* scale_ring = ml + Cfg::kMl / 4;
+  TaskDesc* desc = reinterpret_cast<TaskDesc*>(q_gen + Cfg::kQ + Cfg::kMl + Cfg::kScales);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(desc + kTaskSlots);
+  int* s_last = reinterpret_cast<int*>(bars + 2 * kStages + 2);
+  int* s_dead = s_last + 1;
+  const uint32_t ring = smem_u32(smem), q_smem = smem_u32(q_gen);
+  const uint32_t full = smem_u32(bars), empty = full + 8 * kStages, task_full = empty + 8 * kStages, task_free = task_full + 8;
+
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  unsigned long long t_start = 0;
+  if (threadIdx.x == 0) {
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(full + 8 * s, 1);
+      mbar_init(empty + 8 * s, kWarpsS);
+    }
+    mbar_init(task_full, 33);  // lane 0 once the description is written, every lane once its Q chunks have landed
+    mbar_init(task_free, kWarpsS);
+    *s_dead = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const int G = a.num_q_heads / a.num_kv_heads;
+
+  if (warp == kWarpsS) {
+    // ================================== producer ==========================================
+    if (lane == 0) {
+      prefetch_tensormap(&k_map);
+      prefetch_tensormap(&v_map);
+    }
+    bool dead = false;
+    if ((ring & 1023u) != 0) {  // the TMA swizzle needs it; dynamic shared memory starts there
+      report_timeout(a);
+      dead = true;
+    }
+    const int ppt = kKeyTile >> a.page_shift;  // pages per tile
+    // bf16: two 64-element boxes per page, lane 2 p + half; fp8: one box per page, lane p
+    const int lane_page = kFp8 ? lane : lane >> 1;
+    const bool has_box = lane_page < ppt;
+    const uint32_t box_bytes = static_cast<uint32_t>(a.page_size) * 128u;
+    const uint32_t box_off = kFp8 ? lane_page * box_bytes : (lane & 1) * 16384u + lane_page * box_bytes;
+    const uint64_t policy = make_l2_policy_evict_first();
+    struct Tile {
+      int kv_head, kt, page;
+      float ks, vs;
+      bool first, valid;
+    };
+    // A cursor over the CTA's (task, key tile) sequence: a tile's block-table entry is requested
+    // three tiles before its copy is issued, which reaches into the next tasks.
+    xy_attn_task t{};
+    ReqInfo rq{};
+    int kt = 0, n_grab = 0;
+    const int32_t* bt = a.block_table;
+    int npages = 1;
+    bool open = false, out = false;
+    auto next_tile = [&]() {
+      Tile x{0, 0, 0, 1.f, 1.f, false, false};
+      if (!open || kt >= t.kt_hi) {
+        open = false;
+        if (out) return x;
+        int k = blockIdx.x;
+        if (n_grab > 0) {
+          if (lane == 0) k = static_cast<int>(gridDim.x) + atomicAdd(a.queue_head, 1);
+          k = __shfl_sync(0xffffffffu, k, 0);
+        }
+        ++n_grab;
+        if (k >= a.num_tasks) {
+          out = true;
+          return x;
+        }
+        const int ti = __ldg(a.queue + k);
+        t = a.tasks[ti];
+        rq = a.reqs[t.req];
+        rq.pad1 = (a.task_unit != nullptr && t.part >= 0) ? __ldg(a.task_unit + ti) : -1;
+        if (lane == 0) desc[(n_grab - 1) % kTaskSlots] = TaskDesc{t, rq};
+        kt = t.kt_lo;
+        npages = (rq.kv_len + rq.q_len + a.page_size - 1) >> a.page_shift;
+        bt = a.block_table + static_cast<int64_t>(rq.bt_row) * a.bt_stride;
+        open = true;
+        x.first = true;
+      }
+      x.valid = true;
+      x.kv_head = t.kv_head;
+      x.kt = kt;
+      if (has_box) x.page = __ldg(bt + min(kt * ppt + lane_page, npages - 1));  // past the end: the last page again
+      ++kt;
+      return x;
+    };
+    auto request_scales = [&](Tile& x) {
+      if constexpr (kFp8) {
+        if (x.valid && has_box) {
+          const int64_t si = static_cast<int64_t>(x.page) * a.num_kv_heads + x.kv_head;
+          x.ks = __ldg(a.k_scale + si);
+          x.vs = __ldg(a.v_scale + si);
+        }
+      }
+    };
+    uint32_t n_tasks = 0;
+    // Hands a task (or, with last, the end) to the consumers: description and Q rows.  The previous
+    // task's are in its consumers' registers by then (task_free).
+    auto publish = [&](bool last) {
+      if (n_tasks > 0 && !mbar_wait_block(task_free, (n_tasks - 1) & 1u, a.status)) {
+        report_timeout(a);
+        dead = true;
+        return;
+      }
+      if (!last) {
+        __syncwarp();
+        const TaskDesc& d = desc[n_tasks % kTaskSlots];
+        const int rows = d.t.ntok * G;
+        const uint16_t* q0 = a.q + static_cast<int64_t>(d.rq.q_start + d.t.tok0) * a.q_token_stride +
+                             static_cast<int64_t>(d.t.kv_head) * G * kHeadDim + (lane & 15) * 8;
+        const int rows8 = rows <= 8 ? 8 : 16;  // rows the consumers read; those past the task are zeros
+        for (int x = lane >> 4; x < rows8; x += 2) {
+          const bool ok = x < rows;
+          const uint16_t* src = ok ? q0 + static_cast<int64_t>(x / G) * a.q_token_stride + (x % G) * kHeadDim : q0;
+          cp_async_16(q_smem + x * 256u + (((lane & 15u) ^ (x & 7u)) << 4), src, ok);
+        }
+      } else if (lane == 0) {
+        desc[n_tasks % kTaskSlots].t.req = -1;
+      }
+      ++n_tasks;
+      cp_async_mbar_arrive(task_full);
+      if (lane == 0) mbar_arrive(task_full);
+    };
+    RingPos pos{0, 0};
+    int n_fill = 0;
+    uint32_t k_fills = 0, used = 0, fill_par = 0;
+    auto fill = [&](const CUtensorMap* map, const Tile& x, bool is_k) {
+      if (n_fill++ == a.debug_skip_fill) {  // failure-path test hook: this stage is never filled
+        pos.advance<kStages>();
+        return;
+      }
+      const uint32_t bit = 1u << pos.stage;
+      if (used & bit) {
+        // wait for the readers of this stage's previous fill
+        if (!mbar_wait_block(empty + 8 * pos.stage, (fill_par >> pos.stage) & 1u, a.status)) {
+          report_timeout(a);
+          dead = true;
+          return;
+        }
+        fill_par ^= bit;
+      }
+      used |= bit;
+      if constexpr (kFp8) {
+        if (is_k) {
+          float* slot = scale_ring + (k_fills % kScaleSlots) * 16;
+          ++k_fills;
+          if (has_box) {
+            slot[lane_page] = x.ks;
+            slot[8 + lane_page] = x.vs;
+          }
+          __syncwarp();
+        }
+      }
+      const uint32_t bar = full + 8 * pos.stage;
+      if (lane == 0) mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
+      __syncwarp();
+      if (has_box)
+        tma_load_4d_hint(ring + pos.stage * Cfg::kStageBytes + box_off, map, bar, kFp8 ? 0 : (lane & 1) * 64, 0, x.kv_head,
+                         x.page, policy);
+      pos.advance<kStages>();
+    };
+    Tile q0 = next_tile(), q1 = next_tile(), q2 = next_tile();
+    request_scales(q0);
+    request_scales(q1);
+    while (q0.valid && !dead) {
+      const Tile cur = q0;
+      if (cur.first) publish(false);
+      q0 = q1;
+      q1 = q2;
+      q2 = next_tile();
+      request_scales(q1);
+      if (!dead) fill(&k_map, cur, true);
+      if (!dead) fill(&v_map, cur, false);
+      dead = __any_sync(0xffffffffu, dead);
+    }
+    if (!dead) publish(true);
+    // No copy of this CTA may still be in flight when it exits (immediate on the normal path).
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    for (int s = 0; s < kStages; ++s)
+      if (used & (1u << s)) mbar_wait_block(full + 8 * s, (fill_par >> s) & 1u, a.status);
+  } else {
+    // ================================== consumers =========================================
+    const float scale_log2 = a.sm_scale * 1.4426950408889634f;
+    const StreamRing sr{ring, Cfg::kStageBytes, full, empty};
+    auto q_addr = [&](uint32_t row, uint32_t ch) { return q_smem + row * 256u + ((ch ^ (row & 7u)) << 4); };
+    RingPos pos{0, 0};
+    bool dead = false;
+    uint32_t tile_seq = 0;
+    for (uint32_t n = 0;; ++n) {
+      if (!dead && !mbar_wait_block(task_full, n & 1u, a.status)) {
+        report_timeout(a);
+        dead = true;
+      }
+      // All warps leave together (a warp whose wait ran out must not keep away from the barriers of
+      // a task the others have started); the barrier also keeps the exchange areas of two tasks apart.
+      if (dead) *s_dead = 1;
+      named_bar_sync(1, kWarpsS * 32);
+      if (*reinterpret_cast<volatile int*>(s_dead) != 0) break;
+      TaskView tv;
+      tv.t = desc[n % kTaskSlots].t;
+      tv.rq = desc[n % kTaskSlots].rq;
+      if (tv.t.req < 0) break;
+      const int unit = tv.rq.pad1;
+      tv.G = G;
+      tv.rows = tv.t.ntok * G;
+      auto take_q = [&](auto& w) {
+        w.init();
+        w.load_q(q_addr, lane);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(task_free);  // description and Q rows are in registers
+      };
+      if (tv.rows <= 8) {
+        StreamWarp<kWarpsS, 1, kFp8> w;
+        take_q(w);
+        stream_task<kWarpsS, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, warp, 1,
+                                               s_last);
+      } else {
+        StreamWarp<kWarpsS, 2, kFp8> w;
+        take_q(w);
+        stream_task<kWarpsS, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, warp, 1,
+                                               s_last);
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && blockIdx.x < static_cast<unsigned>(a.num_workers)) {
+    unsigned long long now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    unsigned long long* w = a.worker_times + 4 * blockIdx.x;
+    w[0] = t_start;
+    w[1] = now;
+    w[2] = 0ull;
+    w[3] = now - t_start;
+  }
+}
+
+}  // namespace
+
+// Up to two CTAs per worker (SM), never more than tasks.
+cudaError_t launch_stream(const RunArgs& a, int64_t num_pages, MetaLaunchCache* cache, cudaStream_t s) {
+  const bool fp8 = a.kv_fp8 != 0;
+  const int smem = fp8 ? StreamCfg<true>::kSmem : StreamCfg<false>::kSmem;
+  auto kernel = fp8 ? stream_attention_kernel<true> : stream_attention_kernel<false>;
+  if (!cache->attr_set[4 + fp8]) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    cache->attr_set[4 + fp8] = true;
+  }
+  const cudaError_t e = pool_maps(a, num_pages, cache);
+  if (e != cudaSuccess) return e;
+  const int grid = a.num_tasks < 2 * a.num_workers ? a.num_tasks : 2 * a.num_workers;
+  kernel<<<grid, kThreadsS, smem, s>>>(a, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
+                                       *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
+  return cudaGetLastError();
+}
+
+}  // namespace xy

@@ -128,7 +128,7 @@ struct RunArgs {
   // dynamic dealing: workers take the next task of `queue` with an atomic counter
   const int32_t* queue;
   int32_t* queue_head;
-  int32_t num_tasks, dynamic;
+  int32_t num_tasks, dynamic, num_workers;
   // split units whose last finishing task merges them inside the kernel (streaming units)
   const int32_t* task_unit;              // per task: unit index or -1 (null: no such unit)
   const xy_attn_merge_unit* units;
