@@ -389,6 +389,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.queue_head = ctx->d_status + kStatusQueueHead;  // second cache line of the status block
   a.num_tasks = static_cast<int32_t>(p.tasks.size());
   a.num_workers = ctx->num_workers;
+  a.num_units = static_cast<int32_t>(p.merges.size());
   // Balanced plans are dealt dynamically by the meta-kernel; paper-mode plans keep the static
   // Task-Table (each worker walks its own list), as does the reference kernel.
   a.dynamic = (cfg.plan_mode == XY_PLAN_BALANCED && cfg.kernel != XY_KERNEL_REFERENCE) ? 1 : 0;
@@ -399,9 +400,11 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.k_scale = k_scale;
   a.v_scale = v_scale;
   a.kv_fp8 = fp8 ? 1 : 0;
-  // Every run starts with a clean status word, queue head and unit counters (one memset): a run
-  // after a device-side timeout is an ordinary run.  The sticky record in front of them is kept.
-  XY_CUDA(ctx, cudaMemsetAsync(a.status, 0, (kStatusUnitCounts + (in_kernel_merges ? p.merges.size() : 0)) * sizeof(int32_t), s));
+  // Every run starts with a clean status word, queue head and unit counters: the last CTA of the run
+  // before has left them so, after a device-side timeout too.  (The CTA-pair kernel leaves that to a
+  // memset.)  The sticky record in front of them is kept.
+  if (ctx->pair)
+    XY_CUDA(ctx, cudaMemsetAsync(a.status, 0, (kStatusUnitCounts + (in_kernel_merges ? p.merges.size() : 0)) * sizeof(int32_t), s));
 
   const bool timed = ctx->timing && ctx->timed_runs < kMaxTimedRuns;
   if (timed) {

@@ -423,9 +423,6 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
 
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    unsigned long long now;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    a.worker_times[4 * blockIdx.x] = now;
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&bars->full[s]), 1);
       mbar_init(smem_u32(&bars->empty[s]), kConsumerWarps);
@@ -449,13 +446,23 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     tmem_alloc(smem_u32(&ub->tmem_base), kTmemCols);
     tmem_relinquish();
   }
+  if (warp == kConsumerWarps && lane == 0) {
+    prefetch_tensormap(&k_map);
+    prefetch_tensormap(&v_map);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_dependency_wait();
+  if (threadIdx.x == 0) {
+    unsigned long long now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    a.worker_times[4 * blockIdx.x] = now;
+  }
   const uint32_t tmem = kUmma ? __shfl_sync(0xffffffffu, ub->tmem_base, 0) : 0u;
 
-  const int t_begin = a.worker_off[blockIdx.x], t_end = a.worker_off[blockIdx.x + 1];
   const bool dynamic = a.dynamic != 0;
+  const int t_begin = dynamic ? 0 : a.worker_off[blockIdx.x], t_end = dynamic ? 0 : a.worker_off[blockIdx.x + 1];
   // Every role but the producer reads its task sequence here: the worker's own Task-Table list
   // (static dealing) or the indices the producer publishes (dynamic dealing).  Warp-uniform.
   int seq_static = t_begin;
@@ -485,8 +492,6 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
     if (warp == kConsumerWarps && lane == 0) {
       // ================================ producer =======================================
-      prefetch_tensormap(&k_map);
-      prefetch_tensormap(&v_map);
       Pipe pipe{0, 0};
       bool dead = false;
       // Who read each stage last (bit set: the tcgen05 path) and the parity to wait for on each
@@ -1245,6 +1250,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       a.worker_times[4 * blockIdx.x + 3] = acct_ns[1];
     }
   }
+  grid_launch_dependents();
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1256,6 +1262,8 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
+  __shared__ int s_flag;
+  end_of_run(a, &s_flag);
 }
 
 #include "kernel_pair.inc"
@@ -1344,9 +1352,9 @@ cudaError_t launch_meta(const RunArgs& a, int64_t num_pages, bool umma, MetaLaun
   const cudaError_t e = pool_maps(a, num_pages, cache);
   if (e != cudaSuccess) return e;
   MetaParams P{a};
-  kernel<<<a.num_workers, kThreads, kSmemTotal, s>>>(P, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
-                                                     *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
-  return cudaGetLastError();
+  const int grid = a.dynamic && a.num_tasks < a.num_workers ? a.num_tasks : a.num_workers;
+  return launch_after(kernel, dim3(grid), kThreads, kSmemTotal, s, P, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
+                      *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
 }
 
 // Dense tasks on CTA pairs: `a.queue` / `a.num_tasks` / `a.queue_head` describe the dense part of the

@@ -67,9 +67,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
   const uint32_t full = smem_u32(bars), empty = full + 8 * kStages, task_full = empty + 8 * kStages, task_free = task_full + 8;
 
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  unsigned long long t_start = 0;
   if (threadIdx.x == 0) {
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
     for (int s = 0; s < kStages; ++s) {
       mbar_init(full + 8 * s, 1);
       mbar_init(empty + 8 * s, kWarpsS);
@@ -79,15 +77,18 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     *s_dead = 0;
     fence_mbar_init();
   }
+  if (warp == kWarpsS && lane == 0) {
+    prefetch_tensormap(&k_map);
+    prefetch_tensormap(&v_map);
+  }
   __syncthreads();
+  grid_dependency_wait();
+  unsigned long long t_start = 0;
+  if (threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
   const int G = a.num_q_heads / a.num_kv_heads;
 
   if (warp == kWarpsS) {
     // ================================== producer ==========================================
-    if (lane == 0) {
-      prefetch_tensormap(&k_map);
-      prefetch_tensormap(&v_map);
-    }
     bool dead = false;
     if ((ring & 1023u) != 0) {  // the TMA swizzle needs it; dynamic shared memory starts there
       report_timeout(a);
@@ -284,6 +285,9 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       }
     }
   }
+  // The next launch's CTAs come in as these leave.  (Letting them in from the start filled the SMs
+  // unevenly: a CTA took whichever slot was free first, 55.3 -> 60.4 us for 64 requests on an fp8 cache.)
+  grid_launch_dependents();
   __syncthreads();
   if (threadIdx.x == 0 && blockIdx.x < static_cast<unsigned>(a.num_workers)) {
     unsigned long long now;
@@ -294,6 +298,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     w[2] = 0ull;
     w[3] = now - t_start;
   }
+  end_of_run(a, s_last);
 }
 
 }  // namespace
@@ -312,9 +317,8 @@ cudaError_t launch_stream(const RunArgs& a, int64_t num_pages, MetaLaunchCache* 
   const cudaError_t e = pool_maps(a, num_pages, cache);
   if (e != cudaSuccess) return e;
   const int grid = a.num_tasks < 2 * a.num_workers ? a.num_tasks : 2 * a.num_workers;
-  kernel<<<grid, kThreadsS, smem, s>>>(a, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
-                                       *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
-  return cudaGetLastError();
+  return launch_after(kernel, dim3(grid), kThreadsS, smem, s, a, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
+                      *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
 }
 
 }  // namespace xy

@@ -6,6 +6,7 @@
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
 
+#include "ptx.cuh"
 #include "xy_kernels.h"
 
 namespace xy {
@@ -126,6 +127,8 @@ constexpr int kMergeLaneParts = 8;     // partials per lane on the shuffle path:
 // worker); that path holds eight partial rows in registers and is kept out of the common kernel.
 template <bool kWide>
 __global__ void __launch_bounds__(128) merge_units_kernel(MergeArgs a) {
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
   const xy_attn_merge_unit u = a.units[blockIdx.x];
   const int G = a.num_q_heads / a.num_kv_heads;
   const int rows = u.ntok * G;
@@ -363,6 +366,8 @@ __global__ void __launch_bounds__(128) append_kv_kernel(const uint16_t* qkv, int
                                                         const int32_t* block_table, int bt_stride,
                                                         const ReqInfo* reqs, int num_reqs, int Hq, int Hkv,
                                                         int page_size, int page_shift) {
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
   const int t = blockIdx.x;
   int lo = 0, hi = num_reqs - 1;  // last request whose start position is <= t
   while (lo < hi) {
@@ -392,10 +397,8 @@ cudaError_t launch_append_kv(const uint16_t* qkv, int64_t qkv_token_stride, uint
                              const int32_t* block_table, int bt_stride, const ReqInfo* reqs, int num_reqs,
                              int total_q, int Hq, int Hkv, int page_size, int page_shift, cudaStream_t s) {
   if (total_q == 0) return cudaSuccess;
-  append_kv_kernel<<<total_q, 128, 0, s>>>(qkv, qkv_token_stride, k_pool, v_pool, page_stride, head_stride,
-                                           token_stride, block_table, bt_stride, reqs, num_reqs, Hq, Hkv,
-                                           page_size, page_shift);
-  return cudaGetLastError();
+  return launch_after(append_kv_kernel, dim3(total_q), 128, 0, s, qkv, qkv_token_stride, k_pool, v_pool, page_stride, head_stride,
+                      token_stride, block_table, bt_stride, reqs, num_reqs, Hq, Hkv, page_size, page_shift);
 }
 
 cudaError_t launch_reference(const RunArgs& a, int num_workers, cudaStream_t s) {
@@ -409,10 +412,8 @@ cudaError_t launch_merge_units(const MergeArgs& a, int num_units, int max_rows, 
   int by = (max_rows + 3) / 4;
   by = by < 1 ? 1 : (by > kMergeBlocksPerUnit ? kMergeBlocksPerUnit : by);
   if (max_parts > 32)
-    merge_units_kernel<true><<<dim3(num_units, by), 128, 0, s>>>(a);
-  else
-    merge_units_kernel<false><<<dim3(num_units, by), 128, 0, s>>>(a);
-  return cudaGetLastError();
+    return launch_after(merge_units_kernel<true>, dim3(num_units, by), 128, 0, s, a);
+  return launch_after(merge_units_kernel<false>, dim3(num_units, by), 128, 0, s, a);
 }
 
 cudaError_t launch_merge_plain(const float* o_part, const float* lse_part, int num_splits,

@@ -71,6 +71,13 @@ __device__ __forceinline__ bool elect_one() {
   return ok != 0;
 }
 
+// Programmatic dependent launch.  A kernel launched with launch_after (xy_kernels.h) may start while
+// its predecessor on the stream is still running: it sets up its barriers and tensor memory, and
+// grid_dependency_wait holds it until the predecessor has completed and its writes are visible.
+// grid_launch_dependents lets the successor be scheduled once every CTA of this grid has said so.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -53,6 +53,29 @@ __device__ __forceinline__ void report_timeout(const RunArgs& a) {
   atomicExch(a.status + kStatusSticky, XY_ERR_DEVICE_TIMEOUT);
 }
 
+// Called by all threads of a CTA that is through with its tasks, behind a barrier.  The last CTA of
+// the grid returns the status block to zeros for the next run (so that no memset has to stand between
+// two runs) and clears the time stamps of workers that had no CTA.
+__device__ __forceinline__ void end_of_run(const RunArgs& a, int* s_flag) {
+  if (threadIdx.x == 0) {
+    __threadfence();
+    *s_flag = atomicAdd(a.status + kStatusExits, 1) == static_cast<int>(gridDim.x) - 1 ? 1 : 0;
+  }
+  __syncthreads();
+  if (*s_flag == 0) return;
+  __threadfence();
+  const bool failed = *const_cast<volatile int32_t*>(a.status) != 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a.status[0] = 0;
+    a.status[kStatusExits] = 0;
+    *a.queue_head = 0;
+  }
+  if (failed)  // otherwise every counter was put back by the task that completed its unit
+    for (int i = threadIdx.x; i < a.num_units; i += blockDim.x) a.unit_count[i] = 0;
+  for (int w = gridDim.x * 4 + threadIdx.x; w < a.num_workers * 4; w += blockDim.x) a.worker_times[w] = 0ull;
+}
+
 // A ring of shared-memory stages as its readers see it.
 struct RingPos {
   int stage;
@@ -606,7 +629,9 @@ __device__ __forceinline__ void stream_task(const RunArgs& a, const TaskView& tv
     named_bar_sync(bar_id, kWarps * 32);
     if (warp == 0 && lane == 0) {
       const int ns = a.units[unit].nsplit;
-      *s_last = atomicAdd(a.unit_count + unit, 1) == ns - 1 ? 1 : 0;
+      const bool last = atomicAdd(a.unit_count + unit, 1) == ns - 1;
+      if (last) a.unit_count[unit] = 0;
+      *s_last = last ? 1 : 0;
     }
     named_bar_sync(bar_id, kWarps * 32);
     if (*s_last) {

@@ -15,11 +15,14 @@ constexpr int kStreamRowsMax = 16;
 // The status block, indexed from the word the kernels receive as `status`:
 //   [0]   the current run's status, polled by every bounded wait
 //   [16]  the queue head of dynamic dealing (its own cache line)
+//   [18]  CTAs that have finished
 //   [32 ..] one completion counter per merge unit
-// all of which one memset clears when a run starts; and in front of them, untouched by that,
+// all of which are zero when a run starts: the last CTA of a run puts them back (end_of_run; the
+// CTA-pair kernel has them cleared by a memset instead); and in front of them, untouched by that,
 //   [-8]  the sticky record of failures that xy_attn_device_status reports and clears
 //   [-7]  the number of polls after which a bounded wait gives up (ptx.cuh reads the same word).
 constexpr int kStatusQueueHead = 16;
+constexpr int kStatusExits = 18;
 constexpr int kStatusUnitCounts = 32;
 constexpr int kStatusSticky = -8;
 constexpr int kStatusWaitLimit = -7;
@@ -128,11 +131,11 @@ struct RunArgs {
   // dynamic dealing: workers take the next task of `queue` with an atomic counter
   const int32_t* queue;
   int32_t* queue_head;
-  int32_t num_tasks, dynamic, num_workers;
+  int32_t num_tasks, dynamic, num_workers, num_units;
   // split units whose last finishing task merges them inside the kernel (streaming units)
   const int32_t* task_unit;              // per task: unit index or -1 (null: no such unit)
   const xy_attn_merge_unit* units;
-  int32_t* unit_count;                   // per unit: tasks finished so far (returns to 0 by itself)
+  int32_t* unit_count;                   // per unit: tasks finished so far
   // fp8 KV cache: k_pool / v_pool hold e4m3 bytes (strides in bytes) and these are the fp32 scales
   // [pages, Hkv] of K and V
   const float* k_scale;
