@@ -92,11 +92,12 @@ EXPORTS = (
 )
 
 _lib = None
+_fast = None  # native forms of the per-step calls (csrc/fastcall.cpp)
 
 
 def load() -> ctypes.CDLL:
     """Loads libxy_attn.so (built in-tree by `python -m paper_2412_18106_b200.build`)."""
-    global _lib
+    global _lib, _fast
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -139,6 +140,12 @@ def load() -> ctypes.CDLL:
     for name in EXPORTS:
         if name != "xy_attn_last_error":
             getattr(L, name).restype = ctypes.c_int
+    from . import _fastcall  # built beside the library; a missing one fails loudly too
+    from . import gemm
+    gemm.declare(L)
+    _fastcall.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
+        L.xy_attn_plan, L.xy_attn_run, L.xy_attn_run_fp8kv, L.xy_attn_append_kv, L.xy_gemm_run_ws)))
+    _fast = _fastcall
     _lib = L
     return L
 
@@ -174,11 +181,14 @@ class XYAttn:
         if rc != XY_OK:
             raise XYAttnError(rc, "xy_attn_create failed")
         self.info = xy_attn_plan_info()
+        self._h, self._d, self._info_addr = self._ctx.value, int(head_dim), ctypes.addressof(self.info)
+        self._host_only = device < 0
 
     def close(self):
         if self._ctx and self._ctx.value:
             self.lib.xy_attn_destroy(self._ctx)
             self._ctx = ctypes.c_void_p(0)
+            self._h = 0
 
     def __del__(self):
         try:
@@ -193,6 +203,11 @@ class XYAttn:
     # -- xy_attn_plan
     def plan(self, q_len: Sequence[int], kv_len: Sequence[int], mask_kind: Sequence[int],
              parent_off: Sequence[int], parents=None, stream=None) -> xy_attn_plan_info:
+        rc = _fast.plan(self._h, q_len, kv_len, mask_kind, parent_off, parents,
+                        (0 if self._host_only else None) if stream is None else stream.cuda_stream, self._info_addr)
+        if rc is not None:
+            self._check(rc)
+            return self.info
         R = len(q_len)
         reqs = (xy_attn_request * max(R, 1))()
         for r in range(R):
@@ -243,6 +258,10 @@ class XYAttn:
     def run(self, q: torch.Tensor, k_pool: torch.Tensor, v_pool: torch.Tensor,
             block_table: torch.Tensor, sm_scale: float, o: torch.Tensor, lse: torch.Tensor,
             tree_mask: Optional[torch.Tensor] = None, stream=None) -> None:
+        rc = _fast.run(self._h, self._d, q, k_pool, v_pool, block_table, sm_scale, o, lse, tree_mask,
+                       None if stream is None else stream.cuda_stream)
+        if rc is not None:
+            return self._check(rc)
         for t in (q, k_pool, v_pool, block_table, o, lse):
             if not t.is_cuda:
                 raise XYAttnError(XY_ERR_INVALID_ARG, "run needs CUDA tensors (there is no CPU path)")
@@ -264,6 +283,10 @@ class XYAttn:
                   v_scale: torch.Tensor, block_table: torch.Tensor, sm_scale: float, o: torch.Tensor,
                   lse: torch.Tensor, tree_mask: Optional[torch.Tensor] = None, stream=None) -> None:
         """k_pool / v_pool uint8 (e4m3 bytes) [P, Hkv, B, D], k_scale / v_scale fp32 [P, Hkv]."""
+        rc = _fast.run(self._h, self._d, q, k_pool, v_pool, block_table, sm_scale, o, lse, tree_mask,
+                       None if stream is None else stream.cuda_stream, k_scale, v_scale)
+        if rc is not None:
+            return self._check(rc)
         for t in (q, k_pool, v_pool, k_scale, v_scale, block_table, o, lse):
             if not t.is_cuda:
                 raise XYAttnError(XY_ERR_INVALID_ARG, "run_fp8kv needs CUDA tensors (there is no CPU path)")
@@ -287,6 +310,10 @@ class XYAttn:
     def append_kv(self, qkv: torch.Tensor, k_pool: torch.Tensor, v_pool: torch.Tensor, block_table: torch.Tensor,
                   stream=None) -> None:
         """Copies the K / V heads of the fused bf16 [T, Hq + 2 Hkv, D] tensor into the paged cache."""
+        rc = _fast.append_kv(self._h, self._d, qkv, k_pool, v_pool, block_table,
+                             None if stream is None else stream.cuda_stream)
+        if rc is not None:
+            return self._check(rc)
         for t in (qkv, k_pool, v_pool, block_table):
             if not t.is_cuda:
                 raise XYAttnError(XY_ERR_INVALID_ARG, "append_kv needs CUDA tensors (there is no CPU path)")

@@ -3,7 +3,8 @@
     python -m paper_2412_18106_b200.build [--force]
 
 The shared object lands beside this file (libxy_attn.so); nvcc cross-compiles
-without a GPU.
+without a GPU.  The binding's native calls (_fastcall.so, a CPython extension against
+torch's headers) are compiled beside it with the host compiler.
 """
 from __future__ import annotations
 
@@ -16,6 +17,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libxy_attn.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -38,7 +40,42 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _fastcall_stale() -> bool:
+    if not os.path.exists(FASTCALL):
+        return True
+    deps = [os.path.join(CSRC, "fastcall.cpp")] + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    return any(os.path.getmtime(d) > os.path.getmtime(FASTCALL) for d in deps)
+
+
+def start_fastcall():
+    """Starts the compiler on the CPython extension; returns (process, temporary output)."""
+    import sysconfig
+
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = FASTCALL + ".tmp.%d" % os.getpid()
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-w",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-I", os.path.join(ROOT, "include"), "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-I", sysconfig.get_paths()["include"], "-I", "/usr/local/cuda/include",
+           os.path.join(CSRC, "fastcall.cpp"), "-o", tmp, "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT), tmp
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    fast = start_fastcall() if force or _fastcall_stale() else None
+    try:
+        return _build_lib(force, verbose)
+    finally:
+        if fast is not None:
+            out = fast[0].communicate()[0].decode()
+            if fast[0].returncode != 0:
+                raise RuntimeError("compiling fastcall.cpp failed:\n" + out[-3000:])
+            os.replace(fast[1], FASTCALL)
+
+
+def _build_lib(force: bool, verbose: bool) -> str:
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
