@@ -14,7 +14,9 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <mutex>
 
 #include "ptx.cuh"
 #include "xy_gemm.h"
@@ -651,6 +653,279 @@ smooth_gemm_splitk_kernel(const SplitKParams P, const __grid_constant__ CUtensor
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// Weight-major variant for up to about a thousand tokens: the product is computed transposed.  A CTA
+// pair multiplies 256 rows of W (the 256-row side of tcgen05.mma.cta_group::2, 128 in each CTA) by all
+// tokens of its token tile, up to 512, which are the columns: one accumulator of up to 256 columns or
+// two.  What bounds a CTA here is the 64 bytes per clock an SM takes in: a K chunk costs 16 KiB of W and
+// 64 bytes per token, against 32 KiB for a 128 x 128 tile, no token rows are padded beyond a multiple
+// of 16, and W is read once.  When the tiles are fewer than the SMs, `splits` pairs of a cluster share
+// a tile's K: every pair leaves the fp32 sums of the tokens it does not own in the caller's scratch
+// (through L2), and after a cluster barrier adds the others' sums of its own tokens in a fixed order.
+struct SwapParams {
+  uint16_t* c;
+  int64_t ldc;
+  int32_t M, N, K;
+  int32_t m_tiles, n_tiles;  // tiles of `tok` tokens x 256 rows of W
+  int32_t tok, halves;       // tok = halves * (columns of one MMA)
+  int32_t stages, splits, chunks_per_split, bufs;
+  uint32_t tmem_cols;
+  float4* ws;  // splits > 1: [tile][split][rank][tok / 4][128]
+};
+constexpr int kSwapMaxStages = 12;
+constexpr int kSwapMaxSplits = 4;  // a cluster of eight CTAs
+constexpr int kSwapRing = 212992;  // bytes of ring at most
+constexpr int kSwapSmem = 1024 + kSwapRing + 512;
+
+struct __align__(8) SwapBarriers {
+  uint64_t full[kSwapMaxStages], empty[kSwapMaxStages];
+  uint64_t acc_full[2], acc_empty[2];
+  uint32_t tmem_base;
+};
+
+// Stores 16 tokens of this thread's output column n: neighbouring lanes swap values so that each
+// writes two columns of every other token.
+__device__ __forceinline__ void swap_store16(const SwapParams& P, const float (&v)[16], int m, int m_end, int n, int lane) {
+#pragma unroll
+  for (int j = 0; j < 16; j += 2) {
+    const bool odd = lane & 1;
+    const float got = __shfl_xor_sync(0xffffffffu, odd ? v[j] : v[j + 1], 1);
+    const int row = m + j + (odd ? 1 : 0);
+    if (row < m_end && n < P.N)
+      *reinterpret_cast<uint32_t*>(P.c + static_cast<int64_t>(row) * P.ldc + (n & ~1)) =
+          odd ? pack_bf16(got, v[j + 1]) : pack_bf16(v[j], got);
+  }
+}
+
+__global__ void __launch_bounds__(kGemmThreads, 1)
+smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_constant__ CUtensorMap a_map,
+                        const __grid_constant__ CUtensorMap w_map) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  SwapBarriers* bars = reinterpret_cast<SwapBarriers*>(smem_raw + (base - smem_u32(smem_raw)) + kSwapRing);
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const uint32_t ctarank = cluster_ctarank();
+  const uint32_t leader_rank = ctarank & ~1u;
+  const int rank = static_cast<int>(ctarank & 1u), split = static_cast<int>(ctarank >> 1);
+  const bool leader = rank == 0;
+  const uint16_t pair_mask = static_cast<uint16_t>(3u << leader_rank);
+  const volatile int32_t* status = &g_gemm_status;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < P.stages; ++s) {
+      mbar_init(smem_u32(&bars->full[s]), 1);   // leader: one arming arrive, bytes of both CTAs
+      mbar_init(smem_u32(&bars->empty[s]), 1);  // each CTA: one commit
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&bars->acc_full[b]), 1);   // each CTA: one commit
+      mbar_init(smem_u32(&bars->acc_empty[b]), 8);  // leader: four epilogue warps of each CTA
+    }
+    fence_mbar_init();
+  }
+  const int k_chunks = (P.K + kChunkK - 1) / kChunkK;
+  const int num_tiles = P.m_tiles * P.n_tiles;
+  const int cluster = static_cast<int>(blockIdx.x) / (2 * P.splits), clusters = static_cast<int>(gridDim.x) / (2 * P.splits);
+  const int kc_lo = split * P.chunks_per_split, kc_hi = min(k_chunks, kc_lo + P.chunks_per_split);
+  const int nh = P.tok / P.halves;  // columns of one MMA
+  const uint32_t stage_bytes = kABytes + P.tok * 64;
+  if (warp == 0 && lane == 0) {
+    prefetch_tensormap(&a_map);
+    prefetch_tensormap(&w_map);
+    // The first weights start on their way to L2 while the kernel before this one is still running.
+    const int n0 = (cluster / P.m_tiles) * 256 + 128 * rank;
+    for (int i = 0; i < P.stages && kc_lo + i < kc_hi; ++i) tma_prefetch_2d(&w_map, (kc_lo + i) * kChunkK, n0);
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(&bars->tmem_base), P.tmem_cols);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // the peer's barriers exist before anything arrives on them
+  tc_fence_after();
+  grid_dependency_wait();
+  const uint32_t tmem = bars->tmem_base;
+  auto wait_cluster = [&](uint32_t bar, uint32_t parity) {
+    for (uint32_t i = 0; i < (1u << 22); ++i) {
+      if (mbar_try_wait_cluster(bar, parity)) return true;
+      if ((i & 4095u) == 4095u && status[0] != 0) return false;
+    }
+    return false;
+  };
+
+  bool ok = true;  // epilogue warps: this CTA's sums are there
+  if (warp == 0 && lane == 0) {
+    // ---------------------------------------------------------------- producer (both CTAs)
+    const uint32_t full_leader = cluster_map(smem_u32(&bars->full[0]), leader_rank);
+    uint32_t s = 0, phase = 1;
+    bool dead = false;
+    for (int t = cluster; t < num_tiles && !dead; t += clusters) {
+      const int m0 = (t % P.m_tiles) * P.tok, n0 = (t / P.m_tiles) * 256 + 128 * rank;
+      for (int kc = kc_lo; kc < kc_hi; ++kc) {
+        // (a fresh barrier's previous phase counts as complete: the first round of stages passes)
+        if (!wait_cluster(smem_u32(&bars->empty[s]), phase)) {
+          atomicExch(&g_gemm_status, XY_ERR_DEVICE_TIMEOUT);
+          dead = true;
+          break;
+        }
+        if (leader) mbar_arrive_expect_tx(smem_u32(&bars->full[s]), 2 * stage_bytes);
+        const uint32_t dst = base + s * stage_bytes, bar = full_leader + s * 8u;
+        tma_load_2d_pair(dst, &w_map, bar, kc * kChunkK, n0);  // rows past N arrive as zeros
+        for (int h = 0; h < P.halves; ++h)                      // rows past M likewise
+          tma_load_2d_pair(dst + kABytes + h * nh * 64, &a_map, bar, kc * kChunkK, m0 + h * nh + rank * (nh / 2));
+        if (++s == static_cast<uint32_t>(P.stages)) {
+          s = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+    grid_launch_dependents();
+  } else if (warp == 1 && leader) {
+    // ---------------------------------------------------------------- MMA issuer (leader)
+    constexpr uint64_t kDescHi = static_cast<uint64_t>((1024u >> 4) | (1u << 14) | (2u << 29)) << 32;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((static_cast<uint32_t>(nh) >> 3) << 17) | ((256u >> 4) << 24);
+    const bool elected = elect_one();
+    uint32_t s = 0, phase = 0, local = 0;
+    bool dead = false;
+    for (int t = cluster; t < num_tiles && !dead; t += clusters, ++local) {
+      const uint32_t buf = P.bufs == 2 ? local & 1u : 0u, use = P.bufs == 2 ? local >> 1 : local;
+      if (use > 0 && !wait_cluster(smem_u32(&bars->acc_empty[buf]), (use - 1) & 1u)) {
+        atomicExch(&g_gemm_status, XY_ERR_DEVICE_TIMEOUT);
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem + buf * P.tok;
+      for (int kc = kc_lo; kc < kc_hi; ++kc) {
+        if (!wait_cluster(smem_u32(&bars->full[s]), phase)) {
+          atomicExch(&g_gemm_status, XY_ERR_DEVICE_TIMEOUT);
+          dead = true;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t w_lo = (((base + s * stage_bytes) >> 4) & 0x3FFFu) | (1u << 16);
+        const uint32_t a_lo = (((base + s * stage_bytes + kABytes) >> 4) & 0x3FFFu) | (1u << 16);
+        if (elected) {
+          for (int h = 0; h < P.halves; ++h) {
+#pragma unroll
+            for (int k16 = 0; k16 < 4; ++k16)
+              umma2_ss64(d_tmem + h * nh, kDescHi | (w_lo + k16 * 2), kDescHi | (a_lo + h * nh * 4 + k16 * 2), idesc,
+                         (kc > kc_lo || k16) ? 1u : 0u);
+          }
+          umma2_commit_mask(smem_u32(&bars->empty[s]), pair_mask);  // the stage is free in both CTAs
+        }
+        if (++s == static_cast<uint32_t>(P.stages)) {
+          s = 0;
+          phase ^= 1u;
+        }
+      }
+      if (!dead && elected) umma2_commit_mask(smem_u32(&bars->acc_full[buf]), pair_mask);
+    }
+  } else if (warp >= 2) {
+    // ---------------------------------------------------------------- epilogue (both CTAs)
+    const int q = warp & 3, row = q * 32 + lane;
+    const uint32_t acc_empty_leader = cluster_map(smem_u32(&bars->acc_empty[0]), leader_rank);
+    uint32_t local = 0;
+    for (int t = cluster; t < num_tiles; t += clusters, ++local) {
+      const uint32_t buf = P.bufs == 2 ? local & 1u : 0u, use = P.bufs == 2 ? local >> 1 : local;
+      if (!wait_cluster(smem_u32(&bars->acc_full[buf]), use & 1u)) {
+        atomicExch(&g_gemm_status, XY_ERR_DEVICE_TIMEOUT);
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const int m0 = (t % P.m_tiles) * P.tok, n = (t / P.m_tiles) * 256 + 128 * rank + row;
+      const int m_end = min(P.M, m0 + P.tok);
+      const uint32_t t_acc = tmem + (static_cast<uint32_t>(q * 32) << 16) + buf * P.tok;
+      if (P.splits == 1) {
+#pragma unroll 2
+        for (int c0 = 0; c0 < P.tok && m0 + c0 < m_end; c0 += 16) {
+          uint32_t v[16];
+          tmem_ld_32x32b_x16(t_acc + c0, v);
+          tmem_wait_ld();
+          float f[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+          swap_store16(P, f, m0 + c0, m_end, n, lane);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (leader) mbar_arrive(smem_u32(&bars->acc_empty[buf])); else mbar_arrive_remote(acc_empty_leader + buf * 8u);
+        }
+      } else {
+        // (one tile per cluster) the sums of the tokens that other pairs own -> scratch
+        const int own = (((m_end - m0 + P.splits - 1) / P.splits + 15) / 16) * 16;  // tokens per pair
+        float4* mine = P.ws + (static_cast<int64_t>((t * P.splits + split) * 2 + rank) * (P.tok / 4)) * 128 + row;
+#pragma unroll 2
+        for (int c0 = 0; c0 < P.tok && m0 + c0 < m_end; c0 += 16) {
+          if (c0 / own == split) continue;
+          uint32_t v[16];
+          tmem_ld_32x32b_x16(t_acc + c0, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int g = 0; g < 4; ++g)
+            __stcg(mine + (c0 / 4 + g) * 128, make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]),
+                                                          __uint_as_float(v[4 * g + 2]), __uint_as_float(v[4 * g + 3])));
+        }
+      }
+    }
+  }
+  if (P.splits > 1) {
+    __syncwarp();
+    cluster_sync_all();
+    if (warp >= 2 && ok) {
+      const int q = warp & 3, row = q * 32 + lane, t = cluster;
+      const int m0 = (t % P.m_tiles) * P.tok, n = (t / P.m_tiles) * 256 + 128 * rank + row;
+      const int m_end = min(P.M, m0 + P.tok);
+      const int own = (((m_end - m0 + P.splits - 1) / P.splits + 15) / 16) * 16;
+      const uint32_t t_acc = tmem + (static_cast<uint32_t>(q * 32) << 16);
+      const int64_t slot = static_cast<int64_t>(P.tok / 4) * 128;
+      const float4* part = P.ws + (static_cast<int64_t>(t * P.splits) * 2 + rank) * slot + row;
+      tc_fence_after();
+      for (int c0 = split * own; c0 < (split + 1) * own && m0 + c0 < m_end; c0 += 16) {
+        uint32_t v[16];
+        tmem_ld_32x32b_x16(t_acc + c0, v);
+        float4 x[kSwapMaxSplits - 1][4];
+#pragma unroll
+        for (int o = 0; o < kSwapMaxSplits - 1; ++o)
+          if (o < P.splits - 1) {
+            const float4* src = part + (o < split ? o : o + 1) * 2 * slot + c0 / 4 * 128;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) x[o][g] = __ldcg(src + g * 128);
+          }
+        tmem_wait_ld();
+        float f[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) f[j] = 0.f;
+        // in the order of the splits, this pair's own sums in their place
+#pragma unroll
+        for (int o = 0; o < kSwapMaxSplits; ++o) {
+          if (o == split) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) f[j] += __uint_as_float(v[j]);
+          }
+          if (o < kSwapMaxSplits - 1 && o < P.splits - 1) {
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              f[4 * g] += x[o][g].x;
+              f[4 * g + 1] += x[o][g].y;
+              f[4 * g + 2] += x[o][g].z;
+              f[4 * g + 3] += x[o][g].w;
+            }
+          }
+        }
+        swap_store16(P, f, m0 + c0, m_end, n, lane);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // neither CTA leaves while the other may still touch its memory
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, P.tmem_cols);
+  }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -814,6 +1089,116 @@ cudaError_t launch_gemm_splitk(const void* a, int64_t lda, const void* w, int64_
   return cudaLaunchKernelEx(&cfg, smooth_gemm_splitk_kernel, P, a_map, w_map);
 }
 
+// How a problem is cut for the weight-major kernel, and the time the model below expects.
+struct SwapPlan {
+  int m_tiles = 0, tok = 0, halves = 1, splits = 1;
+  float us = 1e30f;
+};
+
+// The model is fitted to measurements at 64 - 1300 tokens on the Linear shapes of three models (hidden
+// 3584, 4096, 8192; within 5 % for most, up to 25 % short where power limits the clock).  Per K chunk a
+// CTA pair takes its MMAs (64 cycles per instruction at least, 1.3 of the nominal rate) or the SM's
+// intake of 50 B a clock, whichever is longer; every wave of tiles also takes its weights' time in HBM;
+// a store of the sums is not overlapped when they fill tensor memory; splitting K costs the exchange of
+// sums, and pays only while every cluster fits the device at once.
+SwapPlan swap_plan(int M, int N, int K, int64_t workspace_bytes, const int* max_clusters) {
+  SwapPlan best;
+  const int n_tiles = (N + 255) / 256, k_chunks = (K + kChunkK - 1) / kChunkK;
+  const int m_lo = (M + 511) / 512;
+  for (int m_tiles = m_lo; m_tiles <= m_lo + 4; ++m_tiles) {
+    const int per = (M + m_tiles - 1) / m_tiles;
+    const int halves = per > 256 ? 2 : 1;
+    const int tok = (per + 16 * halves - 1) / (16 * halves) * 16 * halves;
+    if ((m_tiles - 1) * tok >= M) continue;
+    for (int splits = 1; splits <= kSwapMaxSplits; ++splits) {
+      const int tiles = m_tiles * n_tiles, cps = (k_chunks + splits - 1) / splits, fit = max_clusters[splits - 1];
+      if (fit < 1) continue;
+      if (splits > 1 && (tiles > fit || cps < 8 || (splits - 1) * cps >= k_chunks ||
+                         static_cast<int64_t>(tiles) * splits * tok * 1024 > workspace_bytes))
+        continue;
+      const float mma = 4.f * halves * std::max(64.f, 0.5f * tok / halves) * 1.3f, intake = (kABytes + 64.f * tok) / 50.f;
+      const float chain = cps * std::max(mma, intake) / 1900.f + (2 * tok > 512 ? tok * 0.010f : 0.f);
+      auto wave = [&](int t) {  // the token tiles of a weight tile share its bytes
+        return std::max(chain, 512.f * K * t / (6.3e6f * m_tiles));
+      };
+      const float us = (tiles / fit) * wave(fit) + (tiles % fit ? wave(tiles % fit) : 0.f) + 4.f + tok * 0.006f +
+                       (splits > 1 ? 1.5f + tok * 0.010f : 0.f);
+      if (us < 0.98f * best.us) best = SwapPlan{m_tiles, tok, halves, splits, us};
+    }
+  }
+  return best;
+}
+
+cudaError_t launch_gemm_swap(const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int M, int N, int K,
+                             const SwapPlan& plan, int clusters, void* workspace, cudaStream_t s) {
+  CUtensorMap a_map, w_map;
+  SwapParams P = {};
+  const int nh = plan.tok / plan.halves;
+  if (!encode_matrix_map(&a_map, a, M, K, lda, nh / 2) || !encode_matrix_map(&w_map, w, N, K, ldw, 128))
+    return cudaErrorInvalidValue;
+  P.c = static_cast<uint16_t*>(c);
+  P.ldc = ldc;
+  P.M = M;
+  P.N = N;
+  P.K = K;
+  P.m_tiles = plan.m_tiles;
+  P.n_tiles = (N + 255) / 256;
+  P.tok = plan.tok;
+  P.halves = plan.halves;
+  P.stages = std::min(kSwapMaxStages, kSwapRing / (kABytes + plan.tok * 64));
+  P.splits = plan.splits;
+  const int k_chunks = (K + kChunkK - 1) / kChunkK, tiles = P.m_tiles * P.n_tiles;
+  P.chunks_per_split = (k_chunks + plan.splits - 1) / plan.splits;
+  P.bufs = plan.splits == 1 && 2 * plan.tok <= 512 ? 2 : 1;
+  P.tmem_cols = 32;
+  while (P.tmem_cols < static_cast<uint32_t>(P.bufs * plan.tok)) P.tmem_cols *= 2;
+  P.ws = static_cast<float4*>(workspace);
+  const int grid = 2 * plan.splits * (plan.splits > 1 ? tiles : std::min(tiles, clusters));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
+  cfg.blockDim = dim3(kGemmThreads, 1, 1);
+  cfg.dynamicSmemBytes = kSwapSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(2 * plan.splits);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, smooth_gemm_swap_kernel, P, a_map, w_map);
+}
+
+// Clusters of 2, 4, 6 and 8 CTAs of the weight-major kernel that fit the device at once (asked once per
+// device, together with the kernel's opt-in to large shared memory).
+cudaError_t swap_clusters(int dev, const int** out) {
+  static int counts[64][kSwapMaxSplits];
+  static std::once_flag once[64];
+  static cudaError_t err[64];
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::call_once(once[dev], [&] {
+    err[dev] = cudaFuncSetAttribute(smooth_gemm_swap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwapSmem);
+    for (int sp = 1; sp <= kSwapMaxSplits && err[dev] == cudaSuccess; ++sp) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(static_cast<unsigned>(2 * sp * 64), 1, 1);
+      cfg.blockDim = dim3(kGemmThreads, 1, 1);
+      cfg.dynamicSmemBytes = kSwapSmem;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = static_cast<unsigned>(2 * sp);
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      err[dev] = cudaOccupancyMaxActiveClusters(&counts[dev][sp - 1], smooth_gemm_swap_kernel, &cfg);
+    }
+  });
+  *out = counts[dev];
+  return err[dev];
+}
+
 }  // namespace
 }  // namespace xy
 
@@ -856,6 +1241,22 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
       return XY_ERR_CUDA;
     if (dev >= 0 && dev < 64) sm_count[dev] = sms;
+  }
+  if (tile_n == 0 && !pair && sms >= 2 && M > 128 && M <= 1536) {
+    // The weight-major kernel when its model beats that of 256 x 256 tiles (0.35 us per K chunk and wave).
+    // Measured, here / the choices below: hidden 4096, 333 tokens QKV 21.1 / 23.3 us, OProj 17.7 / 21.7,
+    // GateUp 73 / 86, Down 40 / 63; 777 tokens 33 / 53, 24 / 28, 149 / 170, 75 / 88; from about 1500
+    // tokens on both are bound by the MMAs, and the 256 x 256 tiles overlap their stores.
+    const int* clusters = nullptr;
+    if (xy::swap_clusters(dev, &clusters) != cudaSuccess) return XY_ERR_CUDA;
+    const xy::SwapPlan plan = xy::swap_plan(M, N, K, workspace != nullptr ? workspace_bytes : 0, clusters);
+    const int tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = sms / 2;
+    const float pair_us = static_cast<float>((tiles + pairs - 1) / pairs) * ((K + 63) / 64) * 0.35f + 5.f;
+    if (plan.us < 0.97f * pair_us) {
+      const cudaError_t e = xy::launch_gemm_swap(a, lda, w, ldw, c, ldc, M, N, K, plan, clusters[plan.splits - 1], workspace,
+                                                 static_cast<cudaStream_t>(stream));
+      return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
+    }
   }
   if (tile_n == 0 && !pair && sms >= 2 && M > 128) {
     // 256 x 256 tiles on CTA pairs when the padding of M to 256 rows stays under 15 % and the tiles

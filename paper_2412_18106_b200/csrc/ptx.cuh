@@ -171,6 +171,18 @@ __device__ __forceinline__ void umma2_commit_both(uint32_t bar) {
                ::"r"(bar), "h"(static_cast<uint16_t>(3))
                : "memory");
 }
+// The same for a pair inside a larger cluster: `mask` has the bits of the pair's two CTAs.
+__device__ __forceinline__ void umma2_commit_mask(uint32_t bar, uint16_t mask) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+               ::"r"(bar), "h"(mask)
+               : "memory");
+}
+// Asks for a tile to be brought into L2 (a hint: nothing is read into the SM).
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* m, int c0, int c1) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
+               ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1)
+               : "memory");
+}
 // Tile load into this CTA's shared memory whose completion bytes are counted on a barrier of the
 // pair's leader (a shared::cluster address).  No multicast: every CTA fetches its own tile.
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* m, uint32_t leader_bar, int c0, int c1,

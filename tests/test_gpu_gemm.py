@@ -156,3 +156,30 @@ def test_random_shapes_and_tile_choices(seed):
     lda = K + 8 * int(rng.integers(0, 3))
     ldc = N + 8 * int(rng.integers(0, 3))
     check(M, N, K, tile_n, seed=100 + seed, lda=lda, ldc=ldc)
+
+
+@pytest.mark.parametrize("M,N,K", [(129, 256, 512), (144, 520, 1032), (255, 1000, 4096), (257, 4096, 2048),
+                                   (333, 776, 4096), (512, 2048, 1096), (513, 1800, 520), (700, 392, 328),
+                                   (1000, 2568, 640)])
+def test_weight_major_kernel_matches_oracle_and_repeats_bitwise(M, N, K):
+    """129 .. about 1000 tokens take the weight-major CTA-pair kernel: one or two accumulators per tile,
+    several token tiles, K split over the pairs of a cluster when there is scratch; ragged M, N and K.
+    Nothing outside [0, M) x [0, N) is written."""
+    g = torch.Generator().manual_seed(M + N + K)
+    a = torch.randn((M, K), generator=g).to(torch.bfloat16)
+    w = torch.randn((N, K), generator=g).to(torch.bfloat16)
+    ref = G.linear(a, w)
+    ad, wd = a.cuda(), w.cuda()
+    ws = xg.xy_gemm_workspace("cuda")
+    for scratch in (None, ws):
+        out = []
+        for _ in range(2):
+            full = torch.full((M + 3, N + 8), 7.0, dtype=torch.bfloat16, device="cuda")
+            xg.xy_gemm_run(ad, wd, full[:M, :N], workspace=scratch)
+            torch.cuda.synchronize()
+            assert xg.xy_gemm_device_status() == 0
+            assert torch.all(full[M:] == 7.0) and torch.all(full[:, N:] == 7.0)
+            out.append(full[:M, :N].clone())
+        assert torch.equal(out[0], out[1])
+        d = np.abs(out[0].float().cpu().numpy().astype(np.float64) - ref)
+        assert np.all(d <= 2.0 ** -8 * np.abs(ref) + 2.0 ** -14 * np.sqrt(K)), d.max()
