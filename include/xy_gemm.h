@@ -33,10 +33,12 @@ extern "C" {
  *   pointers 16-byte aligned
  *   tile_n  columns per tile: 32, 64, 128, 256 (128-row tiles on single CTAs), XY_GEMM_PAIR | 128
  *           or XY_GEMM_PAIR | 256 (256-row tiles on CTA pairs), or 0 to let the library choose:
- *           256 x 256 pair tiles when M > 128 pads to a multiple of 256 with at most 15 % waste
- *           and those tiles number at least a quarter of the SMs; else, for M <= 512 with few
- *           tiles, a split of K over a thread-block cluster (2..8 CTAs per 128 x 128 tile, partial
- *           sums added through distributed shared memory), which puts the idle SMs to work; else
+ *           up to 128 tokens a kernel that streams W (128 rows of W per CTA, all tokens as the
+ *           columns, K split over a thread-block cluster); up to about 1500 tokens 256 rows of W on
+ *           a CTA pair with up to 512 tokens as the columns, K split over the pairs of a cluster when
+ *           there is scratch (xy_gemm_run_ws); without scratch, for M <= 512 with few tiles, 128 x 128
+ *           tiles whose K is split over a cluster; else 256 x 256 pair tiles when M pads to a multiple
+ *           of 256 with at most 15 % waste and those tiles number at least a quarter of the SMs; else
  *           128 x 256 tiles when they give half of the SMs a tile, else 128 x 128
  * Returns XY_OK, XY_ERR_INVALID_ARG (null pointer, bad size or alignment), XY_ERR_UNSUPPORTED
  * (tile_n not one of the values above) or XY_ERR_CUDA.  Calls on one stream are ordered; the caller
@@ -44,8 +46,9 @@ extern "C" {
 int xy_gemm_run(const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int32_t M,
                 int32_t N, int32_t K, int32_t tile_n, void* stream);
 
-/* The same with DEVICE scratch memory, which lets the last, partial wave of tiles be split along K
- * over every SM when K is long (K >= 8192 and a last wave of at most 0.6 of the SMs; measured
+/* The same with DEVICE scratch memory, which lets CTA pairs share the K of a tile for 129 to about 1500
+ * tokens (the pairs of a cluster leave fp32 sums in it and add them in a fixed order), and lets the
+ * last, partial wave of larger problems be split along K over every SM when K is long (K >= 8192 and a last wave of at most 0.6 of the SMs; measured
  * rule): each SM multiplies a run of K chunks of one or two of those tiles and leaves fp32 partial
  * sums in the scratch; a second, small kernel on the same stream adds a tile's partial sums in a
  * fixed order (bit-reproducible) and stores the tile.  No thread waits for another CTA.

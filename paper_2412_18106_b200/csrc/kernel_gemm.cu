@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(128) gemm_fixup_kernel(const GemmParams P) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Split-K variant for small token counts (few tiles).  A whole-K tile is one serial
+// Split-K variant for 129 .. 512 tokens without scratch (few tiles).  A whole-K tile is one serial
 // chain of K/64 chunks on one SM, and with fewer tiles than SMs most of the chip idles while the
 // weights stream through a few SMs.  Here a cluster of `splits` CTAs shares one 128 x 128 tile:
 // CTA r computes the partial product over its slice of K, writes the valid rows of its fp32
@@ -683,18 +683,23 @@ struct __align__(8) SwapBarriers {
   uint32_t tmem_base;
 };
 
-// Stores 16 tokens of this thread's output column n: neighbouring lanes swap values so that each
-// writes two columns of every other token.
-__device__ __forceinline__ void swap_store16(const SwapParams& P, const float (&v)[16], int m, int m_end, int n, int lane) {
+// Stores four (sixteen) tokens m .. of this thread's output column n: neighbouring lanes swap values so
+// that each writes two columns of every other token.
+__device__ __forceinline__ void store4_columns(uint16_t* c, int64_t ldc, const float* v, int m, int m_end, int n, int N, int lane) {
+  const bool odd = lane & 1;
 #pragma unroll
-  for (int j = 0; j < 16; j += 2) {
-    const bool odd = lane & 1;
+  for (int j = 0; j < 4; j += 2) {
     const float got = __shfl_xor_sync(0xffffffffu, odd ? v[j] : v[j + 1], 1);
     const int row = m + j + (odd ? 1 : 0);
-    if (row < m_end && n < P.N)
-      *reinterpret_cast<uint32_t*>(P.c + static_cast<int64_t>(row) * P.ldc + (n & ~1)) =
+    if (row < m_end && n < N)
+      *reinterpret_cast<uint32_t*>(c + static_cast<int64_t>(row) * ldc + (n & ~1)) =
           odd ? pack_bf16(got, v[j + 1]) : pack_bf16(v[j], got);
   }
+}
+__device__ __forceinline__ void store16_columns(uint16_t* c, int64_t ldc, const float (&v)[16], int m, int m_end, int n, int N,
+                                                int lane) {
+#pragma unroll
+  for (int j = 0; j < 16; j += 4) store4_columns(c, ldc, v + j, m + j, m_end, n, N, lane);
 }
 
 __global__ void __launch_bounds__(kGemmThreads, 1)
@@ -844,7 +849,7 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
           float f[16];
 #pragma unroll
           for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
-          swap_store16(P, f, m0 + c0, m_end, n, lane);
+          store16_columns(P.c, P.ldc, f, m0 + c0, m_end, n, P.N, lane);
         }
         tc_fence_before();
         __syncwarp();
@@ -913,7 +918,7 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
             }
           }
         }
-        swap_store16(P, f, m0 + c0, m_end, n, lane);
+        store16_columns(P.c, P.ldc, f, m0 + c0, m_end, n, P.N, lane);
       }
     }
   }
@@ -923,6 +928,171 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem, P.tmem_cols);
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// Weight-major variant for up to 128 tokens, bound by the bytes of W: every CTA multiplies a run of K
+// chunks of 128 rows of W (the 128-row side of the MMA) by all tokens (its columns, padded to 16).  Two
+// CTAs share an SM, so loads are in flight while one of them starts or stores, and the CTAs of
+// the next launch are let in early and ask for their first weights to be brought into L2 before they
+// wait for this launch.  K is cut over a cluster of up to eight CTAs so that about two CTAs per SM run;
+// their fp32 sums (512 bytes per token) are added in a fixed order through distributed shared memory.
+struct SmallParams {
+  uint16_t* c;
+  int64_t ldc;
+  int32_t M, N, K;
+  int32_t tok, stages, splits, cps;
+  uint32_t tmem_cols;
+};
+constexpr int kSmallMaxStages = 8;
+constexpr int kSmallMaxSplits = 8;
+
+struct __align__(8) SmallBarriers {
+  uint64_t full[kSmallMaxStages], empty[kSmallMaxStages];
+  uint64_t acc_full;
+  uint32_t tmem_base;
+};
+
+__global__ void __launch_bounds__(kGemmThreads)
+smooth_gemm_small_kernel(const __grid_constant__ SmallParams P, const __grid_constant__ CUtensorMap a_map,
+                         const __grid_constant__ CUtensorMap w_map) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));
+  const uint32_t stage_bytes = kABytes + P.tok * 128;
+  SmallBarriers* bars = reinterpret_cast<SmallBarriers*>(gen_base + P.stages * stage_bytes);
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const volatile int32_t* status = &g_gemm_status;
+  const int rank = P.splits > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const int n0 = static_cast<int>(blockIdx.x) / P.splits * 128;
+  const int k_chunks = (P.K + kChunkK - 1) / kChunkK;
+  const int kc_lo = rank * P.cps, kc_hi = min(k_chunks, kc_lo + P.cps);
+  if (threadIdx.x == 0) {
+    prefetch_tensormap(&a_map);
+    prefetch_tensormap(&w_map);
+    for (int i = kc_lo; i < min(kc_hi, kc_lo + 8); ++i) tma_prefetch_2d(&w_map, i * kChunkK, n0);
+    for (int s = 0; s < P.stages; ++s) {
+      mbar_init(smem_u32(&bars->full[s]), 1);
+      mbar_init(smem_u32(&bars->empty[s]), 1);
+    }
+    mbar_init(smem_u32(&bars->acc_full), 1);
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&bars->tmem_base), P.tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  grid_dependency_wait();
+  grid_launch_dependents();
+  const uint32_t tmem = bars->tmem_base;
+
+  if (warp == 0 && lane == 0) {
+    // ---------------------------------------------------------------- producer
+    uint32_t s = 0, phase = 1;
+    for (int kc = kc_lo; kc < kc_hi; ++kc) {
+      if (!mbar_wait(smem_u32(&bars->empty[s]), phase, status)) {  // (the first round passes)
+        atomicExch(&g_gemm_status, XY_ERR_DEVICE_TIMEOUT);
+        break;
+      }
+      const uint32_t full = smem_u32(&bars->full[s]), dst = base + s * stage_bytes;
+      mbar_arrive_expect_tx(full, stage_bytes);
+      tma_load_2d(dst, &w_map, full, kc * kChunkK, n0);            // rows past N arrive as zeros
+      tma_load_2d(dst + kABytes, &a_map, full, kc * kChunkK, 0);   // rows past M likewise
+      if (++s == static_cast<uint32_t>(P.stages)) {
+        s = 0;
+        phase ^= 1u;
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer
+    constexpr uint64_t kDescHi = static_cast<uint64_t>((1024u >> 4) | (1u << 14) | (2u << 29)) << 32;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((static_cast<uint32_t>(P.tok) >> 3) << 17) | ((128u >> 4) << 24);
+    const bool elected = elect_one();
+    uint32_t s = 0, phase = 0;
+    bool dead = false;
+    for (int kc = kc_lo; kc < kc_hi; ++kc) {
+      if (!mbar_wait(smem_u32(&bars->full[s]), phase, status)) {
+        atomicExch(&g_gemm_status, XY_ERR_DEVICE_TIMEOUT);
+        dead = true;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t w_lo = (((base + s * stage_bytes) >> 4) & 0x3FFFu) | (1u << 16);
+      const uint32_t a_lo = (((base + s * stage_bytes + kABytes) >> 4) & 0x3FFFu) | (1u << 16);
+      if (elected) {
+#pragma unroll
+        for (int k16 = 0; k16 < 4; ++k16)
+          umma_ss64(tmem, kDescHi | (w_lo + k16 * 2), kDescHi | (a_lo + k16 * 2), idesc, (kc > kc_lo || k16) ? 1u : 0u);
+        umma_commit(smem_u32(&bars->empty[s]));
+      }
+      if (++s == static_cast<uint32_t>(P.stages)) {
+        s = 0;
+        phase ^= 1u;
+      }
+    }
+    if (!dead && elected) umma_commit(smem_u32(&bars->acc_full));
+  }
+  bool ok = true;
+  const int q = warp & 3, row = q * 32 + lane, n = n0 + row;
+  if (warp >= 2) {
+    // ---------------------------------------------------------------- epilogue
+    if (!mbar_wait(smem_u32(&bars->acc_full), 0u, status)) {
+      atomicExch(&g_gemm_status, XY_ERR_DEVICE_TIMEOUT);
+      ok = false;
+    }
+    tc_fence_after();
+    const uint32_t t_acc = tmem + (static_cast<uint32_t>(q * 32) << 16);
+    for (int c0 = 0; ok && c0 < P.tok && c0 < P.M; c0 += 16) {
+      uint32_t v[16];
+      tmem_ld_32x32b_x16(t_acc + c0, v);
+      tmem_wait_ld();
+      if (P.splits == 1) {
+        float f[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+        store16_columns(P.c, P.ldc, f, c0, P.M, n, P.N, lane);
+      } else {
+        // the ring is free: every MMA has read its stage.  Four tokens of row n at (group, row) * 16 B.
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+          sts128(base + ((c0 / 4 + g) * 128 + row) * 16, make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]));
+      }
+    }
+  }
+  if (P.splits > 1) {
+    tc_fence_before();
+    __syncwarp();
+    cluster_sync_all();
+    if (warp >= 2 && ok) {
+      for (int g = rank; g * 4 < P.M; g += P.splits) {  // CTA r adds every splits-th group of four tokens
+        float4 x[kSmallMaxSplits];
+#pragma unroll
+        for (int r = 0; r < kSmallMaxSplits; ++r)
+          if (r < P.splits) x[r] = ld_cluster_f4(cluster_map(base + (g * 128 + row) * 16, static_cast<uint32_t>(r)));
+        float f[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int r = 0; r < kSmallMaxSplits; ++r)
+          if (r < P.splits) {
+            f[0] += x[r].x;
+            f[1] += x[r].y;
+            f[2] += x[r].z;
+            f[3] += x[r].w;
+          }
+        store4_columns(P.c, P.ldc, f, g * 4, P.M, n, P.N, lane);
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();  // every CTA's sums stay until all have read them
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, P.tmem_cols);
   }
 }
 
@@ -1089,6 +1259,23 @@ cudaError_t launch_gemm_splitk(const void* a, int64_t lda, const void* w, int64_
   return cudaLaunchKernelEx(&cfg, smooth_gemm_splitk_kernel, P, a_map, w_map);
 }
 
+// Clusters of `size` CTAs of a GEMM kernel with `smem` bytes each that fit the device at once.
+template <class Kernel>
+cudaError_t max_clusters(Kernel kernel, int size, int smem, int* count) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(size * 64), 1, 1);
+  cfg.blockDim = dim3(kGemmThreads, 1, 1);
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(size);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(count, kernel, &cfg);
+}
+
 // How a problem is cut for the weight-major kernel, and the time the model below expects.
 struct SwapPlan {
   int m_tiles = 0, tok = 0, halves = 1, splits = 1;
@@ -1101,7 +1288,7 @@ struct SwapPlan {
 // intake of 50 B a clock, whichever is longer; every wave of tiles also takes its weights' time in HBM;
 // a store of the sums is not overlapped when they fill tensor memory; splitting K costs the exchange of
 // sums, and pays only while every cluster fits the device at once.
-SwapPlan swap_plan(int M, int N, int K, int64_t workspace_bytes, const int* max_clusters) {
+SwapPlan swap_plan(int M, int N, int K, int64_t workspace_bytes, const int* clusters) {
   SwapPlan best;
   const int n_tiles = (N + 255) / 256, k_chunks = (K + kChunkK - 1) / kChunkK;
   const int m_lo = (M + 511) / 512;
@@ -1111,7 +1298,7 @@ SwapPlan swap_plan(int M, int N, int K, int64_t workspace_bytes, const int* max_
     const int tok = (per + 16 * halves - 1) / (16 * halves) * 16 * halves;
     if ((m_tiles - 1) * tok >= M) continue;
     for (int splits = 1; splits <= kSwapMaxSplits; ++splits) {
-      const int tiles = m_tiles * n_tiles, cps = (k_chunks + splits - 1) / splits, fit = max_clusters[splits - 1];
+      const int tiles = m_tiles * n_tiles, cps = (k_chunks + splits - 1) / splits, fit = clusters[splits - 1];
       if (fit < 1) continue;
       if (splits > 1 && (tiles > fit || cps < 8 || (splits - 1) * cps >= k_chunks ||
                          static_cast<int64_t>(tiles) * splits * tok * 1024 > workspace_bytes))
@@ -1180,23 +1367,71 @@ cudaError_t swap_clusters(int dev, const int** out) {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::call_once(once[dev], [&] {
     err[dev] = cudaFuncSetAttribute(smooth_gemm_swap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwapSmem);
-    for (int sp = 1; sp <= kSwapMaxSplits && err[dev] == cudaSuccess; ++sp) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(static_cast<unsigned>(2 * sp * 64), 1, 1);
-      cfg.blockDim = dim3(kGemmThreads, 1, 1);
-      cfg.dynamicSmemBytes = kSwapSmem;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = static_cast<unsigned>(2 * sp);
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      err[dev] = cudaOccupancyMaxActiveClusters(&counts[dev][sp - 1], smooth_gemm_swap_kernel, &cfg);
-    }
+    for (int sp = 1; sp <= kSwapMaxSplits && err[dev] == cudaSuccess; ++sp)
+      err[dev] = max_clusters(smooth_gemm_swap_kernel, 2 * sp, kSwapSmem, &counts[dev][sp - 1]);
   });
   *out = counts[dev];
   return err[dev];
+}
+
+cudaError_t launch_gemm_small(int dev, const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int M, int N,
+                              int K, int num_sms, cudaStream_t s) {
+  constexpr int kMaxSmem = 115712;  // two CTAs per SM
+  // Clusters of 1 .. 8 CTAs that fit the device at once (asked once per device; the answer counts one CTA
+  // per SM, two run).
+  static int fit[64][kSmallMaxSplits];
+  static std::once_flag once[64];
+  static cudaError_t err[64];
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::call_once(once[dev], [&] {
+    err[dev] = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (err[dev] == cudaSuccess)
+      err[dev] = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    for (int sp = 2; sp <= kSmallMaxSplits && err[dev] == cudaSuccess; ++sp) {
+      err[dev] = max_clusters(smooth_gemm_small_kernel, sp, kMaxSmem, &fit[dev][sp - 1]);
+      fit[dev][sp - 1] *= 2;
+    }
+  });
+  if (err[dev] != cudaSuccess) return err[dev];
+  SmallParams P = {};
+  P.c = static_cast<uint16_t*>(c);
+  P.ldc = ldc;
+  P.M = M;
+  P.N = N;
+  P.K = K;
+  P.tok = (M + 15) / 16 * 16;
+  CUtensorMap a_map, w_map;
+  if (!encode_matrix_map(&a_map, a, M, K, lda, P.tok) || !encode_matrix_map(&w_map, w, N, K, ldw, 128)) return cudaErrorInvalidValue;
+  const int stage = kABytes + P.tok * 128;
+  P.stages = std::min(kSmallMaxStages, (kMaxSmem - 1024 - static_cast<int>(sizeof(SmallBarriers))) / stage);
+  const int tiles = (N + 127) / 128, k_chunks = (K + kChunkK - 1) / kChunkK;
+  // Two CTAs per SM with the deeper ring (three with a shorter one: GateUp at 64 tokens 45.4 against 41.5
+  // us, Down 26.2 / 23.5), and the most CTAs per tile whose clusters fit at once but for one or two: a
+  // second wave costs more than the shorter chains save (QKV, 48 tiles, at 64 tokens: clusters of five, of
+  // which 52 fit, 12.8 us, of six, 44, 18.9; Down, 32 tiles: of eight, 30, 23.5, of six 25.0).  At least six
+  // chunks per CTA.
+  P.splits = 1;
+  for (int sp = 2; sp <= kSmallMaxSplits && sp * 6 <= k_chunks; ++sp)
+    if (tiles * 15 <= fit[dev][sp - 1] * 16) P.splits = sp;
+  P.cps = (k_chunks + P.splits - 1) / P.splits;
+  P.splits = (k_chunks + P.cps - 1) / P.cps;  // no CTA without a chunk
+  P.tmem_cols = 32;
+  while (P.tmem_cols < static_cast<uint32_t>(P.tok)) P.tmem_cols *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(tiles * P.splits), 1, 1);
+  cfg.blockDim = dim3(kGemmThreads, 1, 1);
+  cfg.dynamicSmemBytes = 1024 + P.stages * stage + sizeof(SmallBarriers);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(P.splits);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = P.splits > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, smooth_gemm_small_kernel, P, a_map, w_map);
 }
 
 }  // namespace
@@ -1242,6 +1477,29 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
       return XY_ERR_CUDA;
     if (dev >= 0 && dev < 64) sm_count[dev] = sms;
   }
+  if (tile_n == 0 && !pair && M <= 128) {
+    // Up to 128 tokens are bound by the bytes of W; the kernel for that.  Measured, here / before (whole
+    // tiles or a split of K with padded token rows): hidden 4096, 16 tokens QKV 10.7 / 14.2 us, OProj 8.4 /
+    // 10.6, GateUp 39.7 / 42.9, Down 20.3 / 23.9; hidden 3584, QKV 8.5 / 19.8, OProj 7.3 / 19.2, Down 24 / 53.
+    const cudaError_t e = xy::launch_gemm_small(dev, a, lda, w, ldw, c, ldc, M, N, K, sms, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
+  }
+  if (tile_n == 0 && !pair && workspace == nullptr && M > 128 && M <= 512) {
+    // No scratch, few tiles and one long serial chain over K per tile: split K over a cluster when that
+    // puts several times as many SMs to work (Down / OProj projections of a short chunk; Down at 200
+    // tokens 38.8 us, the weight-major kernel with whole chains about 70, with scratch 31).  Measured: four or more slices pay off from 16 chunks per slice on; two or three
+    // only when the chain is long (32 chunks per slice), else the reduction costs what the
+    // shorter chain saves.
+    const int tiles = ((M + 127) / 128) * ((N + 127) / 128), k_chunks = (K + 63) / 64;
+    int splits = sms / tiles;
+    if (splits > 8) splits = 8;
+    while (splits >= 2 && k_chunks / splits < (splits >= 4 ? 16 : 32)) --splits;
+    if (splits >= 2) {
+      const cudaError_t e =
+          xy::launch_gemm_splitk(a, lda, w, ldw, c, ldc, M, N, K, splits, static_cast<cudaStream_t>(stream));
+      return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
+    }
+  }
   if (tile_n == 0 && !pair && sms >= 2 && M > 128 && M <= 1536) {
     // The weight-major kernel when its model beats that of 256 x 256 tiles (0.35 us per K chunk and wave).
     // Measured, here / the choices below: hidden 4096, 333 tokens QKV 21.1 / 23.3 us, OProj 17.7 / 21.7,
@@ -1261,9 +1519,7 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
   if (tile_n == 0 && !pair && sms >= 2 && M > 128) {
     // 256 x 256 tiles on CTA pairs when the padding of M to 256 rows stays under 15 % and the tiles
     // give at least half of the pairs work: measured best or level with the best from 1024 tokens
-    // on (at 4096 tokens QKV 155 -> 143 us, OProj 105 -> 96, GateUp 667 -> 609, Down 369 -> 339), and
-    // at 256 tokens for GateUp only (112 tiles: 67 -> 61 us; the shapes with 16 - 24 tiles stay with
-    // 128-column tiles or the cluster split of K).
+    // on (at 4096 tokens QKV 155 -> 143 us, OProj 105 -> 96, GateUp 667 -> 609, Down 369 -> 339).
     const int mp = (M + 255) / 256, np = (N + 255) / 256;
     if ((mp * 256 - M) * 100 <= 15 * mp * 256 && mp * np * 4 >= sms) {
       pair = true;
@@ -1276,22 +1532,6 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
         tile_n == 256 ? xy::launch_gemm_pair<256>(a, lda, w, ldw, c, ldc, M, N, K, sms, static_cast<cudaStream_t>(stream))
                       : xy::launch_gemm_pair<128>(a, lda, w, ldw, c, ldc, M, N, K, sms, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
-  }
-  if (tile_n == 0 && M <= 512) {
-    // Few tiles and one long serial chain over K per tile: split K over a cluster when that puts
-    // several times as many SMs to work (Down / OProj projections of a decode batch or a short
-    // chunk).  Measured: four or more slices pay off from 16 chunks per slice on; two or three
-    // only when the chain is long (32 chunks per slice), else the reduction costs what the
-    // shorter chain saves.
-    const int tiles = ((M + 127) / 128) * ((N + 127) / 128), k_chunks = (K + 63) / 64;
-    int splits = sms / tiles;
-    if (splits > 8) splits = 8;
-    while (splits >= 2 && k_chunks / splits < (splits >= 4 ? 16 : 32)) --splits;
-    if (splits >= 2) {
-      const cudaError_t e =
-          xy::launch_gemm_splitk(a, lda, w, ldw, c, ldc, M, N, K, splits, static_cast<cudaStream_t>(stream));
-      return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
-    }
   }
   if (tile_n == 0) {
     // 128 x 256 tiles read the least of A and W per flop; they are used when they give at least

@@ -183,3 +183,26 @@ def test_weight_major_kernel_matches_oracle_and_repeats_bitwise(M, N, K):
         assert torch.equal(out[0], out[1])
         d = np.abs(out[0].float().cpu().numpy().astype(np.float64) - ref)
         assert np.all(d <= 2.0 ** -8 * np.abs(ref) + 2.0 ** -14 * np.sqrt(K)), d.max()
+
+
+@pytest.mark.parametrize("M", [1, 2, 15, 16, 17, 33, 64, 65, 127, 128])
+@pytest.mark.parametrize("N,K", [(128, 72), (520, 1032), (4096, 512), (1032, 4096), (6144, 2056), (40000, 136)])
+def test_weight_streaming_kernel_matches_oracle_and_repeats_bitwise(M, N, K):
+    """Up to 128 tokens: every number of CTAs per cluster from one to eight, ragged rows of W, tokens and
+    K, more tiles than fit at once; nothing outside [0, M) x [0, N) is written."""
+    g = torch.Generator().manual_seed(M * 3 + N + K)
+    a = torch.randn((M, K), generator=g).to(torch.bfloat16)
+    w = torch.randn((N, K), generator=g).to(torch.bfloat16)
+    ad, wd = a.cuda(), w.cuda()
+    out = []
+    for _ in range(2):
+        full = torch.full((M + 3, N + 8), 7.0, dtype=torch.bfloat16, device="cuda")
+        xg.xy_gemm_run(ad, wd, full[:M, :N])
+        torch.cuda.synchronize()
+        assert xg.xy_gemm_device_status() == 0
+        assert torch.all(full[M:] == 7.0) and torch.all(full[:, N:] == 7.0)
+        out.append(full[:M, :N].clone())
+    assert torch.equal(out[0], out[1])
+    ref = G.linear(a, w)
+    d = np.abs(out[0].float().cpu().numpy().astype(np.float64) - ref)
+    assert np.all(d <= 2.0 ** -8 * np.abs(ref) + 2.0 ** -14 * np.sqrt(K)), d.max()
