@@ -388,6 +388,8 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.queue_head = ctx->d_status + kStatusQueueHead;  // second cache line of the status block
   a.num_tasks = static_cast<int32_t>(p.tasks.size());
   a.num_workers = ctx->num_workers;
+  a.exits = ctx->d_status + kStatusExits;
+  a.side_by_side = 0;
   a.num_units = static_cast<int32_t>(p.merges.size());
   // Balanced plans are dealt dynamically by the meta-kernel; paper-mode plans keep the static
   // Task-Table (each worker walks its own list), as does the reference kernel.
@@ -418,19 +420,29 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   if (cfg.kernel == XY_KERNEL_REFERENCE) {
     XY_CUDA(ctx, launch_reference(a, ctx->num_workers, s));
   } else if (p.queue_dense >= 0 && !fp8) {
-    // pair plan: the dense tasks on CTA pairs, then the streaming tasks on single CTAs
+    // two launches: the dense tasks (pair plan: on CTA pairs), then the streaming tasks
     RunArgs d = a;
     d.num_tasks = p.queue_dense;
+    const bool beside = !ctx->pair && p.queue_dense > 0 && p.queue_dense < a.num_tasks;
+    d.side_by_side = beside ? 1 : 0;
     if (d.num_tasks > 0) {
-      XY_CUDA(ctx, launch_pair_dense(d, ctx->num_workers, num_pages, &ctx->launch_cache, s));
+      if (ctx->pair)
+        XY_CUDA(ctx, launch_pair_dense(d, ctx->num_workers, num_pages, &ctx->launch_cache, s));
+      else
+        XY_CUDA(ctx, launch_meta(d, num_pages, true, &ctx->launch_cache, s));
       ctx->last_launches += 1;
     }
     RunArgs st = a;
     st.queue = a.queue + p.queue_dense;
     st.num_tasks = a.num_tasks - p.queue_dense;
-    st.queue_head = a.queue_head + 1;  // its own head word, cleared by the same memset
+    st.side_by_side = beside ? 2 : 0;
+    st.exits = a.exits + 1;
+    st.queue_head = a.queue_head + 1;  // its own head word
     if (st.num_tasks > 0) {
-      XY_CUDA(ctx, launch_meta(st, num_pages, false, &ctx->launch_cache, s));
+      if (ctx->pair)
+        XY_CUDA(ctx, launch_meta(st, num_pages, false, &ctx->launch_cache, s));
+      else
+        XY_CUDA(ctx, launch_stream(st, num_pages, &ctx->launch_cache, s));
       ctx->last_launches += 1;
     }
     ctx->last_launches -= 1;  // counted once more below

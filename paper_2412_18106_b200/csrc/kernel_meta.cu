@@ -454,6 +454,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   __syncthreads();
   tc_fence_after();
   grid_dependency_wait();
+  if (a.side_by_side) grid_launch_dependents();  // every launch before this one is complete: the second may run
   if (threadIdx.x == 0) {
     unsigned long long now;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));

@@ -82,7 +82,8 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     prefetch_tensormap(&v_map);
   }
   __syncthreads();
-  grid_dependency_wait();
+  // (beside the dense launch: its CTAs have let this one in only after their own wait)
+  if (!a.side_by_side) grid_dependency_wait();
   unsigned long long t_start = 0;
   if (threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
   const int G = a.num_q_heads / a.num_kv_heads;
@@ -285,6 +286,8 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       }
     }
   }
+  // Beside the dense launch: that one is waited for here, so that whoever follows this launch follows both.
+  if (a.side_by_side) grid_dependency_wait();
   // The next launch's CTAs come in as these leave.  (Letting them in from the start filled the SMs
   // unevenly: a CTA took whichever slot was free first, 55.3 -> 60.4 us for 64 requests on an fp8 cache.)
   grid_launch_dependents();

@@ -30,6 +30,9 @@ constexpr float kDenseVisitUs = 2.30f;
 constexpr float kStreamVisitUs = 1.00f;
 constexpr float kPairVisitUs = 1.35f;
 constexpr float kTaskFixedUs = 3.0f;
+constexpr double kStreamTaskUs = 3.8;      // around a streaming task of the meta-kernel: descriptors, Q, merge of the warps
+constexpr double kStreamTileHbmUs = 0.0104;  // 64 KiB at 6.3 TB/s
+constexpr double kSecondLaunchUs = 3.0;
 constexpr int kMinChunkTiles = 4;
 // A task may cost at most this fraction of the mean per-worker load before its KV range is
 // split (measured on the five benchmark batches: finer splits lose more to per-task overhead
@@ -303,6 +306,28 @@ int build_plan(const xy_attn_config& cfg, int num_workers, int64_t partial_row_c
   float cap_kind[2] = {static_cast<float>(total_kind[0] / std::max(1, num_workers) * kTaskCapFraction),
                        static_cast<float>(total_kind[1] / std::max(1, num_workers) * kTaskCapFraction)};
   const float dense_factor = kDenseCapFactor;
+  // Two launches side by side (dense tasks on the meta-kernel, streaming tasks on the streaming kernel) or
+  // one mixed queue?  In the mix a streaming tile takes its SM kStreamVisitUs and a task kStreamTaskUs
+  // around it; the streaming kernel runs at the pace of HBM but has its SMs only as the dense tasks
+  // leave them, so the dense part must be small.  Measured, one queue / two launches: decode on shared
+  // prefixes, 128 requests on 8192 + 0 .. 1024 tokens 99.4 / 93.2 us, 210 on 3840 + 0 .. 362 114 / 86; with
+  // the dense tasks 0.59 of the work 85.5 / 88.4; a 2048-token chunk beside 48 decode requests 373 / 491.
+  bool two_launches = false;
+  if (!paper && !pair && cfg.kernel == XY_KERNEL_AUTO && cfg.kv_dtype == XY_KV_BF16) {
+    double dense = 0.0, tiles = 0.0, tasks = 0.0;
+    for (const Unit& u : units) {
+      if (u.kind == 1) {
+        tiles += u.nkt - u.kt0;
+        tasks += 1.0;
+      } else {
+        dense += kTaskFixedUs + u.visit_cost * (u.nkt - u.kt0);
+      }
+    }
+    const double mixed = (dense + kStreamVisitUs * tiles + kStreamTaskUs * tasks) / num_workers;
+    const double apart = dense / num_workers + kSecondLaunchUs +
+                         std::max(tiles * kStreamTileHbmUs, (kStreamVisitUs * tiles + kStreamTaskUs * tasks) * 0.5 / num_workers);
+    two_launches = dense > 0.0 && tasks > 0.0 && apart < 0.95 * mixed && dense < 0.45 * mixed * num_workers;
+  }
   std::vector<int> chunk_tiles(units.size(), 0);
   for (int attempt = 0; attempt < 64; ++attempt) {
     int64_t prow = 0;
@@ -490,10 +515,10 @@ int build_plan(const xy_attn_config& cfg, int num_workers, int64_t partial_row_c
       d.swap(regrouped);
     }
     size_t next[2] = {0, 0};
-    if (pair) out->queue_dense = static_cast<int32_t>(by_kind[0].size());
+    if (pair || two_launches) out->queue_dense = static_cast<int32_t>(by_kind[0].size());
     for (size_t pos = 0; pos < order.size(); ++pos) {
       int kd;
-      if (pair) kd = next[0] < by_kind[0].size() ? 0 : 1;  // two launches: all dense tasks, then all streaming tasks
+      if (pair || two_launches) kd = next[0] < by_kind[0].size() ? 0 : 1;  // all dense tasks, then all streaming tasks
       else if (next[0] >= by_kind[0].size()) kd = 1;
       else if (next[1] >= by_kind[1].size()) kd = 0;
       else {

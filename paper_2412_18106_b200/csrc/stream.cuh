@@ -59,7 +59,7 @@ __device__ __forceinline__ void report_timeout(const RunArgs& a) {
 __device__ __forceinline__ void end_of_run(const RunArgs& a, int* s_flag) {
   if (threadIdx.x == 0) {
     __threadfence();
-    *s_flag = atomicAdd(a.status + kStatusExits, 1) == static_cast<int>(gridDim.x) - 1 ? 1 : 0;
+    *s_flag = atomicAdd(a.exits, 1) == static_cast<int>(gridDim.x) - 1 ? 1 : 0;
   }
   __syncthreads();
   if (*s_flag == 0) return;
@@ -67,10 +67,11 @@ __device__ __forceinline__ void end_of_run(const RunArgs& a, int* s_flag) {
   const bool failed = *const_cast<volatile int32_t*>(a.status) != 0;
   __syncthreads();
   if (threadIdx.x == 0) {
-    a.status[0] = 0;
-    a.status[kStatusExits] = 0;
+    *a.exits = 0;
     *a.queue_head = 0;
+    if (a.side_by_side != 1) a.status[0] = 0;
   }
+  if (a.side_by_side == 1) return;  // the second launch is still running; it ends behind this one
   if (failed)  // otherwise every counter was put back by the task that completed its unit
     for (int i = threadIdx.x; i < a.num_units; i += blockDim.x) a.unit_count[i] = 0;
   for (int w = gridDim.x * 4 + threadIdx.x; w < a.num_workers * 4; w += blockDim.x) a.worker_times[w] = 0ull;

@@ -15,6 +15,7 @@ constexpr int kStreamRowsMax = 16;
 // The status block, indexed from the word the kernels receive as `status`:
 //   [0]   the current run's status, polled by every bounded wait
 //   [16]  the queue head of dynamic dealing (its own cache line)
+//   [17], [19]  the same two words for the second of two launches
 //   [18]  CTAs that have finished
 //   [32 ..] one completion counter per merge unit
 // all of which are zero when a run starts: the last CTA of a run puts them back (end_of_run; the
@@ -50,8 +51,8 @@ struct PlanResult {
   std::vector<float> task_cost;            // parallel to tasks
   std::vector<int32_t> worker_off;         // num_workers + 1
   std::vector<int32_t> queue;              // task indices by descending cost (dynamic dealing)
-  int32_t queue_dense = -1;                // pair plans: the first queue_dense entries are the dense tasks (for the
-                                           // CTA-pair launch), the rest the streaming tasks; -1: one mixed queue
+  int32_t queue_dense = -1;                // plans for two launches: the first queue_dense entries are the dense tasks,
+                                           // the rest the streaming tasks; -1: one mixed queue
   std::vector<xy_attn_merge_unit> merges;  // units merged by the merge kernel first, then those merged in the attention kernel
   std::vector<int32_t> task_unit;          // parallel to tasks: index in `merges` of the unit the last finisher merges
                                            // inside the attention kernel, or -1
@@ -132,6 +133,8 @@ struct RunArgs {
   const int32_t* queue;
   int32_t* queue_head;
   int32_t num_tasks, dynamic, num_workers, num_units;
+  int32_t* exits;          // word of the status block that counts the CTAs that have finished
+  int32_t side_by_side;    // 1, 2: first (dense) and second (streaming) of two launches that run at the same time
   // split units whose last finishing task merges them inside the kernel (streaming units)
   const int32_t* task_unit;              // per task: unit index or -1 (null: no such unit)
   const xy_attn_merge_unit* units;

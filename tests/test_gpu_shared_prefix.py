@@ -108,3 +108,23 @@ def test_groups_found_from_the_block_table():
     O_ref, LSE_ref = oracle.attention(b, t, H.SCALE)
     H.check_against_oracle(O, LSE, O_ref, LSE_ref, "auto groups")
     ctx.close()
+
+
+@pytest.mark.parametrize("page,members,workers", [(128, 42, 0), (16, 42, 0), (128, 30, 7)])
+def test_dense_and_streaming_launches_side_by_side_match_oracle(page, members, workers):
+    """Many members with keys of their own on short common prefixes: the planner gives the group tiles
+    and the members' own keys a launch each, which run at the same time; then the merge."""
+    b, groups = W.shared_prefix_decode(seed=page + members, num_groups=5, members=members, prefix=512, suffix_hi=400,
+                                       hq=16, hkv=4, page_size=page)
+    t = W.make_tensors(b)
+    ctx = H.make_ctx(b, num_workers=workers, max_requests=512)
+    ctx.plan_batch(b, groups=groups)
+    O_ref, LSE_ref = oracle.attention(b, t, H.SCALE)
+    first = None
+    for _ in range(3):
+        O, LSE = H.run_gpu(b, t, ctx=ctx)
+        assert ctx.last_launches() == 3
+        H.check_against_oracle(O, LSE, O_ref, LSE_ref, "two launches")
+        assert first is None or (np.array_equal(O, first[0]) and np.array_equal(LSE, first[1]))
+        first = (O, LSE)
+    ctx.close()
