@@ -1510,7 +1510,11 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
     const xy::SwapPlan plan = xy::swap_plan(M, N, K, workspace != nullptr ? workspace_bytes : 0, clusters);
     const int tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = sms / 2;
     const float pair_us = static_cast<float>((tiles + pairs - 1) / pairs) * ((K + 63) / 64) * 0.35f + 5.f;
-    if (plan.us < 0.97f * pair_us) {
+    // Up to 217 tokens a tile of 256 rows would be more than 15 % padding and is not taken below, so that the
+    // weight-major kernel stands against 128 x 256 tiles, which lose everywhere: GateUp at 200 tokens
+    // 51 / 63 us, N 28672 x K 4096 at 129 tokens 49 / 62, N 57344 x K 8192 at 129 tokens 181 / 234.  (With more
+    // tokens they do not: GateUp at 600 tokens 127 / 105.)
+    if (M <= 217 || plan.us < 0.97f * pair_us) {
       const cudaError_t e = xy::launch_gemm_swap(a, lda, w, ldw, c, ldc, M, N, K, plan, clusters[plan.splits - 1], workspace,
                                                  static_cast<cudaStream_t>(stream));
       return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;

@@ -160,7 +160,7 @@ def test_random_shapes_and_tile_choices(seed):
 
 @pytest.mark.parametrize("M,N,K", [(129, 256, 512), (144, 520, 1032), (255, 1000, 4096), (257, 4096, 2048),
                                    (333, 776, 4096), (512, 2048, 1096), (513, 1800, 520), (700, 392, 328),
-                                   (1000, 2568, 640)])
+                                   (1000, 2568, 640), (129, 28672, 264), (217, 20000, 520)])
 def test_weight_major_kernel_matches_oracle_and_repeats_bitwise(M, N, K):
     """129 .. about 1000 tokens take the weight-major CTA-pair kernel: one or two accumulators per tile,
     several token tiles, K split over the pairs of a cluster when there is scratch; ragged M, N and K.
