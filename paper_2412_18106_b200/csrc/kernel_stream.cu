@@ -82,6 +82,18 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     prefetch_tensormap(&v_map);
   }
   __syncthreads();
+  // The producer reads the description of the first task while the launch before is still running: the
+  // plan's tables come over by a copy, which this launch is ordered behind in full.  (13 requests of 300 -
+  // 2500 keys 21.7 -> 20.6 us, 64 requests up to 8192 keys 96.4 -> 94.8, fp8 cache 55.2 -> 54.7; with the
+  // same in the append kernel, a step of eight layers with appends 190 -> 183.)
+  xy_attn_task t{};
+  ReqInfo rq{};
+  if (warp == kWarpsS) {
+    const int ti = __ldg(a.queue + blockIdx.x);
+    t = a.tasks[ti];
+    rq = a.reqs[t.req];
+    rq.pad1 = (a.task_unit != nullptr && t.part >= 0) ? __ldg(a.task_unit + ti) : -1;
+  }
   // (beside the dense launch: its CTAs have let this one in only after their own wait)
   if (!a.side_by_side) grid_dependency_wait();
   unsigned long long t_start = 0;
@@ -109,8 +121,6 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     };
     // A cursor over the CTA's (task, key tile) sequence: a tile's block-table entry is requested
     // three tiles before its copy is issued, which reaches into the next tasks.
-    xy_attn_task t{};
-    ReqInfo rq{};
     int kt = 0, n_grab = 0;
     const int32_t* bt = a.block_table;
     int npages = 1;
@@ -120,20 +130,20 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       if (!open || kt >= t.kt_hi) {
         open = false;
         if (out) return x;
-        int k = blockIdx.x;
-        if (n_grab > 0) {
+        if (n_grab > 0) {  // (the grid has no more CTAs than there are tasks)
+          int k = 0;
           if (lane == 0) k = static_cast<int>(gridDim.x) + atomicAdd(a.queue_head, 1);
           k = __shfl_sync(0xffffffffu, k, 0);
+          if (k >= a.num_tasks) {
+            out = true;
+            return x;
+          }
+          const int ti = __ldg(a.queue + k);
+          t = a.tasks[ti];
+          rq = a.reqs[t.req];
+          rq.pad1 = (a.task_unit != nullptr && t.part >= 0) ? __ldg(a.task_unit + ti) : -1;
         }
         ++n_grab;
-        if (k >= a.num_tasks) {
-          out = true;
-          return x;
-        }
-        const int ti = __ldg(a.queue + k);
-        t = a.tasks[ti];
-        rq = a.reqs[t.req];
-        rq.pad1 = (a.task_unit != nullptr && t.part >= 0) ? __ldg(a.task_unit + ti) : -1;
         if (lane == 0) desc[(n_grab - 1) % kTaskSlots] = TaskDesc{t, rq};
         kt = t.kt_lo;
         npages = (rq.kv_len + rq.q_len + a.page_size - 1) >> a.page_shift;

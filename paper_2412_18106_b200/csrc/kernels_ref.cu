@@ -366,8 +366,6 @@ __global__ void __launch_bounds__(128) append_kv_kernel(const uint16_t* qkv, int
                                                         const int32_t* block_table, int bt_stride,
                                                         const ReqInfo* reqs, int num_reqs, int Hq, int Hkv,
                                                         int page_size, int page_shift) {
-  ptx::grid_dependency_wait();
-  ptx::grid_launch_dependents();
   const int t = blockIdx.x;
   int lo = 0, hi = num_reqs - 1;  // last request whose start position is <= t
   while (lo < hi) {
@@ -375,6 +373,10 @@ __global__ void __launch_bounds__(128) append_kv_kernel(const uint16_t* qkv, int
     if (reqs[mid].q_start <= t) lo = mid; else hi = mid - 1;
   }
   const ReqInfo rq = reqs[lo];
+  // The plan's tables come over by a copy, which this launch is ordered behind in full: they are read
+  // while the kernel before is still running.
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
   const int j = rq.kv_len + (t - rq.q_start);
   const int64_t page = block_table[static_cast<int64_t>(lo) * bt_stride + (j >> page_shift)];
   const int64_t slot_off = page * page_stride + static_cast<int64_t>(j & (page_size - 1)) * token_stride;

@@ -7,7 +7,8 @@
 
 namespace xy {
 
-// Launches a kernel that calls grid_dependency_wait before it touches global memory.
+// Launches a kernel that calls grid_dependency_wait before it touches anything that a kernel before it
+// wrote, or writes global memory itself.
 template <class... P, class... A>
 inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg = {};
