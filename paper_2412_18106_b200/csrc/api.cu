@@ -401,9 +401,9 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.k_scale = k_scale;
   a.v_scale = v_scale;
   a.kv_fp8 = fp8 ? 1 : 0;
-  // Every run starts with a clean status word, queue head and unit counters: the last CTA of the run
-  // before has left them so, after a device-side timeout too.  (The CTA-pair kernel leaves that to a
-  // memset.)  The sticky record in front of them is kept.
+  // Every run starts with a clean status word, queue head and unit counters: the run before has left
+  // them so, after a device-side timeout too.  (The CTA-pair kernel leaves that to a memset.)  The
+  // sticky record in front of them is kept.
   if (ctx->pair)
     XY_CUDA(ctx, cudaMemsetAsync(a.status, 0, (kStatusUnitCounts + (in_kernel_merges ? p.merges.size() : 0)) * sizeof(int32_t), s));
 

@@ -613,7 +613,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         if (!dynamic) return f_ti < t_end ? f_ti++ : -1;
         if (f_done) return -1;
         int ti = -1;
-        const int k = atomicAdd(a.queue_head, 1);
+        const int k = static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
         if (k < a.num_tasks) ti = __ldg(a.queue + k);
         const uint32_t slot = n_pub % kTaskRing;
         if (n_pub >= kTaskRing &&
@@ -1232,13 +1232,13 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           w.init();
           w.load_q(q_addr, lane);
           stream_task<kConsumerWarps, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq,
-                                                        unit, warp, 1, &s_last);
+                                                        unit, warp, 1, &s_last, nullptr);
         } else {
           StreamWarp<kConsumerWarps, 2, kFp8> w;
           w.init();
           w.load_q(q_addr, lane);
           stream_task<kConsumerWarps, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq,
-                                                        unit, warp, 1, &s_last);
+                                                        unit, warp, 1, &s_last, nullptr);
         }
         pipe.stage = pos.stage;
         pipe.phase = pos.phase;
@@ -1264,7 +1264,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     tmem_dealloc(tmem, kTmemCols);
   }
   __shared__ int s_flag;
-  end_of_run(a, &s_flag);
+  end_of_run(a, &s_flag, nullptr);
 }
 
 #include "kernel_pair.inc"
@@ -1354,6 +1354,7 @@ cudaError_t launch_meta(const RunArgs& a, int64_t num_pages, bool umma, MetaLaun
   if (e != cudaSuccess) return e;
   MetaParams P{a};
   const int grid = a.dynamic && a.num_tasks < a.num_workers ? a.num_tasks : a.num_workers;
+  P.a.queue_wrap = static_cast<uint32_t>(a.num_tasks + grid - 1);  // every CTA grabs in vain once
   return launch_after(kernel, dim3(grid), kThreads, kSmemTotal, s, P, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
                       *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
 }

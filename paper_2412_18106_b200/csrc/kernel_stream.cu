@@ -62,7 +62,8 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
   TaskDesc* desc = reinterpret_cast<TaskDesc*>(q_gen + Cfg::kQ + Cfg::kMl + Cfg::kScales);
   uint64_t* bars = reinterpret_cast<uint64_t*>(desc + kTaskSlots);
   int* s_last = reinterpret_cast<int*>(bars + 2 * kStages + 2);
-  int* s_dead = s_last + 1;
+  int* s_failed = s_last + 1;  // a thread has reported a timeout
+  int* s_dead = s_last + 2;    // the consumers leave together
   const uint32_t ring = smem_u32(smem), q_smem = smem_u32(q_gen);
   const uint32_t full = smem_u32(bars), empty = full + 8 * kStages, task_full = empty + 8 * kStages, task_free = task_full + 8;
 
@@ -74,6 +75,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     }
     mbar_init(task_full, 33);  // lane 0 once the description is written, every lane once its Q chunks have landed
     mbar_init(task_free, kWarpsS);
+    *s_failed = 0;
     *s_dead = 0;
     fence_mbar_init();
   }
@@ -104,7 +106,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     // ================================== producer ==========================================
     bool dead = false;
     if ((ring & 1023u) != 0) {  // the TMA swizzle needs it; dynamic shared memory starts there
-      report_timeout(a);
+      report_timeout(a, s_failed);
       dead = true;
     }
     const int ppt = kKeyTile >> a.page_shift;  // pages per tile
@@ -131,8 +133,10 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
         open = false;
         if (out) return x;
         if (n_grab > 0) {  // (the grid has no more CTAs than there are tasks)
-          int k = 0;
-          if (lane == 0) k = static_cast<int>(gridDim.x) + atomicAdd(a.queue_head, 1);
+          const int grid = static_cast<int>(gridDim.x);
+          int k = a.num_tasks;
+          if (lane == 0 && a.num_tasks > grid)
+            k = grid + static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
           k = __shfl_sync(0xffffffffu, k, 0);
           if (k >= a.num_tasks) {
             out = true;
@@ -172,7 +176,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     // task's are in its consumers' registers by then (task_free).
     auto publish = [&](bool last) {
       if (n_tasks > 0 && !mbar_wait_block(task_free, (n_tasks - 1) & 1u, a.status)) {
-        report_timeout(a);
+        report_timeout(a, s_failed);
         dead = true;
         return;
       }
@@ -207,7 +211,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       if (used & bit) {
         // wait for the readers of this stage's previous fill
         if (!mbar_wait_block(empty + 8 * pos.stage, (fill_par >> pos.stage) & 1u, a.status)) {
-          report_timeout(a);
+          report_timeout(a, s_failed);
           dead = true;
           return;
         }
@@ -262,7 +266,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     uint32_t tile_seq = 0;
     for (uint32_t n = 0;; ++n) {
       if (!dead && !mbar_wait_block(task_full, n & 1u, a.status)) {
-        report_timeout(a);
+        report_timeout(a, s_failed);
         dead = true;
       }
       // All warps leave together (a warp whose wait ran out must not keep away from the barriers of
@@ -287,12 +291,12 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
         StreamWarp<kWarpsS, 1, kFp8> w;
         take_q(w);
         stream_task<kWarpsS, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, warp, 1,
-                                               s_last);
+                                               s_last, s_failed);
       } else {
         StreamWarp<kWarpsS, 2, kFp8> w;
         take_q(w);
         stream_task<kWarpsS, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, warp, 1,
-                                               s_last);
+                                               s_last, s_failed);
       }
     }
   }
@@ -311,7 +315,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     w[2] = 0ull;
     w[3] = now - t_start;
   }
-  end_of_run(a, s_last);
+  end_of_run(a, s_last, s_failed);
 }
 
 }  // namespace
@@ -330,7 +334,9 @@ cudaError_t launch_stream(const RunArgs& a, int64_t num_pages, MetaLaunchCache* 
   const cudaError_t e = pool_maps(a, num_pages, cache);
   if (e != cudaSuccess) return e;
   const int grid = a.num_tasks < 2 * a.num_workers ? a.num_tasks : 2 * a.num_workers;
-  return launch_after(kernel, dim3(grid), kThreadsS, smem, s, a, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
+  RunArgs args = a;
+  args.queue_wrap = static_cast<uint32_t>(a.num_tasks - 1);  // one grab less per CTA for its first task, one more in vain
+  return launch_after(kernel, dim3(grid), kThreadsS, smem, s, args, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
                       *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
 }
 

@@ -17,13 +17,15 @@ constexpr int kStreamRowsMax = 16;
 //   [16]  the queue head of dynamic dealing (its own cache line)
 //   [17], [19]  the same two words for the second of two launches
 //   [18]  CTAs that have finished
+//   [20]  whether a CTA has taken on the cleaning after a failure
 //   [32 ..] one completion counter per merge unit
-// all of which are zero when a run starts: the last CTA of a run puts them back (end_of_run; the
-// CTA-pair kernel has them cleared by a memset instead); and in front of them, untouched by that,
+// all of which are zero when a run starts: they wrap or are put back by the run before (end_of_run;
+// the CTA-pair kernel has them cleared by a memset instead); and in front of them, untouched by that,
 //   [-8]  the sticky record of failures that xy_attn_device_status reports and clears
 //   [-7]  the number of polls after which a bounded wait gives up (ptx.cuh reads the same word).
 constexpr int kStatusQueueHead = 16;
 constexpr int kStatusExits = 18;
+constexpr int kStatusCleaner = 20;
 constexpr int kStatusUnitCounts = 32;
 constexpr int kStatusSticky = -8;
 constexpr int kStatusWaitLimit = -7;
@@ -133,6 +135,7 @@ struct RunArgs {
   const int32_t* queue;
   int32_t* queue_head;
   int32_t num_tasks, dynamic, num_workers, num_units;
+  uint32_t queue_wrap;     // index of the launch's last grab, which wraps the head to zero
   int32_t* exits;          // word of the status block that counts the CTAs that have finished
   int32_t side_by_side;    // 1, 2: first (dense) and second (streaming) of two launches that run at the same time
   // split units whose last finishing task merges them inside the kernel (streaming units)

@@ -73,3 +73,37 @@ def test_debug_context_rejects_a_bad_block_table_before_launching():
     H.check_against_oracle(d.o.float().cpu().numpy().astype(np.float64), d.lse.cpu().numpy().astype(np.float64),
                            O_ref, LSE_ref, "debug context")
     ctx.close()
+
+
+@pytest.mark.parametrize("workers,decode", [(3, True), (40, True), (0, True), (5, False), (0, False)],
+                         ids=["stream-6", "stream-80", "stream-all", "meta-5", "meta-all"])
+def test_many_ctas_that_give_up_leave_a_clean_context(workers, decode):
+    """Every CTA gives up after a fill that never comes, with split units half counted and the queue half
+    dealt: the next ordinary run, with and without reading the status in between, is right, and bitwise
+    what the runs before the failure gave."""
+    b = W.config2_decode(num_requests=9, kv_lo=300, kv_hi=3000) if decode else W.config1_tiny()
+    t = W.make_tensors(b)
+    ctx = H.make_ctx(b, num_workers=workers)
+    ctx.plan_batch(b)
+    d = H.DeviceBatch(b, t)
+
+    def run():
+        o, lse = torch.full_like(d.o, float("nan")), torch.full_like(d.lse, float("nan"))
+        ctx.run(d.q, d.k_pool, d.v_pool, d.block_table, H.SCALE, o, lse)
+        return o, lse
+
+    good = [run() for _ in range(3)]
+    for read in (True, False):
+        ctx.debug_inject(wait_limit_polls=20000, skip_fill=1)
+        run()
+        ctx.debug_inject(0, -1)
+        if read:
+            assert ctx.device_status() == xb.XY_ERR_DEVICE_TIMEOUT
+        good += [run() for _ in range(2)]
+    assert ctx.device_status() == xb.XY_ERR_DEVICE_TIMEOUT and ctx.device_status() == 0
+    O_ref, LSE_ref = oracle.attention(b, t, H.SCALE)
+    for o, lse in good:
+        assert torch.equal(lse, good[0][1])
+    o, lse = good[-1]
+    H.check_against_oracle(o.float().cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64), O_ref, LSE_ref,
+                           "run after a timeout")
