@@ -52,7 +52,9 @@ enum { XY_MASK_CAUSAL = 0, XY_MASK_TREE = 1 };
 enum {
   XY_KERNEL_AUTO = 0,      /* the product path: tcgen05 dense tiles (prefill, verify; 256 packed rows per
                               task) side by side with streaming tiles (decode) in one launch, tasks
-                              dealt from one mixed queue */
+                              dealt from one mixed queue; a batch without dense tiles on a kernel of its
+                              own with two CTAs per SM; shared-prefix groups with a small dense part as
+                              two launches that run at the same time */
   XY_KERNEL_REFERENCE = 1, /* plain SIMT kernel for every tile: slow, kept for bisecting */
   XY_KERNEL_MMA = 2,       /* warp-level mma.sync tiles for every task (dense tasks too) */
   XY_KERNEL_PAIR = 3       /* experimental: dense tiles on CTA pairs (tcgen05 cta_group::2, 512 packed
@@ -342,7 +344,8 @@ int xy_attn_debug_gather(xy_attn_ctx* ctx, int32_t req, int32_t kv_head, const v
  * and copies 4 x num_workers values to `out` (HOST): for each persistent worker its entry and
  * exit time stamps (nanoseconds of the GPU's global timer) and the nanoseconds it spent in dense
  * and in streaming tasks.  Returns the number of entries; copies only if `cap`
- * is large enough.  Only the attention meta-kernel records them (not XY_KERNEL_REFERENCE). */
+ * is large enough.  XY_KERNEL_REFERENCE records none; of the streaming kernel's up to two CTAs per
+ * worker the first num_workers are recorded. */
 int xy_attn_worker_times(xy_attn_ctx* ctx, uint64_t* out, int32_t cap);
 
 /* Debug tracing (only in a library built with -DXY_ENABLE_TRACE, i.e. XY_BUILD_TRACE=1 for
