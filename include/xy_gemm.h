@@ -34,11 +34,11 @@ extern "C" {
  *   tile_n  columns per tile: 32, 64, 128, 256 (128-row tiles on single CTAs), XY_GEMM_PAIR | 128
  *           or XY_GEMM_PAIR | 256 (256-row tiles on CTA pairs), or 0 to let the library choose:
  *           up to 128 tokens a kernel that streams W (128 rows of W per CTA, all tokens as the
- *           columns, K split over a thread-block cluster); up to about 1500 tokens 256 rows of W on
- *           a CTA pair with up to 512 tokens as the columns, K split over the pairs of a cluster when
- *           there is scratch (xy_gemm_run_ws); without scratch, for M <= 512 with few tiles, 128 x 128
- *           tiles whose K is split over a cluster; else 256 x 256 pair tiles when M pads to a multiple
- *           of 256 with at most 15 % waste and those tiles number at least a quarter of the SMs; else
+ *           columns, K split over a thread-block cluster); up to 1536 tokens, where a time model finds it
+ *           the faster one, 256 rows of W on a CTA pair with up to 512 tokens as the columns, K split over
+ *           the pairs of a cluster when there is scratch (xy_gemm_run_ws); else 256 x 256 pair tiles when M
+ *           pads to a multiple of 256 with at most 15 % waste and those tiles number at least a quarter of
+ *           the SMs; else, for M <= 512 with few tiles, 128 x 128 tiles whose K is split over a cluster; else
  *           128 x 256 tiles when they give half of the SMs a tile, else 128 x 128
  * Returns XY_OK, XY_ERR_INVALID_ARG (null pointer, bad size or alignment), XY_ERR_UNSUPPORTED
  * (tile_n not one of the values above) or XY_ERR_CUDA.  Calls on one stream are ordered; the caller
@@ -62,6 +62,17 @@ int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t ldw, void*
 /* Bytes of scratch xy_gemm_run_ws can use on the current device (2 slots of a 128 x 256 fp32 tile
  * per SM: 38.8 MB with 148 SMs), or -1 if the device cannot be queried. */
 int64_t xy_gemm_workspace_bytes(void);
+
+/* Which kernel a call with tile_n = 0 and this much scratch takes, and how it cuts the problem.  Host
+ * arithmetic; for tests and tools.
+ *   device  HOST, 13 numbers that describe a device: its SMs; thread-block clusters of 1 .. 8 CTAs that fit
+ *           at once with one CTA per SM (8 numbers); clusters of 1 .. 4 CTA pairs (4 numbers).  NULL: the
+ *           current device is asked.
+ *   out     HOST, 6 numbers: kernel (0 tiles of 128 x tile_n, 1 tiles of 256 x tile_n on CTA pairs, 2
+ *           128 x 128 tiles with K split over a cluster, 3 weight-major on CTA pairs, 4 weight-streaming),
+ *           tile_n, slices of K, and for kernel 3 the token tiles, their tokens and MMAs per K step
+ * Returns XY_OK, XY_ERR_INVALID_ARG or XY_ERR_CUDA. */
+int xy_gemm_choice(int32_t M, int32_t N, int32_t K, int64_t workspace_bytes, const int32_t* device, int32_t* out);
 
 /* Status of the device-side waits of the GEMM kernels on the current device since the last call of
  * this function: 0, or XY_ERR_DEVICE_TIMEOUT if a bounded wait inside a kernel gave up (the

@@ -18,6 +18,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "gemm_choice.h"
 #include "ptx.cuh"
 #include "xy_gemm.h"
 
@@ -475,7 +476,7 @@ __global__ void __launch_bounds__(128) gemm_fixup_kernel(const GemmParams P) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Split-K variant for 129 .. 512 tokens without scratch (few tiles).  A whole-K tile is one serial
+// Split-K variant for 129 .. 512 tokens (few tiles).  A whole-K tile is one serial
 // chain of K/64 chunks on one SM, and with fewer tiles than SMs most of the chip idles while the
 // weights stream through a few SMs.  Here a cluster of `splits` CTAs shares one 128 x 128 tile:
 // CTA r computes the partial product over its slice of K, writes the valid rows of its fp32
@@ -673,7 +674,6 @@ struct SwapParams {
   float4* ws;  // splits > 1: [tile][split][rank][tok / 4][128]
 };
 constexpr int kSwapMaxStages = 12;
-constexpr int kSwapMaxSplits = 4;  // a cluster of eight CTAs
 constexpr int kSwapRing = 212992;  // bytes of ring at most
 constexpr int kSwapSmem = 1024 + kSwapRing + 512;
 
@@ -946,7 +946,8 @@ struct SmallParams {
   uint32_t tmem_cols;
 };
 constexpr int kSmallMaxStages = 8;
-constexpr int kSmallMaxSplits = 8;
+constexpr int kSmallMaxSplits = kClusterMaxCtas;
+constexpr int kSmallSmem = 115712;  // two CTAs per SM
 
 struct __align__(8) SmallBarriers {
   uint64_t full[kSmallMaxStages], empty[kSmallMaxStages];
@@ -1276,46 +1277,6 @@ cudaError_t max_clusters(Kernel kernel, int size, int smem, int* count) {
   return cudaOccupancyMaxActiveClusters(count, kernel, &cfg);
 }
 
-// How a problem is cut for the weight-major kernel, and the time the model below expects.
-struct SwapPlan {
-  int m_tiles = 0, tok = 0, halves = 1, splits = 1;
-  float us = 1e30f;
-};
-
-// The model is fitted to measurements at 64 - 1300 tokens on the Linear shapes of three models (hidden
-// 3584, 4096, 8192; within 5 % for most, up to 25 % short where power limits the clock).  Per K chunk a
-// CTA pair takes its MMAs (64 cycles per instruction at least, 1.3 of the nominal rate) or the SM's
-// intake of 50 B a clock, whichever is longer; every wave of tiles also takes its weights' time in HBM;
-// a store of the sums is not overlapped when they fill tensor memory; splitting K costs the exchange of
-// sums, and pays only while every cluster fits the device at once.
-SwapPlan swap_plan(int M, int N, int K, int64_t workspace_bytes, const int* clusters) {
-  SwapPlan best;
-  const int n_tiles = (N + 255) / 256, k_chunks = (K + kChunkK - 1) / kChunkK;
-  const int m_lo = (M + 511) / 512;
-  for (int m_tiles = m_lo; m_tiles <= m_lo + 4; ++m_tiles) {
-    const int per = (M + m_tiles - 1) / m_tiles;
-    const int halves = per > 256 ? 2 : 1;
-    const int tok = (per + 16 * halves - 1) / (16 * halves) * 16 * halves;
-    if ((m_tiles - 1) * tok >= M) continue;
-    for (int splits = 1; splits <= kSwapMaxSplits; ++splits) {
-      const int tiles = m_tiles * n_tiles, cps = (k_chunks + splits - 1) / splits, fit = clusters[splits - 1];
-      if (fit < 1) continue;
-      if (splits > 1 && (tiles > fit || cps < 8 || (splits - 1) * cps >= k_chunks ||
-                         static_cast<int64_t>(tiles) * splits * tok * 1024 > workspace_bytes))
-        continue;
-      const float mma = 4.f * halves * std::max(64.f, 0.5f * tok / halves) * 1.3f, intake = (kABytes + 64.f * tok) / 50.f;
-      const float chain = cps * std::max(mma, intake) / 1900.f + (2 * tok > 512 ? tok * 0.010f : 0.f);
-      auto wave = [&](int t) {  // the token tiles of a weight tile share its bytes
-        return std::max(chain, 512.f * K * t / (6.3e6f * m_tiles));
-      };
-      const float us = (tiles / fit) * wave(fit) + (tiles % fit ? wave(tiles % fit) : 0.f) + 4.f + tok * 0.006f +
-                       (splits > 1 ? 1.5f + tok * 0.010f : 0.f);
-      if (us < 0.98f * best.us) best = SwapPlan{m_tiles, tok, halves, splits, us};
-    }
-  }
-  return best;
-}
-
 cudaError_t launch_gemm_swap(const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int M, int N, int K,
                              const SwapPlan& plan, int clusters, void* workspace, cudaStream_t s) {
   CUtensorMap a_map, w_map;
@@ -1358,41 +1319,32 @@ cudaError_t launch_gemm_swap(const void* a, int64_t lda, const void* w, int64_t 
   return cudaLaunchKernelEx(&cfg, smooth_gemm_swap_kernel, P, a_map, w_map);
 }
 
-// Clusters of 2, 4, 6 and 8 CTAs of the weight-major kernel that fit the device at once (asked once per
-// device, together with the kernel's opt-in to large shared memory).
-cudaError_t swap_clusters(int dev, const int** out) {
-  static int counts[64][kSwapMaxSplits];
+// Asks once per device how many clusters fit, and opts the cluster kernels in to large shared memory.
+cudaError_t query_device(int sms, GemmDevice* d) {
+  d->sms = sms;
+  cudaError_t e = cudaFuncSetAttribute(smooth_gemm_swap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwapSmem);
+  for (int sp = 1; sp <= kSwapMaxSplits && e == cudaSuccess; ++sp)
+    e = max_clusters(smooth_gemm_swap_kernel, 2 * sp, kSwapSmem, &d->pair_clusters[sp - 1]);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  d->clusters[0] = sms;
+  for (int n = 2; n <= kClusterMaxCtas && e == cudaSuccess; ++n)  // (the answer counts one CTA per SM; two run)
+    e = max_clusters(smooth_gemm_small_kernel, n, kSmallSmem, &d->clusters[n - 1]);
+  return e;
+}
+
+cudaError_t gemm_device(int dev, int sms, GemmDevice* out) {
+  static GemmDevice known[64];
   static std::once_flag once[64];
   static cudaError_t err[64];
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::call_once(once[dev], [&] {
-    err[dev] = cudaFuncSetAttribute(smooth_gemm_swap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwapSmem);
-    for (int sp = 1; sp <= kSwapMaxSplits && err[dev] == cudaSuccess; ++sp)
-      err[dev] = max_clusters(smooth_gemm_swap_kernel, 2 * sp, kSwapSmem, &counts[dev][sp - 1]);
-  });
-  *out = counts[dev];
+  if (dev < 0 || dev >= 64) return query_device(sms, out);
+  std::call_once(once[dev], [&] { err[dev] = query_device(sms, &known[dev]); });
+  *out = known[dev];
   return err[dev];
 }
 
-cudaError_t launch_gemm_small(int dev, const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int M, int N,
-                              int K, int num_sms, cudaStream_t s) {
-  constexpr int kMaxSmem = 115712;  // two CTAs per SM
-  // Clusters of 1 .. 8 CTAs that fit the device at once (asked once per device; the answer counts one CTA
-  // per SM, two run).
-  static int fit[64][kSmallMaxSplits];
-  static std::once_flag once[64];
-  static cudaError_t err[64];
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::call_once(once[dev], [&] {
-    err[dev] = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-    if (err[dev] == cudaSuccess)
-      err[dev] = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    for (int sp = 2; sp <= kSmallMaxSplits && err[dev] == cudaSuccess; ++sp) {
-      err[dev] = max_clusters(smooth_gemm_small_kernel, sp, kMaxSmem, &fit[dev][sp - 1]);
-      fit[dev][sp - 1] *= 2;
-    }
-  });
-  if (err[dev] != cudaSuccess) return err[dev];
+cudaError_t launch_gemm_small(const GemmDevice& dev, const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc,
+                              int M, int N, int K, cudaStream_t s) {
   SmallParams P = {};
   P.c = static_cast<uint16_t*>(c);
   P.ldc = ldc;
@@ -1403,7 +1355,7 @@ cudaError_t launch_gemm_small(int dev, const void* a, int64_t lda, const void* w
   CUtensorMap a_map, w_map;
   if (!encode_matrix_map(&a_map, a, M, K, lda, P.tok) || !encode_matrix_map(&w_map, w, N, K, ldw, 128)) return cudaErrorInvalidValue;
   const int stage = kABytes + P.tok * 128;
-  P.stages = std::min(kSmallMaxStages, (kMaxSmem - 1024 - static_cast<int>(sizeof(SmallBarriers))) / stage);
+  P.stages = std::min(kSmallMaxStages, (kSmallSmem - 1024 - static_cast<int>(sizeof(SmallBarriers))) / stage);
   const int tiles = (N + 127) / 128, k_chunks = (K + kChunkK - 1) / kChunkK;
   // Two CTAs per SM with the deeper ring (three with a shorter one: GateUp at 64 tokens 45.4 against 41.5
   // us, Down 26.2 / 23.5), and the most CTAs per tile whose clusters fit at once but for one or two: a
@@ -1412,7 +1364,7 @@ cudaError_t launch_gemm_small(int dev, const void* a, int64_t lda, const void* w
   // chunks per CTA.
   P.splits = 1;
   for (int sp = 2; sp <= kSmallMaxSplits && sp * 6 <= k_chunks; ++sp)
-    if (tiles * 15 <= fit[dev][sp - 1] * 16) P.splits = sp;
+    if (tiles * 15 <= 2 * dev.clusters[sp - 1] * 16) P.splits = sp;
   P.cps = (k_chunks + P.splits - 1) / P.splits;
   P.splits = (k_chunks + P.cps - 1) / P.cps;  // no CTA without a chunk
   P.tmem_cols = 32;
@@ -1477,76 +1429,35 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
       return XY_ERR_CUDA;
     if (dev >= 0 && dev < 64) sm_count[dev] = sms;
   }
-  if (tile_n == 0 && !pair && M <= 128) {
-    // Up to 128 tokens are bound by the bytes of W; the kernel for that.  Measured, here / before (whole
-    // tiles or a split of K with padded token rows): hidden 4096, 16 tokens QKV 10.7 / 14.2 us, OProj 8.4 /
-    // 10.6, GateUp 39.7 / 42.9, Down 20.3 / 23.9; hidden 3584, QKV 8.5 / 19.8, OProj 7.3 / 19.2, Down 24 / 53.
-    const cudaError_t e = xy::launch_gemm_small(dev, a, lda, w, ldw, c, ldc, M, N, K, sms, static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
-  }
-  if (tile_n == 0 && !pair && workspace == nullptr && M > 128 && M <= 512) {
-    // No scratch, few tiles and one long serial chain over K per tile: split K over a cluster when that
-    // puts several times as many SMs to work (Down / OProj projections of a short chunk; Down at 200
-    // tokens 38.8 us, the weight-major kernel with whole chains about 70, with scratch 31).  Measured: four or more slices pay off from 16 chunks per slice on; two or three
-    // only when the chain is long (32 chunks per slice), else the reduction costs what the
-    // shorter chain saves.
-    const int tiles = ((M + 127) / 128) * ((N + 127) / 128), k_chunks = (K + 63) / 64;
-    int splits = sms / tiles;
-    if (splits > 8) splits = 8;
-    while (splits >= 2 && k_chunks / splits < (splits >= 4 ? 16 : 32)) --splits;
-    if (splits >= 2) {
-      const cudaError_t e =
-          xy::launch_gemm_splitk(a, lda, w, ldw, c, ldc, M, N, K, splits, static_cast<cudaStream_t>(stream));
-      return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
-    }
-  }
-  if (tile_n == 0 && !pair && sms >= 2 && M > 128 && M <= 1536) {
-    // The weight-major kernel when its model beats that of 256 x 256 tiles (0.35 us per K chunk and wave).
-    // Measured, here / the choices below: hidden 4096, 333 tokens QKV 21.1 / 23.3 us, OProj 17.7 / 21.7,
-    // GateUp 73 / 86, Down 40 / 63; 777 tokens 33 / 53, 24 / 28, 149 / 170, 75 / 88; from about 1500
-    // tokens on both are bound by the MMAs, and the 256 x 256 tiles overlap their stores.
-    const int* clusters = nullptr;
-    if (xy::swap_clusters(dev, &clusters) != cudaSuccess) return XY_ERR_CUDA;
-    const xy::SwapPlan plan = xy::swap_plan(M, N, K, workspace != nullptr ? workspace_bytes : 0, clusters);
-    const int tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = sms / 2;
-    const float pair_us = static_cast<float>((tiles + pairs - 1) / pairs) * ((K + 63) / 64) * 0.35f + 5.f;
-    // Up to 217 tokens a tile of 256 rows would be more than 15 % padding and is not taken below, so that the
-    // weight-major kernel stands against 128 x 256 tiles, which lose everywhere: GateUp at 200 tokens
-    // 51 / 63 us, N 28672 x K 4096 at 129 tokens 49 / 62, N 57344 x K 8192 at 129 tokens 181 / 234.  (With more
-    // tokens they do not: GateUp at 600 tokens 127 / 105.)
-    if (M <= 217 || plan.us < 0.97f * pair_us) {
-      const cudaError_t e = xy::launch_gemm_swap(a, lda, w, ldw, c, ldc, M, N, K, plan, clusters[plan.splits - 1], workspace,
-                                                 static_cast<cudaStream_t>(stream));
-      return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
-    }
-  }
-  if (tile_n == 0 && !pair && sms >= 2 && M > 128) {
-    // 256 x 256 tiles on CTA pairs when the padding of M to 256 rows stays under 15 % and the tiles
-    // give at least half of the pairs work: measured best or level with the best from 1024 tokens
-    // on (at 4096 tokens QKV 155 -> 143 us, OProj 105 -> 96, GateUp 667 -> 609, Down 369 -> 339).
-    const int mp = (M + 255) / 256, np = (N + 255) / 256;
-    if ((mp * 256 - M) * 100 <= 15 * mp * 256 && mp * np * 4 >= sms) {
-      pair = true;
-      tile_n = 256;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  cudaError_t e;
+  if (tile_n == 0) {
+    xy::GemmDevice gd;
+    if (xy::gemm_device(dev, sms, &gd) != cudaSuccess) return XY_ERR_CUDA;
+    const xy::GemmChoice ch = xy::choose_gemm(M, N, K, workspace != nullptr ? workspace_bytes : 0, gd);
+    switch (ch.kernel) {
+      case xy::kGemmSmall:
+        // Up to 128 tokens are bound by the bytes of W; the kernel for that.  Measured, here / before (whole
+        // tiles or a split of K with padded token rows): hidden 4096, 16 tokens QKV 10.7 / 14.2 us, OProj 8.4 /
+        // 10.6, GateUp 39.7 / 42.9, Down 20.3 / 23.9; hidden 3584, QKV 8.5 / 19.8, OProj 7.3 / 19.2, Down 24 / 53.
+        e = xy::launch_gemm_small(gd, a, lda, w, ldw, c, ldc, M, N, K, s);
+        return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
+      case xy::kGemmSwap:
+        e = xy::launch_gemm_swap(a, lda, w, ldw, c, ldc, M, N, K, ch.swap, gd.pair_clusters[ch.splits - 1], workspace, s);
+        return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
+      case xy::kGemmSplitK:
+        e = xy::launch_gemm_splitk(a, lda, w, ldw, c, ldc, M, N, K, ch.splits, s);
+        return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
+      case xy::kGemmPair: pair = true; [[fallthrough]];
+      default: tile_n = ch.tile_n;
     }
   }
   if (pair) {
     if (sms < 2) return XY_ERR_UNSUPPORTED;
-    const cudaError_t e =
-        tile_n == 256 ? xy::launch_gemm_pair<256>(a, lda, w, ldw, c, ldc, M, N, K, sms, static_cast<cudaStream_t>(stream))
-                      : xy::launch_gemm_pair<128>(a, lda, w, ldw, c, ldc, M, N, K, sms, static_cast<cudaStream_t>(stream));
+    e = tile_n == 256 ? xy::launch_gemm_pair<256>(a, lda, w, ldw, c, ldc, M, N, K, sms, s)
+                      : xy::launch_gemm_pair<128>(a, lda, w, ldw, c, ldc, M, N, K, sms, s);
     return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
   }
-  if (tile_n == 0) {
-    // 128 x 256 tiles read the least of A and W per flop; they are used when they give at least
-    // half of the SMs a tile (measured: OProj at 1024 tokens, 128 such tiles, 28 us against 44 us
-    // with 128 x 128; GateUp at 16 tokens 44 against 49 us).  Below that 128 x 128 (narrower tiles
-    // are not faster for small M, where the time is launch and pipeline-fill latency).
-    const int64_t tiles256 = static_cast<int64_t>((M + 127) / 128) * ((N + 255) / 256);
-    tile_n = tiles256 * 2 >= sms ? 256 : 128;
-  }
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e;
   switch (tile_n) {
     case 256: e = xy::launch_gemm<256>(a, lda, w, ldw, c, ldc, M, N, K, sms, workspace, workspace_bytes, s); break;
     case 128: e = xy::launch_gemm<128>(a, lda, w, ldw, c, ldc, M, N, K, sms, workspace, workspace_bytes, s); break;
@@ -1554,6 +1465,31 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
     default: e = xy::launch_gemm<32>(a, lda, w, ldw, c, ldc, M, N, K, sms, workspace, workspace_bytes, s); break;
   }
   return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
+}
+
+extern "C" int xy_gemm_choice(int32_t M, int32_t N, int32_t K, int64_t workspace_bytes, const int32_t* device, int32_t* out) {
+  if (out == nullptr || M < 1 || N < 8 || K < 8 || workspace_bytes < 0) return XY_ERR_INVALID_ARG;
+  xy::GemmDevice gd;
+  if (device != nullptr) {
+    if (device[0] < 1) return XY_ERR_INVALID_ARG;
+    gd.sms = device[0];
+    for (int i = 0; i < xy::kClusterMaxCtas; ++i) gd.clusters[i] = device[1 + i];
+    for (int i = 0; i < xy::kSwapMaxSplits; ++i) gd.pair_clusters[i] = device[1 + xy::kClusterMaxCtas + i];
+  } else {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1 ||
+        xy::gemm_device(dev, sms, &gd) != cudaSuccess)
+      return XY_ERR_CUDA;
+  }
+  const xy::GemmChoice ch = xy::choose_gemm(M, N, K, workspace_bytes, gd);
+  out[0] = ch.kernel;
+  out[1] = ch.tile_n;
+  out[2] = ch.splits;
+  out[3] = ch.swap.m_tiles;
+  out[4] = ch.swap.tok;
+  out[5] = ch.swap.halves;
+  return XY_OK;
 }
 
 extern "C" int xy_gemm_device_status(int32_t* status) {

@@ -2,13 +2,13 @@
 from __future__ import annotations
 
 import ctypes
-from typing import Optional
+from typing import Optional, Sequence
 
 import torch
 
 from . import binding as xb
 
-GEMM_EXPORTS = ("xy_gemm_run", "xy_gemm_run_ws", "xy_gemm_workspace_bytes", "xy_gemm_device_status")
+GEMM_EXPORTS = ("xy_gemm_run", "xy_gemm_run_ws", "xy_gemm_workspace_bytes", "xy_gemm_choice", "xy_gemm_device_status")
 
 XY_GEMM_PAIR = 0x1000  # tile_n flag: 256-row tiles on CTA pairs
 
@@ -22,6 +22,8 @@ def declare(L) -> None:
     L.xy_gemm_run_ws.restype = ctypes.c_int
     L.xy_gemm_workspace_bytes.argtypes = []
     L.xy_gemm_workspace_bytes.restype = i64
+    L.xy_gemm_choice.argtypes = [i32, i32, i32, i64, vp, vp]
+    L.xy_gemm_choice.restype = ctypes.c_int
     L.xy_gemm_device_status.argtypes = [ctypes.POINTER(i32)]
     L.xy_gemm_device_status.restype = ctypes.c_int
 
@@ -68,6 +70,20 @@ def xy_gemm_run(a: torch.Tensor, w: torch.Tensor, c: torch.Tensor, tile_n: int =
                                    int(tile_n), workspace.data_ptr(), workspace.numel(), xb._stream_ptr(stream))
     if rc != 0:
         raise xb.XYAttnError(rc, "xy_gemm_run failed")
+
+
+GEMM_KERNELS = ("tile", "pair", "split_k", "weight_major", "weight_streaming")
+
+
+def xy_gemm_choice(M: int, N: int, K: int, workspace_bytes: int = 0, device: Optional[Sequence[int]] = None) -> dict:
+    """What xy_gemm_run(tile_n=0) takes for these sizes, on the current device or on one described by 13
+    numbers (see include/xy_gemm.h; nothing is asked of a GPU then)."""
+    dev = (ctypes.c_int32 * 13)(*device) if device is not None else None
+    out = (ctypes.c_int32 * 6)()
+    rc = _lib().xy_gemm_choice(M, N, K, workspace_bytes, dev, out)
+    if rc != 0:
+        raise xb.XYAttnError(rc, "xy_gemm_choice failed")
+    return dict(kernel=GEMM_KERNELS[out[0]], tile_n=out[1], splits=out[2], m_tiles=out[3], tok=out[4], halves=out[5])
 
 
 def xy_gemm_device_status() -> int:

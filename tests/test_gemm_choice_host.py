@@ -1,0 +1,64 @@
+"""Which kernel SmoothGEMM takes (xy_gemm_choice), for the device the time models were fitted on: 148 SMs,
+clusters of 1 .. 8 CTAs and of 1 .. 4 pairs as the occupancy query counts them there."""
+import pytest
+
+from paper_2412_18106_b200 import gemm as xg
+
+B200 = [148, 148, 74, 45, 33, 26, 22, 15, 15, 74, 33, 22, 15]
+SCRATCH = 2 * 148 * 128 * 256 * 4
+
+
+def choice(M, N, K, scratch=SCRATCH, device=B200):
+    return xg.xy_gemm_choice(M, N, K, scratch, device)
+
+
+# Measured (us): what is chosen against the weight-major kernel.
+@pytest.mark.parametrize("M,N,K,scratch,kernel,tile_n", [
+    (352, 10240, 8192, 0, "tile", 256),        # 64 / 74
+    (384, 10240, 8192, SCRATCH, "tile", 256),  # 64 / 73
+    (448, 4096, 512, 0, "tile", 128),          # 6.8 / 8.5
+    (512, 4096, 512, SCRATCH, "tile", 128),    # 6.8 / 8.8
+    (1025, 4096, 512, 0, "tile", 256),         # 8.6 / 12.2
+    (1500, 1032, 2304, 0, "tile", 128),        # 14 / 18
+    (333, 256, 28672, SCRATCH, "split_k", 128),  # 22 / 30
+    (1024, 8, 512, SCRATCH, "tile", 128),      # 5.3 / 8.6
+    (820, 10240, 8192, 0, "tile", 256),        # 119 / 124
+])
+def test_kernels_that_beat_the_weight_major_one_are_taken(M, N, K, scratch, kernel, tile_n):
+    c = choice(M, N, K, scratch)
+    assert (c["kernel"], c["tile_n"]) == (kernel, tile_n), c
+
+
+# Measured (us): the weight-major kernel against the one that would run otherwise.
+@pytest.mark.parametrize("M,N,K,scratch", [
+    (600, 28672, 4096, 0),              # 112 / 130
+    (333, 28672, 4096, SCRATCH),        # 73 / 86
+    (333, 4096, 14336, SCRATCH),        # 40 / 63
+    (333, 6144, 4096, SCRATCH),         # 21 / 23
+    (129, 57344, 8192, 0),              # 181 / 234
+    (820, 3584, 18944, SCRATCH),        # 93 / 134
+])
+def test_the_weight_major_kernel_is_taken_where_it_is_faster(M, N, K, scratch):
+    assert choice(M, N, K, scratch)["kernel"] == "weight_major"
+
+
+def test_a_device_without_room_for_pairs_takes_the_other_kernels():
+    c = choice(333, 28672, 4096, device=B200[:9] + [0, 0, 0, 0])
+    assert c["kernel"] == "tile" and c["tok"] == 0
+    assert choice(333, 28672, 4096, device=[1] + [1] + [0] * 7 + [0] * 4)["kernel"] == "tile"
+
+
+@pytest.mark.parametrize("M", [1, 128, 129, 255, 333, 512, 513, 1025, 1536, 1537, 4096])
+@pytest.mark.parametrize("N,K", [(8, 8), (4096, 14336), (131072, 8192), (1032, 2304)])
+def test_cuts_cover_the_tokens_and_fit(M, N, K):
+    for scratch in (0, SCRATCH):
+        c = choice(M, N, K, scratch)
+        if c["kernel"] != "weight_major":
+            continue
+        assert 128 < M <= 1536
+        assert (c["m_tiles"] - 1) * c["tok"] < M <= c["m_tiles"] * c["tok"]
+        assert c["tok"] % (16 * c["halves"]) == 0 and c["tok"] // c["halves"] <= 256 and c["halves"] in (1, 2)
+        n_tiles = (N + 255) // 256
+        if c["splits"] > 1:
+            assert c["m_tiles"] * n_tiles * c["splits"] * c["tok"] * 1024 <= scratch
+            assert c["m_tiles"] * n_tiles <= B200[8 + c["splits"]]
