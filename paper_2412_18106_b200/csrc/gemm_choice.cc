@@ -142,6 +142,7 @@ SwapPlan swap_plan(int M, int N, int K, int64_t workspace_bytes, const GemmDevic
 }  // namespace
 
 GemmChoice choose_gemm(int M, int N, int K, int64_t workspace_bytes, const GemmDevice& dev) {
+  if (workspace_bytes < gemm_scratch_bytes(dev.sms)) workspace_bytes = 0;
   GemmChoice c = token_major(M, N, K, dev);
   if (M <= 128) {
     c.kernel = kGemmSmall;

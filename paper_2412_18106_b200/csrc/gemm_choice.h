@@ -24,6 +24,9 @@ struct GemmDevice {
   int pair_clusters[kSwapMaxSplits] = {0};   // clusters of 1 .. 4 pairs of the weight-major kernel
 };
 
+// Scratch the kernels can use, in bytes: two slots of a 128 x 256 fp32 tile per SM.  Less is none.
+constexpr int64_t gemm_scratch_bytes(int sms) { return static_cast<int64_t>(sms) * 2 * 128 * 256 * 4; }
+
 // How a problem is cut for the weight-major kernel (tok = 0: no cut fits the device).
 struct SwapPlan {
   int m_tiles = 0, tok = 0, halves = 1, splits = 1;

@@ -1394,7 +1394,7 @@ extern "C" int64_t xy_gemm_workspace_bytes(void) {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return -1;
-  return xy::gemm_workspace_bytes(256, sms);
+  return xy::gemm_scratch_bytes(sms);
 }
 
 extern "C" int xy_gemm_run(const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int32_t M,

@@ -62,3 +62,9 @@ def test_cuts_cover_the_tokens_and_fit(M, N, K):
         if c["splits"] > 1:
             assert c["m_tiles"] * n_tiles * c["splits"] * c["tok"] * 1024 <= scratch
             assert c["m_tiles"] * n_tiles <= B200[8 + c["splits"]]
+
+
+@pytest.mark.parametrize("scratch", [1024, SCRATCH // 2, SCRATCH - 16])
+@pytest.mark.parametrize("M,N,K", [(200, 4096, 14336), (333, 4096, 14336), (200, 4096, 4096), (700, 2048, 4096)])
+def test_too_little_scratch_is_none(M, N, K, scratch):
+    assert choice(M, N, K, scratch) == choice(M, N, K, 0)

@@ -206,3 +206,18 @@ def test_weight_streaming_kernel_matches_oracle_and_repeats_bitwise(M, N, K):
     ref = G.linear(a, w)
     d = np.abs(out[0].float().cpu().numpy().astype(np.float64) - ref)
     assert np.all(d <= 2.0 ** -8 * np.abs(ref) + 2.0 ** -14 * np.sqrt(K)), d.max()
+
+
+@pytest.mark.parametrize("size", [1024, 8 << 20])
+def test_too_little_scratch_gives_the_result_without_scratch(size):
+    """200 tokens, where both a cluster split and pairs that share K through scratch can run; what lies behind a
+    too small buffer is not written, nor is the buffer."""
+    M, N, K = 200, 4096, 4104
+    g = torch.Generator().manual_seed(8)
+    a, w = (torch.randn(s, generator=g).to(torch.bfloat16).cuda() for s in ((M, K), (N, K)))
+    buf = torch.full((xg.xy_gemm_workspace("cuda").numel(),), 0x5A, dtype=torch.uint8, device="cuda")
+    c, ref = (torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    xg.xy_gemm_run(a, w, c, workspace=buf[:size])
+    xg.xy_gemm_run(a, w, ref)
+    assert xg.xy_gemm_device_status() == 0
+    assert torch.equal(c, ref) and bool((buf == 0x5A).all())
