@@ -33,12 +33,12 @@ extern "C" {
  *   pointers 16-byte aligned
  *   tile_n  columns per tile: 32, 64, 128, 256 (128-row tiles on single CTAs), XY_GEMM_PAIR | 128
  *           or XY_GEMM_PAIR | 256 (256-row tiles on CTA pairs), or 0 to let the library choose:
- *           up to 128 tokens a kernel that streams W (128 rows of W per CTA, all tokens as the
- *           columns, K split over a thread-block cluster); up to 1536 tokens, where a time model finds it
- *           the faster one, 256 rows of W on a CTA pair with up to 512 tokens as the columns, K split over
- *           the pairs of a cluster when there is scratch (xy_gemm_run_ws); else 256 x 256 pair tiles when M
- *           pads to a multiple of 256 with at most 15 % waste and those tiles number at least a quarter of
- *           the SMs; else, for M <= 512 with few tiles, 128 x 128 tiles whose K is split over a cluster; else
+ *           where a time model finds it the faster one, up to 128 tokens a kernel that streams W (128 rows
+ *           of W per CTA, all tokens as the columns, K split over a thread-block cluster), up to 1536
+ *           tokens 256 rows of W on a CTA pair with up to 512 tokens as the columns, K split over the pairs
+ *           of a cluster when there is scratch (xy_gemm_run_ws); else 256 x 256 pair tiles when M pads to a
+ *           multiple of 256 with at most 15 % waste and those tiles number at least a quarter of the SMs;
+ *           else, for M <= 512 with few tiles, 128 x 128 tiles whose K is split over a cluster; else
  *           128 x 256 tiles when they give half of the SMs a tile, else 128 x 128
  * Returns XY_OK, XY_ERR_INVALID_ARG (null pointer, bad size or alignment), XY_ERR_UNSUPPORTED
  * (tile_n not one of the values above) or XY_ERR_CUDA.  Calls on one stream are ordered; the caller

@@ -139,13 +139,58 @@ SwapPlan swap_plan(int M, int N, int K, int64_t workspace_bytes, const GemmDevic
   return best;
 }
 
+// Weight-streaming kernel: clusters of n CTAs, two CTAs on an SM, that run at once.  Clusters of an even number
+// need whole SMs of a GPC, so that as many fit as clusters of half the size at one CTA per SM; the doubled
+// answer for their own size is the safe count else.  Measured on a B200 (the first tile count that takes
+// a second wave, less one): 148, 92, 71, 55, 45, 37, 33 clusters of 2 .. 8; this says 148, 90, 70, 52, 45, 30, 32.
+int small_fit(const GemmDevice& dev, int n) {
+  if (n == 1) return 2 * dev.sms;
+  const int twice = 2 * dev.clusters[n - 1];
+  return n % 2 ? twice : std::min(dev.clusters[n / 2 - 1], twice * 16 / 15);
+}
+
+// A CTA's chain of K chunks (what it takes in: 128 rows of W and all tokens, shared between the CTAs of an SM)
+// or its wave's weights from HBM, then the exchange of sums or the store.
+float small_us(int M, int N, int K, int splits, const GemmDevice& dev) {
+  const int tiles = div_up(N, 128), chunks = div_up(div_up(K, 64), splits), tok = div_up(M, 16) * 16, fit = small_fit(dev, splits);
+  const float after = splits > 1 ? 1.15f + 5.34f * tok / 128 : 4.50f * tok / 128;
+  auto wave = [&](int n) {
+    const float per_sm = std::min(2.f, std::max(1.f, static_cast<float>(n) * splits / dev.sms));
+    return join(chunks * 0.00421f * (1.54f + per_sm) * (16.f + 0.128f * tok), 256e-6f * n * K / 6.47f) + after;
+  };
+  const float us = 1.33f + (tiles / fit) * wave(fit) + (tiles % fit ? wave(tiles % fit) : 0.f);
+  return splits > 1 || tiles > dev.sms ? us : 1.1f * us;  // a whole chain alone on its SM
+}
+
 }  // namespace
 
 GemmChoice choose_gemm(int M, int N, int K, int64_t workspace_bytes, const GemmDevice& dev) {
   if (workspace_bytes < gemm_scratch_bytes(dev.sms)) workspace_bytes = 0;
   GemmChoice c = token_major(M, N, K, dev);
   if (M <= 128) {
-    c.kernel = kGemmSmall;
+    // Up to 128 tokens are bound by the bytes of W, and the kernel that streams them is the faster one but for
+    // short chains with many tokens, where its stores and its exchange of sums weigh (us, it / the other:
+    // N 16384, K 1024, 128 tokens 14.4 / 10.2; N 12288, K 4096, 128 tokens 27.0 / 24.8).  Its K is cut by the
+    // model, at least six chunks per CTA (N 12288, K 4096, 16 tokens: two slices 20.1, three 24.7, whose 96
+    // clusters do not fit).  The line, over 640 problems: at 1.03 of the
+    // models 7 are more than 2 % slower than the other kernel, at 1.0 one, but 11 that were faster go to the other.
+    int best = 0;
+    float best_us = 1.03f * c.us;
+    const int k_chunks = div_up(K, 64);
+    for (int sp = 1; sp <= kClusterMaxCtas && (sp == 1 || sp * 6 <= k_chunks); ++sp) {
+      if (small_fit(dev, sp) < 1 || (sp - 1) * div_up(k_chunks, sp) >= k_chunks) continue;  // no CTA without a chunk
+      const float us = small_us(M, N, K, sp, dev);
+      if (us < best_us) {
+        best = sp;
+        best_us = us;
+      }
+    }
+    if (best > 0) {
+      c.kernel = kGemmSmall;
+      c.splits = best;
+      c.tile_n = 0;
+      c.us = best_us;
+    }
     return c;
   }
   if (M <= 1536) {

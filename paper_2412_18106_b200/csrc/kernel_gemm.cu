@@ -1343,8 +1343,8 @@ cudaError_t gemm_device(int dev, int sms, GemmDevice* out) {
   return err[dev];
 }
 
-cudaError_t launch_gemm_small(const GemmDevice& dev, const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc,
-                              int M, int N, int K, cudaStream_t s) {
+cudaError_t launch_gemm_small(const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int M, int N, int K,
+                              int splits, cudaStream_t s) {
   SmallParams P = {};
   P.c = static_cast<uint16_t*>(c);
   P.ldc = ldc;
@@ -1358,15 +1358,9 @@ cudaError_t launch_gemm_small(const GemmDevice& dev, const void* a, int64_t lda,
   P.stages = std::min(kSmallMaxStages, (kSmallSmem - 1024 - static_cast<int>(sizeof(SmallBarriers))) / stage);
   const int tiles = (N + 127) / 128, k_chunks = (K + kChunkK - 1) / kChunkK;
   // Two CTAs per SM with the deeper ring (three with a shorter one: GateUp at 64 tokens 45.4 against 41.5
-  // us, Down 26.2 / 23.5), and the most CTAs per tile whose clusters fit at once but for one or two: a
-  // second wave costs more than the shorter chains save (QKV, 48 tiles, at 64 tokens: clusters of five, of
-  // which 52 fit, 12.8 us, of six, 44, 18.9; Down, 32 tiles: of eight, 30, 23.5, of six 25.0).  At least six
-  // chunks per CTA.
-  P.splits = 1;
-  for (int sp = 2; sp <= kSmallMaxSplits && sp * 6 <= k_chunks; ++sp)
-    if (tiles * 15 <= 2 * dev.clusters[sp - 1] * 16) P.splits = sp;
-  P.cps = (k_chunks + P.splits - 1) / P.splits;
-  P.splits = (k_chunks + P.cps - 1) / P.cps;  // no CTA without a chunk
+  // us, Down 26.2 / 23.5).
+  P.splits = splits;
+  P.cps = (k_chunks + splits - 1) / splits;
   P.tmem_cols = 32;
   while (P.tmem_cols < static_cast<uint32_t>(P.tok)) P.tmem_cols *= 2;
   cudaLaunchConfig_t cfg = {};
@@ -1437,10 +1431,10 @@ extern "C" int xy_gemm_run_ws(const void* a, int64_t lda, const void* w, int64_t
     const xy::GemmChoice ch = xy::choose_gemm(M, N, K, workspace != nullptr ? workspace_bytes : 0, gd);
     switch (ch.kernel) {
       case xy::kGemmSmall:
-        // Up to 128 tokens are bound by the bytes of W; the kernel for that.  Measured, here / before (whole
-        // tiles or a split of K with padded token rows): hidden 4096, 16 tokens QKV 10.7 / 14.2 us, OProj 8.4 /
-        // 10.6, GateUp 39.7 / 42.9, Down 20.3 / 23.9; hidden 3584, QKV 8.5 / 19.8, OProj 7.3 / 19.2, Down 24 / 53.
-        e = xy::launch_gemm_small(gd, a, lda, w, ldw, c, ldc, M, N, K, s);
+        // Measured, here / before (whole tiles or a split of K with padded token rows): hidden 4096, 16 tokens QKV
+        // 10.7 / 14.2 us, OProj 8.4 / 10.6, GateUp 39.7 / 42.9, Down 20.3 / 23.9; hidden 3584, QKV 8.5 / 19.8, OProj
+        // 7.3 / 19.2, Down 24 / 53.
+        e = xy::launch_gemm_small(a, lda, w, ldw, c, ldc, M, N, K, ch.splits, s);
         return e == cudaSuccess ? XY_OK : XY_ERR_CUDA;
       case xy::kGemmSwap:
         e = xy::launch_gemm_swap(a, lda, w, ldw, c, ldc, M, N, K, ch.swap, gd.pair_clusters[ch.splits - 1], workspace, s);

@@ -68,3 +68,44 @@ def test_cuts_cover_the_tokens_and_fit(M, N, K):
 @pytest.mark.parametrize("M,N,K", [(200, 4096, 14336), (333, 4096, 14336), (200, 4096, 4096), (700, 2048, 4096)])
 def test_too_little_scratch_is_none(M, N, K, scratch):
     assert choice(M, N, K, scratch) == choice(M, N, K, 0)
+
+
+# Up to 128 tokens: what is chosen against the weight-streaming kernel (measured, us) ...
+@pytest.mark.parametrize("M,N,K,kernel,tile_n", [
+    (128, 16384, 1024, "tile", 128),     # 10.2 / 14.4
+    (80, 16384, 1024, "tile", 128),      # 9.9 / 11.8
+    (128, 12288, 4096, "tile", 128),     # 24.8 / 27.0
+    (128, 4096, 512, "tile", 128),       # 6.6 / 7.5
+    (128, 8, 512, "tile", 128),          # 5.2 / 6.9
+    (128, 256, 28672, "split_k", 128),   # 21.3 / 24.8
+])
+def test_kernels_that_beat_the_weight_streaming_one_are_taken(M, N, K, kernel, tile_n):
+    c = choice(M, N, K)
+    assert (c["kernel"], c["tile_n"]) == (kernel, tile_n), c
+
+
+# ... and where that one is faster, with slices of K whose clusters run at once.
+@pytest.mark.parametrize("M,N,K,splits", [
+    (16, 12288, 4096, (2,)),        # 20.1; three slices 24.7
+    (16, 6144, 4096, (4, 5)),
+    (16, 28672, 4096, (1,)),        # 39.8; two 40.7
+    (16, 4096, 14336, (7, 8)),      # 20.6; six 22.1
+    (1, 4096, 512, (1,)),
+    (64, 4096, 4096, (6, 8)),
+])
+def test_the_weight_streaming_kernel_is_cut_to_what_fits(M, N, K, splits):
+    c = choice(M, N, K)
+    assert c["kernel"] == "weight_streaming" and c["splits"] in splits, c
+
+
+@pytest.mark.parametrize("device", [B200, [132, 132, 66, 42, 32, 25, 20, 16, 14, 66, 32, 20, 14],
+                                    [148] + [148] + [0] * 7 + [0] * 4])
+@pytest.mark.parametrize("M", [1, 17, 64, 128])
+def test_no_slice_of_k_is_empty(M, device):
+    for N in (8, 128, 4096, 12288, 40000, 131072):
+        for K in list(range(8, 4200, 88)) + [14336, 28672]:
+            c = choice(M, N, K, device=device)
+            if c["kernel"] == "weight_streaming":
+                chunks = (K + 63) // 64
+                assert 1 <= c["splits"] <= 8 and device[c["splits"]] > 0
+                assert (c["splits"] - 1) * -(-chunks // c["splits"]) < chunks
