@@ -402,8 +402,9 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.v_scale = v_scale;
   a.kv_fp8 = fp8 ? 1 : 0;
   // Every run starts with a clean status word, queue head and unit counters: the run before has left
-  // them so, after a device-side timeout too.  (The CTA-pair kernel leaves that to a memset.)  The
-  // sticky record in front of them is kept.
+  // them so, after a device-side timeout too unless its cleaning ran into a timeout itself (end_of_run), which
+  // reading the status then makes up for.  (The CTA-pair kernel leaves that to a memset.)  The sticky record
+  // in front of them is kept.
   if (ctx->pair)
     XY_CUDA(ctx, cudaMemsetAsync(a.status, 0, (kStatusUnitCounts + (in_kernel_merges ? p.merges.size() : 0)) * sizeof(int32_t), s));
 
@@ -754,14 +755,15 @@ int xy_attn_device_status(xy_attn_ctx* ctx, int32_t* status_out) {
   if (ctx->host_only) return set_err(ctx, XY_ERR_UNSUPPORTED, "host-only context");
   XY_CUDA(ctx, cudaSetDevice(ctx->cfg.device));
   XY_CUDA(ctx, cudaDeviceSynchronize());
-  // word 0 is the last run's status (cleared by every run), word kStatusSticky the record of
-  // every failure since the last call of this function: report it and clear both.
+  // Word kStatusSticky is the record of every failure since the last call of this function, word 0 a status
+  // that no run has cleared: report, and clear both and whatever else the CTA that cleans up has left if it
+  // gave up (queue heads, counts of CTAs and units).  No run is in flight here.
   int32_t st[kStatusLead + 1];
   XY_CUDA(ctx, cudaMemcpy(st, ctx->d_status_base, sizeof st, cudaMemcpyDeviceToHost));
   const int32_t sticky = st[kStatusLead + kStatusSticky], last = st[kStatusLead];
   const int32_t seen = sticky != 0 ? sticky : last;
   if (seen != 0) {
-    XY_CUDA(ctx, cudaMemset(ctx->d_status, 0, sizeof(int32_t)));
+    XY_CUDA(ctx, cudaMemset(ctx->d_status, 0, sizeof(int32_t) * (kStatusUnitCounts + ctx->cap_merges)));
     XY_CUDA(ctx, cudaMemset(ctx->d_status + kStatusSticky, 0, sizeof(int32_t)));
   }
   *status_out = seen;

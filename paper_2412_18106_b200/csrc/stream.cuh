@@ -63,7 +63,10 @@ __device__ __forceinline__ void report_timeout(const RunArgs& a, int* s_failed =
 // wrapped to zero by themselves, and the task that completed a unit has put its counter back.  (Finding
 // the last CTA instead, to let it clean up, takes a fence and an atomic whose result is waited for: 1.3 -
 // 1.7 us on each launch, 10.8 -> 9.5 us for 13 requests of 500 keys.)  After a failure one of the CTAs
-// that know of it waits (with a limit) until all others have counted themselves, and cleans up.
+// that know of it waits (with a limit) until all others have counted themselves, and cleans up.  If it gives
+// up (the others may wait for an SM that another stream's kernels hold), the next one that knows tries; if
+// none succeeds the block stays as it is, the sticky word says that a run has failed, and reading that
+// (xy_attn_device_status) clears the whole block.
 __device__ __forceinline__ void end_of_run(const RunArgs& a, int* s_flag, const int* s_failed) {
   if (blockIdx.x == 0 && a.side_by_side != 1)
     for (int w = gridDim.x * 4 + threadIdx.x; w < a.num_workers * 4; w += blockDim.x) a.worker_times[w] = 0ull;
@@ -97,11 +100,14 @@ __device__ __forceinline__ void end_of_run(const RunArgs& a, int* s_flag, const 
   int clean = 0;
   if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicExch(a.status + kStatusCleaner, 1) == 0)
-      for (int i = 0; i < (1 << 22) && !clean; ++i) {
+    if (atomicExch(a.status + kStatusCleaner, 1) == 0) {
+      const int limit = *const_cast<volatile const int32_t*>(a.status + kStatusWaitLimit);
+      for (int i = 1; i < limit && !clean; ++i) {  // (a limit of one poll, from a test: none)
         clean = *const_cast<volatile unsigned*>(exits) == others ? 1 : 0;
         if (!clean) __nanosleep(256);
       }
+      if (!clean) atomicExch(a.status + kStatusCleaner, 0);
+    }
     __threadfence();
   }
   if (__shfl_sync(0xffffffffu, clean, 0)) {

@@ -107,3 +107,30 @@ def test_many_ctas_that_give_up_leave_a_clean_context(workers, decode):
     o, lse = good[-1]
     H.check_against_oracle(o.float().cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64), O_ref, LSE_ref,
                            "run after a timeout")
+
+
+@pytest.mark.parametrize("workers,skip,decode", [(3, 20, True), (3, 45, True), (20, 1, True), (2, 2, False), (7, 20, False),
+                                                 (100, 1, False)])
+def test_status_read_clears_what_a_cleaner_that_gave_up_has_left(workers, skip, decode):
+    """With a wait limit of one poll the CTA that cleans up after a failure does not wait for the others (as if they
+    could not get an SM).  Queue head and counters then stay as they are; reading the status clears them, so that
+    the runs behind it are ordinary ones."""
+    b = (W.config2_decode(num_requests=9, kv_lo=300, kv_hi=3000) if decode else
+         W.config3_splitfuse(chunk=300, prefix=300, num_decode=9, kv_lo=200, kv_hi=1500))
+    t = W.make_tensors(b)
+    O_ref, LSE_ref = oracle.attention(b, t, H.SCALE)
+    ctx = H.make_ctx(b, num_workers=workers)
+    ctx.plan_batch(b)
+    d = H.DeviceBatch(b, t)
+    for _ in range(3):
+        ctx.debug_inject(wait_limit_polls=1, skip_fill=skip)
+        ctx.run(d.q, d.k_pool, d.v_pool, d.block_table, H.SCALE, d.o, d.lse)
+        ctx.debug_inject(0, -1)
+        assert ctx.device_status() == xb.XY_ERR_DEVICE_TIMEOUT
+        for _ in range(2):
+            o, lse = torch.full_like(d.o, float("nan")), torch.full_like(d.lse, float("nan"))
+            ctx.run(d.q, d.k_pool, d.v_pool, d.block_table, H.SCALE, o, lse)
+            assert ctx.device_status() == 0
+            H.check_against_oracle(o.float().cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64), O_ref,
+                                   LSE_ref, "run after a status read")
+    ctx.close()
