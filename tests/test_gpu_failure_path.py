@@ -134,3 +134,67 @@ def test_status_read_clears_what_a_cleaner_that_gave_up_has_left(workers, skip, 
             H.check_against_oracle(o.float().cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64), O_ref,
                                    LSE_ref, "run after a status read")
     ctx.close()
+
+
+@pytest.mark.parametrize("workers", [0, 7])
+@pytest.mark.parametrize("skip", [0, 1, 6])
+def test_two_launches_side_by_side_give_up_and_leave_a_clean_context(skip, workers):
+    """The dense and the streaming launch of a shared-prefix plan share the status word and the unit counters:
+    after a wait that ran out in either, the next ordinary runs are bitwise what they were before."""
+    b, groups = W.shared_prefix_decode(seed=7, num_groups=5, members=42, prefix=512, suffix_hi=400, hq=16, hkv=4)
+    t = W.make_tensors(b)
+    ctx = H.make_ctx(b, num_workers=workers, max_requests=512)
+    ctx.plan_batch(b, groups=groups)
+    d = H.DeviceBatch(b, t)
+
+    def run():
+        o, lse = torch.full_like(d.o, float("nan")), torch.full_like(d.lse, float("nan"))
+        ctx.run(d.q, d.k_pool, d.v_pool, d.block_table, H.SCALE, o, lse)
+        assert ctx.last_launches() == 3
+        return o, lse
+
+    good = run()
+    H.check_against_oracle(good[0].float().cpu().numpy().astype(np.float64), good[1].cpu().numpy().astype(np.float64),
+                           *oracle.attention(b, t, H.SCALE), "two launches")
+    for read in (True, False):
+        ctx.debug_inject(wait_limit_polls=20000, skip_fill=skip)
+        run()
+        ctx.debug_inject(0, -1)
+        if read:
+            assert ctx.device_status() == xb.XY_ERR_DEVICE_TIMEOUT
+        for _ in range(2):
+            o, lse = run()
+            assert torch.equal(o, good[0]) and torch.equal(lse, good[1])
+    assert ctx.device_status() == xb.XY_ERR_DEVICE_TIMEOUT and ctx.device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("decode,workers", [(True, 3), (True, 0), (False, 5)], ids=["stream-6", "stream-all", "meta-5"])
+@pytest.mark.parametrize("skip", [1, 11])
+def test_fp8_run_gives_up_and_the_context_recovers(decode, workers, skip):
+    b = W.config2_decode(num_requests=9, kv_lo=300, kv_hi=3000) if decode else W.config1_tiny()
+    t8 = W.to_fp8_kv(W.make_tensors(b))
+    ctx = H.make_ctx(b, num_workers=workers, kv_dtype=xb.XY_KV_FP8_E4M3)
+    ctx.plan_batch(b)
+    q, k, v, ks, vs = (x.cuda() for x in (t8.q, t8.k_pool, t8.v_pool, t8.k_scale, t8.v_scale))
+    bt = torch.from_numpy(np.where(b.block_table < 0, 0, b.block_table).astype(np.int32)).cuda()
+
+    def run():
+        o = torch.full((b.total_q, b.num_q_heads, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((b.total_q, b.num_q_heads), float("nan"), dtype=torch.float32, device="cuda")
+        ctx.run_fp8kv(q, k, v, ks, vs, bt, H.SCALE, o, lse)
+        return o, lse
+
+    good = run()
+    H.check_against_oracle(good[0].float().cpu().numpy().astype(np.float64), good[1].cpu().numpy().astype(np.float64),
+                           *oracle.attention_fp8(b, t8, H.SCALE), "fp8")
+    for read in (True, False):
+        ctx.debug_inject(wait_limit_polls=20000, skip_fill=skip)
+        run()
+        ctx.debug_inject(0, -1)
+        if read:
+            assert ctx.device_status() == xb.XY_ERR_DEVICE_TIMEOUT
+        for _ in range(2):
+            o, lse = run()
+            assert torch.equal(o, good[0]) and torch.equal(lse, good[1])
+    ctx.close()
