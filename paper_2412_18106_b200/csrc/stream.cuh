@@ -92,10 +92,15 @@ __device__ __forceinline__ void end_of_run(const RunArgs& a, int* s_flag, const 
     return;
   }
   if (threadIdx.x >= 32) return;
-  // One lane's reading for the whole warp: another CTA may report a failure between two lanes' loads, and the
-  // lanes have to take the same way.
-  int failed = threadIdx.x == 0 ? *const_cast<volatile const int*>(s_failed != nullptr ? s_failed : a.status) : 0;
-  failed = __shfl_sync(0xffffffffu, failed, 0);
+  int failed;
+  if (s_failed != nullptr) {
+    failed = *const_cast<volatile const int*>(s_failed);
+  } else {
+    // One lane's reading for the whole warp: another CTA may report a failure between two lanes' loads, and
+    // the lanes have to take the same way.
+    failed = threadIdx.x == 0 ? *const_cast<volatile const int32_t*>(a.status) : 0;
+    failed = __shfl_sync(0xffffffffu, failed, 0);
+  }
   if (failed == 0) {
     if (threadIdx.x == 0) atomicInc(exits, others);
     return;
