@@ -345,7 +345,8 @@ int xy_attn_debug_gather(xy_attn_ctx* ctx, int32_t req, int32_t kv_head, const v
  * exit time stamps (nanoseconds of the GPU's global timer) and the nanoseconds it spent in dense
  * and in streaming tasks.  Returns the number of entries; copies only if `cap`
  * is large enough.  XY_KERNEL_REFERENCE records none; of the streaming kernel's up to two CTAs per
- * worker the first num_workers are recorded. */
+ * worker the first num_workers are recorded.  A run of two launches at the same time leaves in an entry the
+ * earlier start, the later end and the times of both (CTAs of the same index, not of the same SM). */
 int xy_attn_worker_times(xy_attn_ctx* ctx, uint64_t* out, int32_t cap);
 
 /* Debug tracing (only in a library built with -DXY_ENABLE_TRACE, i.e. XY_BUILD_TRACE=1 for

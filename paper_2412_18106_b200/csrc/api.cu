@@ -390,6 +390,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.num_workers = ctx->num_workers;
   a.exits = ctx->d_status + kStatusExits;
   a.side_by_side = 0;
+  a.dense_ctas = 0;
   a.num_units = static_cast<int32_t>(p.merges.size());
   // Balanced plans are dealt dynamically by the meta-kernel; paper-mode plans keep the static
   // Task-Table (each worker walks its own list), as does the reference kernel.
@@ -426,6 +427,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
     d.num_tasks = p.queue_dense;
     const bool beside = !ctx->pair && p.queue_dense > 0 && p.queue_dense < a.num_tasks;
     d.side_by_side = beside ? 1 : 0;
+    a.dense_ctas = beside ? std::min(d.num_tasks, ctx->num_workers) : 0;
     if (d.num_tasks > 0) {
       if (ctx->pair)
         XY_CUDA(ctx, launch_pair_dense(d, ctx->num_workers, num_pages, &ctx->launch_cache, s));

@@ -301,7 +301,11 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     }
   }
   // Beside the dense launch: that one is waited for here, so that whoever follows this launch follows both.
-  if (a.side_by_side) grid_dependency_wait();
+  unsigned long long t_end = 0;
+  if (a.side_by_side) {
+    if (threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_end));
+    grid_dependency_wait();
+  }
   // The next launch's CTAs come in as these leave.  (Letting them in from the start filled the SMs
   // unevenly: a CTA took whichever slot was free first, 55.3 -> 60.4 us for 64 requests on an fp8 cache.)
   grid_launch_dependents();
@@ -310,10 +314,11 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     unsigned long long now;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
     unsigned long long* w = a.worker_times + 4 * blockIdx.x;
-    w[0] = t_start;
+    const bool add = a.side_by_side != 0 && blockIdx.x < static_cast<unsigned>(a.dense_ctas);  // the dense launch's is there
+    if (add) atomicMin(w, t_start); else w[0] = t_start;
     w[1] = now;
-    w[2] = 0ull;
-    w[3] = now - t_start;
+    if (!add) w[2] = 0ull;
+    w[3] = (a.side_by_side ? t_end : now) - t_start;
   }
   end_of_run(a, s_last, s_failed);
 }

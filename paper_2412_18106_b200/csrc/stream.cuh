@@ -69,7 +69,7 @@ __device__ __forceinline__ void report_timeout(const RunArgs& a, int* s_failed =
 // (xy_attn_device_status) clears the whole block.
 __device__ __forceinline__ void end_of_run(const RunArgs& a, int* s_flag, const int* s_failed) {
   if (blockIdx.x == 0 && a.side_by_side != 1)
-    for (int w = gridDim.x * 4 + threadIdx.x; w < a.num_workers * 4; w += blockDim.x) a.worker_times[w] = 0ull;
+    for (int w = max(static_cast<int>(gridDim.x), a.dense_ctas) * 4 + threadIdx.x; w < a.num_workers * 4; w += blockDim.x) a.worker_times[w] = 0ull;
   unsigned* exits = reinterpret_cast<unsigned*>(a.exits);
   const unsigned others = gridDim.x - 1;
   if (a.side_by_side) {

@@ -128,3 +128,21 @@ def test_dense_and_streaming_launches_side_by_side_match_oracle(page, members, w
         assert first is None or (np.array_equal(O, first[0]) and np.array_equal(LSE, first[1]))
         first = (O, LSE)
     ctx.close()
+
+
+def test_worker_times_of_two_launches_hold_both():
+    """Dense time of the first launch and streaming time of the second stand beside each other."""
+    b, groups = W.shared_prefix_decode(seed=3, num_groups=5, members=42, prefix=512, suffix_hi=400, hq=16, hkv=4)
+    t = W.make_tensors(b)
+    ctx = H.make_ctx(b, max_requests=512)
+    ctx.plan_batch(b, groups=groups)
+    dense = int((ctx.get_tasks()["kind"] == 0).sum())
+    for _ in range(2):
+        H.run_gpu(b, t, ctx=ctx)
+        assert ctx.last_launches() == 3
+        w = ctx.worker_times().astype(np.int64)
+        used = w[:, 1] > 0
+        assert w[:, 2].sum() > 0 and (w[dense:, 2] == 0).all()
+        assert w[:, 3].sum() > 0 and (w[~used] == 0).all()
+        assert (w[used, 1] >= w[used, 0]).all() and (w[used, 2:].max(axis=1) <= w[used, 1] - w[used, 0]).all()
+    ctx.close()
