@@ -4,7 +4,8 @@
 // lookups and conversions for `run`, as much as the kernels of a small batch; this takes about 1 us
 // (two steps of a four-request batch, planned and run: 108 -> 43 us; two steps of 13 decode requests over
 // eight layers 554 -> 387 us, which is the device's time).
-// A call whose arguments do not pass returns None: the Python form then raises what is wrong.
+// A call whose arguments do not pass returns None: the Python form then raises what is wrong.  So does one
+// whose arguments throw when they are looked at (guarded); no C++ exception leaves an entry point.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -14,6 +15,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <new>
 #include <vector>
 
 #include "xy_attn.h"
@@ -45,11 +47,23 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return none();
 }
 
+template <class Body>
+PyObject* guarded(Body body) {
+  try {
+    return body();
+  } catch (const std::bad_alloc&) {
+    return PyErr_NoMemory();
+  } catch (...) {
+    PyErr_Clear();  // (an exception of a Python tensor subclass is a set Python error too)
+    return none();
+  }
+}
+
 // A CUDA tensor of the given type and number of dimensions whose last one is contiguous.
 const at::Tensor* cuda_tensor(PyObject* o, at::ScalarType type, int64_t dim) {
   if (!THPVariable_Check(o)) return nullptr;
   const at::Tensor& t = THPVariable_Unpack(o);
-  if (!t.is_cuda() || t.scalar_type() != type || t.dim() != dim || t.stride(dim - 1) != 1) return nullptr;
+  if (!t.is_cuda() || t.layout() != at::kStrided || t.scalar_type() != type || t.dim() != dim || t.stride(dim - 1) != 1) return nullptr;
   return &t;
 }
 
@@ -63,12 +77,18 @@ bool stream_of(PyObject* o, void*& s) {
   return !PyErr_Occurred();
 }
 
+// Calls into the library without the GIL: `call` only passes on pointers and numbers that it holds.
 template <class Call>
 PyObject* status(Call call) {
+  struct Unlocked {  // the lock is taken again on every way out
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+  };
   int rc;
-  Py_BEGIN_ALLOW_THREADS;
-  rc = call();
-  Py_END_ALLOW_THREADS;
+  {
+    Unlocked u;
+    rc = call();
+  }
   return PyLong_FromLong(rc);
 }
 
@@ -95,7 +115,7 @@ PyObject* run(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const at::Tensor* o = cuda_tensor(a[7], at::kBFloat16, 3);
   if (!q || !o || !pools(a[3], a[4], a[5], fp8 ? at::kByte : at::kBFloat16, p) || !THPVariable_Check(a[8])) return none();
   const at::Tensor& lse = THPVariable_Unpack(a[8]);
-  if (!lse.is_cuda() || lse.scalar_type() != at::kFloat || !lse.is_contiguous()) return none();
+  if (!lse.is_cuda() || lse.layout() != at::kStrided || lse.scalar_type() != at::kFloat || !lse.is_contiguous()) return none();
   if (q->stride(1) != D || o->stride(1) != D) return none();
   const uint64_t* mask = nullptr;
   if (a[9] != Py_None) {
@@ -104,23 +124,21 @@ PyObject* run(PyObject*, PyObject* const* a, Py_ssize_t n) {
   }
   void* s;
   if (!stream_of(a[10], s)) return nullptr;
-  const at::Tensor &k = *p.k, &v = *p.v, &bt = *p.bt;
-  if (!fp8)
-    return status([&] {
-      return f_run(ctx, q->data_ptr(), q->stride(0), k.data_ptr(), v.data_ptr(), k.size(0), k.stride(0), k.stride(1), k.stride(2),
-                   static_cast<const int32_t*>(bt.data_ptr()), static_cast<int32_t>(bt.stride(0)), mask, static_cast<float>(scale),
-                   o->data_ptr(), o->stride(0), static_cast<float*>(lse.data_ptr()), s);
-    });
+  const at::Tensor &k = *p.k, &bt = *p.bt;
+  const void *qp = q->data_ptr(), *kp = k.data_ptr(), *vp = p.v->data_ptr();
+  void* op = o->data_ptr();
+  auto* lp = static_cast<float*>(lse.data_ptr());
+  auto* btp = static_cast<const int32_t*>(bt.data_ptr());
+  const int64_t qs = q->stride(0), os = o->stride(0), pages = k.size(0), ps = k.stride(0), hs = k.stride(1), ts = k.stride(2);
+  const auto bts = static_cast<int32_t>(bt.stride(0));
+  const auto sc = static_cast<float>(scale);
+  if (!fp8) return status([=] { return f_run(ctx, qp, qs, kp, vp, pages, ps, hs, ts, btp, bts, mask, sc, op, os, lp, s); });
   const at::Tensor *ks = cuda_tensor(a[11], at::kFloat, 2), *vs = cuda_tensor(a[12], at::kFloat, 2);
   if (!ks || !vs || !ks->is_contiguous() || !vs->is_contiguous() || ks->sizes() != vs->sizes() || ks->size(0) != k.size(0) ||
       ks->size(1) != k.size(1))
     return none();
-  return status([&] {
-    return f_run_fp8(ctx, q->data_ptr(), q->stride(0), k.data_ptr(), v.data_ptr(), static_cast<const float*>(ks->data_ptr()),
-                     static_cast<const float*>(vs->data_ptr()), k.size(0), k.stride(0), k.stride(1), k.stride(2),
-                     static_cast<const int32_t*>(bt.data_ptr()), static_cast<int32_t>(bt.stride(0)), mask,
-                     static_cast<float>(scale), o->data_ptr(), o->stride(0), static_cast<float*>(lse.data_ptr()), s);
-  });
+  auto *ksp = static_cast<const float*>(ks->data_ptr()), *vsp = static_cast<const float*>(vs->data_ptr());
+  return status([=] { return f_run_fp8(ctx, qp, qs, kp, vp, ksp, vsp, pages, ps, hs, ts, btp, bts, mask, sc, op, os, lp, s); });
 }
 
 // append_kv(ctx, head_dim, qkv, k_pool, v_pool, block_table, stream)
@@ -134,11 +152,12 @@ PyObject* append_kv(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!qkv || qkv->stride(1) != D || !pools(a[3], a[4], a[5], at::kBFloat16, p)) return none();
   void* s;
   if (!stream_of(a[6], s)) return nullptr;
-  return status([&] {
-    return f_append(ctx, qkv->data_ptr(), qkv->stride(0), p.k->data_ptr(), p.v->data_ptr(), p.k->size(0), p.k->stride(0),
-                    p.k->stride(1), p.k->stride(2), static_cast<const int32_t*>(p.bt->data_ptr()),
-                    static_cast<int32_t>(p.bt->stride(0)), s);
-  });
+  const void* src = qkv->data_ptr();
+  void *kp = p.k->data_ptr(), *vp = p.v->data_ptr();
+  auto* btp = static_cast<const int32_t*>(p.bt->data_ptr());
+  const int64_t ss = qkv->stride(0), pages = p.k->size(0), ps = p.k->stride(0), hs = p.k->stride(1), ts = p.k->stride(2);
+  const auto bts = static_cast<int32_t>(p.bt->stride(0));
+  return status([=] { return f_append(ctx, src, ss, kp, vp, pages, ps, hs, ts, btp, bts, s); });
 }
 
 // gemm(a, w, c, tile_n, stream, workspace)
@@ -163,10 +182,12 @@ PyObject* gemm(PyObject*, PyObject* const* x, Py_ssize_t n) {
   if (!stream_of(x[4], s)) return nullptr;
   // the row stride of a single row says nothing
   const int64_t lda = M > 1 ? a->stride(0) : std::max(K, a->stride(0)), ldc = M > 1 ? c->stride(0) : std::max(N, c->stride(0));
-  return status([&] {
-    return f_gemm(a->data_ptr(), lda, w->data_ptr(), w->stride(0), c->data_ptr(), ldc, static_cast<int32_t>(M),
-                  static_cast<int32_t>(N), static_cast<int32_t>(K), static_cast<int32_t>(tile_n), ws, ws_bytes, s);
-  });
+  const void *ap = a->data_ptr(), *wp = w->data_ptr();
+  void* cp = c->data_ptr();
+  const int64_t ldw = w->stride(0);
+  const auto m32 = static_cast<int32_t>(M), n32 = static_cast<int32_t>(N), k32 = static_cast<int32_t>(K),
+             tn = static_cast<int32_t>(tile_n);
+  return status([=] { return f_gemm(ap, lda, wp, ldw, cp, ldc, m32, n32, k32, tn, ws, ws_bytes, s); });
 }
 
 // Contiguous one-dimensional int32 buffer (a numpy array).
@@ -204,19 +225,24 @@ PyObject* plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void* s;
   if (!stream_of(a[6], s)) return nullptr;
   const int32_t np = trees ? static_cast<int32_t>(par.size()) : 0;
-  return status([&] {
-    std::vector<xy_attn_request> reqs(static_cast<size_t>(R > 0 ? R : 1));
-    for (Py_ssize_t r = 0; r < R; ++r) reqs[r] = xy_attn_request{q.data()[r], kv.data()[r], kind.data()[r], off.data()[r]};
-    return f_plan(ctx, reqs.data(), static_cast<int32_t>(R), np > 0 ? par.data() : nullptr, np, s, info);
-  });
+  std::vector<xy_attn_request> reqs(static_cast<size_t>(R > 0 ? R : 1));
+  for (Py_ssize_t r = 0; r < R; ++r) reqs[r] = xy_attn_request{q.data()[r], kv.data()[r], kind.data()[r], off.data()[r]};
+  const int32_t* parents = np > 0 ? par.data() : nullptr;
+  return status([&] { return f_plan(ctx, reqs.data(), static_cast<int32_t>(R), parents, np, s, info); });
+}
+
+// the entry points: a body behind guarded()
+template <PyObject* (*body)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* entry(PyObject* self, PyObject* const* a, Py_ssize_t n) {
+  return guarded([&] { return body(self, a, n); });
 }
 
 PyMethodDef methods[] = {
-    {"bind", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&bind)), METH_FASTCALL, nullptr},
-    {"plan", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&plan)), METH_FASTCALL, nullptr},
-    {"run", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&run)), METH_FASTCALL, nullptr},
-    {"append_kv", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&append_kv)), METH_FASTCALL, nullptr},
-    {"gemm", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&gemm)), METH_FASTCALL, nullptr},
+    {"bind", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<bind>)), METH_FASTCALL, nullptr},
+    {"plan", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<plan>)), METH_FASTCALL, nullptr},
+    {"run", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<run>)), METH_FASTCALL, nullptr},
+    {"append_kv", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<append_kv>)), METH_FASTCALL, nullptr},
+    {"gemm", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<gemm>)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fastcall", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
