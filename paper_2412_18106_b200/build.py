@@ -3,12 +3,14 @@
     python -m paper_2412_18106_b200.build [--force]
 
 The shared object lands beside this file (libxy_attn.so); nvcc cross-compiles
-without a GPU.  The binding's native calls (_fastcall.so, a CPython extension against
-torch's headers) are compiled beside it with the host compiler.
+without a GPU and without torch.  The binding's native calls (_fastcall.so, a CPython
+extension against torch's headers) are compiled beside it with the host compiler, where
+torch is installed, and again when its version changes.
 """
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -18,6 +20,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libxy_attn.so")
 FASTCALL = os.path.join(HERE, "_fastcall.so")
+FASTCALL_STAMP = os.path.join(HERE, "build", "fastcall.torch")  # the torch version it was compiled against
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -40,9 +43,20 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def torch_version():
+    """The installed torch's version (torch is not imported), or None."""
+    try:
+        return importlib.metadata.version("torch")
+    except importlib.metadata.PackageNotFoundError:
+        return None
+
+
 def _fastcall_stale() -> bool:
-    if not os.path.exists(FASTCALL):
+    if not os.path.exists(FASTCALL) or not os.path.exists(FASTCALL_STAMP):
         return True
+    with open(FASTCALL_STAMP) as f:
+        if f.read() != torch_version():
+            return True
     deps = [os.path.join(CSRC, "fastcall.cpp")] + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > os.path.getmtime(FASTCALL) for d in deps)
 
@@ -64,15 +78,27 @@ def start_fastcall():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    fast = start_fastcall() if force or _fastcall_stale() else None
+    fast = None
+    if torch_version() is None:
+        sys.stderr.write("torch is not installed: building the C library only\n")
+    elif force or _fastcall_stale():
+        try:
+            fast = start_fastcall()
+        except Exception as e:  # the library is built all the same
+            fast = e
     try:
         return _build_lib(force, verbose)
     finally:
+        if isinstance(fast, Exception):
+            raise RuntimeError("compiling fastcall.cpp failed") from fast
         if fast is not None:
             out = fast[0].communicate()[0].decode()
             if fast[0].returncode != 0:
                 raise RuntimeError("compiling fastcall.cpp failed:\n" + out[-3000:])
             os.replace(fast[1], FASTCALL)
+            os.makedirs(os.path.dirname(FASTCALL_STAMP), exist_ok=True)
+            with open(FASTCALL_STAMP, "w") as f:
+                f.write(torch_version())
 
 
 def _build_lib(force: bool, verbose: bool) -> str:
