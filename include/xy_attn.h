@@ -93,7 +93,8 @@ typedef struct {
   int32_t max_pages_per_req; /* capacity: pages a single request may reference */
   int32_t max_tree_nodes;    /* capacity: nodes of one verify tree */
   int32_t device;            /* CUDA device ordinal; -1 = host-only context (plan works, run fails) */
-  int32_t num_workers;       /* 0 = one worker per SM of the device (148 on B200) */
+  int32_t num_workers;       /* 0 = one worker per SM of the device (148 on B200); with fewer, attention keeps to
+                              * that many SMs */
   int32_t kernel;            /* XY_KERNEL_* */
   int32_t plan_mode;         /* XY_PLAN_* */
   int32_t tile_tokens;       /* XY_PLAN_PAPER only: tileSize in tokens (0 = 128 / (Hq/Hkv)) */
@@ -395,11 +396,16 @@ int xy_attn_debug_check_block_table(xy_attn_ctx* ctx, const int32_t* block_table
  * skip_fill-th K/V stage fill of the following runs (-1: none), so that the readers of that stage
  * never see it filled and their waits run out.  Nothing faults and nothing spins without bound:
  * the kernel returns, frees its tensor memory, and the status shows the timeout; O and LSE of
- * such a run are unspecified.  The next run on the context starts from a clean status word. */
+ * such a run are unspecified.  The next run on the context starts from a clean status word, unless the
+ * CTA that cleans up has run into a timeout itself: then xy_attn_device_status cleans. */
 int xy_attn_debug_inject(xy_attn_ctx* ctx, int32_t wait_limit_polls, int32_t skip_fill);
 
 /* Number of kernel launches the last xy_attn_run enqueued. */
 int xy_attn_last_launches(const xy_attn_ctx* ctx);
+
+/* Attention CTAs of the last xy_attn_run that may run at the same time: at most num_workers where that is
+ * below the device's SMs (but for XY_KERNEL_PAIR, whose CTAs come in pairs). */
+int xy_attn_last_ctas(const xy_attn_ctx* ctx);
 
 /* Message of the last error on this context (never null). */
 const char* xy_attn_last_error(const xy_attn_ctx* ctx);

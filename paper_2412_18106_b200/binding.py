@@ -88,7 +88,7 @@ EXPORTS = (
     "xy_attn_append_kv", "xy_attn_worker_times", "xy_attn_get_queue", "xy_attn_plan_cache",
     "xy_attn_plan_shared", "xy_attn_shard_context", "xy_attn_merge_shards",
     "xy_attn_find_prefix_groups", "xy_attn_debug_check_block_table", "xy_attn_debug_inject",
-    "xy_attn_run_fp8kv",
+    "xy_attn_run_fp8kv", "xy_attn_last_ctas",
 )
 
 _lib = None
@@ -134,6 +134,7 @@ def load() -> ctypes.CDLL:
     L.xy_attn_debug_check_block_table.argtypes = [vp, vp, i32, i64]
     L.xy_attn_debug_inject.argtypes = [vp, i32, i32]
     L.xy_attn_last_launches.argtypes = [vp]
+    L.xy_attn_last_ctas.argtypes = [vp]
     L.xy_attn_last_error.argtypes = [vp]
     L.xy_attn_last_error.restype = ctypes.c_char_p
     L.xy_attn_device_status.argtypes = [vp, ctypes.POINTER(i32)]
@@ -404,6 +405,10 @@ class XYAttn:
 
     def last_launches(self) -> int:
         return int(self.lib.xy_attn_last_launches(self._ctx))
+
+    def last_ctas(self) -> int:
+        """Attention CTAs of the last run that may run at the same time."""
+        return int(self.lib.xy_attn_last_ctas(self._ctx))
 
     def last_error(self) -> str:
         return self.lib.xy_attn_last_error(self._ctx).decode()

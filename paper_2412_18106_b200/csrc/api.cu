@@ -19,6 +19,7 @@ using namespace xy;
 struct xy_attn_ctx {
   xy_attn_config cfg{};
   int num_workers = 0;
+  int num_sms = 0;
   bool host_only = false;
   int page_shift = 0;
   bool planned = false;
@@ -45,7 +46,7 @@ struct xy_attn_ctx {
   int32_t* d_status = nullptr;
   unsigned long long* d_trace = nullptr;
   unsigned long long* d_worker_times = nullptr;
-  int last_launches = 0;
+  int last_launches = 0, last_ctas = 0;
   MetaLaunchCache launch_cache;     // tensor maps of the last pools seen, kernel attributes set once
   int32_t dbg_skip_fill = -1;       // -1: none
   bool pair = false;                // dense tasks run on CTA pairs (two launches per run: dense pairs, then streaming)
@@ -125,15 +126,12 @@ int xy_attn_create(const xy_attn_config* cfg, xy_attn_ctx** out) {
       delete c;
       return XY_ERR_CUDA;
     }
-    if (c->num_workers == 0) {
-      int sms = 0;
-      e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cfg->device);
-      if (e != cudaSuccess || sms <= 0) {
-        delete c;
-        return XY_ERR_CUDA;
-      }
-      c->num_workers = sms;
+    e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
+    if (e != cudaSuccess || c->num_sms <= 0) {
+      delete c;
+      return XY_ERR_CUDA;
     }
+    if (c->num_workers == 0) c->num_workers = c->num_sms;
   } else if (c->num_workers == 0) {
     c->num_workers = 148;
   }
@@ -315,7 +313,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
              const uint64_t* tree_mask, float sm_scale, void* o, int64_t o_token_stride,
              float* lse, void* stream) {
   if (ctx == nullptr) return XY_ERR_INVALID_ARG;
-  ctx->last_launches = 0;
+  ctx->last_launches = ctx->last_ctas = 0;
   if (ctx->host_only) return set_err(ctx, XY_ERR_UNSUPPORTED, "host-only context cannot run");
   if (!ctx->planned) return set_err(ctx, XY_ERR_NOT_PLANNED, "xy_attn_run before xy_attn_plan");
   const bool fp8 = k_scale != nullptr;
@@ -391,6 +389,10 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.exits = ctx->d_status + kStatusExits;
   a.side_by_side = 0;
   a.dense_ctas = 0;
+  // With fewer workers than SMs the caller leaves SMs to others: then a run keeps to as many as it has
+  // workers, with one streaming CTA each and the two launches of a plan one after the other.
+  const bool whole_device = ctx->num_workers >= ctx->num_sms;
+  a.ctas_per_worker = whole_device ? 2 : 1;
   a.num_units = static_cast<int32_t>(p.merges.size());
   // Balanced plans are dealt dynamically by the meta-kernel; paper-mode plans keep the static
   // Task-Table (each worker walks its own list), as does the reference kernel.
@@ -425,15 +427,16 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
     // two launches: the dense tasks (pair plan: on CTA pairs), then the streaming tasks
     RunArgs d = a;
     d.num_tasks = p.queue_dense;
-    const bool beside = !ctx->pair && p.queue_dense > 0 && p.queue_dense < a.num_tasks;
+    const bool two = !ctx->pair && p.queue_dense > 0 && p.queue_dense < a.num_tasks, beside = two && whole_device;
     d.side_by_side = beside ? 1 : 0;
-    a.dense_ctas = beside ? std::min(d.num_tasks, ctx->num_workers) : 0;
+    a.dense_ctas = two ? std::min(d.num_tasks, ctx->num_workers) : 0;
     if (d.num_tasks > 0) {
       if (ctx->pair)
         XY_CUDA(ctx, launch_pair_dense(d, ctx->num_workers, num_pages, &ctx->launch_cache, s));
       else
         XY_CUDA(ctx, launch_meta(d, num_pages, true, &ctx->launch_cache, s));
       ctx->last_launches += 1;
+      ctx->last_ctas = ctx->launch_cache.ctas;
     }
     RunArgs st = a;
     st.queue = a.queue + p.queue_dense;
@@ -447,6 +450,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
       else
         XY_CUDA(ctx, launch_stream(st, num_pages, &ctx->launch_cache, s));
       ctx->last_launches += 1;
+      ctx->last_ctas = beside ? ctx->last_ctas + ctx->launch_cache.ctas : std::max(ctx->last_ctas, ctx->launch_cache.ctas);
     }
     ctx->last_launches -= 1;  // counted once more below
   } else if (cfg.kernel == XY_KERNEL_AUTO && a.dynamic && p.info.num_dense_tasks == 0) {
@@ -460,6 +464,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
                              &ctx->launch_cache, s));
   }
   ctx->last_launches += 1;
+  if (ctx->last_ctas == 0) ctx->last_ctas = cfg.kernel == XY_KERNEL_REFERENCE ? ctx->num_workers : ctx->launch_cache.ctas;
   if (timed) XY_CUDA(ctx, cudaEventRecord(ctx->events[3 * ctx->timed_runs + 1], s));
 
   if (p.num_launch_merges > 0) {
@@ -749,6 +754,8 @@ int xy_attn_debug_inject(xy_attn_ctx* ctx, int32_t wait_limit_polls, int32_t ski
 }
 
 int xy_attn_last_launches(const xy_attn_ctx* ctx) { return ctx ? ctx->last_launches : XY_ERR_INVALID_ARG; }
+
+int xy_attn_last_ctas(const xy_attn_ctx* ctx) { return ctx ? ctx->last_ctas : XY_ERR_INVALID_ARG; }
 
 const char* xy_attn_last_error(const xy_attn_ctx* ctx) { return ctx ? ctx->err.c_str() : "null context"; }
 

@@ -1354,6 +1354,7 @@ cudaError_t launch_meta(const RunArgs& a, int64_t num_pages, bool umma, MetaLaun
   if (e != cudaSuccess) return e;
   MetaParams P{a};
   const int grid = a.dynamic && a.num_tasks < a.num_workers ? a.num_tasks : a.num_workers;
+  cache->ctas = grid;
   P.a.queue_wrap = static_cast<uint32_t>(a.num_tasks + grid - 1);  // every CTA grabs in vain once
   return launch_after(kernel, dim3(grid), kThreads, kSmemTotal, s, P, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
                       *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));
@@ -1394,6 +1395,7 @@ cudaError_t launch_pair_dense(const RunArgs& a, int num_workers, int64_t num_pag
     cache->pair_valid = true;
   }
   MetaParams P{a};
+  cache->ctas = num_workers & ~1;
   pair_dense_kernel<<<num_workers & ~1, kThreads, kSmemTotal, s>>>(P, *k_map, *v_map);
   return cudaGetLastError();
 }

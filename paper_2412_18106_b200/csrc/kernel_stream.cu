@@ -314,7 +314,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     unsigned long long now;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
     unsigned long long* w = a.worker_times + 4 * blockIdx.x;
-    const bool add = a.side_by_side != 0 && blockIdx.x < static_cast<unsigned>(a.dense_ctas);  // the dense launch's is there
+    const bool add = blockIdx.x < static_cast<unsigned>(a.dense_ctas);  // the dense launch's is there
     if (add) atomicMin(w, t_start); else w[0] = t_start;
     w[1] = now;
     if (!add) w[2] = 0ull;
@@ -325,7 +325,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
 
 }  // namespace
 
-// Up to two CTAs per worker (SM), never more than tasks.
+// Up to ctas_per_worker CTAs per worker, never more than tasks.
 cudaError_t launch_stream(const RunArgs& a, int64_t num_pages, MetaLaunchCache* cache, cudaStream_t s) {
   const bool fp8 = a.kv_fp8 != 0;
   const int smem = fp8 ? StreamCfg<true>::kSmem : StreamCfg<false>::kSmem;
@@ -338,7 +338,9 @@ cudaError_t launch_stream(const RunArgs& a, int64_t num_pages, MetaLaunchCache* 
   }
   const cudaError_t e = pool_maps(a, num_pages, cache);
   if (e != cudaSuccess) return e;
-  const int grid = a.num_tasks < 2 * a.num_workers ? a.num_tasks : 2 * a.num_workers;
+  const int slots = a.ctas_per_worker * a.num_workers;
+  const int grid = a.num_tasks < slots ? a.num_tasks : slots;
+  cache->ctas = grid;
   RunArgs args = a;
   args.queue_wrap = static_cast<uint32_t>(a.num_tasks - 1);  // one grab less per CTA for its first task, one more in vain
   return launch_after(kernel, dim3(grid), kThreadsS, smem, s, args, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),

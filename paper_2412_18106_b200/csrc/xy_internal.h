@@ -138,7 +138,8 @@ struct RunArgs {
   uint32_t queue_wrap;     // index of the launch's last grab, which wraps the head to zero
   int32_t* exits;          // word of the status block that counts the CTAs that have finished
   int32_t side_by_side;    // 1, 2: first (dense) and second (streaming) of two launches that run at the same time
-  int32_t dense_ctas;      // CTAs of the first of them, whose time stamps the second one adds to
+  int32_t dense_ctas;      // CTAs of the first of two launches, whose time stamps the second one adds to
+  int32_t ctas_per_worker;  // the streaming kernel's: two fit an SM, but a worker counts as one SM
   // split units whose last finishing task merges them inside the kernel (streaming units)
   const int32_t* task_unit;              // per task: unit index or -1 (null: no such unit)
   const xy_attn_merge_unit* units;

@@ -46,6 +46,7 @@ struct MetaLaunchCache {
   int32_t num_kv_heads = 0, page_size = 0;
   bool valid = false, fp8 = false;
   bool attr_set[6] = {false, false, false, false, false, false};
+  int32_t ctas = 0;  // of the last launch
   // the CTA-pair kernel's maps (K in boxes of at most 64 tokens)
   alignas(64) unsigned char pair_maps[2][128];
   const void* pk_pool = nullptr;

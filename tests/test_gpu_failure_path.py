@@ -76,7 +76,7 @@ def test_debug_context_rejects_a_bad_block_table_before_launching():
 
 
 @pytest.mark.parametrize("workers,decode", [(3, True), (40, True), (0, True), (5, False), (0, False)],
-                         ids=["stream-6", "stream-80", "stream-all", "meta-5", "meta-all"])
+                         ids=["stream-3", "stream-40", "stream-all", "meta-5", "meta-all"])
 def test_many_ctas_that_give_up_leave_a_clean_context(workers, decode):
     """Every CTA gives up after a fill that never comes, with split units half counted and the queue half
     dealt: the next ordinary run, with and without reading the status in between, is right, and bitwise
@@ -139,8 +139,9 @@ def test_status_read_clears_what_a_cleaner_that_gave_up_has_left(workers, skip, 
 @pytest.mark.parametrize("workers", [0, 7])
 @pytest.mark.parametrize("skip", [0, 1, 6])
 def test_two_launches_side_by_side_give_up_and_leave_a_clean_context(skip, workers):
-    """The dense and the streaming launch of a shared-prefix plan share the status word and the unit counters:
-    after a wait that ran out in either, the next ordinary runs are bitwise what they were before."""
+    """The dense and the streaming launch of a shared-prefix plan share the status word and the unit counters,
+    side by side as one after the other (7 workers): after a wait that ran out in either, the next ordinary runs
+    are bitwise what they were before."""
     b, groups = W.shared_prefix_decode(seed=7, num_groups=5, members=42, prefix=512, suffix_hi=400, hq=16, hkv=4)
     t = W.make_tensors(b)
     ctx = H.make_ctx(b, num_workers=workers, max_requests=512)
@@ -169,7 +170,7 @@ def test_two_launches_side_by_side_give_up_and_leave_a_clean_context(skip, worke
     ctx.close()
 
 
-@pytest.mark.parametrize("decode,workers", [(True, 3), (True, 0), (False, 5)], ids=["stream-6", "stream-all", "meta-5"])
+@pytest.mark.parametrize("decode,workers", [(True, 3), (True, 0), (False, 5)], ids=["stream-3", "stream-all", "meta-5"])
 @pytest.mark.parametrize("skip", [1, 11])
 def test_fp8_run_gives_up_and_the_context_recovers(decode, workers, skip):
     b = W.config2_decode(num_requests=9, kv_lo=300, kv_hi=3000) if decode else W.config1_tiny()

@@ -113,7 +113,8 @@ def test_groups_found_from_the_block_table():
 @pytest.mark.parametrize("page,members,workers", [(128, 42, 0), (16, 42, 0), (128, 30, 7)])
 def test_dense_and_streaming_launches_side_by_side_match_oracle(page, members, workers):
     """Many members with keys of their own on short common prefixes: the planner gives the group tiles
-    and the members' own keys a launch each, which run at the same time; then the merge."""
+    and the members' own keys a launch each, which run at the same time (with fewer workers than SMs one after
+    the other); then the merge."""
     b, groups = W.shared_prefix_decode(seed=page + members, num_groups=5, members=members, prefix=512, suffix_hi=400,
                                        hq=16, hkv=4, page_size=page)
     t = W.make_tensors(b)
