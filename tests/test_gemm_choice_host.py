@@ -8,6 +8,15 @@ B200 = [148, 148, 74, 45, 33, 26, 22, 15, 15, 74, 33, 22, 15]
 SCRATCH = 2 * 148 * 128 * 256 * 4
 
 
+# Shapes whose cut for the weight-major kernel (with scratch) has this many MMAs per K step and this many pairs that
+# share K: every form the kernel has, in one, two and several token tiles, ragged in M, N and K.
+FORMS = [(130, 12296, 520, 1, 1), (257, 6152, 1096, 1, 1), (200, 264, 328, 1, 1), (130, 6152, 3080, 1, 2), (257, 3080, 3080, 1, 2),
+         (513, 2056, 3080, 1, 2), (130, 4104, 2056, 1, 3), (257, 2056, 2056, 1, 3), (200, 776, 2056, 1, 3), (130, 3080, 2056, 1, 4),
+         (200, 1544, 3080, 1, 4), (130, 264, 2056, 1, 4), (257, 18696, 2056, 2, 1), (518, 6152, 6152, 2, 1), (1500, 3080, 1032, 2, 1),
+         (257, 6152, 8200, 2, 2), (573, 3080, 8200, 2, 2), (781, 2056, 8200, 2, 2), (257, 4104, 6152, 2, 3), (1028, 1544, 6152, 2, 3),
+         (257, 3080, 10248, 2, 4)]
+
+
 def choice(M, N, K, scratch=SCRATCH, device=B200):
     return xg.xy_gemm_choice(M, N, K, scratch, device)
 
@@ -109,3 +118,19 @@ def test_no_slice_of_k_is_empty(M, device):
                 chunks = (K + 63) // 64
                 assert 1 <= c["splits"] <= 8 and device[c["splits"]] > 0
                 assert (c["splits"] - 1) * -(-chunks // c["splits"]) < chunks
+
+
+@pytest.mark.parametrize("M,N,K,halves,splits", FORMS)
+def test_every_form_of_the_weight_major_kernel_has_a_shape(M, N, K, halves, splits):
+    c = choice(M, N, K)
+    assert (c["kernel"], c["halves"], c["splits"]) == ("weight_major", halves, splits), c
+
+
+def test_shapes_of_the_gpu_tests_reach_what_they_name():
+    """Without scratch, tests/test_gpu_gemm.py names the cluster split of K and single-CTA and pair tiles."""
+    reached = [choice(M, N, K, 0)["kernel"] for M in (1, 16, 33, 100, 128, 129, 300, 512)
+               for N, K in ((512, 4096), (4096, 1024), (1032, 2304), (4096, 14336))]
+    assert reached.count("split_k") >= 4 and reached.count("weight_streaming") >= 12
+    assert choice(1024, 4096, 512, 0)["kernel"] == "pair"
+    c = choice(520, 28672, 128, 0)
+    assert (c["kernel"], c["tile_n"]) == ("tile", 256)

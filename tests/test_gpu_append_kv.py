@@ -12,7 +12,7 @@ from tests import helpers as H
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("page", [16, 128])
+@pytest.mark.parametrize("page", [8, 16, 128])
 def test_append_kv_bit_exact_then_attention(page):
     rng = np.random.default_rng(page)
     reqs = [(70, 0, 0, None), (33, 150, 0, None), (1, 257, 0, None), (1, 5, 0, None),

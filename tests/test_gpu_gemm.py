@@ -7,6 +7,7 @@ import torch
 from oracle import gemm_oracle as G
 from paper_2412_18106_b200 import binding as xb
 from paper_2412_18106_b200 import gemm as xg
+from tests.test_gemm_choice_host import FORMS
 
 pytestmark = pytest.mark.gpu
 
@@ -86,18 +87,20 @@ def test_full_size_qkv_projection_sampled():
 @pytest.mark.parametrize("M", [1, 16, 33, 100, 128, 129, 300, 512])
 @pytest.mark.parametrize("N,K", [(512, 4096), (4096, 1024), (1032, 2304), (4096, 14336)])
 def test_small_token_counts_take_the_split_k_path(M, N, K):
-    """tile_n = 0 with M <= 512 and few tiles splits K over a cluster; the sum of the slices
+    """Few tiles and a long K: the library's choice splits K over a cluster, on 128 x 128 tiles from 129 tokens on
+    (and for the narrowest problems below), in the weight-streaming kernel below; the sum of the slices
     must match the oracle like the single-CTA product does (ragged N, K not a multiple of the
     split, rows past M untouched)."""
     check(M, N, K, 0, seed=M + N)
 
 
-@pytest.mark.parametrize("shape", [(600, 4000, 8264, 128), (640, 7936, 8200, 256), (1100, 4096, 8192, 0)])
+@pytest.mark.parametrize("shape", [(600, 4000, 8264, 128), (640, 7936, 8200, 256), (1100, 4096, 8192, 0),
+                                   (1100, 5120, 8192, 256)])
 def test_last_wave_split_along_k_with_scratch_matches_oracle_and_repeats_bitwise(shape):
     """More tiles than SMs, a thin last wave and a long K: with scratch memory the last wave's
     tiles are split along K over all SMs and a fix-up kernel adds the partial sums.  Ragged M, N
     and K included; the result must match the oracle, repeat bit for bit, and stay inside
-    [0, M) x [0, N)."""
+    [0, M) x [0, N).  (The library's own choice for the third shape is the weight-major kernel.)"""
     M, N, K, tile_n = shape
     g = torch.Generator().manual_seed(K)
     a = torch.randn((M, K), generator=g).to(torch.bfloat16)
@@ -160,11 +163,12 @@ def test_random_shapes_and_tile_choices(seed):
 
 @pytest.mark.parametrize("M,N,K", [(129, 256, 512), (144, 520, 1032), (255, 1000, 4096), (257, 4096, 2048),
                                    (333, 776, 4096), (512, 2048, 1096), (513, 1800, 520), (700, 392, 328),
-                                   (1000, 2568, 640), (129, 28672, 264), (217, 20000, 520)])
+                                   (1000, 2568, 640), (129, 28672, 264), (217, 20000, 520)] + [f[:3] for f in FORMS])
 def test_weight_major_kernel_matches_oracle_and_repeats_bitwise(M, N, K):
-    """129 .. about 1000 tokens take the weight-major CTA-pair kernel: one or two accumulators per tile,
-    several token tiles, K split over the pairs of a cluster when there is scratch; ragged M, N and K.
-    Nothing outside [0, M) x [0, N) is written."""
+    """129 .. 1536 tokens, the library's choice without and with scratch: the weight-major CTA-pair kernel in every
+    form (FORMS, whose cuts tests/test_gemm_choice_host.py pins: one or two MMAs per K step, one or two sets of
+    sums, one to several token tiles, K split over one to four pairs when there is scratch) and, for some
+    of the first shapes, what is chosen instead of it.  Nothing outside [0, M) x [0, N) is written."""
     g = torch.Generator().manual_seed(M + N + K)
     a = torch.randn((M, K), generator=g).to(torch.bfloat16)
     w = torch.randn((N, K), generator=g).to(torch.bfloat16)

@@ -27,12 +27,19 @@ def test_config1_tiny_hybrid(kernel):
 
 
 @pytest.mark.parametrize("kernel", KERNELS, ids=lambda k: KNAMES[k])
-@pytest.mark.parametrize("page", [16, 32, 64, 128])
+@pytest.mark.parametrize("page", [8, 16, 32, 64, 128])
 def test_page_sizes(kernel, page):
     rng = np.random.default_rng(page)
     reqs = [(70, 0, 0, None), (33, 150, 0, None), (1, 257, 0, None), (1, 5, 0, None),
             (20, 300, 1, W.random_tree(rng, 20, 6)), (2, 129, 1, [-1, 0])]
     H.parity(W.custom("pages%d" % page, 8, 2, page, reqs, seed=page), kernel=kernel)
+
+
+@pytest.mark.parametrize("page", [8, 16, 32, 64])
+def test_page_sizes_without_dense_tiles(page):
+    """The streaming kernel: a lane per box of a tile's pages, all 32 lanes at 8 tokens a page; KV splits."""
+    reqs = [(1, h, 0, None) for h in (0, 5, 127, 128, 257, 4000)] + [(2, 129, 1, [-1, 0]), (4, 300, 1, [-1, 0, 0, 2])]
+    H.parity(W.custom("stream%d" % page, 8, 2, page, reqs, seed=page), num_workers=148)
 
 
 @pytest.mark.parametrize("kernel", KERNELS, ids=lambda k: KNAMES[k])
