@@ -228,22 +228,13 @@ def run_reference(args):
     return 0
 
 
-# DRAM bytes (read + write) of one launch of the attention meta-kernel, from the ncu captures
-# summarised under profiles/ (same workload, seed 0), each stamped with the commit of the kernel
-# that was captured and the date; a kernel change that may move traffic needs a new capture.
-NCU_TRAFFIC = {
-    # full_mix: the 5 GB pool is beyond what a multi-pass capture should hold; the dense path and the
-    # queue order that decide its traffic have not changed since this capture
-    "full_mix": {"bytes": 6.00e9, "commit": "29136c8", "date": "2026-11-24", "summary": "profiles/launch_list_full_mix.md"},
-    "splitfuse_mix": {"bytes": 1.666e9, "commit": "e5bad30", "date": "2026-11-25",
-                      "summary": "profiles/meta_attention_splitfuse_mix.md"},
-    "verify_trees": {"bytes": 2.503e9, "commit": "e5bad30", "date": "2026-11-25",
-                     "summary": "profiles/meta_attention_verify_trees.md"},
-    "decode_only": {"bytes": 0.593e9, "commit": "e5bad30", "date": "2026-11-25",
-                    "summary": "profiles/meta_attention_decode_only.md"},
-    "long_context_decode": {"bytes": 3.202e9, "commit": "29136c8", "date": "2026-11-24",
-                            "summary": "profiles/meta_attention_long_context_decode.md"},
-}
+# DRAM bytes (read + write) of the attention launch of a run, from the ncu captures summarised under
+# profiles/ (same workload, seed 0), stamped with the commit of the kernels that were captured and the
+# date; a kernel change that may move traffic needs a new capture.
+NCU_TRAFFIC = {name: {"bytes": nbytes, "commit": "8a3210e", "date": "2026-12-02",
+                      "summary": "profiles/stream_attention_decode_only.md"}
+               for name, nbytes in (("full_mix", 6.02e9), ("splitfuse_mix", 1.67e9), ("verify_trees", 2.45e9),
+                                    ("decode_only", 0.593e9), ("long_context_decode", 3.20e9))}
 
 
 def ncu_traffic(name):

@@ -20,17 +20,19 @@
 namespace xy {
 namespace {
 
-// Per-SM time model in microseconds (free design constants; parity does not depend on them).
-// Measured on B200 from the per-worker time each kind of task takes: a dense task advances one
-// key tile per 2.2 - 2.6 us whether one or both of its 128-row sub-tiles are in use (the softmax
-// -> MMA chain of a sub-tile sets the pace and the two sub-tiles overlap each other); a streaming
-// task one key tile per ~1.0 us while HBM is not saturated (1.4 us when every SM streams); a
-// task boundary costs ~3 us (Q load, pipeline refill, epilogue).
+// Per-SM cost model in microseconds (free design constants; parity does not depend on them): what the
+// splits, the order of the mixed queue and the static Task-Table weigh tasks by.  The values are those of
+// the kernels' first forms: a dense task advanced one key tile per 2.2 - 2.6 us whether one or both of
+// its 128-row sub-tiles are in use, a streaming task one per ~1.0 us, and a task boundary cost ~3 us.  (With
+// one tcgen05 issuer a dense tile takes 2.0 us; only ratios matter to a plan, and these ones are what its
+// other constants were tuned with.)
 constexpr float kDenseVisitUs = 2.30f;
 constexpr float kStreamVisitUs = 1.00f;
 constexpr float kPairVisitUs = 1.35f;
 constexpr float kTaskFixedUs = 3.0f;
-constexpr double kStreamTaskUs = 3.8;      // around a streaming task of the meta-kernel: descriptors, Q, merge of the warps
+// For the choice between one mixed queue and two launches only, whose figures are beside it: around a
+// streaming task of the meta-kernel (descriptors, Q, merge of the warps), a tile at the pace of HBM, a launch.
+constexpr double kStreamTaskUs = 3.8;
 constexpr double kStreamTileHbmUs = 0.0104;  // 64 KiB at 6.3 TB/s
 constexpr double kSecondLaunchUs = 3.0;
 constexpr int kMinChunkTiles = 4;
