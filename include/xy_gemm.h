@@ -3,13 +3,13 @@
  *
  *     C[M, N] = A[M, K] * W[N, K]^T      bf16 inputs, fp32 accumulation, bf16 output
  *
- * The kernel always computes whole 128 x tile_n tiles (Section 5.1: computation on fixed shapes).
- * M is padded virtually: the tile loads read rows past M as zeros on chip (selective read; no
- * padded copy of A exists in global memory) and the epilogue stores only rows below M (selective
- * write).  N and K come from the model (Section 5.2) and need no padding beyond 8-element
- * alignment; a last partial tile in N or K is handled the same way (zeros in, clipped store).
- * Tiles are handed to the SMs with the M tiles of one N tile next to each other, so the SMs that
- * run at the same time share the weight tile through L2 (Section 5.3's task order).
+ * The kernels compute whole tiles of fixed shape (Section 5.1): 128 x tile_n or 256 x tile_n, or, for up
+ * to 1536 tokens, 128 or 256 rows of W by a number of tokens padded to 16.  M is padded virtually: the tile
+ * loads read rows past M as zeros on chip (selective read; no padded copy of A exists in global memory) and
+ * the epilogue stores only rows below M (selective write).  N and K come from the model (Section 5.2) and
+ * need no padding beyond 8-element alignment; a last partial tile in N or K is handled the same way (zeros
+ * in, clipped store).  Tiles are handed to the SMs with the M tiles of one N tile next to each other, so the
+ * SMs that run at the same time share the weight tile through L2 (Section 5.3's task order).
  */
 #ifndef XY_GEMM_H_
 #define XY_GEMM_H_
@@ -46,12 +46,13 @@ extern "C" {
 int xy_gemm_run(const void* a, int64_t lda, const void* w, int64_t ldw, void* c, int64_t ldc, int32_t M,
                 int32_t N, int32_t K, int32_t tile_n, void* stream);
 
-/* The same with DEVICE scratch memory, which lets CTA pairs share the K of a tile for 129 to about 1500
- * tokens (the pairs of a cluster leave fp32 sums in it and add them in a fixed order), and lets the
- * last, partial wave of larger problems be split along K over every SM when K is long (K >= 8192 and a last wave of at most 0.6 of the SMs; measured
- * rule): each SM multiplies a run of K chunks of one or two of those tiles and leaves fp32 partial
- * sums in the scratch; a second, small kernel on the same stream adds a tile's partial sums in a
- * fixed order (bit-reproducible) and stores the tile.  No thread waits for another CTA.
+/* The same with DEVICE scratch memory.  It lets CTA pairs share the K of a tile for 129 to 1536 tokens: the
+ * pairs of a cluster leave fp32 sums in it, meet at a cluster barrier and add them in a fixed order.  And it
+ * lets the last, partial wave of 128-row tiles be split along K over every SM when K is long (K >= 8192 and a
+ * last wave of at most 0.6 of the SMs; measured rule): each SM multiplies a run of K chunks of one or two of
+ * those tiles and leaves fp32 partial sums; a second, small kernel on the same stream adds a tile's partial
+ * sums in a fixed order and stores the tile, so that no thread waits for another CTA there.  Both are
+ * bit-reproducible.
  *   workspace        DEVICE, 16-byte aligned, at least xy_gemm_workspace_bytes() bytes (a smaller
  *                    one, or NULL, gives xy_gemm_run's behaviour); contents do not matter.  Calls
  *                    that may run at the same time need scratch of their own.

@@ -65,17 +65,6 @@ __device__ __forceinline__ uint32_t swz(uint32_t row, uint32_t chunk16 /*0..15*/
   return (chunk16 >> 3) * kHalfBytes + row * 128u + (((chunk16 & 7u) ^ (row & 7u)) << 4);
 }
 
-struct Pipe {
-  int stage;
-  uint32_t phase;
-  __device__ __forceinline__ void advance() {
-    if (++stage == kStages) {
-      stage = 0;
-      phase ^= 1u;
-    }
-  }
-};
-
 struct MetaParams {
   RunArgs a;
 };
@@ -469,7 +458,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   int seq_static = t_begin;
   uint32_t n_read = 0;
   bool feed_dead = false;
-  auto next_task = [&](bool whole_warp) -> int {  // whole_warp: called by all 32 lanes (else by one)
+  auto next_task = [&]() -> int {  // called by all 32 lanes
     if (!dynamic) return seq_static < t_end ? seq_static++ : -1;
     const uint32_t slot = n_read % kTaskRing;
     if (!feed_dead && !mbar_wait_block(smem_u32(&tq->full[slot]), (n_read / kTaskRing) & 1u, a.status)) {
@@ -477,12 +466,8 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       feed_dead = true;
     }
     const int ti = feed_dead ? -1 : tq->ti[slot];
-    if (whole_warp) {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&tq->empty[slot]));
-    } else {
-      mbar_arrive(smem_u32(&tq->empty[slot]));
-    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&tq->empty[slot]));
     ++n_read;
     return ti;
   };
@@ -493,7 +478,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
     if (warp == kConsumerWarps && lane == 0) {
       // ================================ producer =======================================
-      Pipe pipe{0, 0};
+      RingPos pipe{0, 0};
       bool dead = false;
       // Who read each stage last (bit set: the tcgen05 path) and the parity to wait for on each
       // of the two empty barriers of a stage; a stage that was never filled needs no wait.
@@ -512,7 +497,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         // Failure-path test hook (xy_attn_debug_inject): this worker leaves out one fill, so the
         // stage's `full` barrier never completes and the readers' bounded waits run out.
         if (n_fill++ == a.debug_skip_fill) {
-          pipe.advance();
+          pipe.advance<kStages>();
           return;
         }
         const uint32_t bit = 1u << pipe.stage;
@@ -574,7 +559,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
             for (int p = 0; p < 8; ++p)
               if (p < ppt) tma_load_4d(dst + kHalfBytes + p * page_bytes, map, full, 0, 0, kv_head, pages[p]);
           }
-          pipe.advance();
+          pipe.advance<kStages>();
           return;
         }
         mbar_arrive_expect_tx(full, kTileBytes);
@@ -592,7 +577,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
             tma_load_4d(dst + kHalfBytes + p * page_bytes, map, full, 64, 0, kv_head, page);
           }
         }
-        pipe.advance();
+        pipe.advance<kStages>();
       };
       // A cursor over the worker's (task, key tile) sequence.  The block-table entry of a tile is
       // requested three tiles before the tile is issued, so its global-memory latency (and the
@@ -752,7 +737,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           }
         }
       };
-      for (int ti = next_task(true); ti >= 0; ti = next_task(true)) {
+      for (int ti = next_task(); ti >= 0; ti = next_task()) {
         const xy_attn_task t = a.tasks[ti];
         const uint32_t n_all = t.kt_hi - t.kt_lo;
         const uint32_t pos0 = pos;
@@ -810,7 +795,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsConsumer));
     // ================================ consumers ========================================
-    Pipe pipe{0, 0};
+    RingPos pipe{0, 0};
     bool dead = false;
     uint32_t ph_s = 0, ph_o = 0;  // this warpgroup's s_full / o_done parities
     uint32_t tile_seq = 0;        // key tiles consumed so far (fp8: selects the scale slot)
@@ -832,7 +817,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       acct_prev = now;
       acct_kind = kind_now;
     };
-    for (int ti = next_task(true); ti >= 0; ti = next_task(true)) {
+    for (int ti = next_task(); ti >= 0; ti = next_task()) {
       TaskView tv;
       tv.t = a.tasks[ti];
       tv.rq = a.reqs[tv.t.req];
@@ -1182,7 +1167,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           if constexpr (kFp8) fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
-          pipe.advance();
+          pipe.advance<kStages>();
           if (work) {
             const bool need_mask = tree ? (col0 + kKeyTile > h) : (col0 + kKeyTile > h + i_min + 1);
             w.softmax(a, tv.rq, s, p, col0, i_lo, i_hi, need_mask, scale_log2, lane, &fs, 0);
@@ -1199,7 +1184,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           if constexpr (kFp8) fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
-          pipe.advance();
+          pipe.advance<kStages>();
         }
         if (active) {
           w.reduce_l();
@@ -1226,22 +1211,19 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         const int unit = (a.task_unit != nullptr && tv.t.part >= 0) ? a.task_unit[ti] : -1;
         const StreamRing sr{ring + (kFp8 ? kHalfBytes : 0), kTileBytes, smem_u32(&bars->full[0]), smem_u32(&bars->empty[0])};
         auto q_addr = [&](uint32_t row, uint32_t ch) { return q_smem + swz(row, ch); };
-        RingPos pos{pipe.stage, pipe.phase};
         if (tv.rows <= 8) {
           StreamWarp<kConsumerWarps, 1, kFp8> w;
           w.init();
           w.load_q(q_addr, lane);
-          stream_task<kConsumerWarps, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq,
+          stream_task<kConsumerWarps, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pipe, dead, scale_log2, scale_ring, tile_seq,
                                                         unit, warp, 1, &s_last, nullptr);
         } else {
           StreamWarp<kConsumerWarps, 2, kFp8> w;
           w.init();
           w.load_q(q_addr, lane);
-          stream_task<kConsumerWarps, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq,
+          stream_task<kConsumerWarps, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pipe, dead, scale_log2, scale_ring, tile_seq,
                                                         unit, warp, 1, &s_last, nullptr);
         }
-        pipe.stage = pos.stage;
-        pipe.phase = pos.phase;
         named_bar_sync(1, kConsumerThreads);
       }
     }
