@@ -101,7 +101,7 @@ float swap_us(int N, int K, const SwapPlan& p, int fit) {
 }
 
 // Which cut of a problem the weight-major kernel takes.  These simpler terms find the better cuts (us, with
-// them / with the model above as the judge: N 6144, K 4096 at 1216 tokens 49.5 / 54.0, N 3584, K 18944 at 820
+// them / with the model above: N 6144, K 4096 at 1216 tokens 49.5 / 54.0, N 3584, K 18944 at 820
 // 93 / 101, N 16384, K 1024 at 352 16.6 / 18.7); the model above is closer to the kernel's time.  Per K
 // chunk a pair takes its MMAs (1.3 of the nominal rate) or an intake of 50 B a clock, whichever is longer;
 // splitting pays only while every cluster fits the device at once.
