@@ -34,6 +34,7 @@ struct xy_attn_ctx {
   size_t dev_front = 0;                  // bytes in front of the Task-Table part
   std::vector<unsigned char> stage;      // host image of the tables while a plan uploads them
   ReqInfo* d_reqs = nullptr;
+  TaskDesc* d_first = nullptr;           // descriptions of a streaming launch's first tasks
   xy_attn_task* d_tasks = nullptr;
   int32_t* d_worker_off = nullptr;
   int32_t* d_queue = nullptr;
@@ -163,7 +164,7 @@ int xy_attn_create(const xy_attn_config* cfg, xy_attn_ctx** out) {
     // the tables of a plan, back to back (16-byte aligned each)
     c->cap_table_bytes = static_cast<int64_t>(sizeof(ReqInfo)) * cfg->max_requests + sizeof(uint64_t) * c->cap_tree_words +
                          (sizeof(xy_attn_task) + 2 * sizeof(int32_t)) * c->cap_tasks + sizeof(int32_t) * (c->num_workers + 1) +
-                         sizeof(xy_attn_merge_unit) * c->cap_merges + 16 * 8;
+                         sizeof(xy_attn_merge_unit) * c->cap_merges + sizeof(TaskDesc) * 2 * c->num_workers + 16 * 9;
     alloc(reinterpret_cast<void**>(&c->d_tables), c->cap_table_bytes);
     alloc(reinterpret_cast<void**>(&c->d_o_part), sizeof(float) * kHeadDim * c->cap_partial_rows);
     alloc(reinterpret_cast<void**>(&c->d_lse_part), sizeof(float) * c->cap_partial_rows);
@@ -248,12 +249,31 @@ int xy_attn_plan_shared(xy_attn_ctx* ctx, const xy_attn_request* reqs, int32_t n
       return at;
     };
     const size_t reqs_at = put(p.reqs), tree_at = put(p.tree_mask);
+    // What the CTAs of a streaming launch start with: one read instead of a chain of three.
+    const int32_t first_at = std::max(p.queue_dense, 0);
+    const int32_t n_first = p.queue_dense >= 0 || p.info.num_dense_tasks == 0
+                                ? std::min<int32_t>(static_cast<int32_t>(p.queue.size()) - first_at, 2 * ctx->num_workers) : 0;
+    const size_t desc_at = (st.size() + 15) & ~size_t{15};
+    st.resize(desc_at + std::max(n_first, 0) * sizeof(TaskDesc));
+    for (int32_t k = 0; k < n_first; ++k) {
+      const int32_t ti = p.queue[first_at + k];
+      TaskDesc d{};
+      d.t = p.tasks[ti];
+      d.rq = p.reqs[d.t.req];
+      d.rq.pad1 = d.t.part >= 0 ? p.task_unit[ti] : -1;
+      if (d.rq.pad1 >= 0) {
+        d.nsplit = p.merges[d.rq.pad1].nsplit;
+        d.part0 = p.merges[d.rq.pad1].part0;
+      }
+      std::memcpy(st.data() + desc_at + k * sizeof(TaskDesc), &d, sizeof d);
+    }
     const size_t front = (st.size() + 15) & ~size_t{15};
     const bool same_tables = ctx->dev_shape_valid && ctx->dev_front == front && ctx->dev_shape == p.shape;
     ctx->dev_shape_valid = false;
     auto at = [&](size_t off) { return ctx->d_tables + off; };
     ctx->d_reqs = reinterpret_cast<ReqInfo*>(at(reqs_at));
     ctx->d_tree = reinterpret_cast<uint64_t*>(at(tree_at));
+    ctx->d_first = reinterpret_cast<TaskDesc*>(at(desc_at));
     if (!same_tables) {
       ctx->d_tasks = reinterpret_cast<xy_attn_task*>(at(put(p.tasks)));
       ctx->d_queue = reinterpret_cast<int32_t*>(at(put(p.queue)));
@@ -371,6 +391,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
   a.lse = lse;
   a.reqs = ctx->d_reqs;
   a.tasks = ctx->d_tasks;
+  a.first = ctx->d_first;
   a.worker_off = ctx->d_worker_off;
   a.o_part = ctx->d_o_part;
   a.lse_part = ctx->d_lse_part;

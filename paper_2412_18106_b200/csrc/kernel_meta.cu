@@ -1211,18 +1211,19 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         const int unit = (a.task_unit != nullptr && tv.t.part >= 0) ? a.task_unit[ti] : -1;
         const StreamRing sr{ring + (kFp8 ? kHalfBytes : 0), kTileBytes, smem_u32(&bars->full[0]), smem_u32(&bars->empty[0])};
         auto q_addr = [&](uint32_t row, uint32_t ch) { return q_smem + swz(row, ch); };
+        auto unit_ref = [&]() { return UnitRef{a.units[unit].nsplit, a.units[unit].part0}; };
         if (tv.rows <= 8) {
           StreamWarp<kConsumerWarps, 1, kFp8> w;
           w.init();
           w.load_q(q_addr, lane);
           stream_task<kConsumerWarps, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pipe, dead, scale_log2, scale_ring, tile_seq,
-                                                        unit, warp, 1, &s_last, nullptr);
+                                                        unit, unit_ref, warp, 1, &s_last, nullptr);
         } else {
           StreamWarp<kConsumerWarps, 2, kFp8> w;
           w.init();
           w.load_q(q_addr, lane);
           stream_task<kConsumerWarps, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pipe, dead, scale_log2, scale_ring, tile_seq,
-                                                        unit, warp, 1, &s_last, nullptr);
+                                                        unit, unit_ref, warp, 1, &s_last, nullptr);
         }
         named_bar_sync(1, kConsumerThreads);
       }

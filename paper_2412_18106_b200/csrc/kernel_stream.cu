@@ -29,6 +29,8 @@ constexpr int kWarpsS = 4;
 constexpr int kThreadsS = (kWarpsS + 1) * 32;
 // Descriptions of tasks: the one being worked on and up to three that the look-ahead has reached.
 constexpr int kTaskSlots = 4;
+// Key tiles of the first task that are asked for while the launch before is still running.
+constexpr int kPrefetchTiles = 2;
 
 template <bool kFp8>
 struct StreamCfg {
@@ -39,14 +41,8 @@ struct StreamCfg {
   static constexpr int kQ = 16 * 256;
   static constexpr int kMl = kWarpsS * 16 * 8;
   static constexpr int kScales = kFp8 ? kScaleSlots * 64 : 0;
-  static constexpr int kSmem = kRing + kXch + kQ + kMl + kScales + kTaskSlots * 64 + 16 * kStages + 32;
+  static constexpr int kSmem = kRing + kXch + kQ + kMl + kScales + kTaskSlots * static_cast<int>(sizeof(TaskDesc)) + 16 * kStages + 32;
 };
-
-struct TaskDesc {
-  xy_attn_task t;
-  ReqInfo rq;  // pad1: index of the unit the last finisher merges, or -1
-};
-static_assert(sizeof(TaskDesc) == 64, "the shared-memory layout reserves 64 bytes per description");
 
 template <bool kFp8>
 __global__ void __launch_bounds__(kThreadsS, 2)
@@ -85,16 +81,33 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
   }
   __syncthreads();
   // The producer reads the description of the first task while the launch before is still running: the
-  // plan's tables come over by a copy, which this launch is ordered behind in full.  (13 requests of 300 -
-  // 2500 keys 21.7 -> 20.6 us, 64 requests up to 8192 keys 96.4 -> 94.8, fp8 cache 55.2 -> 54.7; with the
-  // same in the append kernel, a step of eight layers with appends 190 -> 183.)
-  xy_attn_task t{};
-  ReqInfo rq{};
+  // plan's tables come over by a copy, which this launch is ordered behind in full.
+  TaskDesc d{};
   if (warp == kWarpsS) {
-    const int ti = __ldg(a.queue + blockIdx.x);
-    t = a.tasks[ti];
-    rq = a.reqs[t.req];
-    rq.pad1 = (a.task_unit != nullptr && t.part >= 0) ? __ldg(a.task_unit + ti) : -1;
+    d = a.first[blockIdx.x];
+    // Its first key tiles are brought into L2 meanwhile, when HBM would idle: beside the append kernel and
+    // between the launches.  The block table may still be written by a kernel before: this is a hint, made from
+    // whatever the table holds, with page ids outside the pool left out; the copies below read the table again
+    // behind the wait.  For it to come early enough the description is one read, not a chain of three (queue,
+    // task, request).  Two steps of eight layers, 13 requests of 300 - 2500 keys with appends: 349 us -> 340 with
+    // the hint alone, 313 with both (one tile 312, three 318); 64 requests up to 8192 keys 98 -> 95.5, over an fp8
+    // cache 55.9 -> 54.8 (one tile 55.4, three 54.7).  An append kernel that lets this one in before its own wait: 323.
+    const int lane_page = kFp8 ? lane : lane >> 1, ppt = kKeyTile >> a.page_shift;
+    if (!a.side_by_side && lane_page < ppt) {
+      const int npages = (d.rq.kv_len + d.rq.q_len + a.page_size - 1) >> a.page_shift;
+      const int32_t* bt = a.block_table + static_cast<int64_t>(d.rq.bt_row) * a.bt_stride;
+      int page[kPrefetchTiles];
+#pragma unroll
+      for (int i = 0; i < kPrefetchTiles; ++i) page[i] = ld_l2(bt + min((d.t.kt_lo + i) * ppt + lane_page, npages - 1));
+#pragma unroll
+      for (int i = 0; i < kPrefetchTiles; ++i) {
+        if (d.t.kt_lo + i < d.t.kt_hi && page[i] >= 0 && page[i] < a.num_pages) {
+          tma_prefetch_4d(&k_map, kFp8 ? 0 : (lane & 1) * 64, 0, d.t.kv_head, page[i]);
+          tma_prefetch_4d(&v_map, kFp8 ? 0 : (lane & 1) * 64, 0, d.t.kv_head, page[i]);
+        }
+      }
+    }
+    __syncwarp();
   }
   // (beside the dense launch: its CTAs have let this one in only after their own wait)
   if (!a.side_by_side) grid_dependency_wait();
@@ -129,7 +142,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     bool open = false, out = false;
     auto next_tile = [&]() {
       Tile x{0, 0, 0, 1.f, 1.f, false, false};
-      if (!open || kt >= t.kt_hi) {
+      if (!open || kt >= d.t.kt_hi) {
         open = false;
         if (out) return x;
         if (n_grab > 0) {  // (the grid has no more CTAs than there are tasks)
@@ -143,20 +156,24 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
             return x;
           }
           const int ti = __ldg(a.queue + k);
-          t = a.tasks[ti];
-          rq = a.reqs[t.req];
-          rq.pad1 = (a.task_unit != nullptr && t.part >= 0) ? __ldg(a.task_unit + ti) : -1;
+          d.t = a.tasks[ti];
+          d.rq = a.reqs[d.t.req];
+          d.rq.pad1 = (a.task_unit != nullptr && d.t.part >= 0) ? __ldg(a.task_unit + ti) : -1;
+          if (d.rq.pad1 >= 0) {
+            d.nsplit = a.units[d.rq.pad1].nsplit;
+            d.part0 = a.units[d.rq.pad1].part0;
+          }
         }
         ++n_grab;
-        if (lane == 0) desc[(n_grab - 1) % kTaskSlots] = TaskDesc{t, rq};
-        kt = t.kt_lo;
-        npages = (rq.kv_len + rq.q_len + a.page_size - 1) >> a.page_shift;
-        bt = a.block_table + static_cast<int64_t>(rq.bt_row) * a.bt_stride;
+        if (lane == 0) desc[(n_grab - 1) % kTaskSlots] = d;
+        kt = d.t.kt_lo;
+        npages = (d.rq.kv_len + d.rq.q_len + a.page_size - 1) >> a.page_shift;
+        bt = a.block_table + static_cast<int64_t>(d.rq.bt_row) * a.bt_stride;
         open = true;
         x.first = true;
       }
       x.valid = true;
-      x.kv_head = t.kv_head;
+      x.kv_head = d.t.kv_head;
       x.kt = kt;
       if (has_box) x.page = __ldg(bt + min(kt * ppt + lane_page, npages - 1));  // past the end: the last page again
       ++kt;
@@ -182,10 +199,10 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       }
       if (!last) {
         __syncwarp();
-        const TaskDesc& d = desc[n_tasks % kTaskSlots];
-        const int rows = d.t.ntok * G;
-        const uint16_t* q0 = a.q + static_cast<int64_t>(d.rq.q_start + d.t.tok0) * a.q_token_stride +
-                             static_cast<int64_t>(d.t.kv_head) * G * kHeadDim + (lane & 15) * 8;
+        const TaskDesc& nd = desc[n_tasks % kTaskSlots];
+        const int rows = nd.t.ntok * G;
+        const uint16_t* q0 = a.q + static_cast<int64_t>(nd.rq.q_start + nd.t.tok0) * a.q_token_stride +
+                             static_cast<int64_t>(nd.t.kv_head) * G * kHeadDim + (lane & 15) * 8;
         const int rows8 = rows <= 8 ? 8 : 16;  // rows the consumers read; those past the task are zeros
         for (int x = lane >> 4; x < rows8; x += 2) {
           const bool ok = x < rows;
@@ -279,6 +296,8 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       tv.rq = desc[n % kTaskSlots].rq;
       if (tv.t.req < 0) break;
       const int unit = tv.rq.pad1;
+      const UnitRef ref{desc[n % kTaskSlots].nsplit, desc[n % kTaskSlots].part0};
+      auto unit_ref = [&]() { return ref; };
       tv.G = G;
       tv.rows = tv.t.ntok * G;
       auto take_q = [&](auto& w) {
@@ -290,12 +309,12 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       if (tv.rows <= 8) {
         StreamWarp<kWarpsS, 1, kFp8> w;
         take_q(w);
-        stream_task<kWarpsS, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, warp, 1,
+        stream_task<kWarpsS, 1, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, unit_ref, warp, 1,
                                                s_last, s_failed);
       } else {
         StreamWarp<kWarpsS, 2, kFp8> w;
         take_q(w);
-        stream_task<kWarpsS, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, warp, 1,
+        stream_task<kWarpsS, 2, kFp8, kStages>(a, tv, w, sr, xch, ml, pos, dead, scale_log2, scale_ring, tile_seq, unit, unit_ref, warp, 1,
                                                s_last, s_failed);
       }
     }
@@ -342,6 +361,7 @@ cudaError_t launch_stream(const RunArgs& a, int64_t num_pages, MetaLaunchCache* 
   const int grid = a.num_tasks < slots ? a.num_tasks : slots;
   cache->ctas = grid;
   RunArgs args = a;
+  args.num_pages = num_pages;
   args.queue_wrap = static_cast<uint32_t>(a.num_tasks - 1);  // one grab less per CTA for its first task, one more in vain
   return launch_after(kernel, dim3(grid), kThreadsS, smem, s, args, *reinterpret_cast<const CUtensorMap*>(cache->maps[0]),
                       *reinterpret_cast<const CUtensorMap*>(cache->maps[1]));

@@ -382,13 +382,25 @@ __global__ void __launch_bounds__(128) append_kv_kernel(const uint16_t* qkv, int
   const int64_t slot_off = page * page_stride + static_cast<int64_t>(j & (page_size - 1)) * token_stride;
   const uint16_t* src = qkv + static_cast<int64_t>(t) * qkv_token_stride + static_cast<int64_t>(Hq) * kHeadDim;
   const int chunks = 2 * Hkv * (kHeadDim / 8);  // 16-byte chunks of this token's K then V heads
-  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-    const int hv = c / (kHeadDim / 8), d8 = c % (kHeadDim / 8);  // head index within [K heads | V heads]
-    const bool is_v = hv >= Hkv;
-    const int g = is_v ? hv - Hkv : hv;
-    const uint4 val = *reinterpret_cast<const uint4*>(src + static_cast<int64_t>(hv) * kHeadDim + d8 * 8);
-    uint16_t* pool = is_v ? v_pool : k_pool;
-    *reinterpret_cast<uint4*>(pool + slot_off + static_cast<int64_t>(g) * head_stride + d8 * 8) = val;
+  // A thread's loads first (they do not wait for the page id), then its stores.
+  constexpr int kBatch = 4;
+  for (int c0 = threadIdx.x; c0 < chunks; c0 += kBatch * blockDim.x) {
+    uint4 val[kBatch];
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const int c = c0 + b * blockDim.x;
+      if (c < chunks) val[b] = *reinterpret_cast<const uint4*>(src + static_cast<int64_t>(c) * 8);
+    }
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const int c = c0 + b * blockDim.x;
+      if (c >= chunks) break;
+      const int hv = c / (kHeadDim / 8), d8 = c % (kHeadDim / 8);  // head index within [K heads | V heads]
+      const bool is_v = hv >= Hkv;
+      const int g = is_v ? hv - Hkv : hv;
+      uint16_t* pool = is_v ? v_pool : k_pool;
+      *reinterpret_cast<uint4*>(pool + slot_off + static_cast<int64_t>(g) * head_stride + d8 * 8) = val[b];
+    }
   }
 }
 

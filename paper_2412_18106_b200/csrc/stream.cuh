@@ -140,13 +140,17 @@ struct RingPos {
   }
 };
 
+// The part of a merge unit that its tasks do not hold themselves.
+struct UnitRef {
+  int nsplit, part0;
+};
+
 // Merge of a split unit (the cross-task Update stage of Section 4.2.1) by the task of the unit that
 // finished last: rows <= 16, one warp per row.  Lane c holds LSE_c of splits c, c + 32, ...; the
 // weights are broadcast, and the partial rows are read eight at a time straight from L2.
 template <int kWarps>
-__device__ __forceinline__ void merge_unit_in_kernel(const RunArgs& a, const xy_attn_merge_unit& u, int q_start, int G,
-                                                     int warp, int lane) {
-  const int rows = u.ntok * G, ns = u.nsplit;
+__device__ __forceinline__ void merge_unit_in_kernel(const RunArgs& a, const UnitRef& u, const TaskView& tv, int warp, int lane) {
+  const int rows = tv.rows, ns = u.nsplit;
   for (int x = warp; x < rows; x += kWarps) {
     const float* lse_c = a.lse_part + u.part0 + x;  // split c: + c * rows
     const float4* o_c = reinterpret_cast<const float4*>(a.o_part) + (static_cast<int64_t>(u.part0) + x) * (kHeadDim / 4) + lane;
@@ -189,8 +193,8 @@ __device__ __forceinline__ void merge_unit_in_kernel(const RunArgs& a, const xy_
         acc.w += w[e] * v[e].w;
       }
     }
-    const int64_t token = q_start + u.tok0 + x / G;
-    const int head = u.kv_head * G + x % G;
+    const int64_t token = tv.rq.q_start + tv.t.tok0 + x / tv.G;
+    const int head = tv.t.kv_head * tv.G + x % tv.G;
     uint2 packed;
     packed.x = pack_bf16(acc.x, acc.y);
     packed.y = pack_bf16(acc.z, acc.w);
@@ -459,11 +463,11 @@ constexpr int kStreamXchFloats = kWarps * (kWarps - 1) * (8 / kWarps) * 128;
 // Update stage of Section 4.2.1): warp w finishes m-tiles [w * 8 / kWarps, + 8 / kWarps), so every
 // thread exchanges with the same lane of the other warps (conflict-free, one barrier per 8 rows).
 // The caller puts a barrier of the warps between two tasks: the exchange area is read to the end.
-template <int kWarps, int NR, bool kFp8, int kStages>
+template <int kWarps, int NR, bool kFp8, int kStages, typename UnitOf>
 __device__ __forceinline__ void stream_task(const RunArgs& a, const TaskView& tv, StreamWarp<kWarps, NR, kFp8>& w,
                                             const StreamRing& ring, float* xch, float* ml, RingPos& pos, bool& dead,
                                             float scale_log2, const float* scale_ring, uint32_t& tile_seq, int unit,
-                                            int warp, int bar_id, int* s_last, int* s_failed) {
+                                            UnitOf&& unit_ref, int warp, int bar_id, int* s_last, int* s_failed) {
   constexpr int U = 8 / kWarps, kMt = 8 / kWarps;
   const int lane = threadIdx.x & 31, g = lane >> 2, t2 = 2 * (lane & 3);
   const int h = tv.rq.kv_len;
@@ -679,7 +683,7 @@ __device__ __forceinline__ void stream_task(const RunArgs& a, const TaskView& tv
     __threadfence();
     named_bar_sync(bar_id, kWarps * 32);
     if (warp == 0 && lane == 0) {
-      const int ns = a.units[unit].nsplit;
+      const int ns = unit_ref().nsplit;
       const bool last = atomicAdd(a.unit_count + unit, 1) == ns - 1;
       if (last) a.unit_count[unit] = 0;
       *s_last = last ? 1 : 0;
@@ -687,7 +691,7 @@ __device__ __forceinline__ void stream_task(const RunArgs& a, const TaskView& tv
     named_bar_sync(bar_id, kWarps * 32);
     if (*s_last) {
       __threadfence();
-      merge_unit_in_kernel<kWarps>(a, a.units[unit], tv.rq.q_start, tv.G, warp, lane);
+      merge_unit_in_kernel<kWarps>(a, unit_ref(), tv, warp, lane);
     }
   }
 }

@@ -45,6 +45,15 @@ struct ReqInfo {
   int32_t pad1;
 };
 
+// A streaming task with all that its CTA has to know of it, in one place.
+struct TaskDesc {
+  xy_attn_task t;
+  ReqInfo rq;               // pad1: index of the unit that the last of its tasks to finish merges, or -1
+  int32_t nsplit, part0;    // that unit's number of splits and its first partial row
+  int32_t pad[2];
+};
+static_assert(sizeof(TaskDesc) == 80, "read as five 16-byte words");
+
 struct PlanResult {
   std::vector<ReqInfo> reqs;
   std::vector<int32_t> q_start;            // num_reqs + 1
@@ -114,6 +123,7 @@ struct RunArgs {
   const uint16_t* k_pool;
   const uint16_t* v_pool;
   int64_t page_stride, head_stride, token_stride;
+  int64_t num_pages;
   const int32_t* block_table;
   int32_t bt_stride;
   const uint64_t* tree_mask;
@@ -124,6 +134,7 @@ struct RunArgs {
   // context-owned
   const ReqInfo* reqs;
   const xy_attn_task* tasks;
+  const TaskDesc* first;  // descriptions of the streaming launch's first tasks, one per CTA
   const int32_t* worker_off;
   float* o_part;
   float* lse_part;
