@@ -84,7 +84,8 @@ GemmChoice token_major(int M, int N, int K, const GemmDevice& dev) {
 // Weight-major kernel.  Per K chunk a CTA pair takes its MMAs (64 cycles per instruction at least) but no
 // less than 0.2 us; every wave of tiles also takes its weights' time in HBM; the store of a tile's sums
 // overlaps the next tile's chain when tensor memory holds two sets of them; splitting K costs the exchange
-// of sums.
+// of sums.  (Fitted when a tile's sums were stored by half as many warps: its time is an upper one, and the lines
+// below keep to what was measured with it.)
 float swap_us(int N, int K, const SwapPlan& p, int fit) {
   const int n_tiles = div_up(N, 256), tiles = p.m_tiles * n_tiles, chunks = div_up(div_up(K, 64), p.splits);
   const bool two_sets = 2 * p.tok <= 512;

@@ -673,6 +673,13 @@ struct SwapParams {
   uint32_t tmem_cols;
   float4* ws;  // splits > 1: [tile][split][rank][tok / 4][128]
 };
+// Two epilogue warps per quarter of the accumulator's rows, on alternate groups of tokens: one per quarter took
+// about 6 us for the sums of 352 tokens, a chain of tensor-memory load, shuffles and stores that nothing overlaps
+// when tensor memory holds one set of sums.  Eight against four (us): hidden 4096 at 333 tokens QKV 21.1 -> 20.2,
+// OProj 18.0 -> 16.4, GateUp 73.6 -> 69.4, Down 38.1 -> 36.9; at 200 tokens 19.7, 16.1, 49.4, 31.6 -> 18.0, 15.1,
+// 48.0, 30.4; at 1024 QKV 39.2 -> 37.2, the others level.
+constexpr int kSwapEpilogueWarps = 8;
+constexpr int kSwapThreads = 64 + 32 * kSwapEpilogueWarps;
 constexpr int kSwapMaxStages = 12;
 constexpr int kSwapRing = 212992;  // bytes of ring at most
 constexpr int kSwapSmem = 1024 + kSwapRing + 512;
@@ -702,7 +709,7 @@ __device__ __forceinline__ void store16_columns(uint16_t* c, int64_t ldc, const 
   for (int j = 0; j < 16; j += 4) store4_columns(c, ldc, v + j, m + j, m_end, n, N, lane);
 }
 
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(kSwapThreads, 1)
 smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_constant__ CUtensorMap a_map,
                         const __grid_constant__ CUtensorMap w_map) {
   extern __shared__ uint8_t smem_raw[];
@@ -722,7 +729,7 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars->acc_full[b]), 1);   // each CTA: one commit
-      mbar_init(smem_u32(&bars->acc_empty[b]), 8);  // leader: four epilogue warps of each CTA
+      mbar_init(smem_u32(&bars->acc_empty[b]), 2 * kSwapEpilogueWarps);  // leader: the epilogue warps of both CTAs
     }
     fence_mbar_init();
   }
@@ -826,7 +833,7 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
     }
   } else if (warp >= 2) {
     // ---------------------------------------------------------------- epilogue (both CTAs)
-    const int q = warp & 3, row = q * 32 + lane;
+    const int q = warp & 3, row = q * 32 + lane, second = (warp - 2) >> 2;
     const uint32_t acc_empty_leader = cluster_map(smem_u32(&bars->acc_empty[0]), leader_rank);
     uint32_t local = 0;
     for (int t = cluster; t < num_tiles; t += clusters, ++local) {
@@ -841,15 +848,19 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
       const int m_end = min(P.M, m0 + P.tok);
       const uint32_t t_acc = tmem + (static_cast<uint32_t>(q * 32) << 16) + buf * P.tok;
       if (P.splits == 1) {
-#pragma unroll 2
-        for (int c0 = 0; c0 < P.tok && m0 + c0 < m_end; c0 += 16) {
-          uint32_t v[16];
-          tmem_ld_32x32b_x16(t_acc + c0, v);
+        for (int c0 = 32 * second; c0 < P.tok && m0 + c0 < m_end; c0 += 64) {
+          uint32_t v[2][16];
+          tmem_ld_32x32b_x16(t_acc + c0, v[0]);
+          if (c0 + 16 < P.tok) tmem_ld_32x32b_x16(t_acc + c0 + 16, v[1]);
           tmem_wait_ld();
-          float f[16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
-          store16_columns(P.c, P.ldc, f, m0 + c0, m_end, n, P.N, lane);
+          for (int g = 0; g < 2; ++g) {
+            if (g == 1 && c0 + 16 >= P.tok) break;
+            float f[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[g][j]);
+            store16_columns(P.c, P.ldc, f, m0 + c0 + 16 * g, m_end, n, P.N, lane);
+          }
         }
         tc_fence_before();
         __syncwarp();
@@ -861,7 +872,7 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
         const int own = (((m_end - m0 + P.splits - 1) / P.splits + 15) / 16) * 16;  // tokens per pair
         float4* mine = P.ws + (static_cast<int64_t>((t * P.splits + split) * 2 + rank) * (P.tok / 4)) * 128 + row;
 #pragma unroll 2
-        for (int c0 = 0; c0 < P.tok && m0 + c0 < m_end; c0 += 16) {
+        for (int c0 = 16 * second; c0 < P.tok && m0 + c0 < m_end; c0 += 32) {
           if (c0 / own == split) continue;
           uint32_t v[16];
           tmem_ld_32x32b_x16(t_acc + c0, v);
@@ -878,7 +889,7 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
     __syncwarp();
     cluster_sync_all();
     if (warp >= 2 && ok) {
-      const int q = warp & 3, row = q * 32 + lane, t = cluster;
+      const int q = warp & 3, row = q * 32 + lane, t = cluster, second = (warp - 2) >> 2;
       const int m0 = (t % P.m_tiles) * P.tok, n = (t / P.m_tiles) * 256 + 128 * rank + row;
       const int m_end = min(P.M, m0 + P.tok);
       const int own = (((m_end - m0 + P.splits - 1) / P.splits + 15) / 16) * 16;
@@ -886,7 +897,7 @@ smooth_gemm_swap_kernel(const __grid_constant__ SwapParams P, const __grid_const
       const int64_t slot = static_cast<int64_t>(P.tok / 4) * 128;
       const float4* part = P.ws + (static_cast<int64_t>(t * P.splits) * 2 + rank) * slot + row;
       tc_fence_after();
-      for (int c0 = split * own; c0 < (split + 1) * own && m0 + c0 < m_end; c0 += 16) {
+      for (int c0 = split * own + 16 * second; c0 < (split + 1) * own && m0 + c0 < m_end; c0 += 32) {
         uint32_t v[16];
         tmem_ld_32x32b_x16(t_acc + c0, v);
         float4 x[kSwapMaxSplits - 1][4];
@@ -1262,10 +1273,10 @@ cudaError_t launch_gemm_splitk(const void* a, int64_t lda, const void* w, int64_
 
 // Clusters of `size` CTAs of a GEMM kernel with `smem` bytes each that fit the device at once.
 template <class Kernel>
-cudaError_t max_clusters(Kernel kernel, int size, int smem, int* count) {
+cudaError_t max_clusters(Kernel kernel, int threads, int size, int smem, int* count) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(size * 64), 1, 1);
-  cfg.blockDim = dim3(kGemmThreads, 1, 1);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
   cfg.dynamicSmemBytes = static_cast<size_t>(smem);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1304,7 +1315,7 @@ cudaError_t launch_gemm_swap(const void* a, int64_t lda, const void* w, int64_t 
   const int grid = 2 * plan.splits * (plan.splits > 1 ? tiles : std::min(tiles, clusters));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
-  cfg.blockDim = dim3(kGemmThreads, 1, 1);
+  cfg.blockDim = dim3(kSwapThreads, 1, 1);
   cfg.dynamicSmemBytes = kSwapSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -1324,12 +1335,12 @@ cudaError_t query_device(int sms, GemmDevice* d) {
   d->sms = sms;
   cudaError_t e = cudaFuncSetAttribute(smooth_gemm_swap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwapSmem);
   for (int sp = 1; sp <= kSwapMaxSplits && e == cudaSuccess; ++sp)
-    e = max_clusters(smooth_gemm_swap_kernel, 2 * sp, kSwapSmem, &d->pair_clusters[sp - 1]);
+    e = max_clusters(smooth_gemm_swap_kernel, kSwapThreads, 2 * sp, kSwapSmem, &d->pair_clusters[sp - 1]);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(smooth_gemm_small_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   d->clusters[0] = sms;
   for (int n = 2; n <= kClusterMaxCtas && e == cudaSuccess; ++n)  // (the answer counts one CTA per SM; two run)
-    e = max_clusters(smooth_gemm_small_kernel, n, kSmallSmem, &d->clusters[n - 1]);
+    e = max_clusters(smooth_gemm_small_kernel, kGemmThreads, n, kSmallSmem, &d->clusters[n - 1]);
   return e;
 }
 
