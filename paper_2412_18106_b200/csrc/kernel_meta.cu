@@ -3,9 +3,9 @@
 // One persistent CTA per worker (SM) of 384 threads runs meta-tasks until none are left: its own
 // Task-Table list (Section 3.3.1) or, for balanced plans, the head of one global queue.  Roles:
 //   warps 0..7  consumers: softmax (and, on the warp-level paths, the MMAs), O / LSE output
-//   warp  8     producer (one lane): takes the next task, looks page ids up in the block table and
-//               stages 128-key K and V tiles (one TMA box per page and 64-element half) into a
-//               ring of four shared-memory stages; it runs ahead across task boundaries
+//   warps 8, 10 producers: take the next task, look page ids up in the block table and stage 128-key
+//               K (warp 8) and V tiles (warp 10; one TMA box per page and 64-element half) into a
+//               ring of four shared-memory stages; they run ahead across task boundaries
 //   warp  9     tcgen05 issuer for both 128-row sub-tiles of a dense task
 // Shared-memory tiles use the 128-byte TMA swizzle: element (row, d) of a tile lives at
 //   (d / 64) * 16 KiB + row * 128 B + (((d % 64) / 8) ^ (row % 8)) * 16 B + (d % 8) * 2 B,
@@ -41,10 +41,10 @@ using namespace ptx;
 
 constexpr int kConsumerWarps = 8;
 constexpr int kConsumerThreads = kConsumerWarps * 32;
-constexpr int kThreads = kConsumerThreads + 128;  // + one warpgroup: producer, MMA issuer, 2 idle
+constexpr int kThreads = kConsumerThreads + 128;  // + one warpgroup: K producer, MMA issuer, V producer, 1 idle
 constexpr int kRegsConsumer = 216;  // setmaxnreg budgets: 256 x 216 + 128 x 72 = 168 x 384, the launch allocation
 constexpr int kRegsOther = 72;
-constexpr int kStages = 4;
+constexpr int kStages = 4;  // K tiles in 0 and 2, V tiles in 1 and 3
 constexpr int kTileBytes = 32768;  // 2 halves x 128 rows x 128 B
 constexpr int kHalfBytes = 16384;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -419,7 +419,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     }
     for (int i = 0; i < kTaskRing; ++i) {
       mbar_init(smem_u32(&tq->full[i]), 1);
-      mbar_init(smem_u32(&tq->empty[i]), kConsumerWarps + (kUmma ? 1 : 0));
+      mbar_init(smem_u32(&tq->empty[i]), kConsumerWarps + (kUmma ? 2 : 1));
     }
     for (int X = 0; X < 2; ++X) {
       mbar_init(smem_u32(&ub->q_full[X]), 4);
@@ -476,155 +476,82 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
 
   if (warp >= kConsumerWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
-    if (warp == kConsumerWarps && lane == 0) {
-      // ================================ producer =======================================
-      RingPos pipe{0, 0};
+    if (warp == kConsumerWarps || warp == kConsumerWarps + 2) {
+      static_assert(kStages == 4, "two stages per producer");
+      // ================================ producers ======================================
+      // Warp 8 stages the K tiles (even stages of the ring), warp 10 the V tiles (odd stages); warp 8 also
+      // takes the tasks and hands them to everyone.  Each lane issues the box of one page and half, side
+      // by side.  (One lane that did all of it, K and V, box after box, needed 1600 - 2400 cycles per fill of an
+      // empty ring, about what a streaming tile takes its SM, and its per-stage state cost the consumers 90 bytes
+      // of spills.  One lane / two warps: 2048-token chunk beside 48 decode requests 429 -> 394 us, serving mix of 96
+      // requests 4950 -> 4684, 4 prompts of 4096 tokens 1111 -> 1065, 32 verify trees 864 -> 830, two planned steps of
+      // a tiny batch 36.9 -> 33.6; a chunk of 512 tokens beside 40 decode requests on pages of 16 tokens 216 ->
+      // 120, of 32 tokens 141 -> 111, on pages of 128 over an fp8 cache 264 -> 256.)
+      const int op = warp == kConsumerWarps ? 0 : 1;
       bool dead = false;
-      // Who read each stage last (bit set: the tcgen05 path) and the parity to wait for on each
-      // of the two empty barriers of a stage; a stage that was never filled needs no wait.
-      uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0;
-      uint32_t fill_par = 0;  // per stage: parity of the `full` phase its latest fill completes
+      // Of this producer's stages (2 i + op): who read the stage last (bit i set: the tcgen05 path), the parity
+      // to wait for on each of its two empty barriers, and of its `full` phase that the latest fill completes;
+      // a stage that was never filled needs no wait.
+      uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0, fill_par = 0;
       Tracer tr;
-      tr.init(a, 3, true);
+      tr.init(a, 3, op == 0 && lane == 0);
       const int ppt = kKeyTile >> a.page_shift;  // pages per 128-key tile
+      const int lane_page = kFp8 ? lane : lane >> 1;
+      const bool has_box = lane_page < ppt;
       const uint32_t page_bytes = static_cast<uint32_t>(a.page_size) * 128u;
+      // bf16: two 64-element boxes per page; e4m3 bytes: one box per page (128 B per key) into the upper half of the stage
+      const uint32_t box_off = (kFp8 ? kHalfBytes : (lane & 1) * kHalfBytes) + lane_page * page_bytes;
+      const int box_x = kFp8 ? 0 : (lane & 1) * 64;
+      const CUtensorMap* map = op == 0 ? &k_map : &v_map;
       const uint64_t pol_stream = make_l2_policy_evict_first(), pol_keep = make_l2_policy_evict_last();
-      // Fill one stage (the K or the V tile) once its previous reader has released it.
-      int n_fill = 0;
-      uint32_t k_fills = 0;  // K tiles filled so far (fp8: selects the scale slot)
-      auto fill = [&](int op, bool by_umma, int kv_head, int kt, const int32_t* bt, int npages, int page0,
-                      float ks0, float vs0) {
-        // Failure-path test hook (xy_attn_debug_inject): this worker leaves out one fill, so the
-        // stage's `full` barrier never completes and the readers' bounded waits run out.
-        if (n_fill++ == a.debug_skip_fill) {
-          pipe.advance<kStages>();
-          return;
-        }
-        const uint32_t bit = 1u << pipe.stage;
-        if (used & bit) {
-          bool ok;
-          if (last_umma & bit) {
-            ok = mbar_wait_block(smem_u32(&bars->empty_umma[pipe.stage]), (ph_umma >> pipe.stage) & 1u, a.status);
-            ph_umma ^= bit;
-          } else {
-            ok = mbar_wait_block(smem_u32(&bars->empty[pipe.stage]), (ph_cons >> pipe.stage) & 1u, a.status);
-            ph_cons ^= bit;
-          }
-          if (!ok) {
-            report_timeout(a);
-            dead = true;
-            return;
-          }
-        }
-        if (used & bit) fill_par ^= bit;
-        used |= bit;
-        last_umma = by_umma ? (last_umma | bit) : (last_umma & ~bit);
-        tr(1 + op);
-        const uint32_t full = smem_u32(&bars->full[pipe.stage]);
-        const uint32_t dst = ring + pipe.stage * kTileBytes;
-        const CUtensorMap* map = op == 0 ? &k_map : &v_map;
-        if constexpr (kFp8) {
-          // e4m3 bytes: one box per page (128 B per key) into the upper half of the stage; the K
-          // fill also leaves the K and V scales of the tile's pages in the tile's scale slot, before
-          // the arrive that the readers' wait synchronises with.
-          int pages[8];
-          pages[0] = page0;
-          if (ppt > 1) {
-#pragma unroll
-            for (int p = 0; p < 8; ++p)
-              if (p < ppt) pages[p] = __ldg(bt + min(kt * ppt + p, npages - 1));  // past the end: reload the last
-          }
-          if (op == 0) {
-            float* slot = scale_ring + (k_fills % kScaleSlots) * 16;
-            ++k_fills;
-            if (ppt == 1) {
-              slot[0] = ks0;
-              slot[8] = vs0;
-            } else {
-#pragma unroll
-              for (int p = 0; p < 8; ++p) {
-                if (p < ppt) {
-                  const int64_t si = static_cast<int64_t>(pages[p]) * a.num_kv_heads + kv_head;
-                  slot[p] = __ldg(a.k_scale + si);
-                  slot[8 + p] = __ldg(a.v_scale + si);
-                }
-              }
-            }
-          }
-          mbar_arrive_expect_tx(full, kHalfBytes);
-          if (ppt == 1) {
-            tma_load_4d_hint(dst + kHalfBytes, map, full, 0, 0, kv_head, page0, pol_stream);
-          } else {
-#pragma unroll
-            for (int p = 0; p < 8; ++p)
-              if (p < ppt) tma_load_4d(dst + kHalfBytes + p * page_bytes, map, full, 0, 0, kv_head, pages[p]);
-          }
-          pipe.advance<kStages>();
-          return;
-        }
-        mbar_arrive_expect_tx(full, kTileBytes);
-        if (ppt == 1) {
-          // K/V of streaming tasks is read once: mark it evict-first in L2 so that it does not
-          // push out the K/V that the q tiles of a prefill share through L2 (kept evict-last).
-          const uint64_t pol = by_umma ? pol_keep : pol_stream;
-          tma_load_4d_hint(dst, map, full, 0, 0, kv_head, page0, pol);
-          tma_load_4d_hint(dst + kHalfBytes, map, full, 64, 0, kv_head, page0, pol);
-        } else {
-          for (int p = 0; p < ppt; ++p) {
-            const int pi = min(kt * ppt + p, npages - 1);  // pages past the end: reload the last
-            const int page = __ldg(bt + pi);
-            tma_load_4d(dst + p * page_bytes, map, full, 0, 0, kv_head, page);
-            tma_load_4d(dst + kHalfBytes + p * page_bytes, map, full, 64, 0, kv_head, page);
-          }
-        }
-        pipe.advance<kStages>();
-      };
-      // A cursor over the worker's (task, key tile) sequence.  The block-table entry of a tile is
-      // requested three tiles before the tile is issued, so its global-memory latency (and the
+      // A cursor over the worker's (task, key tile) sequence.  The block-table entries of a tile are
+      // requested three tiles before the tile is issued, so their global-memory latency (and the
       // task / request loads at a task boundary) never sits between a stage's release and its
       // TMA: that latency would otherwise add to every refill of the ring.
       struct Tile {
-        const int32_t* bt;
-        int kv_head, kt, npages, page;
-        float ks, vs;  // fp8, one page per tile: that page's K and V scale
+        int kv_head, page;  // page: of this lane's box
+        float ks, vs;       // fp8: that page's K and V scale
         bool by_umma, valid;
       };
       int f_ti = t_begin, f_kt = 0, f_hi = 0, f_head = 0, f_npages = 1;
       uint32_t n_pub = 0;
       bool f_done = false;
-      // Next task of this worker: its own list, or the head of the global queue (published to the
+      // Next task of this worker: its own list, or the head of the global queue (published by warp 8 to the
       // other roles through the ring; -1 is published once, when the queue is exhausted).
       auto grab = [&]() -> int {
+        if (op == 1) return next_task();
         if (!dynamic) return f_ti < t_end ? f_ti++ : -1;
-        if (f_done) return -1;
         int ti = -1;
-        const int k = static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
-        if (k < a.num_tasks) ti = __ldg(a.queue + k);
+        if (lane == 0) {
+          const int k = static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
+          if (k < a.num_tasks) ti = __ldg(a.queue + k);
+        }
+        ti = __shfl_sync(0xffffffffu, ti, 0);
         const uint32_t slot = n_pub % kTaskRing;
         if (n_pub >= kTaskRing &&
             !mbar_wait_block(smem_u32(&tq->empty[slot]), ((n_pub / kTaskRing) - 1u) & 1u, a.status)) {
           report_timeout(a);
           dead = true;
         }
-        tq->ti[slot] = ti;
-        mbar_arrive(smem_u32(&tq->full[slot]));
+        __syncwarp();
+        if (lane == 0) {
+          tq->ti[slot] = ti;
+          mbar_arrive(smem_u32(&tq->full[slot]));
+        }
         ++n_pub;
-        if (ti < 0) f_done = true;
         return ti;
       };
       const int32_t* f_bt = a.block_table;
       bool f_umma = false, f_open = false;
       auto next_tile = [&]() {
-        Tile x;
-        x.valid = false;
-        x.bt = f_bt;
-        x.kv_head = x.kt = x.page = 0;
-        x.npages = 1;
-        x.ks = x.vs = 1.f;
-        x.by_umma = false;
+        Tile x{0, 0, 1.f, 1.f, false, false};
         while (!f_open || f_kt >= f_hi) {
+          if (f_done) return x;
           const int ti = grab();
-          if (ti < 0) return x;
+          if (ti < 0) {
+            f_done = true;
+            return x;
+          }
           const xy_attn_task t = a.tasks[ti];
           const ReqInfo rq = a.reqs[t.req];
           f_kt = t.kt_lo;
@@ -636,25 +563,71 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           f_open = true;
         }
         x.valid = true;
-        x.bt = f_bt;
         x.kv_head = f_head;
-        x.kt = f_kt;
-        x.npages = f_npages;
         x.by_umma = f_umma;
-        x.page = __ldg(f_bt + min(f_kt * ppt, f_npages - 1));  // consumed three tiles later
+        if (has_box) x.page = __ldg(f_bt + min(f_kt * ppt + lane_page, f_npages - 1));  // past the end: the last page again
         ++f_kt;
         return x;
       };
-      // fp8, one page per tile: the page's scales are requested one step after its block-table
-      // entry (which they depend on) and used one step later still.
+      // fp8: the page's scales are requested one step after its block-table entry (which they depend
+      // on) and used one step later still.
       auto request_scales = [&](Tile& x) {
         if constexpr (kFp8) {
-          if (ppt == 1 && x.valid) {
+          if (op == 0 && x.valid && has_box) {
             const int64_t si = static_cast<int64_t>(x.page) * a.num_kv_heads + x.kv_head;
             x.ks = __ldg(a.k_scale + si);
             x.vs = __ldg(a.v_scale + si);
           }
         }
+      };
+      // Fill this producer's next stage once its previous reader has released it.
+      int n_fill = 0;
+      auto fill = [&](const Tile& x) {
+        const int n = n_fill++;
+        const uint32_t i = n % (kStages / 2), bit = 1u << i, stage = 2 * i + op;
+        // Failure-path test hook (xy_attn_debug_inject): this worker leaves out one fill, so the
+        // stage's `full` barrier never completes and the readers' bounded waits run out.
+        if (2 * n + op == a.debug_skip_fill) return;
+        if (used & bit) {
+          bool ok;
+          if (last_umma & bit) {
+            ok = mbar_wait_block(smem_u32(&bars->empty_umma[stage]), (ph_umma >> i) & 1u, a.status);
+            ph_umma ^= bit;
+          } else {
+            ok = mbar_wait_block(smem_u32(&bars->empty[stage]), (ph_cons >> i) & 1u, a.status);
+            ph_cons ^= bit;
+          }
+          if (!ok) {
+            report_timeout(a);
+            dead = true;
+          }
+          dead = __any_sync(0xffffffffu, dead);
+          if (dead) return;
+          fill_par ^= bit;
+        }
+        used |= bit;
+        last_umma = x.by_umma ? (last_umma | bit) : (last_umma & ~bit);
+        tr(1 + op);
+        const uint32_t full = smem_u32(&bars->full[stage]);
+        if constexpr (kFp8) {
+          // the K fill also leaves the K and V scales of the tile's pages in the tile's scale slot,
+          // before the arrive that the readers' wait synchronises with
+          if (op == 0) {
+            float* slot = scale_ring + (n % kScaleSlots) * 16;
+            if (has_box) {
+              slot[lane_page] = x.ks;
+              slot[8 + lane_page] = x.vs;
+            }
+            __syncwarp();
+          }
+        }
+        if (lane == 0) mbar_arrive_expect_tx(full, kFp8 ? kHalfBytes : kTileBytes);
+        __syncwarp();
+        // K/V of streaming tasks is read once: mark it evict-first in L2 so that it does not
+        // push out the K/V that the q tiles of a prefill share through L2 (kept evict-last).
+        if (has_box)
+          tma_load_4d_hint(ring + stage * kTileBytes + box_off, map, full, box_x, 0, x.kv_head, x.page,
+                           x.by_umma ? pol_keep : pol_stream);
       };
       Tile q0 = next_tile(), q1 = next_tile(), q2 = next_tile();
       request_scales(q0);
@@ -665,14 +638,14 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         q1 = q2;
         q2 = next_tile();
         request_scales(q1);
-        fill(0, cur.by_umma, cur.kv_head, cur.kt, cur.bt, cur.npages, cur.page, cur.ks, cur.vs);
-        if (!dead) fill(1, cur.by_umma, cur.kv_head, cur.kt, cur.bt, cur.npages, cur.page, cur.ks, cur.vs);
+        fill(cur);
+        dead = __any_sync(0xffffffffu, dead);
       }
       // No bulk copy of this CTA may still be in flight when it exits: the latest fill of every
       // stage has landed once its `full` phase completes (immediate on the normal path, where the
       // readers have long consumed it; a bounded wait after a failure).
-      for (int s = 0; s < kStages; ++s)
-        if (used & (1u << s)) mbar_wait_block(smem_u32(&bars->full[s]), (fill_par >> s) & 1u, a.status);
+      for (int i = 0; i < kStages / 2; ++i)
+        if (used & (1u << i)) mbar_wait_block(smem_u32(&bars->full[2 * i + op]), (fill_par >> i) & 1u, a.status);
     } else if (kUmma && warp == kConsumerWarps + 1) {
       // ================================ tcgen05 MMA issuer ==============================
       // One warp issues for both 128-row sub-tiles.  Each sub-tile is a chain

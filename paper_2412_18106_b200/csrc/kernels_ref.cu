@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(128) append_kv_kernel(const uint16_t* qkv, int
   const uint16_t* src = qkv + static_cast<int64_t>(t) * qkv_token_stride + static_cast<int64_t>(Hq) * kHeadDim;
   const int chunks = 2 * Hkv * (kHeadDim / 8);  // 16-byte chunks of this token's K then V heads
   // A thread's loads first (they do not wait for the page id), then its stores.
-  constexpr int kBatch = 4;
+  constexpr int kBatch = 2;  // (eight kv heads: two chunks per thread)
   for (int c0 = threadIdx.x; c0 < chunks; c0 += kBatch * blockDim.x) {
     uint4 val[kBatch];
 #pragma unroll
