@@ -4,7 +4,7 @@
 // Task-Table list (Section 3.3.1) or, for balanced plans, the head of one global queue.  Roles:
 //   warps 0..7  consumers: softmax (and, on the warp-level paths, the MMAs), O / LSE output
 //   warps 8, 10 producers: take the next task, look page ids up in the block table and stage 128-key
-//               K (warp 8) and V tiles (warp 10; one TMA box per page and 64-element half) into a
+//               K and V tiles (V: warp 10 with tensor memory; a TMA box per page and 64-element half) into a
 //               ring of four shared-memory stages; they run ahead across task boundaries
 //   warp  9     tcgen05 issuer for both 128-row sub-tiles of a dense task
 // Shared-memory tiles use the 128-byte TMA swizzle: element (row, d) of a tile lives at
@@ -406,6 +406,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   UmmaBarriers* ub = reinterpret_cast<UmmaBarriers*>(gen_base + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers));
   TaskRing* tq = reinterpret_cast<TaskRing*>(gen_base + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers) + 128);
   float* xch = reinterpret_cast<float*>(gen_base + kTileBytes);  // streaming merge area, aliases sub-tile B's Q
+  constexpr bool kTwoProducers = kUmma;
   static_assert(!(kUmma && kFp8), "the fp8 KV path runs on the warp-level MMA paths");
   float* qmult = reinterpret_cast<float*>(gen_base + kSmemQ + kSmemRing + kSmemMl + sizeof(SmemBarriers) + 128 + 256);
   float* scale_ring = qmult + 128;  // [kScaleSlots][16]: K scales [0..7], V scales [8..15] of a tile's pages
@@ -419,7 +420,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
     }
     for (int i = 0; i < kTaskRing; ++i) {
       mbar_init(smem_u32(&tq->full[i]), 1);
-      mbar_init(smem_u32(&tq->empty[i]), kConsumerWarps + (kUmma ? 2 : 1));
+      mbar_init(smem_u32(&tq->empty[i]), kConsumerWarps + (kUmma ? 1 : 0) + (kTwoProducers ? 1 : 0));
     }
     for (int X = 0; X < 2; ++X) {
       mbar_init(smem_u32(&ub->q_full[X]), 4);
@@ -476,20 +477,22 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
 
   if (warp >= kConsumerWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
-    if (warp == kConsumerWarps || warp == kConsumerWarps + 2) {
+    if (warp == kConsumerWarps || (kTwoProducers && warp == kConsumerWarps + 2)) {
       static_assert(kStages == 4, "two stages per producer");
       // ================================ producers ======================================
-      // Warp 8 stages the K tiles (even stages of the ring), warp 10 the V tiles (odd stages); warp 8 also
-      // takes the tasks and hands them to everyone.  Each lane issues the box of one page and half, side
-      // by side.  (One lane that did all of it, K and V, box after box, needed 1600 - 2400 cycles per fill of an
+      // With tensor memory warp 8 stages the K tiles (even stages of the ring) and warp 10 the V tiles (odd
+      // stages), without it warp 8 both; warp 8 also takes the tasks and hands them to everyone.  Each lane
+      // issues the box of one page and half, side by side.  (One lane that did all of it, K and V, box after box, needed 1600 - 2400 cycles per fill of an
       // empty ring, about what a streaming tile takes its SM, and its per-stage state cost the consumers 90 bytes
       // of spills.  One lane / two warps: 2048-token chunk beside 48 decode requests 429 -> 394 us, serving mix of 96
       // requests 4950 -> 4684, 4 prompts of 4096 tokens 1111 -> 1065, 32 verify trees 864 -> 830, two planned steps of
       // a tiny batch 36.9 -> 33.6; a chunk of 512 tokens beside 40 decode requests on pages of 16 tokens 216 ->
-      // 120, of 32 tokens 141 -> 111, on pages of 128 over an fp8 cache 264 -> 256.)
+      // 120, of 32 tokens 141 -> 111.  The variants without tensor memory are bound by their consumers' instructions and
+      // slower with two: there warp 8 does both.  That mix on the bf16 variant, one lane / two warps / one warp, 215 /
+      // 226 / 195 us, over an fp8 cache 264 / 260 / 242, on pages of 16 tokens 458 / 265 / 272.)
       const int op = warp == kConsumerWarps ? 0 : 1;
       bool dead = false;
-      // Of this producer's stages (2 i + op): who read the stage last (bit i set: the tcgen05 path), the parity
+      // Of this producer's stages: who read the stage last (bit set: the tcgen05 path), the parity
       // to wait for on each of its two empty barriers, and of its `full` phase that the latest fill completes;
       // a stage that was never filled needs no wait.
       uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0, fill_par = 0;
@@ -502,7 +505,6 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // bf16: two 64-element boxes per page; e4m3 bytes: one box per page (128 B per key) into the upper half of the stage
       const uint32_t box_off = (kFp8 ? kHalfBytes : (lane & 1) * kHalfBytes) + lane_page * page_bytes;
       const int box_x = kFp8 ? 0 : (lane & 1) * 64;
-      const CUtensorMap* map = op == 0 ? &k_map : &v_map;
       const uint64_t pol_stream = make_l2_policy_evict_first(), pol_keep = make_l2_policy_evict_last();
       // A cursor over the worker's (task, key tile) sequence.  The block-table entries of a tile are
       // requested three tiles before the tile is issued, so their global-memory latency (and the
@@ -581,20 +583,23 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         }
       };
       // Fill this producer's next stage once its previous reader has released it.
-      int n_fill = 0;
-      auto fill = [&](const Tile& x) {
-        const int n = n_fill++;
-        const uint32_t i = n % (kStages / 2), bit = 1u << i, stage = 2 * i + op;
+      int n = 0;  // tiles staged so far
+      auto fill = [&](const Tile& x, int op) {
+        const uint32_t stage = 2 * (n % (kStages / 2)) + op, bit = 1u << stage;
         // Failure-path test hook (xy_attn_debug_inject): this worker leaves out one fill, so the
-        // stage's `full` barrier never completes and the readers' bounded waits run out.
-        if (2 * n + op == a.debug_skip_fill) return;
+        // stage's `full` barrier never completes and the readers' bounded waits run out.  (The pause keeps the
+        // workers in step, so that the same number of fills falls to one of them in every such run.)
+        if (a.debug_skip_fill >= 0) {
+          __nanosleep(1500);
+          if (2 * n + op == a.debug_skip_fill) return;
+        }
         if (used & bit) {
           bool ok;
           if (last_umma & bit) {
-            ok = mbar_wait_block(smem_u32(&bars->empty_umma[stage]), (ph_umma >> i) & 1u, a.status);
+            ok = mbar_wait_block(smem_u32(&bars->empty_umma[stage]), (ph_umma >> stage) & 1u, a.status);
             ph_umma ^= bit;
           } else {
-            ok = mbar_wait_block(smem_u32(&bars->empty[stage]), (ph_cons >> i) & 1u, a.status);
+            ok = mbar_wait_block(smem_u32(&bars->empty[stage]), (ph_cons >> stage) & 1u, a.status);
             ph_cons ^= bit;
           }
           if (!ok) {
@@ -626,7 +631,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         // K/V of streaming tasks is read once: mark it evict-first in L2 so that it does not
         // push out the K/V that the q tiles of a prefill share through L2 (kept evict-last).
         if (has_box)
-          tma_load_4d_hint(ring + stage * kTileBytes + box_off, map, full, box_x, 0, x.kv_head, x.page,
+          tma_load_4d_hint(ring + stage * kTileBytes + box_off, op == 0 ? &k_map : &v_map, full, box_x, 0, x.kv_head, x.page,
                            x.by_umma ? pol_keep : pol_stream);
       };
       Tile q0 = next_tile(), q1 = next_tile(), q2 = next_tile();
@@ -638,14 +643,16 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         q1 = q2;
         q2 = next_tile();
         request_scales(q1);
-        fill(cur);
+        fill(cur, op);
+        if (!kTwoProducers && !dead) fill(cur, 1);
+        ++n;
         dead = __any_sync(0xffffffffu, dead);
       }
       // No bulk copy of this CTA may still be in flight when it exits: the latest fill of every
       // stage has landed once its `full` phase completes (immediate on the normal path, where the
       // readers have long consumed it; a bounded wait after a failure).
-      for (int i = 0; i < kStages / 2; ++i)
-        if (used & (1u << i)) mbar_wait_block(smem_u32(&bars->full[2 * i + op]), (fill_par >> i) & 1u, a.status);
+      for (int s = 0; s < kStages; ++s)
+        if (used & (1u << s)) mbar_wait_block(smem_u32(&bars->full[s]), (fill_par >> s) & 1u, a.status);
     } else if (kUmma && warp == kConsumerWarps + 1) {
       // ================================ tcgen05 MMA issuer ==============================
       // One warp issues for both 128-row sub-tiles.  Each sub-tile is a chain
