@@ -454,15 +454,18 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
 
   const bool dynamic = a.dynamic != 0;
   const int t_begin = dynamic ? 0 : a.worker_off[blockIdx.x], t_end = dynamic ? 0 : a.worker_off[blockIdx.x + 1];
-  // Every role but the producer reads its task sequence here: the worker's own Task-Table list
-  // (static dealing) or the indices the producer publishes (dynamic dealing).  Warp-uniform.
+  // Every role but warp 8 reads its task sequence here: the worker's own Task-Table list (static dealing) or
+  // the indices that warp 8 publishes (dynamic dealing).  Warp-uniform.  All readers follow the sequence to its -1,
+  // after a failure too: the consumers meet at barriers inside a task, and one that left alone would keep the
+  // others waiting there.  So only warp 8 ends a sequence early (publish below), and a reader's wait for it does
+  // not give up with the others.
   int seq_static = t_begin;
   uint32_t n_read = 0;
   bool feed_dead = false;
   auto next_task = [&]() -> int {  // called by all 32 lanes
     if (!dynamic) return seq_static < t_end ? seq_static++ : -1;
     const uint32_t slot = n_read % kTaskRing;
-    if (!feed_dead && !mbar_wait_block(smem_u32(&tq->full[slot]), (n_read / kTaskRing) & 1u, a.status)) {
+    if (!feed_dead && !mbar_wait_handoff(smem_u32(&tq->full[slot]), (n_read / kTaskRing) & 1u)) {
       report_timeout(a);
       feed_dead = true;
     }
@@ -491,7 +494,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // slower with two: there warp 8 does both.  That mix on the bf16 variant, one lane / two warps / one warp, 215 /
       // 226 / 195 us, over an fp8 cache 264 / 260 / 242, on pages of 16 tokens 458 / 265 / 272.)
       const int op = warp == kConsumerWarps ? 0 : 1;
-      bool dead = false;
+      bool dead = false;  // the same in all lanes, as is everything that decides the warp's way
       // Of this producer's stages: who read the stage last (bit set: the tcgen05 path), the parity
       // to wait for on each of its two empty barriers, and of its `full` phase that the latest fill completes;
       // a stage that was never filled needs no wait.
@@ -520,18 +523,10 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       bool f_done = false;
       // Next task of this worker: its own list, or the head of the global queue (published by warp 8 to the
       // other roles through the ring; -1 is published once, when the queue is exhausted).
-      auto grab = [&]() -> int {
-        if (op == 1) return next_task();
-        if (!dynamic) return f_ti < t_end ? f_ti++ : -1;
-        int ti = -1;
-        if (lane == 0) {
-          const int k = static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
-          if (k < a.num_tasks) ti = __ldg(a.queue + k);
-        }
-        ti = __shfl_sync(0xffffffffu, ti, 0);
+      auto publish = [&](int ti) {
         const uint32_t slot = n_pub % kTaskRing;
-        if (n_pub >= kTaskRing &&
-            !mbar_wait_block(smem_u32(&tq->empty[slot]), ((n_pub / kTaskRing) - 1u) & 1u, a.status)) {
+        // (the readers come this far whatever fails: they do not stop before the -1)
+        if (n_pub >= kTaskRing && !mbar_wait_handoff(smem_u32(&tq->empty[slot]), ((n_pub / kTaskRing) - 1u) & 1u)) {
           report_timeout(a);
           dead = true;
         }
@@ -541,6 +536,17 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           mbar_arrive(smem_u32(&tq->full[slot]));
         }
         ++n_pub;
+      };
+      auto grab = [&]() -> int {
+        if (op == 1) return next_task();
+        if (!dynamic) return f_ti < t_end ? f_ti++ : -1;
+        int ti = -1;
+        if (lane == 0) {
+          const int k = static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
+          if (k < a.num_tasks) ti = __ldg(a.queue + k);
+        }
+        ti = __shfl_sync(0xffffffffu, ti, 0);
+        publish(ti);
         return ti;
       };
       const int32_t* f_bt = a.block_table;
@@ -596,18 +602,17 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         if (used & bit) {
           bool ok;
           if (last_umma & bit) {
-            ok = mbar_wait_block(smem_u32(&bars->empty_umma[stage]), (ph_umma >> stage) & 1u, a.status);
+            ok = mbar_wait_warp(smem_u32(&bars->empty_umma[stage]), (ph_umma >> stage) & 1u, a.status);
             ph_umma ^= bit;
           } else {
-            ok = mbar_wait_block(smem_u32(&bars->empty[stage]), (ph_cons >> stage) & 1u, a.status);
+            ok = mbar_wait_warp(smem_u32(&bars->empty[stage]), (ph_cons >> stage) & 1u, a.status);
             ph_cons ^= bit;
           }
           if (!ok) {
             report_timeout(a);
             dead = true;
+            return;
           }
-          dead = __any_sync(0xffffffffu, dead);
-          if (dead) return;
           fill_par ^= bit;
         }
         used |= bit;
@@ -646,7 +651,10 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         fill(cur, op);
         if (!kTwoProducers && !dead) fill(cur, 1);
         ++n;
-        dead = __any_sync(0xffffffffu, dead);
+      }
+      if (dynamic && !f_done) {  // after a failure: the others' sequence ends too, and is read to its end
+        if (op == 0) publish(-1);
+        else while (next_task() >= 0) {}
       }
       // No bulk copy of this CTA may still be in flight when it exits: the latest fill of every
       // stage has landed once its `full` phase completes (immediate on the normal path, where the

@@ -117,7 +117,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
 
   if (warp == kWarpsS) {
     // ================================== producer ==========================================
-    bool dead = false;
+    bool dead = false;  // the same in all lanes, as is everything that decides the warp's way
     if ((ring & 1023u) != 0) {  // the TMA swizzle needs it; dynamic shared memory starts there
       report_timeout(a, s_failed);
       dead = true;
@@ -192,7 +192,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     // Hands a task (or, with last, the end) to the consumers: description and Q rows.  The previous
     // task's are in its consumers' registers by then (task_free).
     auto publish = [&](bool last) {
-      if (n_tasks > 0 && !mbar_wait_block(task_free, (n_tasks - 1) & 1u, a.status)) {
+      if (n_tasks > 0 && !mbar_wait_warp(task_free, (n_tasks - 1) & 1u, a.status)) {
         report_timeout(a, s_failed);
         dead = true;
         return;
@@ -227,7 +227,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       const uint32_t bit = 1u << pos.stage;
       if (used & bit) {
         // wait for the readers of this stage's previous fill
-        if (!mbar_wait_block(empty + 8 * pos.stage, (fill_par >> pos.stage) & 1u, a.status)) {
+        if (!mbar_wait_warp(empty + 8 * pos.stage, (fill_par >> pos.stage) & 1u, a.status)) {
           report_timeout(a, s_failed);
           dead = true;
           return;
@@ -266,7 +266,6 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       request_scales(q1);
       if (!dead) fill(&k_map, cur, true);
       if (!dead) fill(&v_map, cur, false);
-      dead = __any_sync(0xffffffffu, dead);
     }
     if (!dead) publish(true);
     // No copy of this CTA may still be in flight when it exits (immediate on the normal path).

@@ -64,6 +64,20 @@ __device__ __forceinline__ bool mbar_wait_block(uint32_t bar, uint32_t parity, c
   return false;
 }
 
+// The same for a whole warp whose lanes go on to votes and warp barriers: all of them leave with one answer.
+// (Each lane decides on its own polls; one may find the barrier complete when its neighbour has just given up.)
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const volatile int32_t* status) {
+  return __all_sync(0xffffffffu, mbar_wait_block(bar, parity, status));
+}
+
+// A wait, by a whole warp, for a hand-off that a role of the same CTA makes in any case, also once a run has failed:
+// four times the limit of that role's own waits, and no look at the status word, so that all who wait for it see it.
+__device__ __forceinline__ bool mbar_wait_handoff(uint32_t bar, uint32_t parity) {
+  bool ok = false;
+  for (uint32_t i = 0; i < (1u << 24) && !ok; ++i) ok = mbar_try_wait(bar, parity);
+  return __all_sync(0xffffffffu, ok);
+}
+
 // One lane of the (converged) warp, the same one on every call.
 __device__ __forceinline__ bool elect_one() {
   uint32_t ok;
