@@ -457,7 +457,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   // Every role but warp 8 reads its task sequence here: the worker's own Task-Table list (static dealing) or
   // the indices that warp 8 publishes (dynamic dealing).  Warp-uniform.  All readers follow the sequence to its -1,
   // after a failure too: the consumers meet at barriers inside a task, and one that left alone would keep the
-  // others waiting there.  So only warp 8 ends a sequence early (publish below), and a reader's wait for it does
+  // others waiting there.  So only warp 8 ends a sequence early (grab below), and a reader's wait for it does
   // not give up with the others.
   int seq_static = t_begin;
   uint32_t n_read = 0;
@@ -495,10 +495,10 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // 226 / 195 us, over an fp8 cache 264 / 260 / 242, on pages of 16 tokens 458 / 265 / 272.)
       const int op = warp == kConsumerWarps ? 0 : 1;
       bool dead = false;  // the same in all lanes, as is everything that decides the warp's way
-      // Of this producer's stages: who read the stage last (bit set: the tcgen05 path), the parity
-      // to wait for on each of its two empty barriers, and of its `full` phase that the latest fill completes;
-      // a stage that was never filled needs no wait.
-      uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0, fill_par = 0;
+      // Of this producer's stages: whether the stage has been handed out, who read it last (bit set: the tcgen05
+      // path), the parity to wait for on each of its two empty barriers; whether a copy has been issued into it, and
+      // the parity of its `full` phase that the latest one completes.
+      uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0, armed = 0, fill_par = 0;
       Tracer tr;
       tr.init(a, 3, op == 0 && lane == 0);
       const int ppt = kKeyTile >> a.page_shift;  // pages per 128-key tile
@@ -523,7 +523,15 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       bool f_done = false;
       // Next task of this worker: its own list, or the head of the global queue (published by warp 8 to the
       // other roles through the ring; -1 is published once, when the queue is exhausted).
-      auto publish = [&](int ti) {
+      auto grab = [&]() -> int {
+        if (op == 1) return next_task();
+        if (!dynamic) return f_ti < t_end ? f_ti++ : -1;
+        int ti = -1;
+        if (lane == 0 && !dead) {
+          const int k = static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
+          if (k < a.num_tasks) ti = __ldg(a.queue + k);
+        }
+        ti = __shfl_sync(0xffffffffu, ti, 0);
         const uint32_t slot = n_pub % kTaskRing;
         // (the readers come this far whatever fails: they do not stop before the -1)
         if (n_pub >= kTaskRing && !mbar_wait_handoff(smem_u32(&tq->empty[slot]), ((n_pub / kTaskRing) - 1u) & 1u)) {
@@ -536,17 +544,6 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           mbar_arrive(smem_u32(&tq->full[slot]));
         }
         ++n_pub;
-      };
-      auto grab = [&]() -> int {
-        if (op == 1) return next_task();
-        if (!dynamic) return f_ti < t_end ? f_ti++ : -1;
-        int ti = -1;
-        if (lane == 0) {
-          const int k = static_cast<int>(atomicInc(reinterpret_cast<unsigned*>(a.queue_head), a.queue_wrap));
-          if (k < a.num_tasks) ti = __ldg(a.queue + k);
-        }
-        ti = __shfl_sync(0xffffffffu, ti, 0);
-        publish(ti);
         return ti;
       };
       const int32_t* f_bt = a.block_table;
@@ -592,13 +589,6 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       int n = 0;  // tiles staged so far
       auto fill = [&](const Tile& x, int op) {
         const uint32_t stage = 2 * (n % (kStages / 2)) + op, bit = 1u << stage;
-        // Failure-path test hook (xy_attn_debug_inject): this worker leaves out one fill, so the
-        // stage's `full` barrier never completes and the readers' bounded waits run out.  (The pause keeps the
-        // workers in step, so that the same number of fills falls to one of them in every such run.)
-        if (a.debug_skip_fill >= 0) {
-          __nanosleep(1500);
-          if (2 * n + op == a.debug_skip_fill) return;
-        }
         if (used & bit) {
           bool ok;
           if (last_umma & bit) {
@@ -613,10 +603,14 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
             dead = true;
             return;
           }
-          fill_par ^= bit;
         }
         used |= bit;
         last_umma = x.by_umma ? (last_umma | bit) : (last_umma & ~bit);
+        // Failure-path test hook (xy_attn_debug_inject): this worker leaves out one copy, so that the stage's `full`
+        // barrier does not complete and the readers' bounded waits run out.
+        if (2 * n + op == a.debug_skip_fill) return;
+        if (armed & bit) fill_par ^= bit;
+        armed |= bit;
         tr(1 + op);
         const uint32_t full = smem_u32(&bars->full[stage]);
         if constexpr (kFp8) {
@@ -642,25 +636,21 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       Tile q0 = next_tile(), q1 = next_tile(), q2 = next_tile();
       request_scales(q0);
       request_scales(q1);
-      while (q0.valid && !dead) {
+      while (q0.valid) {  // (after a failure without copies: the sequence of tasks is ended, or read to its end)
         const Tile cur = q0;
         q0 = q1;
         q1 = q2;
         q2 = next_tile();
         request_scales(q1);
-        fill(cur, op);
+        if (!dead) fill(cur, op);
         if (!kTwoProducers && !dead) fill(cur, 1);
         ++n;
-      }
-      if (dynamic && !f_done) {  // after a failure: the others' sequence ends too, and is read to its end
-        if (op == 0) publish(-1);
-        else while (next_task() >= 0) {}
       }
       // No bulk copy of this CTA may still be in flight when it exits: the latest fill of every
       // stage has landed once its `full` phase completes (immediate on the normal path, where the
       // readers have long consumed it; a bounded wait after a failure).
       for (int s = 0; s < kStages; ++s)
-        if (used & (1u << s)) mbar_wait_block(smem_u32(&bars->full[s]), (fill_par >> s) & 1u, a.status);
+        if (armed & (1u << s)) mbar_wait_block(smem_u32(&bars->full[s]), (fill_par >> s) & 1u, a.status);
     } else if (kUmma && warp == kConsumerWarps + 1) {
       // ================================ tcgen05 MMA issuer ==============================
       // One warp issues for both 128-row sub-tiles.  Each sub-tile is a chain
@@ -695,8 +685,8 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
       constexpr uint64_t kDescHi64 = static_cast<uint64_t>(kDescHi) << 32;
       const uint32_t ring_lo = (ring >> 4) & 0x3FFFu, q_lo = (q_smem >> 4) & 0x3FFFu;
-      auto commit = [&](uint64_t* bar) {
-        if (elected) umma_commit(smem_u32(bar));
+      auto commit = [&](uint64_t* bar) {  // (after a timeout nothing is handed on: those who wait give up too)
+        if (elected && !dead) umma_commit(smem_u32(bar));
       };
       // S_X = Q_X K^T: 8 k-steps of 16 elements, 32 B apart, the second half 16 KiB away
       auto issue_qk = [&](int X, uint32_t p) {
@@ -777,7 +767,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // Tensor memory is freed after the final barrier: no MMA of this thread may still be in
       // flight then.  On the normal path they completed long ago (immediate); after a failure
       // this is a bounded wait.
-      commit(&ub->drained);
+      if (elected) umma_commit(smem_u32(&ub->drained));
       mbar_wait_block(smem_u32(&ub->drained), 0u, a.status);
     }
   } else {
@@ -1154,7 +1144,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           if (work) w.qk(ring + pipe.stage * kTileBytes, 0, lane, s);
           if constexpr (kFp8) fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
+          if (lane == 0 && !dead) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
           pipe.advance<kStages>();
           if (work) {
             const bool need_mask = tree ? (col0 + kKeyTile > h) : (col0 + kKeyTile > h + i_min + 1);
@@ -1171,7 +1161,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           if (work) w.pv(ring + pipe.stage * kTileBytes, 0, lane, p);
           if constexpr (kFp8) fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
+          if (lane == 0 && !dead) mbar_arrive(smem_u32(&bars->empty[pipe.stage]));
           pipe.advance<kStages>();
         }
         if (active) {

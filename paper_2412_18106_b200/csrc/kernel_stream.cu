@@ -117,7 +117,9 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
 
   if (warp == kWarpsS) {
     // ================================== producer ==========================================
-    bool dead = false;  // the same in all lanes, as is everything that decides the warp's way
+    // `dead` is the same in all lanes, as is everything that decides the warp's way; a lane whose wait for a stage has
+    // run out goes on without copies until the vote behind the tile.
+    bool dead = false, failed = false;
     if ((ring & 1023u) != 0) {  // the TMA swizzle needs it; dynamic shared memory starts there
       report_timeout(a, s_failed);
       dead = true;
@@ -218,23 +220,25 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     };
     RingPos pos{0, 0};
     int n_fill = 0;
-    uint32_t k_fills = 0, used = 0, fill_par = 0;
+    // per stage: handed out, parity of its next `empty` wait, copied into, parity of the latest copy's `full` phase
+    uint32_t k_fills = 0, used = 0, ph_empty = 0, armed = 0, fill_par = 0;
     auto fill = [&](const CUtensorMap* map, const Tile& x, bool is_k) {
-      if (n_fill++ == a.debug_skip_fill) {  // failure-path test hook: this stage is never filled
-        pos.advance<kStages>();
-        return;
-      }
       const uint32_t bit = 1u << pos.stage;
       if (used & bit) {
         // wait for the readers of this stage's previous fill
-        if (!mbar_wait_warp(empty + 8 * pos.stage, (fill_par >> pos.stage) & 1u, a.status)) {
+        if (!failed && !mbar_wait_block(empty + 8 * pos.stage, (ph_empty >> pos.stage) & 1u, a.status)) {
           report_timeout(a, s_failed);
-          dead = true;
-          return;
+          failed = true;
         }
-        fill_par ^= bit;
+        ph_empty ^= bit;
       }
       used |= bit;
+      if (n_fill++ == a.debug_skip_fill) {  // failure-path test hook: this copy is left out
+        pos.advance<kStages>();
+        return;
+      }
+      if (armed & bit) fill_par ^= bit;
+      armed |= bit;
       if constexpr (kFp8) {
         if (is_k) {
           float* slot = scale_ring + (k_fills % kScaleSlots) * 16;
@@ -247,9 +251,9 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
         }
       }
       const uint32_t bar = full + 8 * pos.stage;
-      if (lane == 0) mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
+      if (lane == 0 && !failed) mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
       __syncwarp();
-      if (has_box)
+      if (has_box && !failed)
         tma_load_4d_hint(ring + pos.stage * Cfg::kStageBytes + box_off, map, bar, kFp8 ? 0 : (lane & 1) * 64, 0, x.kv_head,
                          x.page, policy);
       pos.advance<kStages>();
@@ -264,14 +268,17 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       q1 = q2;
       q2 = next_tile();
       request_scales(q1);
-      if (!dead) fill(&k_map, cur, true);
-      if (!dead) fill(&v_map, cur, false);
+      if (!dead) {
+        fill(&k_map, cur, true);
+        fill(&v_map, cur, false);
+        dead = __any_sync(0xffffffffu, failed);
+      }
     }
     if (!dead) publish(true);
     // No copy of this CTA may still be in flight when it exits (immediate on the normal path).
     asm volatile("cp.async.wait_all;" ::: "memory");
     for (int s = 0; s < kStages; ++s)
-      if (used & (1u << s)) mbar_wait_block(full + 8 * s, (fill_par >> s) & 1u, a.status);
+      if (armed & (1u << s)) mbar_wait_block(full + 8 * s, (fill_par >> s) & 1u, a.status);
   } else {
     // ================================== consumers =========================================
     const float scale_log2 = a.sm_scale * 1.4426950408889634f;

@@ -490,9 +490,10 @@ __device__ __forceinline__ void stream_task(const RunArgs& a, const TaskView& tv
       dead = true;
     }
   };
+  // (a warp that has given up hands no stage back: its copy may be on the way still, and a stage is not armed twice)
   auto release = [&]() {
     __syncwarp();
-    if (lane == 0) mbar_arrive(ring.empty + 8u * pos.stage);
+    if (lane == 0 && !dead) mbar_arrive(ring.empty + 8u * pos.stage);
     pos.advance<kStages>();
   };
   // Tiles that every row of the task sees in full need neither the mask nor the test whether the

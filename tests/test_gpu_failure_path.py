@@ -170,7 +170,9 @@ def test_two_launches_side_by_side_give_up_and_leave_a_clean_context(skip, worke
     ctx.close()
 
 
-@pytest.mark.parametrize("decode,workers", [(True, 3), (True, 0), (False, 5)], ids=["stream-3", "stream-all", "meta-5"])
+# (The tiny batch has 32 fills: with two workers one of them comes to its twelfth however the tasks fall; with five
+# that would depend on their pace.)
+@pytest.mark.parametrize("decode,workers", [(True, 3), (True, 0), (False, 2)], ids=["stream-3", "stream-all", "meta-2"])
 @pytest.mark.parametrize("skip", [1, 11])
 def test_fp8_run_gives_up_and_the_context_recovers(decode, workers, skip):
     b = W.config2_decode(num_requests=9, kv_lo=300, kv_hi=3000) if decode else W.config1_tiny()
@@ -198,4 +200,56 @@ def test_fp8_run_gives_up_and_the_context_recovers(decode, workers, skip):
         for _ in range(2):
             o, lse = run()
             assert torch.equal(o, good[0]) and torch.equal(lse, good[1])
+    ctx.close()
+
+
+# Batches for one worker, which comes to every fill: a long streaming task beside a chunk, a long dense task beside a
+# short one, and many tasks of one to four tiles.
+AHEAD = {
+    "stream": [(500, 0, 0, None), (1, 6000, 0, None)],
+    "dense": [(64, 5000, 0, None), (1, 90, 0, None)],
+    "short": [(500, 0, 0, None)] + [(1, 20 + 2 * i, 0, None) for i in range(14)],
+}
+
+
+@pytest.mark.parametrize("fp8,kernel", [(False, xb.XY_KERNEL_AUTO), (False, xb.XY_KERNEL_MMA), (True, xb.XY_KERNEL_AUTO)],
+                         ids=["auto", "mma", "fp8"])
+@pytest.mark.parametrize("batch", sorted(AHEAD))
+@pytest.mark.parametrize("skip", [24, 25, 38, 39])
+def test_one_tile_missing_while_the_producers_are_ahead(batch, skip, fp8, kernel):
+    """A K tile (even) or a V tile (odd) is left out deep in a run: the other kind's stages are full, their producer
+    waits for its readers or has tasks in hand that nobody has read, and copies are in flight.  The run ends, every
+    role and warp of it, and the runs behind it are bitwise those before it."""
+    b = W.custom("ahead_" + batch, 8, 2, 64, AHEAD[batch], seed=21)
+    kw = dict(num_workers=1, kernel=kernel)
+    if fp8:
+        kw["kv_dtype"] = xb.XY_KV_FP8_E4M3
+    ctx = H.make_ctx(b, **kw)
+    info = ctx.plan_batch(b)
+    tasks = ctx.get_tasks()
+    assert info.num_dense_tasks > 0 and 2 * int((tasks["kt_hi"] - tasks["kt_lo"]).sum()) > skip
+    t = W.make_tensors(b)
+    t = W.to_fp8_kv(t) if fp8 else t
+    q, k, v = t.q.cuda(), t.k_pool.cuda(), t.v_pool.cuda()
+    scales = (t.k_scale.cuda(), t.v_scale.cuda()) if fp8 else ()
+    bt = torch.from_numpy(np.where(b.block_table < 0, 0, b.block_table).astype(np.int32)).cuda()
+
+    def run():
+        o = torch.full((b.total_q, b.num_q_heads, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((b.total_q, b.num_q_heads), float("nan"), dtype=torch.float32, device="cuda")
+        (ctx.run_fp8kv if fp8 else ctx.run)(q, k, v, *scales, bt, H.SCALE, o, lse)
+        return o, lse
+
+    good = run()
+    assert ctx.last_launches() == 1  # both kinds of task by the meta-kernel
+    ref = oracle.attention_fp8(b, t, H.SCALE) if fp8 else oracle.attention(b, t, H.SCALE)
+    H.check_against_oracle(good[0].float().cpu().numpy().astype(np.float64), good[1].cpu().numpy().astype(np.float64),
+                           *ref, batch)
+    for limit in (20000, 1):
+        ctx.debug_inject(wait_limit_polls=limit, skip_fill=skip)
+        run()
+        ctx.debug_inject(0, -1)
+        assert ctx.device_status() == xb.XY_ERR_DEVICE_TIMEOUT and ctx.device_status() == 0
+        o, lse = run()
+        assert ctx.device_status() == 0 and torch.equal(o, good[0]) and torch.equal(lse, good[1])
     ctx.close()
