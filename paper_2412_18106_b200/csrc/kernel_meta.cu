@@ -443,6 +443,9 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // (What a kernel before may have written, block table, scales, masks, Q, is read by ordinary loads behind this wait.
+  // __ldg is for the plan's tables alone: it asks for data that nobody writes while this kernel lives, and may be
+  // moved across the wait.)
   grid_dependency_wait();
   if (a.side_by_side) grid_launch_dependents();  // every launch before this one is complete: the second may run
   if (threadIdx.x == 0) {
@@ -570,7 +573,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         x.valid = true;
         x.kv_head = f_head;
         x.by_umma = f_umma;
-        if (has_box) x.page = __ldg(f_bt + min(f_kt * ppt + lane_page, f_npages - 1));  // past the end: the last page again
+        if (has_box) x.page = f_bt[min(f_kt * ppt + lane_page, f_npages - 1)];  // past the end: the last page again
         ++f_kt;
         return x;
       };
@@ -580,8 +583,8 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         if constexpr (kFp8) {
           if (op == 0 && x.valid && has_box) {
             const int64_t si = static_cast<int64_t>(x.page) * a.num_kv_heads + x.kv_head;
-            x.ks = __ldg(a.k_scale + si);
-            x.vs = __ldg(a.v_scale + si);
+            x.ks = a.k_scale[si];
+            x.vs = a.v_scale[si];
           }
         }
       };
@@ -907,9 +910,9 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
               const int wbase = max(jp0, 0) >> 6;
               const uint64_t* mrow = a.tree_mask + tv.rq.tree_off + static_cast<int64_t>(i_row) * tv.rq.tree_words;
               uint64_t w0 = 0ull, w1 = 0ull, w2 = 0ull;
-              if (wbase < tv.rq.tree_words) w0 = __ldg(mrow + wbase);
-              if (wbase + 1 < tv.rq.tree_words) w1 = __ldg(mrow + wbase + 1);
-              if (wbase + 2 < tv.rq.tree_words) w2 = __ldg(mrow + wbase + 2);
+              if (wbase < tv.rq.tree_words) w0 = mrow[wbase];
+              if (wbase + 1 < tv.rq.tree_words) w1 = mrow[wbase + 1];
+              if (wbase + 2 < tv.rq.tree_words) w2 = mrow[wbase + 2];
               uint64_t t_lo, t_hi;
               if (jp0 >= 0) {
                 const int sh = jp0 & 63;

@@ -109,7 +109,9 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     }
     __syncwarp();
   }
-  // (beside the dense launch: its CTAs have let this one in only after their own wait)
+  // (Beside the dense launch: its CTAs have let this one in only after their own wait.)  What a kernel before may have
+  // written is read by ordinary loads from here on; __ldg, which may be moved across the wait, reads the plan's
+  // tables alone.
   if (!a.side_by_side) grid_dependency_wait();
   unsigned long long t_start = 0;
   if (threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
@@ -177,7 +179,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       x.valid = true;
       x.kv_head = d.t.kv_head;
       x.kt = kt;
-      if (has_box) x.page = __ldg(bt + min(kt * ppt + lane_page, npages - 1));  // past the end: the last page again
+      if (has_box) x.page = bt[min(kt * ppt + lane_page, npages - 1)];  // past the end: the last page again
       ++kt;
       return x;
     };
@@ -185,8 +187,8 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
       if constexpr (kFp8) {
         if (x.valid && has_box) {
           const int64_t si = static_cast<int64_t>(x.page) * a.num_kv_heads + x.kv_head;
-          x.ks = __ldg(a.k_scale + si);
-          x.vs = __ldg(a.v_scale + si);
+          x.ks = a.k_scale[si];
+          x.vs = a.v_scale[si];
         }
       }
     };

@@ -92,7 +92,7 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Reads a word past L1; unlike __ldg it may be repeated later for a newer value.
+// Reads a word past L1, in place: a word that another kernel may be writing, to be read again behind the wait.
 __device__ __forceinline__ int32_t ld_l2(const int32_t* p) {
   int32_t v;
   asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");

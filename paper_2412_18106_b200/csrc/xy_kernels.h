@@ -7,8 +7,10 @@
 
 namespace xy {
 
-// Launches a kernel that calls grid_dependency_wait before it touches anything that a kernel before it
-// wrote, or writes global memory itself.
+// Launches a kernel that calls grid_dependency_wait before it uses anything that a kernel before it wrote, or writes
+// global memory itself.  (Before the wait the streaming kernel looks at the block table and the GEMM at its weights
+// for L2 prefetches alone, whose outcome is the same whatever they find; tables of a plan may be read, they come
+// over by a copy, which a launch is ordered behind in full.)
 template <class... P, class... A>
 inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg = {};
