@@ -92,6 +92,12 @@ void free_device(xy_attn_ctx* c) {
   cudaFree(c->d_worker_times);
 }
 
+// Whether the streaming kernel runs this plan or, in a plan for two launches, its streaming part.
+bool streaming_launch(const xy_attn_ctx* c) {
+  if (c->cfg.kernel != XY_KERNEL_AUTO || c->cfg.plan_mode != XY_PLAN_BALANCED) return false;
+  return c->plan.info.num_dense_tasks == 0 || (c->plan.queue_dense >= 0 && c->cfg.kv_dtype == XY_KV_BF16);
+}
+
 }  // namespace
 
 extern "C" {
@@ -251,10 +257,10 @@ int xy_attn_plan_shared(xy_attn_ctx* ctx, const xy_attn_request* reqs, int32_t n
     const size_t reqs_at = put(p.reqs), tree_at = put(p.tree_mask);
     // What the CTAs of a streaming launch start with: one read instead of a chain of three.
     const int32_t first_at = std::max(p.queue_dense, 0);
-    const int32_t n_first = p.queue_dense >= 0 || p.info.num_dense_tasks == 0
+    const int32_t n_first = streaming_launch(ctx)
                                 ? std::min<int32_t>(static_cast<int32_t>(p.queue.size()) - first_at, 2 * ctx->num_workers) : 0;
     const size_t desc_at = (st.size() + 15) & ~size_t{15};
-    st.resize(desc_at + std::max(n_first, 0) * sizeof(TaskDesc));
+    st.resize(desc_at + n_first * sizeof(TaskDesc));
     for (int32_t k = 0; k < n_first; ++k) {
       const int32_t ti = p.queue[first_at + k];
       TaskDesc d{};
@@ -474,7 +480,7 @@ int run_impl(xy_attn_ctx* ctx, const void* q, int64_t q_token_stride, const void
       ctx->last_ctas = beside ? ctx->last_ctas + ctx->launch_cache.ctas : std::max(ctx->last_ctas, ctx->launch_cache.ctas);
     }
     ctx->last_launches -= 1;  // counted once more below
-  } else if (cfg.kernel == XY_KERNEL_AUTO && a.dynamic && p.info.num_dense_tasks == 0) {
+  } else if (streaming_launch(ctx)) {
     // Only streaming tasks: the kernel with two small CTAs per SM (faster from one request to a
     // saturated decode batch, figures in kernel_stream.cu).  With dense tasks in the batch the
     // meta-kernel runs both kinds side by side.
