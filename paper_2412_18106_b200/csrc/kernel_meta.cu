@@ -592,6 +592,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       int n = 0;  // tiles staged so far
       auto fill = [&](const Tile& x, int op) {
         const uint32_t stage = 2 * (n % (kStages / 2)) + op, bit = 1u << stage;
+        const uint32_t full = smem_u32(&bars->full[stage]);
         if (used & bit) {
           bool ok;
           if (last_umma & bit) {
@@ -615,7 +616,6 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
         if (armed & bit) fill_par ^= bit;
         armed |= bit;
         tr(1 + op);
-        const uint32_t full = smem_u32(&bars->full[stage]);
         if constexpr (kFp8) {
           // the K fill also leaves the K and V scales of the tile's pages in the tile's scale slot,
           // before the arrive that the readers' wait synchronises with
@@ -667,20 +667,17 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // at the power cap.)
       const bool elected = elect_one();
       uint32_t pos = 0;  // ring position: stage = pos % kStages, parity = (pos / kStages) & 1
-      bool dead = false;
       uint32_t ph_q = 0, ph_p = 0;  // bit X: parity of sub-tile X's next wait
       Tracer tr;
       tr.init(a, 2, elected);
-      auto wait_or_die = [&](uint32_t bar, uint32_t parity) {
-        if (!dead && !mbar_wait_block(bar, parity, a.status)) {
-          report_timeout(a);
-          dead = true;
-        }
-      };
-      auto wait_full = [&](uint32_t p) {
-        wait_or_die(smem_u32(&bars->full[p % kStages]), (p / kStages) & 1u);
+      // Once a wait has run out nothing more is issued or handed on (a stage's copy may be on the way still, and
+      // its producer must not arm it twice): the tasks that are left are only read.
+      auto wait = [&](uint32_t bar, uint32_t parity) {
+        const bool ok = mbar_wait_warp(bar, parity, a.status);
         tc_fence_after();
+        return ok;
       };
+      auto wait_full = [&](uint32_t p) { return wait(smem_u32(&bars->full[p % kStages]), (p / kStages) & 1u); };
       // Descriptor halves.  High word (same for every operand here): 8-row groups 1024 B apart,
       // sm_100 descriptor version, 128-byte swizzle.  Low word: start address >> 4 in bits 0-13,
       // leading byte offset >> 4 in bits 16-29 (16 B for the K-major Q / K tiles; 16 KiB, the
@@ -688,14 +685,14 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
       constexpr uint64_t kDescHi64 = static_cast<uint64_t>(kDescHi) << 32;
       const uint32_t ring_lo = (ring >> 4) & 0x3FFFu, q_lo = (q_smem >> 4) & 0x3FFFu;
-      auto commit = [&](uint64_t* bar) {  // (after a timeout nothing is handed on: those who wait give up too)
-        if (elected && !dead) umma_commit(smem_u32(bar));
+      auto commit = [&](uint64_t* bar) {
+        if (elected) umma_commit(smem_u32(bar));
       };
       // S_X = Q_X K^T: 8 k-steps of 16 elements, 32 B apart, the second half 16 KiB away
       auto issue_qk = [&](int X, uint32_t p) {
         const uint32_t k0 = (ring_lo + (p % kStages) * (kTileBytes >> 4)) | (1u << 16);
         const uint32_t q0 = (q_lo + X * (kTileBytes >> 4)) | (1u << 16);
-        if (elected && !dead) {
+        if (elected) {
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks) {
             const uint32_t off = (ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2;
@@ -709,7 +706,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // keys, 2 KiB apart.
       auto issue_pv = [&](int X, uint32_t p, int half, bool accumulate) {
         const uint32_t v0 = (ring_lo + (p % kStages) * (kTileBytes >> 4)) | ((kHalfBytes >> 4) << 16);
-        if (elected && !dead) {
+        if (elected) {
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const int ks = half * 4 + k;
@@ -718,7 +715,8 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           }
         }
       };
-      for (int ti = next_task(); ti >= 0; ti = next_task()) {
+      int ti = next_task();
+      for (; ti >= 0; ti = next_task()) {
         const xy_attn_task t = a.tasks[ti];
         const uint32_t n_all = t.kt_hi - t.kt_lo;
         const uint32_t pos0 = pos;
@@ -734,27 +732,25 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           // q_full first: streaming tasks are skipped without a look at the ring, so this warp may be
           // several fills of a stage ahead, where the parity of `full` says nothing.  Q is there once
           // the consumers are through with every earlier task, that is, with every earlier fill.
-          wait_or_die(smem_u32(&ub->q_full[X]), (ph_q >> X) & 1u);
+          if (!wait(smem_u32(&ub->q_full[X]), (ph_q >> X) & 1u)) goto given_up;
           ph_q ^= 1u << X;
-          wait_full(pos0);
+          if (!wait_full(pos0)) goto given_up;
           issue_qk(X, pos0);
         }
         commit(&bars->empty_umma[pos0 % kStages]);
         for (int j = 0; j < n_max; ++j) {
           const uint32_t pv = pos0 + 2 * j + 1, pk = pv + 1;
-          wait_full(pv);
+          if (!wait_full(pv)) goto given_up;
 #pragma unroll
           for (int X = 0; X < 2; ++X) {
             if (j >= ds.n[X]) continue;
             const bool more = j + 1 < ds.n[X];
-            wait_or_die(smem_u32(&ub->p_full[X][0]), (ph_p >> X) & 1u);
-            tc_fence_after();
+            if (!wait(smem_u32(&ub->p_full[X][0]), (ph_p >> X) & 1u)) goto given_up;
             tr(12);
             issue_pv(X, pv, 0, j > 0);
-            if (more) wait_full(pk);
-            wait_or_die(smem_u32(&ub->p_full[X][1]), (ph_p >> X) & 1u);  // second half of P
+            if (more && !wait_full(pk)) goto given_up;
+            if (!wait(smem_u32(&ub->p_full[X][1]), (ph_p >> X) & 1u)) goto given_up;  // second half of P
             ph_p ^= 1u << X;
-            tc_fence_after();
             issue_pv(X, pv, 1, true);
             if (!more) commit(&ub->o_done[X]);
             // the stage goes back to the producer behind its last reader
@@ -767,10 +763,13 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
           }
         }
       }
+    given_up:
+      if (ti >= 0) report_timeout(a);
+      while (ti >= 0) ti = next_task();
       // Tensor memory is freed after the final barrier: no MMA of this thread may still be in
       // flight then.  On the normal path they completed long ago (immediate); after a failure
       // this is a bounded wait.
-      if (elected) umma_commit(smem_u32(&ub->drained));
+      commit(&ub->drained);
       mbar_wait_block(smem_u32(&ub->drained), 0u, a.status);
     }
   } else {
@@ -910,9 +909,9 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
               const int wbase = max(jp0, 0) >> 6;
               const uint64_t* mrow = a.tree_mask + tv.rq.tree_off + static_cast<int64_t>(i_row) * tv.rq.tree_words;
               uint64_t w0 = 0ull, w1 = 0ull, w2 = 0ull;
-              if (wbase < tv.rq.tree_words) w0 = mrow[wbase];
-              if (wbase + 1 < tv.rq.tree_words) w1 = mrow[wbase + 1];
-              if (wbase + 2 < tv.rq.tree_words) w2 = mrow[wbase + 2];
+              if (wbase < tv.rq.tree_words) w0 = ld_u64(mrow + wbase);
+              if (wbase + 1 < tv.rq.tree_words) w1 = ld_u64(mrow + wbase + 1);
+              if (wbase + 2 < tv.rq.tree_words) w2 = ld_u64(mrow + wbase + 2);
               uint64_t t_lo, t_hi;
               if (jp0 >= 0) {
                 const int sh = jp0 & 63;

@@ -99,6 +99,14 @@ __device__ __forceinline__ int32_t ld_l2(const int32_t* p) {
   return v;
 }
 
+// An ordinary load that the compiler may merge and move as it may __ldg's: for words that a kernel before has written,
+// at addresses that were themselves read behind the dependency wait.
+__device__ __forceinline__ uint64_t ld_u64(const uint64_t* p) {
+  uint64_t v;
+  asm("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
+  return v;
+}
+
 // ---------------------------------------------------------------- proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

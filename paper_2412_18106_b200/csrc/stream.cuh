@@ -42,7 +42,7 @@ __device__ __forceinline__ bool visible(const RunArgs& a, const ReqInfo& rq, int
   if (col > rq.kv_len + i) return false;  // causal frontier; also excludes everything >= L
   if (col < rq.kv_len || rq.mask_kind == XY_MASK_CAUSAL) return true;
   const int jp = col - rq.kv_len;
-  const uint64_t w = a.tree_mask[rq.tree_off + static_cast<int64_t>(i) * rq.tree_words + (jp >> 6)];
+  const uint64_t w = ld_u64(a.tree_mask + rq.tree_off + static_cast<int64_t>(i) * rq.tree_words + (jp >> 6));
   return (w >> (jp & 63)) & 1ull;
 }
 
