@@ -353,8 +353,9 @@ int xy_attn_worker_times(xy_attn_ctx* ctx, uint64_t* out, int32_t cap);
 /* Debug tracing (only in a library built with -DXY_ENABLE_TRACE, i.e. XY_BUILD_TRACE=1 for
  * paper_2412_18106_b200.build; otherwise no records are written and 0 entries are meaningful).
  * When the environment variable XY_ATTN_TRACE=1 is set at create time, the
- * roles of worker 0 (sub-tile A, sub-tile B, MMA issuer, producer) stamp (tag << 48 | SM cycle
- * counter) records into a context-owned buffer of 4 x 2048 entries per run.  This call
+ * roles of worker 0 (sub-tile A, sub-tile B, MMA issuer, producers) stamp (tag << 48 | SM cycle
+ * counter) records into a context-owned buffer of 4 x 2048 entries per run (where K and V have a
+ * producer each, the first half of the producers' entries is K's, the second V's).  This call
  * synchronises the device and copies them to `out` (HOST); it returns the number of entries
  * (0 when tracing is off) and copies only if `cap` is large enough. */
 int xy_attn_debug_trace(xy_attn_ctx* ctx, uint64_t* out, int32_t cap);

@@ -323,16 +323,18 @@ __device__ __forceinline__ void write_lse(const RunArgs& a, const TaskView& tv, 
 struct Tracer {
 #ifdef XY_ENABLE_TRACE
   unsigned long long* p;
-  int n;
-  __device__ __forceinline__ void init(const RunArgs& a, int role, bool on) {
-    p = (a.trace != nullptr && blockIdx.x == 0 && on) ? a.trace + role * kTraceLen : nullptr;
+  int n, len;
+  // two warps may share a role: each has its half of the records then
+  __device__ __forceinline__ void init(const RunArgs& a, int role, bool on, int half = -1) {
+    len = half < 0 ? kTraceLen : kTraceLen / 2;
+    p = (a.trace != nullptr && blockIdx.x == 0 && on) ? a.trace + role * kTraceLen + max(half, 0) * len : nullptr;
     n = 0;
   }
   __device__ __forceinline__ void operator()(unsigned tag) {
-    if (p != nullptr && n < kTraceLen) p[n++] = (static_cast<unsigned long long>(tag) << 48) | (clock64() & 0xFFFFFFFFFFFFull);
+    if (p != nullptr && n < len) p[n++] = (static_cast<unsigned long long>(tag) << 48) | (clock64() & 0xFFFFFFFFFFFFull);
   }
 #else
-  __device__ __forceinline__ void init(const RunArgs&, int, bool) {}
+  __device__ __forceinline__ void init(const RunArgs&, int, bool, int = -1) {}
   __device__ __forceinline__ void operator()(unsigned) {}
 #endif
 };
@@ -503,7 +505,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // the parity of its `full` phase that the latest one completes.
       uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0, armed = 0, fill_par = 0;
       Tracer tr;
-      tr.init(a, 3, op == 0 && lane == 0);
+      tr.init(a, 3, lane == 0, kTwoProducers ? op : -1);
       const int ppt = kKeyTile >> a.page_shift;  // pages per 128-key tile
       const int lane_page = kFp8 ? lane : lane >> 1;
       const bool has_box = lane_page < ppt;
