@@ -44,6 +44,11 @@ struct StreamCfg {
   static constexpr int kSmem = kRing + kXch + kQ + kMl + kScales + kTaskSlots * static_cast<int>(sizeof(TaskDesc)) + 16 * kStages + 32;
 };
 
+// Two CTAs have to fit the 228 KiB of an SM, each in units of 128 bytes with the 1 KiB that the system takes.
+template <bool kFp8>
+constexpr bool kTwoPerSm = 2 * ((StreamCfg<kFp8>::kSmem + 127) / 128 * 128 + 1024) <= 228 * 1024;
+static_assert(kTwoPerSm<false> && kTwoPerSm<true>, "the grid counts on two CTAs per SM");
+
 template <bool kFp8>
 __global__ void __launch_bounds__(kThreadsS, 2)
 stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant__ CUtensorMap k_map,
@@ -225,7 +230,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     // per stage: handed out, parity of its next `empty` wait, copied into, parity of the latest copy's `full` phase
     uint32_t k_fills = 0, used = 0, ph_empty = 0, armed = 0, fill_par = 0;
     auto fill = [&](const CUtensorMap* map, const Tile& x, bool is_k) {
-      const uint32_t bit = 1u << pos.stage;
+      const uint32_t bit = 1u << pos.stage, bar = full + 8 * pos.stage;
       if (used & bit) {
         // wait for the readers of this stage's previous fill
         if (!failed && !mbar_wait_block(empty + 8 * pos.stage, (ph_empty >> pos.stage) & 1u, a.status)) {
@@ -252,7 +257,6 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
           __syncwarp();
         }
       }
-      const uint32_t bar = full + 8 * pos.stage;
       if (lane == 0 && !failed) mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
       __syncwarp();
       if (has_box && !failed)

@@ -30,7 +30,7 @@ constexpr int kStatusUnitCounts = 32;
 constexpr int kStatusSticky = -8;
 constexpr int kStatusWaitLimit = -7;
 constexpr int kStatusLead = 8;  // words in front of `status`
-constexpr int kTraceRoles = 4;      // sub-tile A, sub-tile B, MMA issuer, producer (worker 0 only)
+constexpr int kTraceRoles = 4;      // sub-tile A, sub-tile B, MMA issuer, producers (worker 0 only)
 constexpr int kTraceLen = 2048;    // records per role and run
 
 // Per-request facts the kernels need (device-visible, 32 bytes).
@@ -46,13 +46,13 @@ struct ReqInfo {
 };
 
 // A streaming task with all that its CTA has to know of it, in one place.
-struct TaskDesc {
+struct alignas(16) TaskDesc {
   xy_attn_task t;
   ReqInfo rq;               // pad1: index of the unit that the last of its tasks to finish merges, or -1
   int32_t nsplit, part0;    // that unit's number of splits and its first partial row
   int32_t pad[2];
 };
-static_assert(sizeof(TaskDesc) == 80, "read as five 16-byte words");
+static_assert(sizeof(TaskDesc) == 80 && alignof(TaskDesc) == 16, "read as five 16-byte words");
 
 struct PlanResult {
   std::vector<ReqInfo> reqs;
