@@ -393,10 +393,10 @@ int xy_attn_debug_check_block_table(xy_attn_ctx* ctx, const int32_t* block_table
 /* Failure-path test hook for the bounded waits of the attention kernel (every wait on a barrier
  * or a turn counter gives up after a limit and records XY_ERR_DEVICE_TIMEOUT, Section 4.2.1's
  * pipelines being chains of such hand-offs).  wait_limit_polls > 0 replaces the limit (0 restores
- * the default of 2^22 polls); skip_fill >= 0 makes the producer of every worker leave out its
- * skip_fill-th K/V stage fill of the following runs (-1: none), so that the readers of that stage
- * never see it filled and their waits run out.  Nothing faults and nothing spins without bound:
- * the kernel returns, frees its tensor memory, and the status shows the timeout; O and LSE of
+ * the default of 2^22 polls); skip_fill >= 0 makes the producers of every worker leave out its
+ * skip_fill-th K/V stage fill of the following runs (-1: none; tile t's K counts as 2 t, its V as
+ * 2 t + 1), so that the readers of that stage never see it filled and their waits run out, while
+ * everything else goes on at its own pace.  Nothing faults and nothing spins without bound: the kernel returns, frees its tensor memory, and the status shows the timeout; O and LSE of
  * such a run are unspecified.  The next run on the context starts from a clean status word, unless the
  * CTA that cleans up has run into a timeout itself: then xy_attn_device_status cleans. */
 int xy_attn_debug_inject(xy_attn_ctx* ctx, int32_t wait_limit_polls, int32_t skip_fill);

@@ -490,14 +490,16 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // ================================ producers ======================================
       // With tensor memory warp 8 stages the K tiles (even stages of the ring) and warp 10 the V tiles (odd
       // stages), without it warp 8 both; warp 8 also takes the tasks and hands them to everyone.  Each lane
-      // issues the box of one page and half, side by side.  (One lane that did all of it, K and V, box after box, needed 1600 - 2400 cycles per fill of an
-      // empty ring, about what a streaming tile takes its SM, and its per-stage state cost the consumers 90 bytes
-      // of spills.  One lane / two warps: 2048-token chunk beside 48 decode requests 429 -> 394 us, serving mix of 96
-      // requests 4950 -> 4684, 4 prompts of 4096 tokens 1111 -> 1065, 32 verify trees 864 -> 830, two planned steps of
-      // a tiny batch 36.9 -> 33.6; a chunk of 512 tokens beside 40 decode requests on pages of 16 tokens 216 ->
-      // 120, of 32 tokens 141 -> 111.  The variants without tensor memory are bound by their consumers' instructions and
-      // slower with two: there warp 8 does both.  That mix on the bf16 variant, one lane / two warps / one warp, 215 /
-      // 226 / 195 us, over an fp8 cache 264 / 260 / 242, on pages of 16 tokens 458 / 265 / 272.)
+      // issues the box of one page and half, side by side.  (One lane that did all of it, K and V, box after box,
+      // needed 1600 - 2400 cycles per fill of an empty ring, about what a streaming tile takes its SM, and its
+      // per-stage state cost the consumers of the variant with tensor memory 90 bytes of spills, now none; the other
+      // two spill about 400 bytes either way.  One lane / two warps: 2048-token chunk beside 48 decode requests 435 ->
+      // 401 us, serving mix of 96 requests 5023 -> 4746, 4 prompts of 4096 tokens 1126 -> 1077, 32 verify trees 878 ->
+      // 854, two planned steps of a tiny batch 36.9 -> 34.0; a chunk of 512 tokens beside 40 decode requests on pages of
+      // 16 tokens 216 -> 120, of 32 tokens 141 -> 111.  The variants without tensor memory are bound by their
+      // consumers' instructions and slower with two: there warp 8 does both.  That mix on the bf16 variant, one
+      // lane / two warps / one warp, 215 / 226 / 195 us, over an fp8 cache 264 / 260 / 242, on pages of 16 tokens
+      // 458 / 265 / 272.)
       const int op = warp == kConsumerWarps ? 0 : 1;
       bool dead = false;  // the same in all lanes, as is everything that decides the warp's way
       // Of this producer's stages: whether the stage has been handed out, who read it last (bit set: the tcgen05
@@ -666,7 +668,9 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // operand is warp-uniform; one elected lane issues.  (Two issuing lanes, one per sub-tile, that
       // took turns through a polled shared-memory word: 3.65 k cycles per pair of 128 x 128 tiles,
       // this form 3.27 k; 4 prompts of 4096 tokens 1172 -> 1136 us, tree verification 916 -> 879 us
-      // at the power cap.)
+      // at the power cap.  Waits that end with a vote and leave the loop on a failure, instead of a flag that each
+      // group of MMAs asks: serving mix of 96 requests 4766 -> 4678 us, 4 prompts 1078 -> 1071; the same flag at
+      // the hand-overs too: tiny batch 33.2 -> 33.9; a predicate that changes on a failure: trees 860 -> 913.)
       const bool elected = elect_one();
       uint32_t pos = 0;  // ring position: stage = pos % kStages, parity = (pos / kStages) & 1
       uint32_t ph_q = 0, ph_p = 0;  // bit X: parity of sub-tile X's next wait

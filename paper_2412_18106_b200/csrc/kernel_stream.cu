@@ -12,7 +12,8 @@
 // Measured (device time of one call) against the meta-kernel, whose single CTA per SM drains between
 // tasks: 13 requests of 300 - 2500 keys, 32/8 heads 34.9 -> 23.8 us; 24 requests up to 3000 keys, 64/8
 // heads 47.5 -> 38.6 us; 64 requests up to 8192 keys, 28/4 heads 101.3 -> 100.0 us, over an fp8 cache 88.5 ->
-// 56.6 us.  (With the tables read before the dependency wait, below: 94.8, 0.9 of the copy bandwidth, and 54.7.)
+// 56.6 us.  (With the first task read and its first tiles asked for before the dependency wait 90.6, 0.97 of the copy
+// bandwidth by the bytes a batch cannot do without, and 52.6.)
 #include <cuda.h>
 #include <cuda_runtime.h>
 

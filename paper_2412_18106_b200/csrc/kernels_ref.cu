@@ -382,8 +382,10 @@ __global__ void __launch_bounds__(128) append_kv_kernel(const uint16_t* qkv, int
   const int64_t slot_off = page * page_stride + static_cast<int64_t>(j & (page_size - 1)) * token_stride;
   const uint16_t* src = qkv + static_cast<int64_t>(t) * qkv_token_stride + static_cast<int64_t>(Hq) * kHeadDim;
   const int chunks = 2 * Hkv * (kHeadDim / 8);  // 16-byte chunks of this token's K then V heads
-  // A thread's loads first (they do not wait for the page id), then its stores.
-  constexpr int kBatch = 2;  // (eight kv heads: two chunks per thread)
+  // A thread's loads first (they do not wait for the page id), then its stores.  Two at a time is all that eight kv
+  // heads have.  One after the other / so: 13 tokens, 8 heads 1.42 -> 1.25 us in a row of appends, 32 heads 2.66 ->
+  // 2.08, 4096 tokens 5.22 -> 5.22 and 22.0 -> 19.5; two steps of eight layers, 13 requests 331 -> 318.
+  constexpr int kBatch = 2;
   for (int c0 = threadIdx.x; c0 < chunks; c0 += kBatch * blockDim.x) {
     uint4 val[kBatch];
 #pragma unroll

@@ -312,8 +312,10 @@ int build_plan(const xy_attn_config& cfg, int num_workers, int64_t partial_row_c
   // one mixed queue?  In the mix a streaming tile takes its SM kStreamVisitUs and a task kStreamTaskUs
   // around it; the streaming kernel runs at the pace of HBM but has its SMs only as the dense tasks
   // leave them, so the dense part must be small.  Measured, one queue / two launches: decode on shared
-  // prefixes, 128 requests on 8192 + 0 .. 1024 tokens 99.4 / 93.2 us, 210 on 3840 + 0 .. 362 114 / 86; with
-  // the dense tasks 0.59 of the work 85.5 / 88.4; a 2048-token chunk beside 48 decode requests 373 / 491.
+  // prefixes, 210 requests on 3840 + 0 .. 362 tokens (the dense tasks are 0.26 of the work) 79.9 / 70.8 us, 210 on
+  // 8192 + 0 .. 362 (0.43) 102.3 / 97.8, 128 on 8192 + 0 .. 1024 (0.40) 89.9 / 90.0, 128 on 12288 + 0 .. 200 (0.63)
+  // 80.7 / 81.2; a 2048-token chunk beside 48 decode requests 383 / 418.  (The costs are those of a meta-kernel
+  // whose staging was one lane; the line still divides these.)
   bool two_launches = false;
   if (!paper && !pair && cfg.kernel == XY_KERNEL_AUTO && cfg.kv_dtype == XY_KV_BF16) {
     double dense = 0.0, tiles = 0.0, tasks = 0.0;
