@@ -495,11 +495,12 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // per-stage state cost the consumers of the variant with tensor memory 90 bytes of spills, now none; the other
       // two spill about 400 bytes either way.  One lane / two warps: 2048-token chunk beside 48 decode requests 435 ->
       // 401 us, serving mix of 96 requests 5023 -> 4746, 4 prompts of 4096 tokens 1126 -> 1077, 32 verify trees 878 ->
-      // 854, two planned steps of a tiny batch 36.9 -> 34.0; a chunk of 512 tokens beside 40 decode requests on pages of
-      // 16 tokens 216 -> 120, of 32 tokens 141 -> 111.  The variants without tensor memory are bound by their
-      // consumers' instructions and slower with two: there warp 8 does both.  That mix on the bf16 variant, one
-      // lane / two warps / one warp, 215 / 226 / 195 us, over an fp8 cache 264 / 260 / 242, on pages of 16 tokens
-      // 458 / 265 / 272.)
+      // 854, two planned steps of a tiny batch 36.9 -> 34.0; a chunk of 512 tokens on 2048 beside 40 decode
+      // requests of 1000 - 8000 on pages of 16 tokens 229 -> 115, of 32 tokens 157 -> 109.  The variants without tensor
+      // memory are bound by their consumers' instructions, and there the second warp is no gain for all: that mix on
+      // the bf16 variant, one lane / one warp / two, 273 / 258 / 255 us, on pages of 16 tokens 376 / 302 / 294, over an
+      // fp8 cache 345 / 291 / 283; but with requests of 200 - 2000 121 / 120 / 127 and 147 / 133 / 156.  One warp does
+      // both there, which nowhere measured is slower than one lane.)
       const int op = warp == kConsumerWarps ? 0 : 1;
       bool dead = false;  // the same in all lanes, as is everything that decides the warp's way
       // Of this producer's stages: whether the stage has been handed out, who read it last (bit set: the tcgen05
