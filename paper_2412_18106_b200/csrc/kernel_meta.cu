@@ -503,10 +503,11 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // both there, which nowhere measured is slower than one lane.)
       const int op = warp == kConsumerWarps ? 0 : 1;
       bool dead = false;  // the same in all lanes, as is everything that decides the warp's way
-      // Of this producer's stages: whether the stage has been handed out, who read it last (bit set: the tcgen05
-      // path), the parity to wait for on each of its two empty barriers; whether a copy has been issued into it, and
-      // the parity of its `full` phase that the latest one completes.
-      uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0, armed = 0, fill_par = 0;
+      // Of this producer's stages: who read the stage last (bit set: the tcgen05 path), the parity
+      // to wait for on each of its two empty barriers, and of its `full` phase that the latest fill completes;
+      // a stage that was never filled needs no wait.
+      uint32_t used = 0, last_umma = 0, ph_cons = 0, ph_umma = 0, fill_par = 0;
+      uint32_t left_out = 0;  // stage whose copy the test hook has left out: nobody hands it back any more
       Tracer tr;
       tr.init(a, 3, lane == 0, kTwoProducers ? op : -1);
       const int ppt = kKeyTile >> a.page_shift;  // pages per 128-key tile
@@ -612,14 +613,16 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
             dead = true;
             return;
           }
+          fill_par ^= bit;
         }
         used |= bit;
         last_umma = x.by_umma ? (last_umma | bit) : (last_umma & ~bit);
         // Failure-path test hook (xy_attn_debug_inject): this worker leaves out one copy, so that the stage's `full`
         // barrier does not complete and the readers' bounded waits run out.
-        if (2 * n + op == a.debug_skip_fill) return;
-        if (armed & bit) fill_par ^= bit;
-        armed |= bit;
+        if (2 * n + op == a.debug_skip_fill) {
+          left_out = bit;
+          return;
+        }
         tr(1 + op);
         if constexpr (kFp8) {
           // the K fill also leaves the K and V scales of the tile's pages in the tile's scale slot,
@@ -658,7 +661,7 @@ meta_attention_kernel(const __grid_constant__ MetaParams P, const __grid_constan
       // stage has landed once its `full` phase completes (immediate on the normal path, where the
       // readers have long consumed it; a bounded wait after a failure).
       for (int s = 0; s < kStages; ++s)
-        if (armed & (1u << s)) mbar_wait_block(smem_u32(&bars->full[s]), (fill_par >> s) & 1u, a.status);
+        if (used & ~left_out & (1u << s)) mbar_wait_block(smem_u32(&bars->full[s]), (fill_par >> s) & 1u, a.status);
     } else if (kUmma && warp == kConsumerWarps + 1) {
       // ================================ tcgen05 MMA issuer ==============================
       // One warp issues for both 128-row sub-tiles.  Each sub-tile is a chain

@@ -228,25 +228,24 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     };
     RingPos pos{0, 0};
     int n_fill = 0;
-    // per stage: handed out, parity of its next `empty` wait, copied into, parity of the latest copy's `full` phase
-    uint32_t k_fills = 0, used = 0, ph_empty = 0, armed = 0, fill_par = 0;
+    uint32_t k_fills = 0, used = 0, fill_par = 0;
+    uint32_t left_out = 0;  // stage whose copy the test hook has left out: nobody hands it back any more
     auto fill = [&](const CUtensorMap* map, const Tile& x, bool is_k) {
       const uint32_t bit = 1u << pos.stage, bar = full + 8 * pos.stage;
       if (used & bit) {
         // wait for the readers of this stage's previous fill
-        if (!failed && !mbar_wait_block(empty + 8 * pos.stage, (ph_empty >> pos.stage) & 1u, a.status)) {
+        if (!failed && !mbar_wait_block(empty + 8 * pos.stage, (fill_par >> pos.stage) & 1u, a.status)) {
           report_timeout(a, s_failed);
           failed = true;
         }
-        ph_empty ^= bit;
+        fill_par ^= bit;
       }
       used |= bit;
       if (n_fill++ == a.debug_skip_fill) {  // failure-path test hook: this copy is left out
+        left_out = bit;
         pos.advance<kStages>();
         return;
       }
-      if (armed & bit) fill_par ^= bit;
-      armed |= bit;
       if constexpr (kFp8) {
         if (is_k) {
           float* slot = scale_ring + (k_fills % kScaleSlots) * 16;
@@ -285,7 +284,7 @@ stream_attention_kernel(const __grid_constant__ RunArgs a, const __grid_constant
     // No copy of this CTA may still be in flight when it exits (immediate on the normal path).
     asm volatile("cp.async.wait_all;" ::: "memory");
     for (int s = 0; s < kStages; ++s)
-      if (armed & (1u << s)) mbar_wait_block(full + 8 * s, (fill_par >> s) & 1u, a.status);
+      if (used & ~left_out & (1u << s)) mbar_wait_block(full + 8 * s, (fill_par >> s) & 1u, a.status);
   } else {
     // ================================== consumers =========================================
     const float scale_log2 = a.sm_scale * 1.4426950408889634f;
